@@ -237,6 +237,11 @@ struct RowArgs {
     int limit = 0;                    // process tiles with tgen <= limit (ASM: all tiles)
     const int32_t *alist = nullptr;   // as LinEpi::alist (not used by ASM, which writes every
     const int32_t *acount = nullptr;  // row of its output)
+    int lim_a = INT32_MAX;            // UPD: qa / qb are zero (and not read) in tiles beyond these
+    int lim_b = INT32_MAX;            // hop distances; ASM, ASMSUB: block k beyond kbase + k
+    int tri_a = 0;                    // UPD: ca is lower triangular
+    int M = 0;                        // columns in use (set by launch_rowblock)
+    int tc = 0;                       // tensor-core kernels allowed (rowblock_tc.cu)
     int kbase = 0;                    // ASM: index of the first block (frontier reach)
     int accumulate = 0;               // ASM: y += product (the accumulator starts from y)
     const int32_t *skip = nullptr;    // the launch does nothing when *skip != 0 (device flag)
@@ -251,7 +256,7 @@ int rowblock_max_grid(int W);
 // (rowblock_tc.cu); launch_rowblock uses it where rowblock_tc_supported says so.  Gram
 // partials: grid <= max_grid rows of [W*W].
 bool rowblock_tc_supported(int mode, int W);
-bool rowblock_tc_enabled();   // KB_TENSOR_CORES=1 in the environment
+bool rowblock_tc_enabled();   // KB_TENSOR_CORES=1 in the environment (asked once per solve)
 int launch_rowblock_tc(int mode, const RowArgs<float> &a, cudaStream_t s, int max_grid, int *grid_out);
 int rowblock_tc_max_grid();
 

@@ -145,6 +145,7 @@ struct Common {
     int spmm = 0;
     Ctrl *hctrl = nullptr;   // host copy of the control block when the caller wants info
     bool frontier = true;    // restrict the per-step kernels to the reached rows
+    int tc = 0;              // tensor-core row-block kernels allowed (asked once per solve)
     const QuadRule *quad = nullptr;   // spline kernel with non-integer s (Lanczos methods)
 };
 
@@ -319,6 +320,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             // diagonal block: H_kk = Q_k^T L Q_k
             int grid = 0;
             RowArgs<T> pa;
+            pa.tc = c.tc;
             pa.n = n; pa.x = b.wbuf; pa.qa = Qk; pa.partials = b.parts; pa.ctrl = b.ctrl;
             pa.tgen = tg; pa.limit = k; pa.alist = tg ? b.alist : nullptr; pa.acount = b.acount;
             KB_TRY(launch_rowblock<T>(RB_PROJ, W, pa, c.s, &grid, M));
@@ -328,9 +330,11 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             // three-term update: X = L Q_k - Q_{k-1} H_{k-1,k} - Q_k H_kk, then Gram X^T X
             T *X = blk(k);
             RowArgs<T> ua;
+            ua.tc = c.tc;
             ua.n = n; ua.x = b.wbuf; ua.qa = Qp; ua.ca = Bp; ua.qb = Qk; ua.cb = Cb;
             ua.out = X; ua.partials = b.parts; ua.ctrl = b.ctrl;
             ua.tgen = tg; ua.limit = k; ua.alist = tg ? b.alist : nullptr; ua.acount = b.acount;
+            ua.lim_a = k - 2; ua.lim_b = k - 1; ua.tri_a = 1;   // (H_{k-1,k} is lower triangular)
             KB_TRY(launch_rowblock<T>(RB_UPD, W, ua, c.s, &grid, M));
             KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl));
             if (c.p.reorth == 2) {
@@ -342,15 +346,18 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                 for (int j = 0; j < 2; ++j) {
                     if (!loc[j]) continue;
                     RowArgs<T> ra;
+                    ra.tc = c.tc;
                     ra.n = n; ra.x = X; ra.qa = loc[j]; ra.partials = b.parts; ra.ctrl = b.ctrl;
                     ra.tgen = tg; ra.limit = k; ra.alist = tg ? b.alist : nullptr; ra.acount = b.acount;
                     KB_TRY(launch_rowblock<T>(RB_PROJ, W, ra, c.s, &grid, M));
                     KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl, Cl + j * WW));
                 }
                 RowArgs<T> la;
+                la.tc = c.tc;
                 la.n = n; la.x = X; la.qa = Qp; la.ca = Cl + WW; la.qb = Qk;
                 la.cb = Cl; la.out = X; la.partials = b.parts; la.ctrl = b.ctrl;
                 la.tgen = tg; la.limit = k; la.alist = tg ? b.alist : nullptr; la.acount = b.acount;
+                la.lim_a = k - 2; la.lim_b = k - 1;
                 KB_TRY(launch_rowblock<T>(RB_UPD, W, la, c.s, &grid, M));
                 KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl));
             }
@@ -365,6 +372,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                     const int32_t *skip = pass == 1 ? b.reo_skip : nullptr;
                     for (int j = 0; j < k; ++j) {
                         RowArgs<T> ra;
+                        ra.tc = c.tc;
                         ra.n = n; ra.x = X; ra.qa = b.basis + j * bs; ra.partials = b.parts;
                         ra.ctrl = b.ctrl; ra.skip = skip;
                         ra.tgen = tg; ra.limit = k; ra.alist = tg ? b.alist : nullptr; ra.acount = b.acount;
@@ -373,6 +381,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                                                 b.Cstk + size_t(j) * W * W, skip));
                     }
                     RowArgs<T> sa;
+                    sa.tc = c.tc;
                     sa.n = n; sa.x = X; sa.basis = b.basis; sa.block_stride = bs; sa.nblk = k;
                     sa.ca = b.Cstk; sa.out = X; sa.partials = b.parts; sa.ctrl = b.ctrl; sa.skip = skip;
                     sa.tgen = tg; sa.limit = k; sa.alist = tg ? b.alist : nullptr; sa.acount = b.acount;
@@ -385,6 +394,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             KB_TRY(launch_chol<C>(b.Gsum, M, W, 1, k, inv_thresh2, piv2, b.R1, S1, nullptr,
                                   nullptr, b.ctrl, c.s));
             RowArgs<T> ma;
+            ma.tc = c.tc;
             ma.n = n; ma.x = X; ma.ca = S1; ma.out = X; ma.partials = b.parts; ma.ctrl = b.ctrl;
             ma.tgen = tg; ma.limit = k; ma.alist = tg ? b.alist : nullptr; ma.acount = b.acount;
             KB_TRY(launch_rowblock<T>(RB_MULGRAM, W, ma, c.s, &grid, M));
@@ -392,6 +402,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             KB_TRY(launch_chol<C>(b.Gsum, M, W, 2, k, inv_thresh2, piv2, b.R1, S2,
                                   b.Hs + size_t(k - 1) * M * M, Bk, b.ctrl, c.s));
             RowArgs<T> qa;
+            qa.tc = c.tc;
             qa.n = n; qa.x = X; qa.ca = S2; qa.out = X; qa.ctrl = b.ctrl;
             qa.tgen = tg; qa.limit = k; qa.alist = tg ? b.alist : nullptr; qa.acount = b.acount;
             KB_TRY(launch_rowblock<T>(RB_MUL, W, qa, c.s, &grid, M));
@@ -432,6 +443,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
         // assembly: Y = [Q_1 .. Q_m] U
         if (!two) {
             RowArgs<T> aa;
+            aa.tc = c.tc;
             aa.n = n; aa.basis = b.basis; aa.block_stride = bs; aa.nblk = m; aa.ca = b.Ut;
             aa.y = Y; aa.ldy = ldy; aa.mo = M; aa.ctrl = b.ctrl; aa.tgen = tg;
             int grid = 0;
@@ -451,6 +463,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                 T *Qk = blk(k - 1);
                 T *Qp = k >= 2 ? blk(k - 2) : nullptr;
                 RowArgs<T> aa;
+                aa.tc = c.tc;
                 aa.n = n; aa.basis = Qk; aa.block_stride = bs; aa.nblk = 1;
                 aa.ca = b.Ut + (k - 1) * WW; aa.y = Y; aa.ldy = ldy; aa.mo = M; aa.tgen = tg;
                 aa.kbase = k - 1; aa.accumulate = k > 1 ? 1 : 0;
@@ -474,17 +487,21 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                 ++c.spmm;
                 T *X = blk(k);
                 RowArgs<T> ua;
+                ua.tc = c.tc;
                 ua.n = n; ua.x = b.wbuf; ua.qa = Qp; ua.ca = k >= 2 ? b.Bs + (k - 2) * WW : nullptr;
                 ua.qb = Qk; ua.cb = b.Cbs + (k - 1) * WW;
                 ua.out = X; ua.partials = b.parts; ua.ctrl = b.ctrl2; ua.tgen = tg; ua.limit = k; ua.alist = tg ? b.alist : nullptr; ua.acount = b.acount;
+                ua.lim_a = k - 2; ua.lim_b = k - 1; ua.tri_a = 1;
                 KB_TRY(launch_rowblock<T>(RB_UPD, W, ua, c.s, &grid, M));
                 if (c.p.reorth == 2) {
                     RowArgs<T> la = ua;
+                    la.tri_a = 0;
                     la.x = X; la.ca = b.Cloc + (2 * (k - 1) + 1) * WW; la.cb = b.Cloc + 2 * (k - 1) * WW;
                     KB_TRY(launch_rowblock<T>(RB_UPD, W, la, c.s, &grid, M));
                 }
                 for (int pass = 0; pass < 2; ++pass) {
                     RowArgs<T> qa;
+                    qa.tc = c.tc;
                     qa.n = n; qa.x = X; qa.ca = (pass == 0 ? b.Rs1 : b.Rs2) + (k - 1) * WW;
                     qa.out = X; qa.ctrl = b.ctrl2; qa.tgen = tg; qa.limit = k; qa.alist = tg ? b.alist : nullptr; qa.acount = b.acount;
                     KB_TRY(launch_rowblock<T>(RB_MUL, W, qa, c.s, &grid, M));
@@ -910,6 +927,7 @@ int apply_device(kb_graph *g, kb_method method, kb_phi phi, const kb_params *par
     // exact restriction of the per-step kernels to rows reached from W (hop distances are
     // kept in 8 bits)
     c.frontier = !params->no_frontier && m <= FRONTIER_MAX_HOPS;
+    c.tc = rowblock_tc_enabled() ? 1 : 0;
     const bool f64 = params->basis == KB_F64;
     const bool bf16 = params->basis == KB_BF16;
     const int chunk = f64 ? 64 : 128;

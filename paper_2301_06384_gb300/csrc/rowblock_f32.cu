@@ -1,0 +1,10 @@
+// Instances of the tall-skinny block kernels (rowblock.cuh), one translation unit per stored
+// type so that they compile in parallel.
+#include "rowblock.cuh"
+
+namespace kb {
+namespace rb {
+template int launch_w<float, 16>(int, const RowArgs<float> &, cudaStream_t, int *);
+template int launch_w<float, 32>(int, const RowArgs<float> &, cudaStream_t, int *);
+}  // namespace rb
+}  // namespace kb
