@@ -116,9 +116,13 @@ bool prof_on();
 
 // ------------------------------------------------------------------ frontier restriction
 // Krylov blocks started from E_W are exactly zero outside the (k-1)-hop ball of W at step
-// k.  gen[i] (uint8) is the hop distance of row i from W (255 = not reached yet); tgen[t]
-// is the minimum over the 32-row activity tile t.  Kernels given tgen skip tiles whose
-// minimum exceeds their limit.
+// k.  gen[i] (uint8) is the hop distance of row i from W (255 = beyond the last hop wanted);
+// tgen[t] is the minimum over the 32-row tile t (0x7f7f7f7f likewise).  Both are known before
+// the first step: alist holds all tiles by rising tgen (equal ones in index order) and
+// acount[k] the number of tiles with tgen <= k, so the tiles active at step k are a prefix.
+// A block that is zero beyond hop b is written on the tiles with tgen <= b only and kept zero
+// on those of the two hops beyond, which the next product's gathers reach; nothing else of
+// it is ever initialised or read.
 constexpr int ACT_ROWS = 32;
 constexpr int FRONTIER_MAX_HOPS = 250;
 __device__ __forceinline__ int tile_min_gen(const int32_t *tgen, int64_t r0, int rows) {
@@ -184,14 +188,12 @@ struct LinEpi {
                                       // the arithmetic is FP32, doubles for FP64)
     const Ctrl *ctrl = nullptr;
     const int32_t *tgen = nullptr;    // frontier tiles (nullptr: all rows)
-    const uint8_t *gen = nullptr;     // hop distance per row (with tgen): a warp whose rows
-                                      // all lie beyond the limit skips them
+    const uint8_t *gen = nullptr;     // hop distance per row (with tgen): rows beyond the limit
+                                      // are written as zeros, without their gathers
     int limit = 0;                    // process tiles with tgen <= limit
-    int zero_inactive = 0;            // write zeros for skipped tiles (final output)
-    const int32_t *alist = nullptr;   // with tgen: the 32-row frontier tiles with tgen <= limit in
-    const int32_t *acount = nullptr;  // increasing order and their number (device); the kernel
-                                      // then visits only the row tiles they cover (ignored when
-                                      // zero_inactive is set: every tile is written then)
+    int zero_inactive = 0;            // write zeros on the tiles beyond the limit (final output)
+    const int32_t *alist = nullptr;   // with tgen: the tiles by rising hop distance and the number
+    const int32_t *acount = nullptr;  // of them within the limit (device)
     ProfCount prof;
 };
 
@@ -235,8 +237,8 @@ struct RowArgs {
     const Ctrl *ctrl = nullptr;
     const int32_t *tgen = nullptr;    // frontier tiles (nullptr: all rows)
     int limit = 0;                    // process tiles with tgen <= limit (ASM: all tiles)
-    const int32_t *alist = nullptr;   // as LinEpi::alist (not used by ASM, which writes every
-    const int32_t *acount = nullptr;  // row of its output)
+    const int32_t *alist = nullptr;   // the frontier tiles by rising hop distance and the number
+    const int32_t *acount = nullptr;  // of them within the limit (ASM walks all of them)
     int lim_a = INT32_MAX;            // UPD: qa / qb are zero (and not read) in tiles beyond these
     int lim_b = INT32_MAX;            // hop distances; ASM, ASMSUB: block k beyond kbase + k
     int tri_a = 0;                    // UPD: ca is lower triangular

@@ -70,7 +70,8 @@ template <typename T>
 int launch_scatter(T *block, int64_t ld, const int32_t *nodes, int M, int col0, T val, cudaStream_t s);
 int launch_marker(int32_t *marker, const int32_t *nodes, int M, cudaStream_t s);
 template <typename T>
-int launch_scale_copy(T *out, const T *in, int64_t count, double scale, cudaStream_t s);
+int launch_scale_copy(T *out, const T *in, int64_t n, int W, double scale, const int32_t *alist,
+                      const int32_t *acount, cudaStream_t s);   // the listed tiles, or all rows
 int launch_fill_nan(float *Y, int64_t n, int64_t ldy, int mo, const Ctrl *ctrl, cudaStream_t s);
 
 template <typename T>
@@ -107,20 +108,30 @@ int axpy_max_grid();
 template <typename T>
 int launch_assemble_diag(int W, const T *basis, int64_t stride, int nblk, const double *omega,
                          int64_t n, float *Y, int64_t ldy, int mo, int64_t M_alg,
-                         const int32_t *tgen, cudaStream_t s, int kbase = 0, int accumulate = 0);
+                         const int32_t *tgen, const Ctrl *ctrl, cudaStream_t s, int kbase = 0,
+                         int accumulate = 0);
 
-// Frontier restriction: hop distances from the node set (uint8, 255 = not reached) and
-// per-32-row tile minima; expand(k) marks the rows at distance k.
-int launch_frontier_init(uint8_t *gen, int32_t *tgen, int64_t n, const int32_t *nodes, int M,
-                         cudaStream_t s);
-// alist / acount (optional): the active-tile list of step k - 1 (launch_frontier_list with
-// limit k - 1), which holds every row at distance k - 1; only those tiles are visited.
-int launch_frontier_expand(const GraphDev &g, uint8_t *gen, int32_t *tgen, int k, cudaStream_t s,
-                           const int32_t *alist = nullptr, const int32_t *acount = nullptr);
-// Compacts the 32-row frontier tiles with tgen <= limit into list (increasing tile order,
-// capacity ceil(n / 32)) and their number into *count; one CTA, deterministic.
-int launch_frontier_list(const int32_t *tgen, int64_t n, int limit, int32_t *list, int32_t *count,
-                         cudaStream_t s);
+// Frontier restriction (frontier.cu).  The arrays of one solve; see kb_internal.cuh for the
+// meaning of gen, tgen, alist and acount.
+struct FrontierBufs {
+    uint8_t *gen = nullptr;
+    int32_t *tgen = nullptr, *alist = nullptr, *acount = nullptr;
+    unsigned char *zeroed = nullptr;   // qlev, tcnt (the barrier behind it) and vis: cleared first
+    size_t zero_bytes = 0;
+    int32_t *qlev = nullptr, *tcnt = nullptr, *queue = nullptr;
+    int32_t *sync = nullptr;           // barrier count, error flag
+    uint32_t *vis = nullptr;
+    int levels = 0;
+    // number of tiles within k hops (device)
+    const int32_t *count(int k) const { return acount + (k < levels ? k : levels); }
+};
+// Lays the arrays out from base (nullptr: sizes only); *bytes receives their size.
+void plan_frontier(FrontierBufs &f, int64_t n, unsigned char *base, size_t *bytes);
+// Hop distances up to `levels` from the nodes, and the tile list.
+int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, int levels, cudaStream_t s);
+// Zeros on the tiles within f.levels hops: see k_zero_tiles.
+int launch_zero_tiles(void *blocks, int64_t block_bytes, int nblk, int row_bytes, int64_t n, bool ring,
+                      const FrontierBufs &f, cudaStream_t s);
 template <typename T>
 int launch_u_convert(const double *U, int M, int W, int m, T *Ut, const Ctrl *ctrl, cudaStream_t s);
 

@@ -120,6 +120,11 @@ struct Arena {
         off += bytes;
         return p;
     }
+    void frontier(FrontierBufs &f, int64_t n) {
+        size_t bytes = 0;
+        plan_frontier(f, n, base ? reinterpret_cast<unsigned char *>(base + off) : nullptr, &bytes);
+        off += bytes;
+    }
 };
 
 void ensure_pool(int dev) {
@@ -206,9 +211,7 @@ struct CblBufs {
     double *reo_d0;      // full reorthogonalisation: squared column norms before the first pass
     int32_t *reo_skip;   // ... and the flag that skips the second pass
     Ctrl *ctrl, *ctrl2, *ctrl_chk;
-    uint8_t *gen;
-    int32_t *tgen;
-    int32_t *alist, *acount;   // active 32-row tiles of the current step (frontier)
+    FrontierBufs fr;
 };
 
 template <typename T>
@@ -242,10 +245,7 @@ void plan_cbl(Arena &ar, CblBufs<T> &b, int64_t n, int M, int W, int m, int rb_g
     b.ctrl = ar.take<Ctrl>(1);
     b.ctrl2 = ar.take<Ctrl>(1);
     b.ctrl_chk = ar.take<Ctrl>(1);
-    b.gen = ar.take<uint8_t>(size_t(n));
-    b.tgen = ar.take<int32_t>(size_t((n + ACT_ROWS - 1) / ACT_ROWS));
-    b.alist = ar.take<int32_t>(size_t((n + ACT_ROWS - 1) / ACT_ROWS));
-    b.acount = ar.take<int32_t>(1);
+    ar.frontier(b.fr, n);
 }
 
 template <typename T>
@@ -271,23 +271,35 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
         const double inv_thresh2 = (tau_inv * lam) * (tau_inv * lam) * M;
         const double piv2 = tau_piv * tau_piv;
         KB_TRY(launch_ctrl_init(b.ctrl, m, c.s));
-        // with the frontier restriction only reached tiles are written, so every block
-        // starts from zeros; otherwise each block is written in full
+        // with the frontier restriction a block is written on the tiles it reaches and zero on
+        // those just beyond; otherwise each block is written in full
         const int nbuf = two ? 3 : m;
-        KB_CUDA_TRY(cudaMemsetAsync(b.basis, 0, sizeof(T) * size_t(n) * W * (c.frontier ? nbuf : 1), c.s));
-        KB_TRY(launch_scatter<T>(b.basis, W, nodes, M, 0, T(1), c.s));
+        const int64_t bs = n * W;
+        auto start_blocks = [&]() -> int {
+            if (!c.frontier) {
+                KB_CUDA_TRY(cudaMemsetAsync(b.basis, 0, sizeof(T) * size_t(bs), c.s));
+            } else if (c.tc) {
+                // (the tensor-core kernels walk 128-row tiles, whose rows beyond the reach they read)
+                KB_CUDA_TRY(cudaMemsetAsync(b.basis, 0, sizeof(T) * size_t(bs) * nbuf, c.s));
+                KB_CUDA_TRY(cudaMemsetAsync(b.wbuf, 0, sizeof(T) * size_t(bs), c.s));
+            } else {
+                KB_TRY(launch_zero_tiles(b.basis, bs * sizeof(T), nbuf, W * int(sizeof(T)), n, !two, b.fr, c.s));
+            }
+            return launch_scatter<T>(b.basis, W, nodes, M, 0, T(1), c.s);
+        };
+        if (c.frontier) KB_TRY(launch_frontier(c.g->dev, b.fr, nodes, M, m + 1, c.s));
+        KB_TRY(start_blocks());
         // slots of steps after a stop are never written: keep them zero
         KB_CUDA_TRY(cudaMemsetAsync(b.Cbs, 0, sizeof(C) * size_t(m) * W * W * 6, c.s));
-        const int32_t *tg = c.frontier ? b.tgen : nullptr;
-        if (c.frontier) {
-            KB_TRY(launch_frontier_init(b.gen, b.tgen, n, nodes, M, c.s));
-            KB_TRY(launch_frontier_list(b.tgen, n, 0, b.alist, b.acount, c.s));
-            // the SpMM and the row-block kernels tile rows differently; rows of L Q_k that
-            // the SpMM skips must read as zero in the row-block kernels (the reached set
-            // only grows, so zeroing once suffices)
-            KB_CUDA_TRY(cudaMemsetAsync(b.wbuf, 0, sizeof(T) * size_t(n) * W, c.s));
-        }
-        const int64_t bs = n * W;
+        // the frontier arguments of a row-block launch over the tiles within k hops
+        const int32_t *tg = c.frontier ? b.fr.tgen : nullptr;
+        auto within = [&](RowArgs<T> &ra, int k) {
+            ra.tc = c.tc;
+            ra.tgen = tg;
+            ra.limit = k;
+            ra.alist = tg ? b.fr.alist : nullptr;
+            ra.acount = tg ? b.fr.count(k) : nullptr;
+        };
         const size_t WW = size_t(W) * W;
         auto blk = [&](int j) { return b.basis + int64_t(two ? j % 3 : j) * bs; };
         int nchk = 0;
@@ -301,28 +313,23 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             C *S1 = b.Rs1 + (k - 1) * WW, *S2 = b.Rs2 + (k - 1) * WW;
             C *Cl = b.Cloc + 2 * (k - 1) * WW;
             // Q_k is supported on rows within k-1 hops of W; L Q_k within k hops
-            if (c.frontier) {
-                KB_TRY(launch_frontier_expand(c.g->dev, b.gen, b.tgen, k, c.s, b.alist, b.acount));
-                KB_TRY(launch_frontier_list(b.tgen, n, k, b.alist, b.acount, c.s));
-            }
             // block SpMM: W = L Q_k
             LinEpi<T> e;
             e.s1 = 1.0;
             e.out = b.wbuf;
             e.ctrl = b.ctrl;
             e.tgen = tg;
-            e.gen = tg ? b.gen : nullptr;
+            e.gen = tg ? b.fr.gen : nullptr;
             e.limit = k;
-            e.alist = tg ? b.alist : nullptr;
-            e.acount = b.acount;
+            e.alist = tg ? b.fr.alist : nullptr;
+            e.acount = tg ? b.fr.count(k) : nullptr;
             KB_TRY(launch_spmm<T>(c.g->dev, W, Qk, e, c.s, nullptr, M, 0));
             ++c.spmm;
             // diagonal block: H_kk = Q_k^T L Q_k
             int grid = 0;
             RowArgs<T> pa;
-            pa.tc = c.tc;
             pa.n = n; pa.x = b.wbuf; pa.qa = Qk; pa.partials = b.parts; pa.ctrl = b.ctrl;
-            pa.tgen = tg; pa.limit = k; pa.alist = tg ? b.alist : nullptr; pa.acount = b.acount;
+            within(pa, k - 1);   // (Q_k is zero elsewhere)
             KB_TRY(launch_rowblock<T>(RB_PROJ, W, pa, c.s, &grid, M));
             KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl));
             KB_TRY(launch_hkk<C>(b.Gsum, M, W, b.Hd + size_t(k - 1) * M * M, Cb, b.ctrl, c.s));
@@ -330,10 +337,9 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             // three-term update: X = L Q_k - Q_{k-1} H_{k-1,k} - Q_k H_kk, then Gram X^T X
             T *X = blk(k);
             RowArgs<T> ua;
-            ua.tc = c.tc;
             ua.n = n; ua.x = b.wbuf; ua.qa = Qp; ua.ca = Bp; ua.qb = Qk; ua.cb = Cb;
             ua.out = X; ua.partials = b.parts; ua.ctrl = b.ctrl;
-            ua.tgen = tg; ua.limit = k; ua.alist = tg ? b.alist : nullptr; ua.acount = b.acount;
+            within(ua, k);
             ua.lim_a = k - 2; ua.lim_b = k - 1; ua.tri_a = 1;   // (H_{k-1,k} is lower triangular)
             KB_TRY(launch_rowblock<T>(RB_UPD, W, ua, c.s, &grid, M));
             KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl));
@@ -346,17 +352,15 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                 for (int j = 0; j < 2; ++j) {
                     if (!loc[j]) continue;
                     RowArgs<T> ra;
-                    ra.tc = c.tc;
                     ra.n = n; ra.x = X; ra.qa = loc[j]; ra.partials = b.parts; ra.ctrl = b.ctrl;
-                    ra.tgen = tg; ra.limit = k; ra.alist = tg ? b.alist : nullptr; ra.acount = b.acount;
+                    within(ra, k - 1 - j);
                     KB_TRY(launch_rowblock<T>(RB_PROJ, W, ra, c.s, &grid, M));
                     KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl, Cl + j * WW));
                 }
                 RowArgs<T> la;
-                la.tc = c.tc;
                 la.n = n; la.x = X; la.qa = Qp; la.ca = Cl + WW; la.qb = Qk;
                 la.cb = Cl; la.out = X; la.partials = b.parts; la.ctrl = b.ctrl;
-                la.tgen = tg; la.limit = k; la.alist = tg ? b.alist : nullptr; la.acount = b.acount;
+                within(la, k);
                 la.lim_a = k - 2; la.lim_b = k - 1;
                 KB_TRY(launch_rowblock<T>(RB_UPD, W, la, c.s, &grid, M));
                 KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl));
@@ -372,19 +376,17 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                     const int32_t *skip = pass == 1 ? b.reo_skip : nullptr;
                     for (int j = 0; j < k; ++j) {
                         RowArgs<T> ra;
-                        ra.tc = c.tc;
                         ra.n = n; ra.x = X; ra.qa = b.basis + j * bs; ra.partials = b.parts;
                         ra.ctrl = b.ctrl; ra.skip = skip;
-                        ra.tgen = tg; ra.limit = k; ra.alist = tg ? b.alist : nullptr; ra.acount = b.acount;
+                        within(ra, j);
                         KB_TRY(launch_rowblock<T>(RB_PROJ, W, ra, c.s, &grid, M));
                         KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl,
                                                 b.Cstk + size_t(j) * W * W, skip));
                     }
                     RowArgs<T> sa;
-                    sa.tc = c.tc;
                     sa.n = n; sa.x = X; sa.basis = b.basis; sa.block_stride = bs; sa.nblk = k;
                     sa.ca = b.Cstk; sa.out = X; sa.partials = b.parts; sa.ctrl = b.ctrl; sa.skip = skip;
-                    sa.tgen = tg; sa.limit = k; sa.alist = tg ? b.alist : nullptr; sa.acount = b.acount;
+                    within(sa, k);
                     KB_TRY(launch_rowblock<T>(RB_ASMSUB, W, sa, c.s, &grid, M));
                     KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl, nullptr, skip));
                     if (pass == 0) KB_TRY(launch_reorth_decide(b.Gsum, b.reo_d0, M, W, b.reo_skip, c.s));
@@ -394,17 +396,15 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             KB_TRY(launch_chol<C>(b.Gsum, M, W, 1, k, inv_thresh2, piv2, b.R1, S1, nullptr,
                                   nullptr, b.ctrl, c.s));
             RowArgs<T> ma;
-            ma.tc = c.tc;
             ma.n = n; ma.x = X; ma.ca = S1; ma.out = X; ma.partials = b.parts; ma.ctrl = b.ctrl;
-            ma.tgen = tg; ma.limit = k; ma.alist = tg ? b.alist : nullptr; ma.acount = b.acount;
+            within(ma, k);
             KB_TRY(launch_rowblock<T>(RB_MULGRAM, W, ma, c.s, &grid, M));
             KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl));
             KB_TRY(launch_chol<C>(b.Gsum, M, W, 2, k, inv_thresh2, piv2, b.R1, S2,
                                   b.Hs + size_t(k - 1) * M * M, Bk, b.ctrl, c.s));
             RowArgs<T> qa;
-            qa.tc = c.tc;
             qa.n = n; qa.x = X; qa.ca = S2; qa.out = X; qa.ctrl = b.ctrl;
-            qa.tgen = tg; qa.limit = k; qa.alist = tg ? b.alist : nullptr; qa.acount = b.acount;
+            within(qa, k);
             KB_TRY(launch_rowblock<T>(RB_MUL, W, qa, c.s, &grid, M));
             // stopping rule: U_k at the check steps, compared with the previous check's
             if (c.p.tol > 0.0 && k < m && (k == 8 || k == 12 || k == 16 || k == 24 || k == 32 ||
@@ -443,54 +443,43 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
         // assembly: Y = [Q_1 .. Q_m] U
         if (!two) {
             RowArgs<T> aa;
-            aa.tc = c.tc;
             aa.n = n; aa.basis = b.basis; aa.block_stride = bs; aa.nblk = m; aa.ca = b.Ut;
-            aa.y = Y; aa.ldy = ldy; aa.mo = M; aa.ctrl = b.ctrl; aa.tgen = tg;
+            aa.y = Y; aa.ldy = ldy; aa.mo = M; aa.ctrl = b.ctrl;
+            within(aa, m);   // (all tiles are written; the list only orders them)
             int grid = 0;
             KB_TRY(launch_rowblock<T>(RB_ASM, W, aa, c.s, &grid, M));
         } else {
             // second pass: the same products and updates with the recorded matrices
             // (bit-identical blocks); Y += Q_k U_k as each block is recomputed
             KB_TRY(launch_ctrl_init(b.ctrl2, m, c.s));
-            KB_CUDA_TRY(cudaMemsetAsync(b.basis, 0, sizeof(T) * size_t(n) * W * (c.frontier ? 3 : 1), c.s));
-            KB_TRY(launch_scatter<T>(b.basis, W, nodes, M, 0, T(1), c.s));
-            if (c.frontier) {
-                KB_TRY(launch_frontier_init(b.gen, b.tgen, n, nodes, M, c.s));
-                KB_TRY(launch_frontier_list(b.tgen, n, 0, b.alist, b.acount, c.s));
-                KB_CUDA_TRY(cudaMemsetAsync(b.wbuf, 0, sizeof(T) * size_t(n) * W, c.s));
-            }
+            KB_TRY(start_blocks());
             for (int k = 1; k <= m; ++k) {
                 T *Qk = blk(k - 1);
                 T *Qp = k >= 2 ? blk(k - 2) : nullptr;
                 RowArgs<T> aa;
-                aa.tc = c.tc;
                 aa.n = n; aa.basis = Qk; aa.block_stride = bs; aa.nblk = 1;
-                aa.ca = b.Ut + (k - 1) * WW; aa.y = Y; aa.ldy = ldy; aa.mo = M; aa.tgen = tg;
+                aa.ca = b.Ut + (k - 1) * WW; aa.y = Y; aa.ldy = ldy; aa.mo = M;
+                within(aa, k - 1);   // (the first launch writes all of Y)
                 aa.kbase = k - 1; aa.accumulate = k > 1 ? 1 : 0;
                 int grid = 0;
                 KB_TRY(launch_rowblock<T>(RB_ASM, W, aa, c.s, &grid, M));
                 if (k == m) break;
-                if (c.frontier) {
-                    KB_TRY(launch_frontier_expand(c.g->dev, b.gen, b.tgen, k, c.s, b.alist, b.acount));
-                    KB_TRY(launch_frontier_list(b.tgen, n, k, b.alist, b.acount, c.s));
-                }
                 LinEpi<T> e;
                 e.s1 = 1.0;
                 e.out = b.wbuf;
                 e.ctrl = b.ctrl2;
                 e.tgen = tg;
-                e.gen = tg ? b.gen : nullptr;
+                e.gen = tg ? b.fr.gen : nullptr;
                 e.limit = k;
-                e.alist = tg ? b.alist : nullptr;
-                e.acount = b.acount;
+                e.alist = tg ? b.fr.alist : nullptr;
+                e.acount = tg ? b.fr.count(k) : nullptr;
                 KB_TRY(launch_spmm<T>(c.g->dev, W, Qk, e, c.s, nullptr, M, 0));
                 ++c.spmm;
                 T *X = blk(k);
                 RowArgs<T> ua;
-                ua.tc = c.tc;
                 ua.n = n; ua.x = b.wbuf; ua.qa = Qp; ua.ca = k >= 2 ? b.Bs + (k - 2) * WW : nullptr;
                 ua.qb = Qk; ua.cb = b.Cbs + (k - 1) * WW;
-                ua.out = X; ua.partials = b.parts; ua.ctrl = b.ctrl2; ua.tgen = tg; ua.limit = k; ua.alist = tg ? b.alist : nullptr; ua.acount = b.acount;
+                ua.out = X; ua.partials = b.parts; ua.ctrl = b.ctrl2; within(ua, k);
                 ua.lim_a = k - 2; ua.lim_b = k - 1; ua.tri_a = 1;
                 KB_TRY(launch_rowblock<T>(RB_UPD, W, ua, c.s, &grid, M));
                 if (c.p.reorth == 2) {
@@ -501,9 +490,8 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                 }
                 for (int pass = 0; pass < 2; ++pass) {
                     RowArgs<T> qa;
-                    qa.tc = c.tc;
                     qa.n = n; qa.x = X; qa.ca = (pass == 0 ? b.Rs1 : b.Rs2) + (k - 1) * WW;
-                    qa.out = X; qa.ctrl = b.ctrl2; qa.tgen = tg; qa.limit = k; qa.alist = tg ? b.alist : nullptr; qa.acount = b.acount;
+                    qa.out = X; qa.ctrl = b.ctrl2; within(qa, k);
                     KB_TRY(launch_rowblock<T>(RB_MUL, W, qa, c.s, &grid, M));
                 }
             }
@@ -529,9 +517,7 @@ struct LzBufs {
     int32_t *alive;
     double *c1, *c2, *aupd, *omega;   // c1, c2, aupd: one row of W per step
     Ctrl *ctrl, *ctrl2;
-    uint8_t *gen;
-    int32_t *tgen;
-    int32_t *alist, *acount;   // active 32-row tiles of the current step (frontier)
+    FrontierBufs fr;
 };
 
 template <typename T>
@@ -551,10 +537,7 @@ void plan_lz(Arena &ar, LzBufs<T> &b, int64_t n, int W, int m, int pgrid, bool t
     b.omega = ar.take<double>(size_t(m) * W);
     b.ctrl = ar.take<Ctrl>(1);
     b.ctrl2 = ar.take<Ctrl>(1);
-    b.gen = ar.take<uint8_t>(size_t(n));
-    b.tgen = ar.take<int32_t>(size_t((n + ACT_ROWS - 1) / ACT_ROWS));
-    b.alist = ar.take<int32_t>(size_t((n + ACT_ROWS - 1) / ACT_ROWS));
-    b.acount = ar.take<int32_t>(1);
+    ar.frontier(b.fr, n);
 }
 
 template <typename T>
@@ -591,13 +574,15 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
         const double thresh = (f64 ? 1e-12 : 1e-6) * c.g->lambda;
         KB_TRY(launch_ctrl_init(b.ctrl, m, c.s));
         const int nbuf = two ? 3 : m + 1;
-        KB_CUDA_TRY(cudaMemsetAsync(b.basis, 0, sizeof(T) * size_t(n) * W * (c.frontier ? nbuf : 1), c.s));
-        KB_TRY(launch_scatter<T>(b.basis, W, nodes, M, 0, T(1), c.s));
-        const int32_t *tg = c.frontier ? b.tgen : nullptr;
-        if (c.frontier) {
-            KB_TRY(launch_frontier_init(b.gen, b.tgen, n, nodes, M, c.s));
-            KB_TRY(launch_frontier_list(b.tgen, n, 0, b.alist, b.acount, c.s));
-        }
+        const int64_t bs = n * W;
+        const int32_t *tg = c.frontier ? b.fr.tgen : nullptr;
+        auto start_blocks = [&]() -> int {
+            if (!c.frontier) KB_CUDA_TRY(cudaMemsetAsync(b.basis, 0, sizeof(T) * size_t(bs), c.s));
+            else KB_TRY(launch_zero_tiles(b.basis, bs * sizeof(T), nbuf, W * int(sizeof(T)), n, !two, b.fr, c.s));
+            return launch_scatter<T>(b.basis, W, nodes, M, 0, T(1), c.s);
+        };
+        if (c.frontier) KB_TRY(launch_frontier(c.g->dev, b.fr, nodes, M, m + 1, c.s));
+        KB_TRY(start_blocks());
         // coefficients of steps after an invariant stop are never written: keep them zero
         KB_CUDA_TRY(cudaMemsetAsync(b.c1, 0, sizeof(double) * size_t(m + 1) * W, c.s));
         KB_CUDA_TRY(cudaMemsetAsync(b.c2, 0, sizeof(double) * size_t(m + 1) * W, c.s));
@@ -606,23 +591,18 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
         KB_CUDA_TRY(cudaMemsetAsync(b.alpha, 0, sizeof(double) * size_t(m + 1) * W, c.s));
         KB_CUDA_TRY(cudaMemsetAsync(b.sigma, 0, sizeof(double) * size_t(m + 1) * W, c.s));
         KB_TRY(launch_lanczos_init(W, M, gbl ? 1 : 0, f64 ? 0 : 1, b.sigma, b.alive, b.c1, b.c2, c.s));
-        const int64_t bs = n * W;
         auto blk = [&](int j) { return b.basis + int64_t(two ? j % 3 : j) * bs; };
         for (int k = 1; k <= m; ++k) {
             T *Pk = blk(k - 1);
             T *Pp = k >= 2 ? blk(k - 2) : nullptr;
             T *X = blk(k);
-            if (c.frontier) {
-                KB_TRY(launch_frontier_expand(c.g->dev, b.gen, b.tgen, k, c.s, b.alist, b.acount));
-                KB_TRY(launch_frontier_list(b.tgen, n, k, b.alist, b.acount, c.s));
-            }
             // X = L Q_k - h_{k,k-1} Q_{k-1}, with Q_k = sigma_k P_k; dots <P_k, X> per column
             LinEpi<T> e;
             e.tgen = tg;
-            e.gen = tg ? b.gen : nullptr;
+            e.gen = tg ? b.fr.gen : nullptr;
             e.limit = k;
-            e.alist = tg ? b.alist : nullptr;
-            e.acount = b.acount;
+            e.alist = tg ? b.fr.alist : nullptr;
+            e.acount = tg ? b.fr.count(k) : nullptr;
             e.a1 = b.c1 + int64_t(k - 1) * W;
             e.a2 = b.c2 + int64_t(k - 1) * W;
             e.s0 = 0.0;
@@ -638,7 +618,7 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
             if (k == m) break;
             int grid2 = 0;
             KB_TRY(launch_axpy_colnorm<T>(W, X, Pk, b.aupd + int64_t(k - 1) * W, n, b.parts, &grid2,
-                                          b.ctrl, tg, k, M, c.s, tg ? b.alist : nullptr, b.acount));
+                                          b.ctrl, tg, k, M, c.s, tg ? b.fr.alist : nullptr, tg ? b.fr.count(k) : nullptr));
             KB_TRY(launch_lanczos_beta(b.parts, grid2, W, M, gbl ? 1 : 0, k - 1, f64 ? 0 : 1, thresh, b.beta,
                                        b.sigma, b.alive, b.c1 + int64_t(k) * W, b.c2 + int64_t(k) * W,
                                        b.ctrl, c.s));
@@ -647,32 +627,23 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
                                   c.p.eps, c.s_int, c.g->lambda_proj, *tc, b.omega, b.work, b.qwork, b.ctrl,
                                   projected_bound(c), c.s, c.phi == KB_PHI_EXP ? &series : nullptr));
         if (!two) {
-            KB_TRY(launch_assemble_diag<T>(W, b.basis, bs, m, b.omega, n, Y, ldy, M, M, tg, c.s));
+            KB_TRY(launch_assemble_diag<T>(W, b.basis, bs, m, b.omega, n, Y, ldy, M, M, tg, b.ctrl, c.s));
         } else {
             // second pass: the same products and updates with the recorded coefficients
             // (bit-identical blocks), each block added to Y as soon as it exists
             KB_TRY(launch_ctrl_init(b.ctrl2, m, c.s));
-            KB_CUDA_TRY(cudaMemsetAsync(b.basis, 0, sizeof(T) * size_t(n) * W * (c.frontier ? 3 : 1), c.s));
-            KB_TRY(launch_scatter<T>(b.basis, W, nodes, M, 0, T(1), c.s));
-            if (c.frontier) {
-                KB_TRY(launch_frontier_init(b.gen, b.tgen, n, nodes, M, c.s));
-                KB_TRY(launch_frontier_list(b.tgen, n, 0, b.alist, b.acount, c.s));
-            }
-            KB_TRY(launch_assemble_diag<T>(W, blk(0), bs, 1, b.omega, n, Y, ldy, M, M, nullptr, c.s, 0, 0));
+            KB_TRY(start_blocks());
+            KB_TRY(launch_assemble_diag<T>(W, blk(0), bs, 1, b.omega, n, Y, ldy, M, M, tg, b.ctrl, c.s, 0, 0));
             for (int k = 1; k < m; ++k) {
                 T *Pk = blk(k - 1);
                 T *Pp = k >= 2 ? blk(k - 2) : nullptr;
                 T *X = blk(k);
-                if (c.frontier) {
-                    KB_TRY(launch_frontier_expand(c.g->dev, b.gen, b.tgen, k, c.s, b.alist, b.acount));
-                    KB_TRY(launch_frontier_list(b.tgen, n, k, b.alist, b.acount, c.s));
-                }
                 LinEpi<T> e;
                 e.tgen = tg;
-                e.gen = tg ? b.gen : nullptr;
+                e.gen = tg ? b.fr.gen : nullptr;
                 e.limit = k;
-                e.alist = tg ? b.alist : nullptr;
-                e.acount = b.acount;
+                e.alist = tg ? b.fr.alist : nullptr;
+                e.acount = tg ? b.fr.count(k) : nullptr;
                 e.a1 = b.c1 + int64_t(k - 1) * W;
                 e.a2 = b.c2 + int64_t(k - 1) * W;
                 e.s0 = 0.0;
@@ -685,9 +656,9 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
                 ++c.spmm;
                 int grid2 = 0;
                 KB_TRY(launch_axpy_colnorm<T>(W, X, Pk, b.aupd + int64_t(k - 1) * W, n, b.parts, &grid2,
-                                              b.ctrl2, tg, k, M, c.s, tg ? b.alist : nullptr, b.acount));
+                                              b.ctrl2, tg, k, M, c.s, tg ? b.fr.alist : nullptr, tg ? b.fr.count(k) : nullptr));
                 KB_TRY(launch_assemble_diag<T>(W, X, bs, 1, b.omega + int64_t(k) * W, n, Y, ldy, M, M,
-                                               tg, c.s, k, 1));
+                                               tg, b.ctrl, c.s, k, 1));
             }
         }
         KB_TRY(launch_fill_nan(Y, n, ldy, M, b.ctrl, c.s));
@@ -706,8 +677,7 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
 template <typename T>
 int cheb_pass(Common &c, const std::vector<double> &coef, double lam, int W, int64_t n,
               const int32_t *marker, const int32_t *nodes, int Mc, const T *Zsrc, T *bufs[3],
-              T *out, float *yout, int64_t ldo, int mo, int64_t M_alg, uint8_t *gen,
-              int32_t *tgen, int hop0, int32_t *alist, int32_t *acount) {
+              T *out, float *yout, int64_t ldo, int mo, int64_t M_alg, const FrontierBufs *fr, int hop0) {
     // weights of sum_k'' c_k T_k (Lobatto interpolation: c_0 and c_m halved)
     const int h = int(coef.size()) - 1;
     std::vector<double> w(coef);
@@ -716,9 +686,10 @@ int cheb_pass(Common &c, const std::vector<double> &coef, double lam, int W, int
     // b_h = w_h S
     int cur_i = 0, prev_i = -1;
     if (Zsrc) {
-        KB_TRY(launch_scale_copy<T>(bufs[0], Zsrc, n * W, w[h], c.s));
+        KB_TRY(launch_scale_copy<T>(bufs[0], Zsrc, n, W, w[h], fr ? fr->alist : nullptr,
+                                    fr ? fr->count(hop0) : nullptr, c.s));
     } else {
-        KB_CUDA_TRY(cudaMemsetAsync(bufs[0], 0, sizeof(T) * size_t(n) * W, c.s));
+        if (!fr) KB_CUDA_TRY(cudaMemsetAsync(bufs[0], 0, sizeof(T) * size_t(n) * W, c.s));
         KB_TRY(launch_scatter<T>(bufs[0], W, nodes, Mc, 0, T(w[h]), c.s));
     }
     // b_k = w_k S + 2 A b_{k+1} - b_{k+2} (k = h-1..1);  result = w_0 S + A b_1 - b_2,
@@ -729,20 +700,13 @@ int cheb_pass(Common &c, const std::vector<double> &coef, double lam, int W, int
         while (dst_i == cur_i || dst_i == prev_i) ++dst_i;
         // b_k is supported on rows within hop0 + (h - k) hops of W
         const int hop = hop0 + (h - k);
-        if (tgen) {
-            // the list of the previous hop holds every row at distance hop - 1; the list of
-            // this hop serves this step's SpMM (the last step writes zeros on inactive tiles
-            // and walks every tile) and the next expansion (the second cheb2 pass)
-            KB_TRY(launch_frontier_expand(c.g->dev, gen, tgen, hop, c.s, alist, acount));
-            KB_TRY(launch_frontier_list(tgen, n, hop, alist, acount, c.s));
-        }
         LinEpi<T> e;
-        e.tgen = tgen;
-        e.gen = tgen ? gen : nullptr;
+        e.tgen = fr ? fr->tgen : nullptr;
+        e.gen = fr ? fr->gen : nullptr;
         e.limit = hop;
-        e.alist = (tgen && !last) ? alist : nullptr;
-        e.acount = acount;
-        e.zero_inactive = last ? 1 : 0;
+        e.alist = fr ? fr->alist : nullptr;
+        e.acount = fr ? fr->count(hop) : nullptr;
+        e.zero_inactive = last && yout ? 1 : 0;
         e.s1 = (last ? -2.0 : -4.0) / lam;
         e.s0 = last ? 1.0 : 2.0;
         e.s2 = -1.0;
@@ -767,15 +731,14 @@ int cheb_pass(Common &c, const std::vector<double> &coef, double lam, int W, int
 
 template <typename T>
 void plan_cheb(Arena &ar, int64_t n, int Mmax, bool squared, T **bufs, T **Z, int32_t **marker,
-               uint8_t **gen, int32_t **tgen, int32_t **alist, int32_t **acount) {
+               FrontierBufs &fr) {
+    // bufs and Z are consecutive blocks of n Wmax elements
     const int Wmax = width_for(Mmax);
-    for (int i = 0; i < 3; ++i) bufs[i] = ar.take<T>(size_t(n) * Wmax);
-    *Z = squared ? ar.take<T>(size_t(n) * Wmax) : nullptr;
+    T *p = ar.take<T>(size_t(squared ? 4 : 3) * n * Wmax);
+    for (int i = 0; i < 3; ++i) bufs[i] = p ? p + size_t(i) * n * Wmax : nullptr;
+    *Z = squared && p ? p + size_t(3) * n * Wmax : nullptr;
     *marker = ar.take<int32_t>(size_t(n));
-    *gen = ar.take<uint8_t>(size_t(n));
-    *tgen = ar.take<int32_t>(size_t((n + ACT_ROWS - 1) / ACT_ROWS));
-    *alist = ar.take<int32_t>(size_t((n + ACT_ROWS - 1) / ACT_ROWS));
-    *acount = ar.take<int32_t>(1);
+    ar.frontier(fr, n);
 }
 
 template <typename T>
@@ -787,36 +750,33 @@ int run_cheb(Common &c, bool squared, const int32_t *nodes, int M, int m, float 
     const int Mmax = std::min(M, sizeof(T) == 8 ? 64 : 128);
     Arena dry;
     T *bufs[3], *Z;
-    int32_t *marker, *tgen, *alist, *acount;
-    uint8_t *gen;
-    plan_cheb<T>(dry, n, Mmax, squared, bufs, &Z, &marker, &gen, &tgen, &alist, &acount);
+    int32_t *marker;
+    FrontierBufs fb;
+    plan_cheb<T>(dry, n, Mmax, squared, bufs, &Z, &marker, fb);
     Arena ar;
     KB_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void **>(&ar.base), dry.off, c.s));
-    plan_cheb<T>(ar, n, Mmax, squared, bufs, &Z, &marker, &gen, &tgen, &alist, &acount);
+    plan_cheb<T>(ar, n, Mmax, squared, bufs, &Z, &marker, fb);
     auto body = [&]() -> int {
         for (int col0 = 0; col0 < M; col0 += Mmax) {
             const int Mc = std::min(Mmax, M - col0);
             const int W = width_for(Mc);
             KB_CUDA_TRY(cudaMemsetAsync(marker, 0xFF, sizeof(int32_t) * size_t(n), c.s));
             KB_TRY(launch_marker(marker, nodes + col0, Mc, c.s));
-            int32_t *tg = nullptr;
+            const FrontierBufs *fr = c.frontier ? &fb : nullptr;
             if (c.frontier) {
-                // Clenshaw blocks are written on reached tiles only: start from zeros
-                for (int i = 0; i < 3; ++i)
-                    KB_CUDA_TRY(cudaMemsetAsync(bufs[i], 0, sizeof(T) * size_t(n) * W, c.s));
-                if (Z) KB_CUDA_TRY(cudaMemsetAsync(Z, 0, sizeof(T) * size_t(n) * W, c.s));
-                KB_TRY(launch_frontier_init(gen, tgen, n, nodes + col0, Mc, c.s));
-                KB_TRY(launch_frontier_list(tgen, n, 0, alist, acount, c.s));
-                tg = tgen;
+                // Clenshaw blocks rotate and are written on reached tiles only: zeros on all of those
+                KB_TRY(launch_frontier(c.g->dev, fb, nodes + col0, Mc, (squared ? 2 * h : h) + 1, c.s));
+                KB_TRY(launch_zero_tiles(bufs[0], int64_t(sizeof(T)) * n * width_for(Mmax), squared ? 4 : 3,
+                                         W * int(sizeof(T)), n, false, fb, c.s));
             }
             if (!squared) {
                 KB_TRY(cheb_pass<T>(c, coef, lam, W, n, marker, nodes + col0, Mc, nullptr, bufs,
-                                    nullptr, Y + col0, ldy, Mc, Mc, gen, tg, 0, alist, acount));
+                                    nullptr, Y + col0, ldy, Mc, Mc, fr, 0));
             } else {
                 KB_TRY(cheb_pass<T>(c, coef, lam, W, n, marker, nodes + col0, Mc, nullptr, bufs, Z,
-                                    nullptr, 0, 0, Mc, gen, tg, 0, alist, acount));
+                                    nullptr, 0, 0, Mc, fr, 0));
                 KB_TRY(cheb_pass<T>(c, coef, lam, W, n, marker, nodes + col0, Mc, Z, bufs,
-                                    nullptr, Y + col0, ldy, Mc, Mc, gen, tg, h, alist, acount));
+                                    nullptr, Y + col0, ldy, Mc, Mc, fr, h));
             }
         }
         return 0;
@@ -850,10 +810,10 @@ size_t workspace_bytes_t(int64_t n, kb_method method, int M, int m, bool two, co
         case KB_CHEB:
         case KB_CHEB2: {
             T *bufs[3], *Z;
-            int32_t *marker, *tgen, *alist, *acount;
-            uint8_t *gen;
-            plan_cheb<T>(dry, n, std::min(M, sizeof(T) == 8 ? 64 : 128), method == KB_CHEB2, bufs, &Z,
-                         &marker, &gen, &tgen, &alist, &acount);
+            int32_t *marker;
+            FrontierBufs fb;
+            plan_cheb<T>(dry, n, std::min(M, sizeof(T) == 8 ? 64 : 128), method == KB_CHEB2, bufs, &Z, &marker,
+                         fb);
             break;
         }
     }
@@ -924,9 +884,15 @@ int apply_device(kb_graph *g, kb_method method, kb_phi phi, const kb_params *par
     if (rc) return rc;
     Common c{g, phi, *params, s_int, static_cast<cudaStream_t>(stream), 0, nullptr, true};
     if (quad->n > 0) c.quad = quad.get();
-    // exact restriction of the per-step kernels to rows reached from W (hop distances are
-    // kept in 8 bits)
-    c.frontier = !params->no_frontier && m <= FRONTIER_MAX_HOPS;
+    // exact restriction of the per-step kernels to rows reached from W (hop distances are kept
+    // in 8 bits).  It costs a breadth-first search and a sort (about 5 us per hop), so blocks
+    // below 16 MiB, which stay in L2, run on all rows: measured with 20 steps on random
+    // geometric graphs, restricted / all rows (us): 16384 rows, M = 64, cheb 308 / 222, cbl
+    // 5061 / 4975; 65536 rows, M = 64 (16 MiB), cheb 456 / 429, cbl 6290 / 7050; 262144 rows,
+    // M = 16 (16 MiB), cheb 321 / 552, cbl 2558 / 3598.  FP64 products cost some 16 times as
+    // much per row.
+    const int64_t blk_bytes = g->dev.n * width_for(std::min(M, 128)) * (params->basis == KB_F64 ? 128 : 4);
+    c.frontier = !params->no_frontier && m <= FRONTIER_MAX_HOPS && blk_bytes >= (int64_t(16) << 20);
     c.tc = rowblock_tc_enabled() ? 1 : 0;
     const bool f64 = params->basis == KB_F64;
     const bool bf16 = params->basis == KB_BF16;

@@ -190,7 +190,8 @@ k_rowblock(RowArgs<T> a) {
     C *sG = PROD ? sO + q.TR * LDO : sO;                            // [NGR * NB][BI * BJ] (W = 128)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t nt = (a.n + ACT_ROWS - 1) / ACT_ROWS;             // frontier tiles of the matrix
-    const int64_t cnt = a.alist ? (MODE == RB_ASM ? nt : int64_t(*a.acount)) : nt;
+    // (ASM writes all of y; a launch that adds to it only the tiles that its block reaches)
+    const int64_t cnt = a.alist && (MODE != RB_ASM || a.accumulate) ? int64_t(*a.acount) : nt;
     auto tile_at = [&](int64_t i) -> int64_t {
         return i >= cnt ? -1 : (a.alist ? int64_t(__ldg(a.alist + i)) : i);
     };

@@ -78,11 +78,24 @@ __global__ void k_marker(int32_t *marker, NodeChunk ch) {
     if (j < ch.cnt) marker[ch.idx[j]] = ch.col0 + j;
 }
 
+// out = scale in on the listed 32-row tiles (all rows without a list), 16 bytes at a time
 template <typename T>
-__global__ void k_scale_copy(T *out, const T *in, int64_t count, double scale) {
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < count;
-         i += int64_t(gridDim.x) * blockDim.x)
-        out[i] = T(scale * to_double(in[i]));
+__global__ void __launch_bounds__(256) k_scale_copy(T *out, const T *in, int64_t n, int W, double scale,
+                                                    const int32_t *__restrict__ alist, const int32_t *acount) {
+    constexpr int V = 16 / int(sizeof(T));
+    const int64_t nt = (n + ACT_ROWS - 1) / ACT_ROWS;
+    const int64_t cnt = alist ? int64_t(*acount) : nt;
+    for (int64_t it = blockIdx.x; it < cnt; it += gridDim.x) {
+        const int64_t r0 = (alist ? int64_t(__ldg(alist + it)) : it) * ACT_ROWS;
+        const int64_t rows = n - r0 < ACT_ROWS ? n - r0 : ACT_ROWS;
+        for (int64_t i = int64_t(threadIdx.x) * V; i < rows * W; i += 256 * V) {
+            uint4 raw = *reinterpret_cast<const uint4 *>(in + r0 * W + i);
+            T *v = reinterpret_cast<T *>(&raw);
+#pragma unroll
+            for (int q = 0; q < V; ++q) v[q] = T(scale * to_double(v[q]));
+            *reinterpret_cast<uint4 *>(out + r0 * W + i) = raw;
+        }
+    }
 }
 
 __global__ void k_fill_nan(float *Y, int64_t n, int64_t ldy, int mo, const Ctrl *ctrl) {
@@ -1191,7 +1204,7 @@ __global__ void __launch_bounds__(256) k_axpy_colnorm(T *X, const T *P, const do
     C acc[4] = {0, 0, 0, 0};
     unsigned long long my_rows = 0;
     if (alist && tgen) {
-        // active 32-row tiles only (listed in increasing order): RPP rows per pass
+        // active 32-row tiles only: RPP rows per pass
         const int cnt = *acount;
         for (int it = blockIdx.x; it < cnt; it += gridDim.x) {
             const int64_t t0 = int64_t(__ldg(alist + it)) * ACT_ROWS;
@@ -1274,10 +1287,13 @@ template <typename T, int W>
 __global__ void __launch_bounds__(256) k_assemble_diag(const T *basis, int64_t stride, int nblk,
                                                         const double *omega, int64_t n, float *Y,
                                                         int64_t ldy, int mo, const int32_t *tgen,
-                                                        int kbase, int accumulate, ProfCount pc) {
+                                                        int kbase, int accumulate, const Ctrl *ctrl,
+                                                        ProfCount pc) {
     constexpr int CG = W / 4;
     constexpr int RPP = 256 / CG;
     using C = typename Cmp<T>::type;
+    // blocks of steps after a stop were never written (their weights are zero)
+    nblk = min(nblk, max(ctrl->steps - kbase, 0));
     extern __shared__ __align__(16) unsigned char sm_raw[];
     C *som = reinterpret_cast<C *>(sm_raw);     // [nblk][W]
     for (int i = threadIdx.x; i < nblk * W; i += blockDim.x) som[i] = C(omega[i]);
@@ -1304,47 +1320,6 @@ __global__ void __launch_bounds__(256) k_assemble_diag(const T *basis, int64_t s
             if (c4 + q < mo) Y[row * ldy + c4 + q] = acc[q];
     }
     if (pc.nnz && cg == 0 && my_units) atomicAdd(pc.nnz, my_units);
-}
-
-// ---------------------------------------------------------------- frontier
-__global__ void k_frontier_seed(uint8_t *gen, int32_t *tgen, NodeChunk ch) {
-    const int j = threadIdx.x + blockIdx.x * blockDim.x;
-    if (j < ch.cnt) {
-        gen[ch.idx[j]] = 0;
-        tgen[ch.idx[j] / ACT_ROWS] = 0;
-    }
-}
-
-// One hop: rows at distance k-1 mark their unreached neighbours with distance k.
-// Marks the unreached neighbours of one frontier row (stored nonzeros beg..end) with
-// distance k, eight at a time: their indices, then their marks, loaded before any store (a
-// mark read as unset that another thread sets meanwhile only repeats the same store).
-__device__ __forceinline__ void expand_row(const GraphDev &g, uint8_t *gen, int32_t *tgen, int k,
-                                           int beg, int end) {
-    for (int p = beg; p < end; p += 8) {
-        int jj[8];
-        uint8_t gj[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) jj[u] = p + u < end ? __ldg(g.col + p + u) : -1;
-#pragma unroll
-        for (int u = 0; u < 8; ++u) gj[u] = jj[u] >= 0 ? gen[jj[u]] : uint8_t(0);
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (gj[u] == 255) {
-                gen[jj[u]] = uint8_t(k);
-                atomicMin(tgen + jj[u] / ACT_ROWS, k);
-            }
-    }
-}
-
-__global__ void __launch_bounds__(256) k_frontier_expand(GraphDev g, uint8_t *gen, int32_t *tgen, int k) {
-    for (int64_t i = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; i < g.n;
-         i += int64_t(gridDim.x) * blockDim.x) {
-        if (__ldg(tgen + i / ACT_ROWS) > k - 1) continue;
-        if (gen[i] != uint8_t(k - 1)) continue;
-        const int beg = __ldg(g.rowptr + i), end = __ldg(g.rowptr + i + 1);
-        expand_row(g, gen, tgen, k, beg, end);
-    }
 }
 
 template <typename T>
@@ -1511,134 +1486,12 @@ int launch_marker(int32_t *marker, const int32_t *nodes, int M, cudaStream_t s) 
 }
 
 template <typename T>
-int launch_scale_copy(T *out, const T *in, int64_t count, double scale, cudaStream_t s) {
-    const int grid = int(std::min<int64_t>((count + 255) / 256, int64_t(num_sms()) * 8));
-    k_scale_copy<T><<<std::max(grid, 1), 256, 0, s>>>(out, in, count, scale);
+int launch_scale_copy(T *out, const T *in, int64_t n, int W, double scale, const int32_t *alist,
+                      const int32_t *acount, cudaStream_t s) {
+    const int grid = int(std::min<int64_t>((n + ACT_ROWS - 1) / ACT_ROWS, int64_t(num_sms()) * 8));
+    k_scale_copy<T><<<std::max(grid, 1), 256, 0, s>>>(out, in, n, W, scale, alist, acount);
     count_launches(1);
     KB_CUDA_TRY(cudaGetLastError());
-    return 0;
-}
-
-int launch_frontier_init(uint8_t *gen, int32_t *tgen, int64_t n, const int32_t *nodes, int M,
-                         cudaStream_t s) {
-    KB_CUDA_TRY(cudaMemsetAsync(gen, 0xFF, size_t(n), s));
-    KB_CUDA_TRY(cudaMemsetAsync(tgen, 0x7F, sizeof(int32_t) * size_t((n + ACT_ROWS - 1) / ACT_ROWS), s));
-    for (int j0 = 0; j0 < M; j0 += NodeChunk::CAP) {
-        NodeChunk ch;
-        ch.cnt = std::min(NodeChunk::CAP, M - j0);
-        ch.col0 = j0;
-        for (int j = 0; j < ch.cnt; ++j) ch.idx[j] = nodes[j0 + j];
-        k_frontier_seed<<<1, NodeChunk::CAP, 0, s>>>(gen, tgen, ch);
-        count_launches(1);
-    }
-    KB_CUDA_TRY(cudaGetLastError());
-    return 0;
-}
-
-// Same as k_frontier_expand, visiting only the rows of the 32-row tiles active at step k-1
-// (the list made after the previous expansion): the rows at distance k-1 lie there.
-__global__ void __launch_bounds__(256) k_frontier_expand_listed(GraphDev g, uint8_t *gen, int32_t *tgen, int k,
-                                                                const int32_t *__restrict__ alist,
-                                                                const int32_t *__restrict__ acount) {
-    const int64_t total = int64_t(*acount) * ACT_ROWS;
-    for (int64_t idx = blockIdx.x * int64_t(blockDim.x) + threadIdx.x; idx < total;
-         idx += int64_t(gridDim.x) * blockDim.x) {
-        const int64_t i = int64_t(__ldg(alist + idx / ACT_ROWS)) * ACT_ROWS + idx % ACT_ROWS;
-        if (i >= g.n || gen[i] != uint8_t(k - 1)) continue;
-        const int beg = __ldg(g.rowptr + i), end = __ldg(g.rowptr + i + 1);
-        expand_row(g, gen, tgen, k, beg, end);
-    }
-}
-
-// Stream compaction of the active 32-row tiles in tile order.  Each warp owns a contiguous
-// range of 32-entry groups and reads them coalesced, eight groups in flight; a ballot gives
-// each group's active lanes, kept in shared memory (up to LIST_MASKS groups, i.e. 2^18 tiles
-// of 32 rows; beyond that the second pass reads the array again).  The warp's count and, in
-// the second pass, each active entry's position (the active lanes below it) come from
-// population counts; a block-wide exclusive scan of the warp counts gives each warp's offset.
-constexpr int LIST_MASKS = 8192;
-__global__ void __launch_bounds__(1024) k_frontier_list(const int32_t *__restrict__ tgen, int64_t nact,
-                                                        int limit, int32_t *__restrict__ list,
-                                                        int32_t *__restrict__ count) {
-    __shared__ int wsum[33];
-    __shared__ unsigned s_mask[LIST_MASKS];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int64_t ngrp = (nact + 31) / 32;
-    const bool cached = ngrp <= LIST_MASKS;
-    const int64_t gper = (ngrp + nw - 1) / nw;
-    const int64_t g0 = int64_t(warp) * gper;
-    const int64_t g1 = g0 + gper < ngrp ? g0 + gper : ngrp;
-    int c = 0;
-    for (int64_t g = g0; g < g1; g += 8) {
-        int32_t v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int64_t a = (g + u) * 32 + lane;
-            v[u] = (g + u < g1 && a < nact) ? __ldg(tgen + a) : INT_MAX;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const unsigned mask = __ballot_sync(0xffffffffu, v[u] <= limit);
-            if (cached && lane == 0 && g + u < g1) s_mask[g + u] = mask;
-            c += __popc(mask);
-        }
-    }
-    if (lane == 0) wsum[warp] = c;
-    __syncthreads();
-    if (warp == 0) {
-        const int own = lane < nw ? wsum[lane] : 0;
-        int incl = own;
-        for (int off = 1; off < 32; off <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += u;
-        }
-        wsum[lane] = incl - own;               // exclusive offset of warp `lane`
-        if (lane == 31) wsum[32] = incl;       // total
-    }
-    __syncthreads();
-    int pos = wsum[warp];
-    const unsigned below = (1u << lane) - 1u;
-    for (int64_t g = g0; g < g1; g += 8) {
-        unsigned mk[8];
-        if (cached) {
-#pragma unroll
-            for (int u = 0; u < 8; ++u) mk[u] = g + u < g1 ? s_mask[g + u] : 0u;
-        } else {
-            int32_t v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int64_t a = (g + u) * 32 + lane;
-                v[u] = (g + u < g1 && a < nact) ? __ldg(tgen + a) : INT_MAX;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) mk[u] = __ballot_sync(0xffffffffu, v[u] <= limit);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if ((mk[u] >> lane) & 1u) list[pos + __popc(mk[u] & below)] = int32_t((g + u) * 32 + lane);
-            pos += __popc(mk[u]);
-        }
-    }
-    if (threadIdx.x == 0) *count = wsum[32];
-}
-
-int launch_frontier_list(const int32_t *tgen, int64_t n, int limit, int32_t *list, int32_t *count,
-                         cudaStream_t s) {
-    prof_begin(KernelClass::OTHER, s);
-    k_frontier_list<<<1, 1024, 0, s>>>(tgen, (n + ACT_ROWS - 1) / ACT_ROWS, limit, list, count);
-    KB_CUDA_TRY(cudaGetLastError());
-    prof_end(KernelClass::OTHER, s, double(n) / ACT_ROWS * 4, 0);
-    return 0;
-}
-
-int launch_frontier_expand(const GraphDev &g, uint8_t *gen, int32_t *tgen, int k, cudaStream_t s,
-                           const int32_t *alist, const int32_t *acount) {
-    const int grid = int(std::max<int64_t>(1, std::min<int64_t>((g.n + 255) / 256, int64_t(num_sms()) * 8)));
-    prof_begin(KernelClass::OTHER, s);
-    if (alist) k_frontier_expand_listed<<<grid, 256, 0, s>>>(g, gen, tgen, k, alist, acount);
-    else k_frontier_expand<<<grid, 256, 0, s>>>(g, gen, tgen, k);
-    KB_CUDA_TRY(cudaGetLastError());
-    prof_end(KernelClass::OTHER, s, double(g.n) / ACT_ROWS * 4, 0);
     return 0;
 }
 
@@ -1771,13 +1624,13 @@ int axpy_max_grid() { return num_sms() * 4; }
         cudaFuncSetAttribute(k_assemble_diag<T, WW>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                              int(smem));                                                      \
         k_assemble_diag<T, WW><<<grid, 256, smem, s>>>(basis, stride, nblk, omega, n, Y, ldy, mo,  \
-                                                       tgen, kbase, accumulate, pc);          \
+                                                       tgen, kbase, accumulate, ctrl, pc);    \
     } while (0)
 
 template <typename T>
 int launch_assemble_diag(int W, const T *basis, int64_t stride, int nblk, const double *omega,
                          int64_t n, float *Y, int64_t ldy, int mo, int64_t M_alg,
-                         const int32_t *tgen, cudaStream_t s, int kbase, int accumulate) {
+                         const int32_t *tgen, const Ctrl *ctrl, cudaStream_t s, int kbase, int accumulate) {
     const int rpp = 256 / (W / 4);
     const int grid = std::max(1, int(std::min<int64_t>((n + rpp - 1) / rpp, int64_t(num_sms()) * 8)));
     const size_t smem = sizeof(typename Cmp<T>::type) * size_t(nblk) * W;
@@ -1809,7 +1662,8 @@ int launch_u_convert(const double *U, int M, int W, int m, T *Ut, const Ctrl *ct
 
 #define KB_INST(T)                                                                              \
     template int launch_scatter<T>(T *, int64_t, const int32_t *, int, int, T, cudaStream_t);   \
-    template int launch_scale_copy<T>(T *, const T *, int64_t, double, cudaStream_t);           \
+    template int launch_scale_copy<T>(T *, const T *, int64_t, int, double, const int32_t *,    \
+                                      const int32_t *, cudaStream_t);                           \
     template int launch_hkk<T>(const double *, int, int, double *, T *, const Ctrl *, cudaStream_t); \
     template int launch_chol<T>(const double *, int, int, int, int, double, double, double *,   \
                                 T *, double *, T *, Ctrl *, cudaStream_t);                      \
@@ -1818,7 +1672,7 @@ int launch_u_convert(const double *U, int M, int W, int m, T *Ut, const Ctrl *ct
                                         cudaStream_t, const int32_t *, const int32_t *);        \
     template int launch_assemble_diag<T>(int, const T *, int64_t, int, const double *, int64_t, \
                                          float *, int64_t, int, int64_t, const int32_t *,       \
-                                         cudaStream_t, int, int);                               \
+                                         const Ctrl *, cudaStream_t, int, int);                             \
     template int launch_u_convert<T>(const double *, int, int, int, T *, const Ctrl *, cudaStream_t);
 KB_INST(float)
 KB_INST(double)
@@ -1826,14 +1680,14 @@ KB_INST(double)
 // BF16 blocks: element-wise kernels on the stored type (small matrices stay FP32)
 template int launch_scatter<__nv_bfloat16>(__nv_bfloat16 *, int64_t, const int32_t *, int, int,
                                            __nv_bfloat16, cudaStream_t);
-template int launch_scale_copy<__nv_bfloat16>(__nv_bfloat16 *, const __nv_bfloat16 *, int64_t,
-                                              double, cudaStream_t);
+template int launch_scale_copy<__nv_bfloat16>(__nv_bfloat16 *, const __nv_bfloat16 *, int64_t, int,
+                                              double, const int32_t *, const int32_t *, cudaStream_t);
 template int launch_axpy_colnorm<__nv_bfloat16>(int, __nv_bfloat16 *, const __nv_bfloat16 *,
                                                 const double *, int64_t, double *, int *,
                                                 const Ctrl *, const int32_t *, int, int64_t,
                                                 cudaStream_t, const int32_t *, const int32_t *);
 template int launch_assemble_diag<__nv_bfloat16>(int, const __nv_bfloat16 *, int64_t, int,
                                                  const double *, int64_t, float *, int64_t, int,
-                                                 int64_t, const int32_t *, cudaStream_t, int, int);
+                                                 int64_t, const int32_t *, const Ctrl *, cudaStream_t, int, int);
 
 }  // namespace kb

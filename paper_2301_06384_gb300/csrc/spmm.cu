@@ -3,15 +3,17 @@
 // This is the "MV" of Table 1 (Section 7), the operation the paper names the most
 // expensive for large graphs; every method performs m of them per solve.
 //
-// Schedule (GB300).  A CTA owns a tile of consecutive rows at a time (persistent grid,
-// a multiple of the SM count).  The tile's row pointers and then all its column indices
-// (and weights) are staged in shared memory with coalesced loads, so a row's neighbour
-// list costs no dependent global round trip.  A row of x is W elements; W/8 lanes cover it
-// with two 16-byte vectors each (float4, or 2 x double2), so each warp works on 32/(W/8)
-// rows at once, one lane group per row; a group reads its neighbour indices from shared
-// memory (broadcast) and gathers two neighbour rows with independent 16-byte loads before
-// consuming them.  The register budget is sized for 5 resident CTAs (40 warps) per SM.  Rows of a tile whose column list does not fit in shared memory
-// (hub rows) read their indices from global memory instead.
+// Schedule (GB300).  A row of x is W elements; W/8 lanes cover it with two 16-byte vectors
+// each (float4, or 2 x double2), so a warp takes 32/(W/8) rows at once, one lane group per
+// row: a warp's unit of work, all in one 32-row frontier tile.  Warps walk their units
+// independently (no barrier, no shared staging) over the active-tile list, or over all rows
+// without one.  Row pointers come one unit ahead; the lanes of a group load a chunk of the
+// row's neighbour indices with one coalesced load and pass them round by shuffles; U rows are
+// gathered with independent 16-byte loads before they are used.  Rows beyond the frontier
+// inside an active tile are written as zeros without their gathers.  Bound by the latency
+// and the L2 bandwidth of the gathers.  Against CTA tiles with row pointers and indices staged
+// in shared memory (three barriers per tile) and 32-row units that left half of the warps idle
+// at W = 32: RGG of 2e4 rows, M = 37, 30 products 447 -> 345 us.
 //
 // The Laplacian is applied in difference form (L x)_i = sum_j w_ij (x_i - x_j) + r_i x_i,
 // which gives L 1 = 0 exactly for D - A and drops the diagonal load for standard
@@ -66,44 +68,17 @@ template <> struct V4<double> {
     }
 };
 
-// Schedule parameters (compile-time; the defaults are the measured best on the RGG bench).
-#ifndef KB_SPMM_CAP
-#define KB_SPMM_CAP 4096
-#endif
-#ifndef KB_SPMM_VPL
-#define KB_SPMM_VPL 2
-#endif
-#ifndef KB_SPMM_U
-#define KB_SPMM_U 4
-#endif
-#ifndef KB_SPMM_PACKED
-#define KB_SPMM_PACKED 1   // FP32 neighbour loop on packed f32x2 pairs
-#endif
-#ifndef KB_SPMM_IDX32
-#define KB_SPMM_IDX32 0
-#endif
 constexpr int SPMM_THREADS = 256;
 constexpr int WARPS = SPMM_THREADS / 32;
-constexpr int CAP = KB_SPMM_CAP;   // staged column indices per tile
-constexpr int VPL = KB_SPMM_VPL;   // 16-byte vectors per lane (4 VPL elements of a row)
-constexpr int U = KB_SPMM_U;       // neighbour rows gathered per lane before use
+constexpr int VPL = 2;          // 16-byte vectors per lane (8 elements of a row)
+constexpr int U = 4;            // neighbour rows gathered per lane before use
 
 template <int W>
 struct SpmmGeo {
-    static constexpr int LPR = W / (4 * VPL) < 1 ? 1 : W / (4 * VPL);   // lanes per row
-    static constexpr int RPW = 32 / LPR;                 // rows per warp
-    static constexpr int NG = WARPS * RPW;               // lane groups per CTA
-    static constexpr int RPG = W >= 64 ? 4 : (W == 32 ? 2 : 1);   // rows per group per tile
-    static constexpr int TR = NG * RPG;                  // rows per tile
+    static constexpr int LPR = W / (4 * VPL);   // lanes per row
+    static constexpr int RPW = 32 / LPR;        // rows of a warp's unit of work
+    static constexpr int UPT = ACT_ROWS / RPW;  // units of a 32-row tile
 };
-
-// Resident CTAs per SM the register budget is sized for: the FP32 kernel without column
-// dot products fits 5 (40 warps), the others fewer.
-// Prefetch the 128-byte line holding p into L2 (no register result, no fault on the
-// addresses used here: every caller passes an address inside an allocated array).
-__device__ __forceinline__ void prefetch_l2(const void *p) {
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
 
 // Packed FP32 pairs (Blackwell add/sub/fma.rn.f32x2): each lane of the pair is rounded as
 // the scalar instruction would round it, so the packed neighbour loop gives bit-identical
@@ -151,44 +126,31 @@ __device__ __forceinline__ void lds4(const C *p, C (&v)[4]) {
     }
 }
 
-#ifndef KB_SPMM_OCC
-#define KB_SPMM_OCC 4   // FP32 / BF16 kernel without column dots
-#endif
-#ifndef KB_SPMM_OCC_DOT
-#define KB_SPMM_OCC_DOT 4   // FP32 / BF16 kernel with column dots
-#endif
+// Resident CTAs per SM the register budget is sized for.  Measured, RGG of 10^6 rows, M = 64,
+// 30 products (ms), four / three / five CTAs: without column dots 1.58 / 1.66 / 1.87; with
+// them (8 more accumulators) 3.62 / 3.45.  Two or eight gathers in flight instead of U = 4:
+// 1.74 / 1.78 and 4.10 / 3.89.
 template <typename T, bool DOT>
 struct SpmmOcc {
-    static constexpr int value = sizeof(typename Cmp<T>::type) == 8 ? 3 : (DOT ? KB_SPMM_OCC_DOT : KB_SPMM_OCC);
+    static constexpr int value = sizeof(typename Cmp<T>::type) == 8 ? 3 : (DOT ? 3 : 4);
 };
 
-// WGT: the graph stores edge weights (false: unit weights, w_ij = 1).  LST: the launch walks
-// the active-tile list (frontier restriction with a list of the active 32-row tiles).
-template <typename T, int W, bool DOT, bool WGT, bool LST>
+// WGT: the graph stores edge weights (false: unit weights, w_ij = 1).
+template <typename T, int W, bool DOT, bool WGT>
 __global__ void __launch_bounds__(SPMM_THREADS, (SpmmOcc<T, DOT>::value))
-k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo) {
+k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo, int mcols) {
     using G = SpmmGeo<W>;
     using C = typename Cmp<T>::type;   // arithmetic type
-    constexpr int LPR = G::LPR, RPW = G::RPW, NG = G::NG, TR = G::TR, RPG = G::RPG;
-    // gathers in flight per lane group: fewer in the variant that also accumulates column
-    // dots (its registers hold the dot partials)
-    constexpr int UU = DOT ? (U < 2 ? U : 2) : U;
-    static_assert(TR >= ACT_ROWS && TR % ACT_ROWS == 0, "row tiles hold whole 32-row frontier tiles");
+    constexpr int LPR = G::LPR, RPW = G::RPW, UPT = G::UPT;
+    constexpr int CPL = LPR >= 8 ? 1 : 8 / LPR;   // neighbour indices a lane loads at once
+    constexpr int CHUNK = LPR * CPL;
     if (e.ctrl && e.ctrl->stop) return;
-    // (arrays a variant does not use take one element: shared memory left to L1 caches the
-    // gathered rows)
-    __shared__ int s_rp[TR + 1];
-    __shared__ int s_col[CAP];
-    __shared__ float s_w[WGT ? CAP : 1];
     __shared__ __align__(16) C s_coef[5][W];       // c1 hi, c1 lo, c0, c2 hi, c2 lo
     __shared__ C s_sc[2];                          // s3, wE in the arithmetic type
     __shared__ double s_dot[DOT ? WARPS : 1][W];
-    __shared__ unsigned long long s_cnt[2];       // rows, stored nonzeros processed
     if (threadIdx.x == 0) {
         s_sc[0] = C(e.s3);
         s_sc[1] = C(e.wE);
-        s_cnt[0] = 0ull;
-        s_cnt[1] = 0ull;
     }
     for (int c = threadIdx.x; c < W; c += blockDim.x) {
         const double d1 = e.a1 ? e.a1[c] : e.s1;
@@ -208,245 +170,177 @@ k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo) {
     // column span (whole 32-byte sectors) of the gathered row
     const int sub = lane % LPR;
 #define KB_COL(v) (((v) * LPR + sub) * 4)
-    const int gid = warp * RPW + grp;
+    // columns past the block's M hold zeros in every operand: neither gathered nor read
+    bool cin[VPL];
+#pragma unroll
+    for (int v = 0; v < VPL; ++v) cin[v] = KB_COL(v) < mcols;
     C dot[VPL][4];
 #pragma unroll
     for (int v = 0; v < VPL; ++v)
 #pragma unroll
         for (int q = 0; q < 4; ++q) dot[v][q] = C(0);
-    const int64_t ntiles = (g.n + TR - 1) / TR;
-    // with the active-tile list, the unit of work is one listed 32-row tile instead of a
-    // TR-row tile: the few active rows of an early step spread over all CTAs
-    constexpr bool listed = LST;
-    const int64_t nloop = listed ? int64_t(*e.acount) : ntiles;
-    // A listed unit is one chunk of 32 rows: its lane groups read their row pointers and
-    // column indices straight from global memory, with no shared staging and no barrier, so
-    // the warps of a CTA move through their units independently.  The coefficients set above
-    // are ordered here.
-    if constexpr (listed) __syncthreads();
-
-    for (int64_t it = blockIdx.x; it < nloop; it += gridDim.x) {
-        const int64_t r0 = listed ? int64_t(__ldg(e.alist + it)) * ACT_ROWS : it * TR;
-        const int urows = listed ? ACT_ROWS : TR;
-        const int rows = (g.n - r0 < urows) ? int(g.n - r0) : urows;
-        if (e.tgen && tile_min_gen(e.tgen, r0, rows) > e.limit) {
-            // every row of the tile is beyond the frontier: its output is exactly zero
-            if (e.zero_inactive) {
-                if (e.yout) {
-                    for (int i = threadIdx.x; i < rows * mo; i += blockDim.x)
-                        e.yout[(r0 + i / mo) * ldo + (i % mo)] = 0.f;
-                } else {
-                    for (int i = threadIdx.x; i < rows * W; i += blockDim.x) e.out[r0 * W + i] = T(0.f);
-                }
-            }
-            continue;
+    unsigned my_rows = 0, my_nnz = 0;
+    // a unit of work is RPW rows of a 32-row tile, one warp's; tiles past `active` (beyond the
+    // frontier limit) are only written, with zeros, where the launch asks for it
+    const int64_t nt = (g.n + ACT_ROWS - 1) / ACT_ROWS;
+    const int64_t active = e.tgen ? int64_t(*e.acount) : nt;
+    const int64_t nunits = (e.tgen && !e.zero_inactive ? active : nt) * UPT;
+    const int64_t step = int64_t(gridDim.x) * WARPS;
+    __syncthreads();
+    // row, its reach flag and its neighbour range for unit `w` (w < nunits)
+    auto row_of = [&](int64_t w) -> int64_t {
+        const int64_t t = w / UPT;
+        return (e.tgen ? int64_t(__ldg(e.alist + t)) : t) * ACT_ROWS + (w % UPT) * RPW + grp;
+    };
+    // The rows come one unit ahead (list entry, hop distance, row pointers), so that a unit's
+    // chain of dependent loads is only neighbour indices -> gathered rows.
+    int64_t row = -1;
+    int beg = 0, end = 0;
+    bool act = false;
+    auto fetch = [&](int64_t w, int64_t &r, int &b, int &en, bool &on) {
+        r = -1;
+        b = en = 0;
+        on = false;
+        if (w >= nunits) return;
+        r = row_of(w);
+        if (r >= g.n) {
+            r = -1;
+            return;
         }
-        int base = 0;
-        bool staged = false;
-        if constexpr (!listed) {
-            // ask L2 for the tile's own dense rows now (x_i at the row start, y / z in the
-            // epilogue) and for the next tile's row pointers, so that those loads, issued
-            // later, do not wait on DRAM
-            const char *xb = reinterpret_cast<const char *>(x + r0 * W);
-            const int64_t tile_bytes = int64_t(rows) * W * int64_t(sizeof(T));
-            constexpr int64_t row_bytes = int64_t(W) * int64_t(sizeof(T));
-            for (int64_t off = int64_t(threadIdx.x) * 128; off < tile_bytes; off += int64_t(blockDim.x) * 128) {
-                // rows of 32-row frontier tiles beyond the limit are skipped below: no prefetch
-                if (e.tgen && __ldg(e.tgen + (r0 + off / row_bytes) / ACT_ROWS) > e.limit) continue;
-                prefetch_l2(xb + off);
-                if (e.y) prefetch_l2(reinterpret_cast<const char *>(e.y + r0 * W) + off);
-                if (e.z) prefetch_l2(reinterpret_cast<const char *>(e.z + r0 * W) + off);
-            }
-            const int64_t nr0 = r0 + int64_t(gridDim.x) * TR;
-            if (threadIdx.x < (TR + 1 + 31) / 32 && nr0 + threadIdx.x * 32 <= g.n)
-                prefetch_l2(g.rowptr + nr0 + threadIdx.x * 32);
-            __syncthreads();   // previous tile done with the shared arrays
-            for (int i = threadIdx.x; i <= rows; i += blockDim.x) s_rp[i] = __ldg(g.rowptr + r0 + i);
-            __syncthreads();
-            base = s_rp[0];
-            const int cnt = s_rp[rows] - base;
-            staged = cnt <= CAP;
-            if (staged) {
-                for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-                    s_col[i] = __ldg(g.col + base + i);
-                    if (WGT) s_w[i] = __ldg(g.w + base + i);
-                }
-            }
-            __syncthreads();
+        on = w / UPT < active && (!e.tgen || int(__ldg(e.gen + r)) <= e.limit);
+        b = __ldg(g.rowptr + r);
+        en = __ldg(g.rowptr + r + 1);
+    };
+    const int64_t w0 = int64_t(blockIdx.x) * WARPS + warp;
+    fetch(w0, row, beg, end, act);
+    for (int64_t w = w0; w < nunits; w += step) {
+        int64_t nrow;
+        int nbeg, nend;
+        bool nact;
+        fetch(w + step, nrow, nbeg, nend, nact);
+        const int deg = act ? end - beg : 0;
+        if (sub == 0 && act) {
+            ++my_rows;
+            my_nnz += unsigned(deg);
         }
-#pragma unroll 1
-        for (int rr = 0; rr < RPG; ++rr) {
-            // rows rr*NG .. rr*NG+NG-1 of the tile (one lane group each); with the frontier
-            // restriction a chunk whose 32-row frontier tiles are all beyond the limit is
-            // exactly zero and skipped (CTA-uniform)
-            const int c0r = rr * NG;
-            if (c0r >= rows) break;
-            const int crows = rows - c0r < NG ? rows - c0r : NG;
-            const int lrow = c0r + gid;
-            bool skip_rows = e.tgen && tile_min_gen(e.tgen, r0 + c0r, crows) > e.limit;
-            if (!skip_rows && e.gen) {
-                // this warp's RPW rows of the chunk: skipped (warp-uniform) when every one
-                // of them lies beyond the limit (the rr loop has no barrier)
-                const int wr0 = c0r + warp * RPW;
-                bool any = false;
+        V4<T> xi[VPL];
+        C acc[VPL][4];
 #pragma unroll
-                for (int q = 0; q < RPW; ++q)
-                    if (wr0 + q < rows && int(__ldg(e.gen + r0 + wr0 + q)) <= e.limit) any = true;
-                skip_rows = !any;
-            } else if (!skip_rows && threadIdx.x == 0 && !listed) {
-                s_cnt[0] += unsigned(crows);
-                s_cnt[1] += unsigned(s_rp[c0r + crows] - s_rp[c0r]);
+        for (int v = 0; v < VPL; ++v) {
+            xi[v] = act && cin[v] ? V4<T>::load(x + row * W + KB_COL(v)) : V4<T>{};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) acc[v][q] = C(0);
+        }
+        // neighbours: the lanes of a group load the indices (and weights) of a chunk of 8 or
+        // LPR; the group then takes them in order by shuffles.  The loop runs to the longest row of the
+        // warp; slots past a row's end contribute x_i - x_i, an exact zero.
+        const int maxdeg = __reduce_max_sync(0xffffffffu, deg);
+        for (int p0 = 0; p0 < maxdeg; p0 += CHUNK) {
+            int mj[CPL];
+            float mw[CPL];
+#pragma unroll
+            for (int q = 0; q < CPL; ++q) {
+                const int p = p0 + q * LPR + sub;
+                mj[q] = p < deg ? __ldg(g.col + beg + p) : 0;
+                if (WGT) mw[q] = p < deg ? __ldg(g.w + beg + p) : 0.f;
             }
-            if (skip_rows) {
-                if (e.zero_inactive && lrow < rows) {
 #pragma unroll
-                    for (int v = 0; v < VPL; ++v)
+            for (int u0 = 0; u0 < CHUNK; u0 += U) {
+                if (p0 + u0 >= maxdeg) break;
+                if constexpr (std::is_same<T, float>::value) {
+                    f2 xj[U][VPL][2], xi2[VPL][2];
+                    f2 wv[U];
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int c = KB_COL(v) + q;
-                            if (e.yout) {
-                                if (c < mo) e.yout[(r0 + lrow) * ldo + c] = 0.f;
-                            } else {
-                                e.out[(r0 + lrow) * W + c] = T(0.f);
-                            }
-                        }
-                }
-                continue;
-            }
-            if (e.gen && lane == 0) {
-                // rows and stored nonzeros this warp processes
-                const int wr0 = c0r + warp * RPW;
-                const int wr1 = wr0 + RPW < rows ? wr0 + RPW : rows;
-                if (wr1 > wr0) {
-                    const int nz = listed ? __ldg(g.rowptr + r0 + wr1) - __ldg(g.rowptr + r0 + wr0)
-                                          : s_rp[wr1] - s_rp[wr0];
-                    atomicAdd(&s_cnt[0], (unsigned long long)(wr1 - wr0));
-                    atomicAdd(&s_cnt[1], (unsigned long long)nz);
-                }
-            }
-            if (lrow >= rows) continue;
-            const int64_t row = r0 + lrow;
-            const int beg = listed ? __ldg(g.rowptr + row) : s_rp[lrow] - base;
-            const int end = listed ? __ldg(g.rowptr + row + 1) : s_rp[lrow + 1] - base;
-            V4<T> xi[VPL];
-            C acc[VPL][4];
+                    for (int v = 0; v < VPL; ++v) {
+                        xi2[v][0] = f2_pack(xi[v].v[0], xi[v].v[1]);
+                        xi2[v][1] = f2_pack(xi[v].v[2], xi[v].v[3]);
+                    }
 #pragma unroll
-            for (int v = 0; v < VPL; ++v) {
-                xi[v] = V4<T>::load(x + row * W + KB_COL(v));
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[v][q] = C(0);
-            }
-            if constexpr (std::is_same<T, float>::value && KB_SPMM_PACKED) {
-                // the same sums on packed pairs: acc += w (x_i - x_j), two columns per
-                // instruction
-                f2 xi2[VPL][2], acc2[VPL][2];
-#pragma unroll
-                for (int v = 0; v < VPL; ++v) {
-                    xi2[v][0] = f2_pack(xi[v].v[0], xi[v].v[1]);
-                    xi2[v][1] = f2_pack(xi[v].v[2], xi[v].v[3]);
-                    acc2[v][0] = 0ull;
-                    acc2[v][1] = 0ull;
-                }
-                for (int p = beg; p < end; p += UU) {
-                    // slots past the row's end gather the row itself (weight 0): x_i - x_i
-                    // adds an exact zero, so the unrolled body needs no per-slot branch
-                    f2 xj2[UU][VPL][2];
-                    f2 wv2[UU];
-                    int jj[UU];
-#pragma unroll
-                    for (int u = 0; u < UU; ++u) {
-                        const bool in = p + u < end;
-                        jj[u] = in ? (staged ? s_col[p + u] : __ldg(g.col + base + p + u)) : int(row);
+                    for (int u = 0; u < U; ++u) {
+                        const int j = __shfl_sync(0xffffffffu, mj[(u0 + u) / LPR], (u0 + u) % LPR, LPR);
                         if (WGT) {
-                            const float w = in ? (staged ? s_w[p + u] : __ldg(g.w + base + p + u)) : 0.f;
-                            wv2[u] = f2_pack(w, w);
+                            const float wj = __shfl_sync(0xffffffffu, mw[(u0 + u) / LPR], (u0 + u) % LPR, LPR);
+                            wv[u] = f2_pack(wj, wj);
+                        }
+                        const bool in = p0 + u0 + u < deg;
+                        const float *xr = reinterpret_cast<const float *>(x) + int64_t(j) * W;
+#pragma unroll
+                        for (int v = 0; v < VPL; ++v) {
+                            xj[u][v][0] = xi2[v][0];
+                            xj[u][v][1] = xi2[v][1];
+                            if (in && cin[v]) ldg_f2x2(xr + KB_COL(v), xj[u][v][0], xj[u][v][1]);
                         }
                     }
 #pragma unroll
-                    for (int u = 0; u < UU; ++u)
+                    for (int v = 0; v < VPL; ++v) {
+                        f2 a0 = f2_pack(acc[v][0], acc[v][1]), a1 = f2_pack(acc[v][2], acc[v][3]);
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            const f2 d0 = f2_sub(xi2[v][0], xj[u][v][0]), d1 = f2_sub(xi2[v][1], xj[u][v][1]);
+                            a0 = WGT ? f2_fma(wv[u], d0, a0) : f2_add(a0, d0);
+                            a1 = WGT ? f2_fma(wv[u], d1, a1) : f2_add(a1, d1);
+                        }
+                        f2_unpack(a0, acc[v][0], acc[v][1]);
+                        f2_unpack(a1, acc[v][2], acc[v][3]);
+                    }
+                } else {
+                    V4<T> xj[U][VPL];
+                    C wv[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        const int j = __shfl_sync(0xffffffffu, mj[(u0 + u) / LPR], (u0 + u) % LPR, LPR);
+                        wv[u] = WGT ? C(__shfl_sync(0xffffffffu, mw[(u0 + u) / LPR], (u0 + u) % LPR, LPR)) : C(1);
+                        const bool in = p0 + u0 + u < deg;
 #pragma unroll
                         for (int v = 0; v < VPL; ++v)
-                            ldg_f2x2(reinterpret_cast<const float *>(x) + int64_t(jj[u]) * W + KB_COL(v),
-                                     xj2[u][v][0], xj2[u][v][1]);
+                            xj[u][v] = in && cin[v] ? V4<T>::load(x + int64_t(j) * W + KB_COL(v)) : xi[v];
+                    }
 #pragma unroll
-                    for (int u = 0; u < UU; ++u)
+                    for (int u = 0; u < U; ++u)
 #pragma unroll
                         for (int v = 0; v < VPL; ++v)
 #pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const f2 d = f2_sub(xi2[v][h], xj2[u][v][h]);
-                                acc2[v][h] = WGT ? f2_fma(wv2[u], d, acc2[v][h]) : f2_add(acc2[v][h], d);
-                            }
+                            for (int q = 0; q < 4; ++q)
+                                acc[v][q] = WGT ? fma(wv[u], xi[v].v[q] - xj[u][v].v[q], acc[v][q])
+                                                : acc[v][q] + (xi[v].v[q] - xj[u][v].v[q]);
                 }
-#pragma unroll
-                for (int v = 0; v < VPL; ++v) {
-                    f2_unpack(acc2[v][0], acc[v][0], acc[v][1]);
-                    f2_unpack(acc2[v][1], acc[v][2], acc[v][3]);
-                    // x_i again from its packed copy (the scalar copy need not live across
-                    // the loop)
-                    f2_unpack(xi2[v][0], xi[v].v[0], xi[v].v[1]);
-                    f2_unpack(xi2[v][1], xi[v].v[2], xi[v].v[3]);
-                }
-            } else {
-            for (int p = beg; p < end; p += UU) {
-                // slots past the row's end gather the row itself (weight 0): x_i - x_i adds
-                // an exact zero, so the unrolled body needs no per-slot branch
-                V4<T> xj[UU][VPL];
-                C wv[UU];
-                int jj[UU];
-#pragma unroll
-                for (int u = 0; u < UU; ++u) {
-                    const bool in = p + u < end;
-                    jj[u] = in ? (staged ? s_col[p + u] : __ldg(g.col + base + p + u)) : int(row);
-                    wv[u] = WGT ? (in ? C(staged ? s_w[p + u] : __ldg(g.w + base + p + u)) : C(0)) : C(1);
-                }
-#pragma unroll
-                for (int u = 0; u < UU; ++u)
-#pragma unroll
-                    for (int v = 0; v < VPL; ++v)
-                        xj[u][v] = V4<T>::load(KB_SPMM_IDX32 ? x + (unsigned(jj[u]) * unsigned(W) + unsigned(KB_COL(v)))
-                                                             : x + int64_t(jj[u]) * W + KB_COL(v));
-#pragma unroll
-                for (int u = 0; u < UU; ++u)
-#pragma unroll
-                    for (int v = 0; v < VPL; ++v)
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            acc[v][q] = WGT ? fma(wv[u], xi[v].v[q] - xj[u][v].v[q], acc[v][q])
-                                            : acc[v][q] + (xi[v].v[q] - xj[u][v].v[q]);
             }
-            }
-            const C r = g.rdiag ? C(__ldg(g.rdiag + row)) : C(0);
-            const int mk = e.marker ? __ldg(e.marker + row) : -1;
+        }
+        if (row >= 0) {
+            const C r = g.rdiag && act ? C(__ldg(g.rdiag + row)) : C(0);
+            const int mk = e.marker && act ? __ldg(e.marker + row) : -1;
 #pragma unroll
             for (int v = 0; v < VPL; ++v) {
                 const int c = KB_COL(v);
-                C o[4], k1h[4], k1l[4], k0[4];
-                lds4(&s_coef[0][c], k1h);
-                lds4(&s_coef[1][c], k1l);
-                lds4(&s_coef[2][c], k0);
+                C o[4] = {0, 0, 0, 0};
+                if (act && cin[v]) {
+                    C k1h[4], k1l[4], k0[4];
+                    lds4(&s_coef[0][c], k1h);
+                    lds4(&s_coef[1][c], k1l);
+                    lds4(&s_coef[2][c], k0);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const C a = fma(r, xi[v].v[q], acc[v][q]);
-                    o[q] = fma(k1h[q], a, fma(k1l[q], a, k0[q] * xi[v].v[q]));
+                    for (int q = 0; q < 4; ++q) {
+                        const C a = fma(r, xi[v].v[q], acc[v][q]);
+                        o[q] = fma(k1h[q], a, fma(k1l[q], a, k0[q] * xi[v].v[q]));
+                    }
+                    if (e.y) {
+                        const V4<T> yi = V4<T>::load(e.y + row * W + c);
+                        C k2h[4], k2l[4];
+                        lds4(&s_coef[3][c], k2h);
+                        lds4(&s_coef[4][c], k2l);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) o[q] = fma(k2h[q], yi.v[q], fma(k2l[q], yi.v[q], o[q]));
+                    }
+                    if (e.z) {
+                        const V4<T> zi = V4<T>::load(e.z + row * W + c);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) o[q] = fma(s_sc[0], zi.v[q], o[q]);
+                    }
+                    // (constant indices: a computed index would put o in local memory)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        if (mk == c + q) o[q] += s_sc[1];
                 }
-                if (e.y) {
-                    const V4<T> yi = V4<T>::load(e.y + row * W + c);
-                    C k2h[4], k2l[4];
-                    lds4(&s_coef[3][c], k2h);
-                    lds4(&s_coef[4][c], k2l);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) o[q] = fma(k2h[q], yi.v[q], fma(k2l[q], yi.v[q], o[q]));
-                }
-                if (e.z) {
-                    const V4<T> zi = V4<T>::load(e.z + row * W + c);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q) o[q] = fma(s_sc[0], zi.v[q], o[q]);
-                }
-                // (constant indices: a computed index would put o in local memory)
-#pragma unroll
-                for (int q = 0; q < 4; ++q)
-                    if (mk == c + q) o[q] += s_sc[1];
                 if (!e.yout) {
                     // narrowed blocks: the dot below is that of the stored values
                     if constexpr (!std::is_same<T, C>::value) {
@@ -458,9 +352,14 @@ k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo) {
                     for (int q = 0; q < 4; ++q) ov.v[q] = o[q];
                     ov.store(e.out + row * W + c);
                 } else {
+                    float *y = e.yout + row * ldo + c;
+                    if (c + 3 < mo && ((ldo & 3) == 0) && (reinterpret_cast<uintptr_t>(y) & 15) == 0) {
+                        *reinterpret_cast<float4 *>(y) = make_float4(float(o[0]), float(o[1]), float(o[2]), float(o[3]));
+                    } else {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        if (c + q < mo) e.yout[row * ldo + c + q] = float(o[q]);
+                        for (int q = 0; q < 4; ++q)
+                            if (c + q < mo) y[q] = float(o[q]);
+                    }
                 }
                 if (DOT) {
 #pragma unroll
@@ -468,10 +367,14 @@ k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo) {
                 }
             }
         }
+        row = nrow;
+        beg = nbeg;
+        end = nend;
+        act = nact;
     }
-    if (threadIdx.x == 0 && e.prof.rows) {
-        atomicAdd(e.prof.rows, s_cnt[0]);
-        atomicAdd(e.prof.nnz, s_cnt[1]);
+    if (e.prof.rows && my_rows) {
+        atomicAdd(e.prof.rows, (unsigned long long)my_rows);
+        atomicAdd(e.prof.nnz, (unsigned long long)my_nnz);
     }
     if constexpr (DOT && std::is_same<C, float>::value) {
         // double-float combination on the FP32 pipe; partials written as DF pairs
@@ -522,35 +425,29 @@ int occupancy_spmm() {
     // function-local static: computed once, thread-safe (several serving workers)
     static const int per_sm = [] {
         int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_spmm<T, W, DOT, true, false>, SPMM_THREADS, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_spmm<T, W, DOT, true>, SPMM_THREADS, 0);
         return v < 1 ? 1 : v;
     }();
     return per_sm;
 }
 
 template <typename T, int W, bool DOT>
-int launch_wd(const GraphDev &g, const T *x, const LinEpi<T> &e, int64_t ldo, int mo,
+int launch_wd(const GraphDev &g, const T *x, const LinEpi<T> &e, int64_t ldo, int mo, int mcols,
               cudaStream_t s, int *grid_out) {
-    const int64_t ntiles = (g.n + SpmmGeo<W>::TR - 1) / SpmmGeo<W>::TR;
-    int grid = int(std::min<int64_t>(ntiles, int64_t(num_sms()) * occupancy_spmm<T, W, DOT>()));
+    const int64_t units = (g.n + SpmmGeo<W>::RPW - 1) / SpmmGeo<W>::RPW;
+    int grid = int(std::min<int64_t>((units + WARPS - 1) / WARPS, int64_t(num_sms()) * occupancy_spmm<T, W, DOT>()));
     if (grid < 1) grid = 1;
     if (grid_out) *grid_out = grid;
-    const bool lst = e.alist && e.tgen && !e.zero_inactive;
-    if (g.w) {
-        if (lst) k_spmm<T, W, DOT, true, true><<<grid, SPMM_THREADS, 0, s>>>(g, x, e, ldo, mo);
-        else k_spmm<T, W, DOT, true, false><<<grid, SPMM_THREADS, 0, s>>>(g, x, e, ldo, mo);
-    } else {
-        if (lst) k_spmm<T, W, DOT, false, true><<<grid, SPMM_THREADS, 0, s>>>(g, x, e, ldo, mo);
-        else k_spmm<T, W, DOT, false, false><<<grid, SPMM_THREADS, 0, s>>>(g, x, e, ldo, mo);
-    }
+    if (g.w) k_spmm<T, W, DOT, true><<<grid, SPMM_THREADS, 0, s>>>(g, x, e, ldo, mo, mcols);
+    else k_spmm<T, W, DOT, false><<<grid, SPMM_THREADS, 0, s>>>(g, x, e, ldo, mo, mcols);
     return 0;
 }
 
 template <typename T, int W>
-int launch_w(const GraphDev &g, const T *x, const LinEpi<T> &e, int64_t ldo, int mo,
+int launch_w(const GraphDev &g, const T *x, const LinEpi<T> &e, int64_t ldo, int mo, int mcols,
              cudaStream_t s, int *grid_out) {
-    return e.dot_partials ? launch_wd<T, W, true>(g, x, e, ldo, mo, s, grid_out)
-                          : launch_wd<T, W, false>(g, x, e, ldo, mo, s, grid_out);
+    return e.dot_partials ? launch_wd<T, W, true>(g, x, e, ldo, mo, mcols, s, grid_out)
+                          : launch_wd<T, W, false>(g, x, e, ldo, mo, mcols, s, grid_out);
 }
 
 }  // namespace
@@ -561,11 +458,12 @@ int launch_spmm(const GraphDev &g, int W, const T *x, const LinEpi<T> &e, cudaSt
     if (ldo <= 0) { ldo = W; mo = W; }
     LinEpi<T> ee = e;
     ee.prof = prof_begin(KernelClass::SPMM, s);
+    const int mcols = int(M_alg);
     switch (W) {
-        case 16: launch_w<T, 16>(g, x, ee, ldo, mo, s, grid_out); break;
-        case 32: launch_w<T, 32>(g, x, ee, ldo, mo, s, grid_out); break;
-        case 64: launch_w<T, 64>(g, x, ee, ldo, mo, s, grid_out); break;
-        case 128: launch_w<T, 128>(g, x, ee, ldo, mo, s, grid_out); break;
+        case 16: launch_w<T, 16>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
+        case 32: launch_w<T, 32>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
+        case 64: launch_w<T, 64>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
+        case 128: launch_w<T, 128>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
         default: return fail(KB_ERR_ARG, "unsupported block width");
     }
     cudaError_t err = cudaGetLastError();
