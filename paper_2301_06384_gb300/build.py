@@ -19,7 +19,7 @@ OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libkb.so")
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 SOURCES = ["graph.cu", "spmm.cu", "rowblock.cu", "rowblock_f32.cu", "rowblock_f32_wide.cu",
-           "rowblock_f64.cu", "rowblock_bf16.cu", "rowblock_tc.cu", "small.cu", "frontier.cu", "projected.cu", "krylov.cu",
+           "rowblock_ordered.cu", "rowblock_f64.cu", "rowblock_bf16.cu", "rowblock_tc.cu", "small.cu", "chol.cu", "chol_ordered.cu", "frontier.cu", "projected.cu", "krylov.cu",
            "fixed_scratch.cu", "server.cu", "rls.cu", "quadrature.cu"]
 
 

@@ -143,18 +143,82 @@ k_bfs(GraphDev g, NodeChunk seeds, int levels, uint8_t *gen, int32_t *tgen, uint
     }
 }
 
-// Tiles at distance b = blockIdx.x (b = levels + 1: all that were not reached) in index order
-// into list[acount[b - 1] ..].  Each warp owns a contiguous range of 32-tile groups and reads
-// them coalesced, eight groups in flight; a ballot gives the group's members, kept in shared
-// memory for the second pass (up to LIST_MASKS groups; beyond that the array is read again),
-// and a block-wide exclusive scan of the warps' counts their offsets.
+// Compaction of the 32-row tiles whose distance satisfies in(tgen) into list[first ..], in index
+// order, by one CTA of 1024 threads; returns their number.  Each warp owns a contiguous range
+// of 32-tile groups and reads them coalesced, eight groups in flight; a ballot gives the group's
+// members, kept in shared memory for the second pass (up to LIST_MASKS groups; beyond that the
+// array is read again), and a block-wide exclusive scan of the warps' counts their offsets.
 constexpr int LIST_MASKS = 8192;
+template <typename P>
+__device__ int compact_tiles(const int32_t *tgen, int64_t nact, const P &in, int first, int32_t *list) {
+    __shared__ int wsum[33];
+    __shared__ unsigned s_mask[LIST_MASKS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int64_t ngrp = (nact + 31) / 32;
+    const bool cached = ngrp <= LIST_MASKS;
+    const int64_t gper = (ngrp + nw - 1) / nw;
+    const int64_t g0 = int64_t(warp) * gper;
+    const int64_t g1 = g0 + gper < ngrp ? g0 + gper : ngrp;
+    auto masks = [&](int64_t g, unsigned (&mk)[8]) {
+        int32_t v[8];
+        bool on[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int64_t a = (g + u) * 32 + lane;
+            on[u] = g + u < g1 && a < nact;
+            v[u] = on[u] ? __ldg(tgen + a) : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) mk[u] = __ballot_sync(0xffffffffu, on[u] && in(v[u]));
+    };
+    int c = 0;
+    for (int64_t g = g0; g < g1; g += 8) {
+        unsigned mk[8];
+        masks(g, mk);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if (cached && lane == 0 && g + u < g1) s_mask[g + u] = mk[u];
+            c += __popc(mk[u]);
+        }
+    }
+    if (lane == 0) wsum[warp] = c;
+    __syncthreads();
+    if (warp == 0) {
+        const int own = lane < nw ? wsum[lane] : 0;
+        int incl = own;
+        for (int off = 1; off < 32; off <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, incl, off);
+            if (lane >= off) incl += u;
+        }
+        wsum[lane] = incl - own;               // exclusive offset of warp `lane`
+        if (lane == 31) wsum[32] = incl;
+    }
+    __syncthreads();
+    int pos = first + wsum[warp];
+    const unsigned below = (1u << lane) - 1u;
+    for (int64_t g = g0; g < g1; g += 8) {
+        unsigned mk[8];
+        if (cached) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) mk[u] = g + u < g1 ? s_mask[g + u] : 0u;
+        } else {
+            masks(g, mk);
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            if ((mk[u] >> lane) & 1u) list[pos + __popc(mk[u] & below)] = int32_t((g + u) * 32 + lane);
+            pos += __popc(mk[u]);
+        }
+    }
+    return wsum[32];
+}
+
+// The list by distance, one CTA per distance: tiles at distance b = blockIdx.x (b = levels + 1:
+// all that were not reached) into list[acount[b - 1] ..].
 __global__ void __launch_bounds__(1024) k_tile_sort(int32_t *tgen, uint8_t *gen, int64_t n, int64_t nact, int levels,
                                                     const int32_t *__restrict__ tcnt, const int32_t *err,
                                                     int32_t *__restrict__ acount, int32_t *__restrict__ list) {
-    __shared__ int wsum[33];
     __shared__ int s_before, s_own;
-    __shared__ unsigned s_mask[LIST_MASKS];
     const int b = blockIdx.x;
     if (*err) {
         // the search gave up: every row counts as reached at once
@@ -179,62 +243,15 @@ __global__ void __launch_bounds__(1024) k_tile_sort(int32_t *tgen, uint8_t *gen,
         }
     }
     __syncthreads();
-    const int first = s_before;
     if (s_own == 0) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int64_t ngrp = (nact + 31) / 32;
-    const bool cached = ngrp <= LIST_MASKS;
-    const int64_t gper = (ngrp + nw - 1) / nw;
-    const int64_t g0 = int64_t(warp) * gper;
-    const int64_t g1 = g0 + gper < ngrp ? g0 + gper : ngrp;
-    auto masks = [&](int64_t g, unsigned (&mk)[8]) {
-        int32_t v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            const int64_t a = (g + u) * 32 + lane;
-            v[u] = (g + u < g1 && a < nact) ? __ldg(tgen + a) : -1;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) mk[u] = __ballot_sync(0xffffffffu, b <= levels ? v[u] == b : v[u] > levels);
-    };
-    int c = 0;
-    for (int64_t g = g0; g < g1; g += 8) {
-        unsigned mk[8];
-        masks(g, mk);
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if (cached && lane == 0 && g + u < g1) s_mask[g + u] = mk[u];
-            c += __popc(mk[u]);
-        }
-    }
-    if (lane == 0) wsum[warp] = c;
-    __syncthreads();
-    if (warp == 0) {
-        const int own = lane < nw ? wsum[lane] : 0;
-        int incl = own;
-        for (int off = 1; off < 32; off <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, incl, off);
-            if (lane >= off) incl += u;
-        }
-        wsum[lane] = incl - own;               // exclusive offset of warp `lane`
-    }
-    __syncthreads();
-    int pos = first + wsum[warp];
-    const unsigned below = (1u << lane) - 1u;
-    for (int64_t g = g0; g < g1; g += 8) {
-        unsigned mk[8];
-        if (cached) {
-#pragma unroll
-            for (int u = 0; u < 8; ++u) mk[u] = g + u < g1 ? s_mask[g + u] : 0u;
-        } else {
-            masks(g, mk);
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-            if ((mk[u] >> lane) & 1u) list[pos + __popc(mk[u] & below)] = int32_t((g + u) * 32 + lane);
-            pos += __popc(mk[u]);
-        }
-    }
+    compact_tiles(tgen, nact, [&](int v) { return b <= levels ? v == b : v > levels; }, s_before, list);
+}
+
+// The tiles within k hops in index order (solves that keep a fixed order of their sums).
+__global__ void __launch_bounds__(1024) k_tile_list(const int32_t *tgen, int64_t nact, int k, int32_t *list,
+                                                    int32_t *count) {
+    const int c = compact_tiles(tgen, nact, [&](int v) { return v <= k; }, 0, list);
+    if (threadIdx.x == 0) *count = c;
 }
 
 // Zeros on the listed tiles.  ring: block b of the stored basis is written on the tiles within
@@ -314,6 +331,14 @@ int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, in
     k_tile_sort<<<levels + 2, 1024, 0, s>>>(f.tgen, f.gen, g.n, nt, levels, f.tcnt, f.sync + 1, f.acount, f.alist);
     KB_CUDA_TRY(cudaGetLastError());
     prof_end(KernelClass::OTHER, s, double(g.n) + 4.0 * double(nt), 0, 2);
+    return 0;
+}
+
+int launch_tile_list(const FrontierBufs &f, int64_t n, int k, int32_t *list, int32_t *count, cudaStream_t s) {
+    prof_begin(KernelClass::OTHER, s);
+    k_tile_list<<<1, 1024, 0, s>>>(f.tgen, (n + ACT_ROWS - 1) / ACT_ROWS, k, list, count);
+    KB_CUDA_TRY(cudaGetLastError());
+    prof_end(KernelClass::OTHER, s, double(n) / ACT_ROWS * 4, 0);
     return 0;
 }
 

@@ -243,6 +243,7 @@ struct RowArgs {
     int lim_b = INT32_MAX;            // hop distances; ASM, ASMSUB: block k beyond kbase + k
     int tri_a = 0;                    // UPD: ca is lower triangular
     int M = 0;                        // columns in use (set by launch_rowblock)
+    int ordered = 0;                  // sums in a fixed order (rowblock.cuh): alist is in index order
     int tc = 0;                       // tensor-core kernels allowed (rowblock_tc.cu)
     int kbase = 0;                    // ASM: index of the first block (frontier reach)
     int accumulate = 0;               // ASM: y += product (the accumulator starts from y)

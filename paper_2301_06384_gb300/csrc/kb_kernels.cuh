@@ -81,6 +81,11 @@ int launch_chol(const double *G, int M, int W, int pass, int step, double inv_th
                 double piv_rel2, double *R1, T *Rinv, double *Hs, T *Bout, Ctrl *ctrl,
                 cudaStream_t s);
 
+// FP32 solves with full reorthogonalisation (chol_ordered.cu)
+int launch_chol_ordered(const double *G, int M, int W, int pass, int step, double inv_thresh2,
+                        double piv_rel2, double *R1, float *Rinv, double *Hs, float *Bout, Ctrl *ctrl,
+                        cudaStream_t s);
+
 int launch_lanczos_init(int W, int M, int gbl, int round32, double *sigma, int32_t *alive,
                         double *c1, double *c2, cudaStream_t s);
 int launch_lanczos_alpha(const double *parts, int nparts, int W, int M, int gbl, int k, int df,
@@ -129,6 +134,8 @@ struct FrontierBufs {
 void plan_frontier(FrontierBufs &f, int64_t n, unsigned char *base, size_t *bytes);
 // Hop distances up to `levels` from the nodes, and the tile list.
 int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, int levels, cudaStream_t s);
+// The tiles within k hops in index order into list, their number into *count.
+int launch_tile_list(const FrontierBufs &f, int64_t n, int k, int32_t *list, int32_t *count, cudaStream_t s);
 // Zeros on the tiles within f.levels hops: see k_zero_tiles.
 int launch_zero_tiles(void *blocks, int64_t block_bytes, int nblk, int row_bytes, int64_t n, bool ring,
                       const FrontierBufs &f, cudaStream_t s);

@@ -20,6 +20,7 @@
 #include <limits>
 #include <memory>
 #include <mutex>
+#include <type_traits>
 
 namespace kb {
 
@@ -151,6 +152,7 @@ struct Common {
     Ctrl *hctrl = nullptr;   // host copy of the control block when the caller wants info
     bool frontier = true;    // restrict the per-step kernels to the reached rows
     int tc = 0;              // tensor-core row-block kernels allowed (asked once per solve)
+    int ordered = 0;         // FP32 cbl with full reorthogonalisation: sums in a fixed order
     const QuadRule *quad = nullptr;   // spline kernel with non-integer s (Lanczos methods)
 };
 
@@ -212,6 +214,7 @@ struct CblBufs {
     int32_t *reo_skip;   // ... and the flag that skips the second pass
     Ctrl *ctrl, *ctrl2, *ctrl_chk;
     FrontierBufs fr;
+    int32_t *olist, *ocount;   // ordered solves: the step's tiles in index order
 };
 
 template <typename T>
@@ -246,6 +249,8 @@ void plan_cbl(Arena &ar, CblBufs<T> &b, int64_t n, int M, int W, int m, int rb_g
     b.ctrl2 = ar.take<Ctrl>(1);
     b.ctrl_chk = ar.take<Ctrl>(1);
     ar.frontier(b.fr, n);
+    b.olist = ar.take<int32_t>(size_t((n + ACT_ROWS - 1) / ACT_ROWS));
+    b.ocount = ar.take<int32_t>(1);
 }
 
 template <typename T>
@@ -275,11 +280,13 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
         // those just beyond; otherwise each block is written in full
         const int nbuf = two ? 3 : m;
         const int64_t bs = n * W;
+        const bool ord = c.ordered != 0;
         auto start_blocks = [&]() -> int {
             if (!c.frontier) {
                 KB_CUDA_TRY(cudaMemsetAsync(b.basis, 0, sizeof(T) * size_t(bs), c.s));
-            } else if (c.tc) {
-                // (the tensor-core kernels walk 128-row tiles, whose rows beyond the reach they read)
+            } else if (c.tc || ord) {
+                // (kernels that walk whole tiles of 64 rows or more, or all tiles for every block,
+                // read rows beyond a block's reach)
                 KB_CUDA_TRY(cudaMemsetAsync(b.basis, 0, sizeof(T) * size_t(bs) * nbuf, c.s));
                 KB_CUDA_TRY(cudaMemsetAsync(b.wbuf, 0, sizeof(T) * size_t(bs), c.s));
             } else {
@@ -295,10 +302,18 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
         const int32_t *tg = c.frontier ? b.fr.tgen : nullptr;
         auto within = [&](RowArgs<T> &ra, int k) {
             ra.tc = c.tc;
+            ra.ordered = c.ordered;
             ra.tgen = tg;
             ra.limit = k;
             ra.alist = tg ? b.fr.alist : nullptr;
             ra.acount = tg ? b.fr.count(k) : nullptr;
+        };
+        // a launch with a Gram in an ordered solve: the tiles of step k in index order
+        auto in_order = [&](RowArgs<T> &ra, int k) {
+            if (!ord || !tg) return;
+            ra.limit = k;
+            ra.alist = b.olist;
+            ra.acount = b.ocount;
         };
         const size_t WW = size_t(W) * W;
         auto blk = [&](int j) { return b.basis + int64_t(two ? j % 3 : j) * bs; };
@@ -312,6 +327,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             C *Bk = b.Bs + (k - 1) * WW;
             C *S1 = b.Rs1 + (k - 1) * WW, *S2 = b.Rs2 + (k - 1) * WW;
             C *Cl = b.Cloc + 2 * (k - 1) * WW;
+            if (ord && tg) KB_TRY(launch_tile_list(b.fr, n, k, b.olist, b.ocount, c.s));
             // Q_k is supported on rows within k-1 hops of W; L Q_k within k hops
             // block SpMM: W = L Q_k
             LinEpi<T> e;
@@ -330,6 +346,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             RowArgs<T> pa;
             pa.n = n; pa.x = b.wbuf; pa.qa = Qk; pa.partials = b.parts; pa.ctrl = b.ctrl;
             within(pa, k - 1);   // (Q_k is zero elsewhere)
+            in_order(pa, k);
             KB_TRY(launch_rowblock<T>(RB_PROJ, W, pa, c.s, &grid, M));
             KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl));
             KB_TRY(launch_hkk<C>(b.Gsum, M, W, b.Hd + size_t(k - 1) * M * M, Cb, b.ctrl, c.s));
@@ -340,6 +357,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             ua.n = n; ua.x = b.wbuf; ua.qa = Qp; ua.ca = Bp; ua.qb = Qk; ua.cb = Cb;
             ua.out = X; ua.partials = b.parts; ua.ctrl = b.ctrl;
             within(ua, k);
+            in_order(ua, k);
             ua.lim_a = k - 2; ua.lim_b = k - 1; ua.tri_a = 1;   // (H_{k-1,k} is lower triangular)
             KB_TRY(launch_rowblock<T>(RB_UPD, W, ua, c.s, &grid, M));
             KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl));
@@ -379,6 +397,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                         ra.n = n; ra.x = X; ra.qa = b.basis + j * bs; ra.partials = b.parts;
                         ra.ctrl = b.ctrl; ra.skip = skip;
                         within(ra, j);
+                        in_order(ra, k);
                         KB_TRY(launch_rowblock<T>(RB_PROJ, W, ra, c.s, &grid, M));
                         KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl,
                                                 b.Cstk + size_t(j) * W * W, skip));
@@ -387,21 +406,29 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                     sa.n = n; sa.x = X; sa.basis = b.basis; sa.block_stride = bs; sa.nblk = k;
                     sa.ca = b.Cstk; sa.out = X; sa.partials = b.parts; sa.ctrl = b.ctrl; sa.skip = skip;
                     within(sa, k);
+                    in_order(sa, k);
                     KB_TRY(launch_rowblock<T>(RB_ASMSUB, W, sa, c.s, &grid, M));
                     KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl, nullptr, skip));
                     if (pass == 0) KB_TRY(launch_reorth_decide(b.Gsum, b.reo_d0, M, W, b.reo_skip, c.s));
                 }
             }
             // reduced QR: X = Q_{k+1} H_{k+1,k} by CholeskyQR2
-            KB_TRY(launch_chol<C>(b.Gsum, M, W, 1, k, inv_thresh2, piv2, b.R1, S1, nullptr,
-                                  nullptr, b.ctrl, c.s));
+            auto chol = [&](int pass, C *Rinv, double *Hs, C *B) -> int {
+                if constexpr (std::is_same<T, float>::value) {
+                    if (ord)
+                        return launch_chol_ordered(b.Gsum, M, W, pass, k, inv_thresh2, piv2, b.R1, Rinv, Hs, B,
+                                                   b.ctrl, c.s);
+                }
+                return launch_chol<C>(b.Gsum, M, W, pass, k, inv_thresh2, piv2, b.R1, Rinv, Hs, B, b.ctrl, c.s);
+            };
+            KB_TRY(chol(1, S1, nullptr, nullptr));
             RowArgs<T> ma;
             ma.n = n; ma.x = X; ma.ca = S1; ma.out = X; ma.partials = b.parts; ma.ctrl = b.ctrl;
             within(ma, k);
+            in_order(ma, k);
             KB_TRY(launch_rowblock<T>(RB_MULGRAM, W, ma, c.s, &grid, M));
             KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl));
-            KB_TRY(launch_chol<C>(b.Gsum, M, W, 2, k, inv_thresh2, piv2, b.R1, S2,
-                                  b.Hs + size_t(k - 1) * M * M, Bk, b.ctrl, c.s));
+            KB_TRY(chol(2, S2, b.Hs + size_t(k - 1) * M * M, Bk));
             RowArgs<T> qa;
             qa.n = n; qa.x = X; qa.ca = S2; qa.out = X; qa.ctrl = b.ctrl;
             within(qa, k);
@@ -892,7 +919,8 @@ int apply_device(kb_graph *g, kb_method method, kb_phi phi, const kb_params *par
     // M = 16 (16 MiB), cheb 321 / 552, cbl 2558 / 3598.  FP64 products cost some 16 times as
     // much per row.
     const int64_t blk_bytes = g->dev.n * width_for(std::min(M, 128)) * (params->basis == KB_F64 ? 128 : 4);
-    c.frontier = !params->no_frontier && m <= FRONTIER_MAX_HOPS && blk_bytes >= (int64_t(16) << 20);
+    c.ordered = method == KB_CBL && params->reorth == 1 && params->basis == KB_F32 ? 1 : 0;
+    c.frontier = !params->no_frontier && m <= FRONTIER_MAX_HOPS && (blk_bytes >= (int64_t(16) << 20) || c.ordered);
     c.tc = rowblock_tc_enabled() ? 1 : 0;
     const bool f64 = params->basis == KB_F64;
     const bool bf16 = params->basis == KB_BF16;

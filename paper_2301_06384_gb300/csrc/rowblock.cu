@@ -12,6 +12,11 @@ KB_RB_EXT(float, 16) KB_RB_EXT(float, 32) KB_RB_EXT(float, 64) KB_RB_EXT(float, 
 KB_RB_EXT(double, 16) KB_RB_EXT(double, 32) KB_RB_EXT(double, 64)
 KB_RB_EXT(__nv_bfloat16, 16) KB_RB_EXT(__nv_bfloat16, 32) KB_RB_EXT(__nv_bfloat16, 64) KB_RB_EXT(__nv_bfloat16, 128)
 #undef KB_RB_EXT
+// rowblock_ordered.cu
+extern template int launch_ordered<16>(int, const RowArgs<float> &, cudaStream_t, int *);
+extern template int launch_ordered<32>(int, const RowArgs<float> &, cudaStream_t, int *);
+extern template int launch_ordered<64>(int, const RowArgs<float> &, cudaStream_t, int *);
+extern template int launch_ordered<128>(int, const RowArgs<float> &, cudaStream_t, int *);
 }  // namespace rb
 
 namespace {
@@ -88,7 +93,20 @@ int launch_rowblock(int mode, int W, const RowArgs<T> &a, cudaStream_t s, int *g
     // (launches under a device skip flag take the SIMT kernels, which read the flag)
     if constexpr (std::is_same<T, float>::value)
         tc = a.tc && !a.skip && rowblock_tc_supported(mode, W);
-    if (tc) {
+    bool done = false;
+    if constexpr (std::is_same<T, float>::value) {
+        if (a.ordered && !tc && mode != RB_MUL && mode != RB_ASM) {
+            done = true;
+            switch (W) {
+                case 16: rc = rb::launch_ordered<16>(mode, aa, s, grid_out); break;
+                case 32: rc = rb::launch_ordered<32>(mode, aa, s, grid_out); break;
+                case 64: rc = rb::launch_ordered<64>(mode, aa, s, grid_out); break;
+                default: rc = rb::launch_ordered<128>(mode, aa, s, grid_out); break;
+            }
+        }
+    }
+    if (done) {
+    } else if (tc) {
         // FP32 blocks of width 64: tensor-core kernel (rowblock_tc.cu)
         if constexpr (std::is_same<T, float>::value)
             rc = launch_rowblock_tc(mode, aa, s, rowblock_max_grid<T>(W), grid_out);

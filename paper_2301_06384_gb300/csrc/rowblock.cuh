@@ -25,6 +25,14 @@
 // FP32 sums have two levels (at most about 64 rows, then across tiles); the row groups are
 // combined in a fixed order at the end, one partial G per CTA, summed by k_reduce.
 //
+// Ordered form (ORD; FP32 solves with full reorthogonalisation).  Full reorthogonalisation is
+// asked for where the result is sensitive to the rounding of the basis: with the spline kernel
+// on hub graphs (BA, 5e5 rows, (0.1 I + L)^{-2}) another order of the Gram sums, no less
+// accurate, moves single entries of Y by 10^-3 to 10^-2 of their root mean square.  Such
+// solves keep one order of every FP32 sum: the rows of a tile of 4096 / W one after the other
+// (one row group), a CTA's tiles by rising index from the step's list in index order, a fixed
+// number of CTAs per SM.  (Products have no freedom: a chain over k per entry.)
+//
 // Bound: the shared-memory data path (8 x 4 register tiles: 12 16-byte loads of 4 wavefronts
 // per 128 FMAs) for W >= 64, HBM below; the FP64 pipe in FP64.
 //
@@ -34,8 +42,8 @@
 //                                    now                      42.3   117.7     63.2    34.5
 //   128^3 grid, M = 32, 40 steps,    before                  242.8   451.8    291.6   155.8
 //                                    now                      71.7   219.6    103.5    59.5
-//   BA 5e5 rows, M = 128,            before                  280.8  1675.7    962.6   665.5
-//                                    now                     327.3  1230.4    678.0   330.8
+//   BA 5e5 rows, M = 128, ordered,   before                  280.8  1675.7    962.6   665.5
+//                                    now                     209.2  1129.1    634.4   329.6
 //   RGG 10^5 rows, M = 33, FP64,     before                  477.6  1193.7    743.4   305.1
 //                                    now                     113.5   234.1    136.6    67.8
 #pragma once
@@ -60,6 +68,22 @@ __device__ __forceinline__ void ld4(const C *p, C (&v)[4]) {
         const double2 a = reinterpret_cast<const double2 *>(p)[0];
         const double2 b = reinterpret_cast<const double2 *>(p)[1];
         v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+    }
+}
+// N consecutive elements (N = 1, 2 or a multiple of 4)
+template <typename C, int N>
+__device__ __forceinline__ void ldn(const C *p, C (&v)[N]) {
+    if constexpr (N % 4 == 0) {
+#pragma unroll
+        for (int u = 0; u < N; u += 4) {
+            C t[4];
+            ld4<C>(p + u, t);
+#pragma unroll
+            for (int w = 0; w < 4; ++w) v[u + w] = t[w];
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < N; ++u) v[u] = p[u];
     }
 }
 template <typename C>
@@ -105,7 +129,7 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-template <typename T, int W>
+template <typename T, int W, bool ORD = false>
 struct Geo {
     using C = typename Cmp<T>::type;
     static constexpr int VEC = 16 / int(sizeof(C));
@@ -115,7 +139,10 @@ struct Geo {
     static constexpr int LDO = W + VEC;
     static constexpr bool TWO = sizeof(C) == 4;           // two-level Gram sums
     static constexpr bool G2S = W == 128;                 // second level in shared memory
-    static constexpr int BI = 8, BJ = G2S ? 8 : 4;        // Gram block of a thread
+    static constexpr int BI = ORD ? W / 16 : 8, BJ = ORD ? W / 16 : G2S ? 8 : 4;   // Gram block of a thread
+    static constexpr int TO = 4096 / W;                   // ORD: rows of a tile
+    static constexpr int SO = W == 128 ? 2 : 1;           // ORD: such tiles of a virtual tile
+    static constexpr int CTAS = W >= 128 ? 2 : W >= 32 ? 4 : 3;   // ORD: CTAs per SM
     static constexpr int PR = 2048 / W;                   // rows of a PROJ chunk
 };
 
@@ -124,9 +151,9 @@ struct RowGeo {
     int Mk, CG, RG, TR;      // columns in use (multiple of 4), column groups, row groups, rows
     int NI, NJ, NB, NGR;     // Gram blocks along i and j, their number, row groups of the Gram
 };
-template <typename T, int W, int MODE, int RPT>
+template <typename T, int W, int MODE, int RPT, bool ORD = false>
 __host__ __device__ inline RowGeo row_geo(int M) {
-    using G = Geo<T, W>;
+    using G = Geo<T, W, ORD>;
     RowGeo r;
     r.Mk = (M + 3) / 4 * 4;
     r.CG = r.Mk / 4;
@@ -134,18 +161,19 @@ __host__ __device__ inline RowGeo row_geo(int M) {
     int tr = (RB_THREADS / r.CG) * RPT;
     tr = (tr < cap ? tr : cap) / 32 * 32;
     r.TR = tr < 32 ? 32 : tr;
+    if (ORD) r.TR = G::TO * G::SO;
     r.RG = r.TR / RPT;
     r.NI = (M + G::BI - 1) / G::BI;
     r.NJ = (M + G::BJ - 1) / G::BJ;
     if (MODE == RB_PROJ) r.NB = r.NI * r.NJ;
-    else if (G::BJ == 8) r.NB = r.NI * (r.NI + 1) / 2;
+    else if (G::BJ == G::BI) r.NB = r.NI * (r.NI + 1) / 2;
     else {
         // blocks (bi, bj) with bj >= 2 bi
         r.NB = 0;
         for (int b = 0; b < r.NI; ++b) r.NB += r.NJ - 2 * b;
     }
     r.NGR = RB_THREADS / r.NB;
-    if (r.NGR < 1) r.NGR = 1;
+    if (ORD || r.NGR < 1) r.NGR = 1;
     return r;
 }
 template <typename T, int W, int MODE>
@@ -154,9 +182,9 @@ __host__ __device__ inline size_t stage_elems(const RowGeo &r) {
     if (MODE == RB_PROJ) return size_t(2) * G::PR * W;
     return size_t(r.TR) * G::LDA + size_t(G::KC) * W;
 }
-template <typename T, int W, int MODE>
+template <typename T, int W, int MODE, bool ORD>
 inline size_t smem_bytes(const RowGeo &r) {
-    using G = Geo<T, W>;
+    using G = Geo<T, W, ORD>;
     using C = typename G::C;
     const bool gram = MODE == RB_PROJ || MODE == RB_UPD || MODE == RB_MULGRAM || MODE == RB_ASMSUB;
     size_t e = NST * stage_elems<T, W, MODE>(r);
@@ -169,10 +197,10 @@ inline size_t smem_bytes(const RowGeo &r) {
     return e * sizeof(C);
 }
 
-template <typename T, int W, int MODE, int RPT>
+template <typename T, int W, int MODE, int RPT, bool ORD>
 __global__ void __launch_bounds__(RB_THREADS, sizeof(typename Cmp<T>::type) == 8 ? 1 : 2)
 k_rowblock(RowArgs<T> a) {
-    using G = Geo<T, W>;
+    using G = Geo<T, W, ORD>;
     using C = typename G::C;
     constexpr bool PROD = MODE != RB_PROJ;
     constexpr bool GRAM = MODE == RB_PROJ || MODE == RB_UPD || MODE == RB_MULGRAM || MODE == RB_ASMSUB;
@@ -184,7 +212,7 @@ k_rowblock(RowArgs<T> a) {
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *sm = reinterpret_cast<C *>(smem_raw);
-    const RowGeo q = row_geo<T, W, MODE, RPT>(a.M);
+    const RowGeo q = row_geo<T, W, MODE, RPT, ORD>(a.M);
     const int SE = int(stage_elems<T, W, MODE>(q));
     C *sO = sm + NST * SE;                                          // [TR][LDO]
     C *sG = PROD ? sO + q.TR * LDO : sO;                            // [NGR * NB][BI * BJ] (W = 128)
@@ -194,6 +222,19 @@ k_rowblock(RowArgs<T> a) {
     const int64_t cnt = a.alist && (MODE != RB_ASM || a.accumulate) ? int64_t(*a.acount) : nt;
     auto tile_at = [&](int64_t i) -> int64_t {
         return i >= cnt ? -1 : (a.alist ? int64_t(__ldg(a.alist + i)) : i);
+    };
+
+    // Ordered form: positions of the step's list (or tiles of TO rows without one); a tile of
+    // several listed frontier tiles is taken at the first of them.
+    constexpr int AO = ORD ? G::TO / ACT_ROWS : 1;
+    const int64_t olen = ORD ? (a.alist ? int64_t(*a.acount) : (a.n + G::TO - 1) / G::TO) : 0;
+    auto otile = [&](int64_t i) -> int64_t {
+        return i >= olen ? -1 : (a.alist ? int64_t(__ldg(a.alist + i)) / AO : i);
+    };
+    auto onorm = [&](int64_t i) -> int64_t {
+        if (AO > 1 && a.alist)
+            while (i < olen && i > 0 && otile(i - 1) == otile(i)) i += gridDim.x;
+        return i;
     };
 
     // ---- Gram state
@@ -256,20 +297,8 @@ k_rowblock(RowArgs<T> a) {
 #pragma unroll 2
                 for (int r = grp; r < R; r += q.NGR) {
                     C av[BI], bv[BJ];
-#pragma unroll
-                    for (int u = 0; u < BI; u += 4) {
-                        C t[4];
-                        ld4<C>(left + r * ld + gi0 + u, t);
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) av[u + v] = t[v];
-                    }
-#pragma unroll
-                    for (int u = 0; u < BJ; u += 4) {
-                        C t[4];
-                        ld4<C>(right + r * ld + gj0 + u, t);
-#pragma unroll
-                        for (int v = 0; v < 4; ++v) bv[u + v] = t[v];
-                    }
+                    ldn<C, BI>(left + r * ld + gi0, av);
+                    ldn<C, BJ>(right + r * ld + gj0, bv);
 #pragma unroll
                     for (int i = 0; i < BI; ++i)
 #pragma unroll
@@ -279,7 +308,7 @@ k_rowblock(RowArgs<T> a) {
                         }
                 }
             }
-            if constexpr (G::TWO) {
+            if constexpr (G::TWO && !ORD) {
                 grows += R / q.NGR;
                 if (grows >= 32) flush();
             }
@@ -325,10 +354,49 @@ k_rowblock(RowArgs<T> a) {
             const int c = q.Mk + i % (W - q.Mk), r = i / (W - q.Mk);
             sm[r * W + c] = C(0);
         }
-        int64_t ch = blockIdx.x;
-        int64_t pf = ch;
-        for (int s = 0; s < NST - 1; ++s, pf += gridDim.x) issue(pf, s);
         int st = 0;
+        if constexpr (ORD) {
+            // the two chunks of each tile, one flush per tile
+            int64_t pvt = onorm(blockIdx.x);
+            int ph = 0;
+            auto issue_o = [&](int s) {
+                if (pvt < olen) {
+                    C *dx = sm + s * SE, *dq = dx + PR * W;
+                    const int64_t r0 = otile(pvt) * G::TO + ph * PR;
+                    for (int i = tid; i < PR * W / VEC; i += RB_THREADS) {
+                        const int r = i / (W / VEC), c = (i % (W / VEC)) * VEC;
+                        if (c >= q.Mk) continue;
+                        const bool in = r0 + r < a.n;
+                        const int64_t off = in ? (r0 + r) * W + c : 0;
+                        cp16(dx + r * W + c, a.x + off, in);
+                        cp16(dq + r * W + c, a.qa + off, in);
+                    }
+                    ph ^= 1;
+                    if (ph == 0) pvt = onorm(pvt + gridDim.x);
+                }
+                cp_commit();
+            };
+            for (int s = 0; s < NST - 1; ++s) issue_o(s);
+            for (int64_t vt = onorm(blockIdx.x); vt < olen; vt = onorm(vt + gridDim.x)) {
+                for (int h = 0; h < G::TO / PR; ++h) {
+                    cp_wait<NST - 2>();
+                    __syncthreads();
+                    issue_o(st == 0 ? NST - 1 : st - 1);
+                    const C *dx = sm + st * SE;
+                    gram_rows(dx + PR * W, dx, W, PR);
+                    st = st + 1 == NST ? 0 : st + 1;
+                }
+                flush();
+                if (tid == 0) {
+                    my_rows += G::TO;
+                    my_units += G::TO;
+                }
+            }
+        }
+        int64_t ch = ORD ? nch : blockIdx.x;
+        int64_t pf = ch;
+        if (!ORD)
+            for (int s = 0; s < NST - 1; ++s, pf += gridDim.x) issue(pf, s);
         for (; ch < nch; ch += gridDim.x, pf += gridDim.x) {
             cp_wait<NST - 2>();
             __syncthreads();
@@ -356,7 +424,21 @@ k_rowblock(RowArgs<T> a) {
             cmax = max(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
         }
         const int nsub = q.TR / ACT_ROWS;
-        const int64_t nvt = (cnt + nsub - 1) / nsub;
+        const int64_t nvt = ORD ? olen : (cnt + nsub - 1) / nsub;
+        const int64_t vt0 = ORD ? onorm(blockIdx.x) : int64_t(blockIdx.x);
+        auto vt_next = [&](int64_t vt) -> int64_t {
+            return ORD ? onorm(vt + int64_t(gridDim.x) * G::SO) : vt + gridDim.x;
+        };
+        // 32-row tile `u` of a virtual tile, -1 past the end
+        auto vt_tile = [&](int64_t vt, int u) -> int64_t {
+            if constexpr (ORD) {
+                const int64_t t = otile(vt + int64_t(u / AO) * gridDim.x);
+                const int64_t f = t * AO + u % AO;
+                return t < 0 || f >= nt ? -1 : f;
+            } else {
+                return tile_at(vt * nsub + u);
+            }
+        };
         int nkb = 1;
         if (MODE == RB_UPD) nkb = a.qa ? 2 : 1;
         if (MODE == RB_ASM) nkb = a.ctrl ? min(a.ctrl->steps, a.nblk) : a.nblk;
@@ -366,19 +448,19 @@ k_rowblock(RowArgs<T> a) {
             if (!MULTI || !a.tgen) return 0;
             int m = INT_MAX;
             for (int u = 0; u < nsub; ++u) {
-                const int64_t t = tile_at(vt * nsub + u);
+                const int64_t t = vt_tile(vt, u);
                 if (t >= 0) m = min(m, __ldg(a.tgen + t));
             }
             return min(max(m - a.kbase, 0), nkb);
         };
         // chunk cursor of the loads
-        int64_t pvt = blockIdx.x;
+        int64_t pvt = vt0;
         int pkb = 0, pk0 = 0;
         auto skip_empty = [&]() {
             while (pvt < nvt) {
                 pkb = first_kb(pvt);
                 if (pkb < nkb) break;
-                pvt += gridDim.x;
+                pvt = vt_next(pvt);
             }
             pk0 = 0;
         };
@@ -408,7 +490,7 @@ k_rowblock(RowArgs<T> a) {
                 for (int i = tid; i < q.TR * VPR; i += RB_THREADS) {
                     const int r = i / VPR, c = (i % VPR) * EPV;
                     if (pk0 + c >= q.Mk) continue;
-                    const int64_t t = tile_at(pvt * nsub + r / ACT_ROWS);
+                    const int64_t t = vt_tile(pvt, r / ACT_ROWS);
                     const int64_t row = t * ACT_ROWS + r % ACT_ROWS;
                     const bool in = t >= 0 && row < a.n && (!a.tgen || lim == INT_MAX || __ldg(a.tgen + t) <= lim);
                     const int64_t off = in ? row * W + pk0 + c : 0;
@@ -427,7 +509,7 @@ k_rowblock(RowArgs<T> a) {
                 if (pk0 >= q.Mk) {
                     pk0 = 0;
                     if (++pkb >= nkb) {
-                        pvt += gridDim.x;
+                        pvt = vt_next(pvt);
                         skip_empty();
                     }
                 }
@@ -439,10 +521,10 @@ k_rowblock(RowArgs<T> a) {
             sO[(i / (LDO - q.Mk)) * LDO + q.Mk + i % (LDO - q.Mk)] = C(0);
         for (int s = 0; s < NST - 1; ++s) issue(s);
         int st = 0;
-        for (int64_t vt = blockIdx.x; vt < nvt; vt += gridDim.x) {
+        for (int64_t vt = vt0; vt < nvt; vt = vt_next(vt)) {
             const int kb0 = first_kb(vt);
             if (tid == 0) {
-                const int64_t rows = min(int64_t(q.TR), (cnt - vt * nsub) * ACT_ROWS);
+                const int64_t rows = ORD ? q.TR : min(int64_t(q.TR), (cnt - vt * nsub) * ACT_ROWS);
                 my_rows += rows;
                 my_units += (unsigned long long)(rows) * (nkb - kb0);
             }
@@ -456,7 +538,7 @@ k_rowblock(RowArgs<T> a) {
 #pragma unroll
                 for (int r = 0; r < RPT; ++r) {
                     const int lr = rg + q.RG * r;
-                    const int64_t t = tile_at(vt * nsub + lr / ACT_ROWS);
+                    const int64_t t = vt_tile(vt, lr / ACT_ROWS);
                     const int64_t row = t * ACT_ROWS + lr % ACT_ROWS;
                     if (t >= 0 && row < a.n)
 #pragma unroll
@@ -509,7 +591,7 @@ k_rowblock(RowArgs<T> a) {
                     const int lr = rg + q.RG * r;
                     C o[4];
                     if (SUBX) {
-                        const int64_t t = tile_at(vt * nsub + lr / ACT_ROWS);
+                        const int64_t t = vt_tile(vt, lr / ACT_ROWS);
                         const int64_t row = t * ACT_ROWS + lr % ACT_ROWS;
                         C xv[4] = {0, 0, 0, 0};
                         if (t >= 0 && row < a.n) ldg4<T>(a.x + row * W + col4, xv);
@@ -532,7 +614,7 @@ k_rowblock(RowArgs<T> a) {
             constexpr int CPR = W / 4;
             for (int i = tid; i < q.TR * CPR; i += RB_THREADS) {
                 const int r = i / CPR, c = (i % CPR) * 4;
-                const int64_t t = tile_at(vt * nsub + r / ACT_ROWS);
+                const int64_t t = vt_tile(vt, r / ACT_ROWS);
                 const int64_t row = t * ACT_ROWS + r % ACT_ROWS;
                 if (t < 0 || row >= a.n) continue;
                 C o[4];
@@ -550,7 +632,15 @@ k_rowblock(RowArgs<T> a) {
                     stg4<T>(a.out + row * W + c, o);
                 }
             }
-            gram_rows(sO, sO, LDO, q.TR);
+            if constexpr (ORD) {
+#pragma unroll
+                for (int u = 0; u < G::SO; ++u) {
+                    gram_rows(sO + u * G::TO * LDO, sO + u * G::TO * LDO, LDO, G::TO);
+                    flush();
+                }
+            } else {
+                gram_rows(sO, sO, LDO, q.TR);
+            }
         }
         cp_wait<0>();
         __syncthreads();
@@ -561,7 +651,7 @@ k_rowblock(RowArgs<T> a) {
     }
     if constexpr (GRAM) {
         // combine the row groups in a fixed order and write this CTA's W x W partial
-        if constexpr (G::TWO) flush();
+        if constexpr (G::TWO && !ORD) flush();
         C *comb = G::G2S ? sG : sm;
         const int nth = q.NB * q.NGR;
         if constexpr (!G::G2S) {
@@ -597,26 +687,28 @@ constexpr int RB_MAX_CTAS = 4;   // per SM: bounds the Gram partials
 
 // Resident CTAs per SM of an instance with smem bytes of dynamic shared memory.  The attribute
 // is raised once per instance to the most any block can take.
-template <typename T, int W, int MODE, int RPT>
+template <typename T, int W, int MODE, int RPT, bool ORD>
 int occupancy(size_t smem) {
     static const cudaError_t attr = cudaFuncSetAttribute(
-        k_rowblock<T, W, MODE, RPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        k_rowblock<T, W, MODE, RPT, ORD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     (void)attr;
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rowblock<T, W, MODE, RPT>, RB_THREADS, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rowblock<T, W, MODE, RPT, ORD>, RB_THREADS, smem);
     return std::max(1, std::min(per_sm, RB_MAX_CTAS));
 }
 
-template <typename T, int W, int MODE, int RPT>
+template <typename T, int W, int MODE, int RPT, bool ORD = false>
 int launch_r(const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
-    const RowGeo q = row_geo<T, W, MODE, RPT>(a.M);
-    const size_t smem = smem_bytes<T, W, MODE>(q);
-    const int64_t unit = MODE == RB_PROJ ? Geo<T, W>::PR : q.TR;
+    using G = Geo<T, W, ORD>;
+    const RowGeo q = row_geo<T, W, MODE, RPT, ORD>(a.M);
+    const size_t smem = smem_bytes<T, W, MODE, ORD>(q);
+    const int64_t unit = ORD ? G::TO : MODE == RB_PROJ ? G::PR : q.TR;
     const int64_t nvt = (a.n + unit - 1) / unit;
-    int grid = int(std::min<int64_t>(nvt, int64_t(num_sms()) * occupancy<T, W, MODE, RPT>(smem)));
+    const int per_sm = occupancy<T, W, MODE, RPT, ORD>(smem);
+    int grid = int(std::min<int64_t>(nvt, int64_t(num_sms()) * (ORD ? G::CTAS : per_sm)));
     if (grid < 1) grid = 1;
     if (grid_out) *grid_out = grid;
-    k_rowblock<T, W, MODE, RPT><<<grid, RB_THREADS, smem, s>>>(a);
+    k_rowblock<T, W, MODE, RPT, ORD><<<grid, RB_THREADS, smem, s>>>(a);
     return 0;
 }
 
@@ -645,6 +737,19 @@ int launch_w(int mode, const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
         case RB_ASMSUB: return launch_mode<T, W, RB_ASMSUB>(a, s, grid_out);
     }
     return fail(KB_ERR_ARG, "bad row-block mode");
+}
+
+// Ordered form: the modes with a Gram.
+template <int W>
+int launch_ordered(int mode, const RowArgs<float> &a, cudaStream_t s, int *grid_out) {
+    constexpr int R = W == 128 ? 8 : 4;
+    switch (mode) {
+        case RB_PROJ: return launch_r<float, W, RB_PROJ, R, true>(a, s, grid_out);
+        case RB_UPD: return launch_r<float, W, RB_UPD, R, true>(a, s, grid_out);
+        case RB_MULGRAM: return launch_r<float, W, RB_MULGRAM, R, true>(a, s, grid_out);
+        case RB_ASMSUB: return launch_r<float, W, RB_ASMSUB, R, true>(a, s, grid_out);
+    }
+    return fail(KB_ERR_ARG, "bad ordered row-block mode");
 }
 
 }  // namespace rb
