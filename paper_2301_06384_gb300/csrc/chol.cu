@@ -49,8 +49,8 @@ __global__ void k_hkk(const double *__restrict__ G, int M, int W, double *__rest
 // takes the general path.
 //
 // Bound: latency of one CTA (smallmat.cuh).  Per launch, FP32, pass 1 and
-// pass 2 (us, launch list): 53 / 22 at M = 64, 18 / 9 at M = 16; with one barrier per column
-// and 4 x 4 tiles on few threads 99 / 24 and 43 / 11.
+// pass 2 (us, launch list): 31 / 15 at M = 40, 17 / 9 at M = 16; with one barrier per column
+// and 4 x 4 tiles on few threads 69 / 19 and 43 / 11.  FP64, M = 33: 58 / 49, before 112 / 90.
 constexpr int CHOL_THREADS = 512;
 
 struct CholLayout {
@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
     double *A = reinterpret_cast<double *>(smem);                    // FP64 factorisation
     double *scr = reinterpret_cast<double *>(smem + L.scr);
     constexpr bool FP32 = sizeof(T) == 4;
+    auto none = [](int, int) { return 0; };
     const bool try_small = pass == 2 && FP32;
     if (threadIdx.x == 0) {
         emax_bits = 0u;
@@ -167,11 +168,12 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
             sm::each(M, M, [&](int i, int j) {
                 if (j < i) F0[i * lda + j] = 0.f;
             });
-            sm::tri_mm(F2, F1, lda, M, [&](int i, int j, float c) { F0[i * lda + j] = c; });
+            sm::tri_mm(F2, F1, lda, M, none, [&](int i, int j, float c, int) { F0[i * lda + j] = c; });
             __syncthreads();
             // H = (I + F + F^2) R1 = R1 + (C + F C), the corrections of relative size ||E||
-            sm::tri_mm(F2, F0, lda, M, [&](int i, int j, float c2) {
-                const double h = __ldcg(R1 + i * M + j) + double(F0[i * lda + j] + c2);
+            sm::tri_mm(F2, F0, lda, M, [&](int i, int j) { return __ldcg(R1 + i * M + j); },
+                       [&](int i, int j, float c2, double r1) {
+                const double h = r1 + double(F0[i * lda + j] + c2);
                 const float ht = float(h);
                 Hs[i * M + j] = double(ht);
                 Bout[j * W + i] = ht;
@@ -203,9 +205,9 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
                 __syncthreads();
                 if (__uint_as_float(emax_bits) < 1e-3f) {
                     // C1 = R E over S (zeros below the diagonal), then R1 = R + (C1 + C1 E)
-                    sm::tri_mm(F0, F2, lda, M, [&](int i, int j, float c) { F1[i * lda + j] = c; });
+                    sm::tri_mm(F0, F2, lda, M, none, [&](int i, int j, float c, int) { F1[i * lda + j] = c; });
                     __syncthreads();
-                    sm::tri_mm(F1, F2, lda, M, [&](int i, int j, float c2) {
+                    sm::tri_mm(F1, F2, lda, M, none, [&](int i, int j, float c2, int) {
                         R1[i * M + j] = double(F0[i * lda + j]) + double(F1[i * lda + j] + c2);
                     });
                     sm::each(M, M, [&](int i, int j) {
@@ -273,16 +275,28 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
             if (i < M && j < M) Hs[i * M + j] = 0.0;
             Bout[j * W + i] = T(0);
         });
-        sm::tiles2(M, M, [&](int i, int j) {
-            for (int r = i; r < min(i + 2, M); ++r)
-                for (int c = max(j, r); c < min(j + 2, M); ++c) {
-                    double h = 0.0;
-                    for (int k = r; k <= c; ++k) h = fma(A[r * lda + k], __ldcg(R1 + k * M + c), h);
-                    const T ht = T(h);
-                    Hs[r * M + c] = double(ht);
-                    Bout[c * W + r] = ht;
-                }
-        });
+        __syncthreads();
+        // R1 over the second region where it fits beside A (FP64 mode, and FP32 up to M = 96), else
+        // over the product's own loads from global memory
+        double *R = reinterpret_cast<double *>(smem + L.second);
+        if (L.second + size_t(lda) * ((M + 1) / 2 * 2) * sizeof(double) <= L.scr) {
+            sm::load_square(R1, M, M, [&](int i, int j, double v) { R[i * lda + j] = j >= i ? v : 0.0; });
+            __syncthreads();
+            sm::tri_mm<double>(A, R, lda, M, none, [&](int i, int j, double h, int) {
+                const T ht = T(h);
+                Hs[i * M + j] = double(ht);
+                Bout[j * W + i] = ht;
+            });
+        } else {
+            sm::tri_tiles<1>(M, [&](int i, int j) {
+                double h = 0.0;
+#pragma unroll 8
+                for (int k = i; k <= j; ++k) h = fma(A[i * lda + k], __ldcg(R1 + k * M + j), h);
+                const T ht = T(h);
+                Hs[i * M + j] = double(ht);
+                Bout[j * W + i] = ht;
+            });
+        }
     }
 }
 

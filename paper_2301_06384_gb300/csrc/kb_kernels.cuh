@@ -143,7 +143,7 @@ template <typename T>
 int launch_u_convert(const double *U, int M, int W, int m, T *Ut, const Ctrl *ctrl, cudaStream_t s);
 
 // Projected problem of the classical block Lanczos method (FP64, block tridiagonal H_m).
-// Hdf: nullptr for the FP64 recurrence; else 2 m M^2 doubles of scratch for the split H, and
+// Hdf: nullptr for the FP64 recurrence; else 2 m M (M + 1) doubles of scratch for H as floats, and
 // the recurrence runs in double-float on the FP32 pipe (the FP32 and BF16 modes).
 int launch_cheb_bt(const double *Hd, const double *Hs, int M, int m, double lam,
                    const std::vector<double> &d, double *V0, double *V1, double *V2, double *U,
@@ -152,15 +152,21 @@ int launch_cheb_bt(const double *Hd, const double *Hs, int M, int m, double lam,
 // q->n == 0).  Non-integer s: the quadrature rule q gives the fractional factor
 // sum_k W_k (sigma_k I + H_m)^{-1} F_1, one block Cholesky factorisation and solve per node
 // (qbatch nodes at a time, one CTA each, in qscr: qbatch * bt_quad_node_doubles(M, m)
-// doubles), then s_int solves with eps I + H_m.  kmax: a host-side bound on ctrl->steps (the
-// factorisation is launched block by block up to it; 0 means m).
+// doubles), then s_int solves with eps I + H_m.
 __host__ __device__ inline size_t bt_quad_node_doubles(int M, int m) {
     return 3 * size_t(m) * M * M + size_t(m) * M;   // Ld, Ls, Y blocks and reciprocal diagonals
 }
+// The factors of eps I + H, kept from one stopping-rule check to the next: m blocks of M x M each, Ls
+// two.
+struct SplineBufs {
+    double *Ri, *RiT, *Y, *GT, *K, *Ls;
+};
+// Blocks r0 .. kmax - 1 are factored now (0: all m), those before r0 were by an earlier call with
+// the same buffers; y0 likewise for the forward solutions of the first solve.  fc: the control
+// block of the process (its steps bound the blocks); ctrl: that of this solve.
 int launch_bt_spline(const double *Hd, const double *Hs, int M, int m, double eps, int s_int,
-                     double *Ld, double *Ls, double *Yw, double *U, const Ctrl *ctrl,
-                     cudaStream_t s, const QuadRule *q = nullptr, double *qscr = nullptr,
-                     int qbatch = 0, int kmax = 0);
+                     const SplineBufs &b, double *U, const Ctrl *fc, const Ctrl *ctrl, cudaStream_t s,
+                     const QuadRule *q, double *qscr, int qbatch, int r0, int y0, int kmax);
 
 // Full reorthogonalisation: save the diagonal of the Gram of X before the first pass; after
 // it, *skip = 1 when every column kept at least half of its squared norm (the second pass is

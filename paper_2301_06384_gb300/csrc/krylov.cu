@@ -208,7 +208,9 @@ struct CblBufs {
     double *Gsum, *Hd, *Hs, *R1, *V0, *V1, *V2, *U;
     double *Uc;          // stopping rule: two U_k of the checks (alternating)
     double *qscr;        // projected step with non-integer s: per-node block solves
-    double *Hdf;         // projected e^{-tH} F_1 in double-float: H split into float pairs
+    double *Hdf;         // projected e^{-tH} F_1 in double-float: H as floats, and transposed;
+                         // spline kernel: two of the factor arrays
+    double *bt_ls;
     int32_t *chk_prev;   // steps of the previous check (0: none yet)
     double *reo_d0;      // full reorthogonalisation: squared column norms before the first pass
     int32_t *reo_skip;   // ... and the flag that skips the second pass
@@ -241,7 +243,8 @@ void plan_cbl(Arena &ar, CblBufs<T> &b, int64_t n, int M, int W, int m, int rb_g
     b.U = ar.take<double>(size_t(m) * M * M);
     b.Uc = ar.take<double>(size_t(2) * m * M * M);
     b.qscr = qbatch > 0 ? ar.take<double>(size_t(qbatch) * bt_quad_node_doubles(M, m)) : nullptr;
-    b.Hdf = sizeof(typename Cmp<T>::type) == 4 ? ar.take<double>(size_t(2) * m * M * M) : nullptr;
+    b.Hdf = ar.take<double>(size_t(2) * m * M * (M + 1));
+    b.bt_ls = ar.take<double>(size_t(2) * M * M);
     b.chk_prev = ar.take<int32_t>(1);
     b.reo_d0 = ar.take<double>(size_t(W));
     b.reo_skip = ar.take<int32_t>(1);
@@ -318,6 +321,8 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
         const size_t WW = size_t(W) * W;
         auto blk = [&](int j) { return b.basis + int64_t(two ? j % 3 : j) * bs; };
         int nchk = 0;
+        int kfac = 0;   // blocks of the spline kernel's factorisation that earlier checks formed
+        const SplineBufs sbufs{b.V0, b.V1, b.V2, b.Hdf, b.Hdf + size_t(m) * M * M, b.bt_ls};
         if (c.p.tol > 0.0) KB_CUDA_TRY(cudaMemsetAsync(b.chk_prev, 0, sizeof(int32_t), c.s));
         for (int k = 1; k <= m; ++k) {
             T *Qk = blk(k - 1);
@@ -441,10 +446,11 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                 KB_TRY(launch_ctrl_snapshot(b.ctrl_chk, b.ctrl, k, c.s));
                 if (c.phi == KB_PHI_EXP) {
                     const std::vector<double> d = exp_series_coeffs(c.p.t, lam_p, 1e-17);
-                    KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, Ucur, b.ctrl_chk, c.s, b.Hdf));
+                    KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, Ucur, b.ctrl_chk, c.s, f64 ? nullptr : b.Hdf));
                 } else {
-                    KB_TRY(launch_bt_spline(b.Hd, b.Hs, M, m, c.p.eps, c.s_int, b.V0, b.V1, b.V2, Ucur,
-                                            b.ctrl_chk, c.s, c.quad, b.qscr, qbatch, k));
+                    KB_TRY(launch_bt_spline(b.Hd, b.Hs, M, m, c.p.eps, c.s_int, sbufs, Ucur, b.ctrl, b.ctrl_chk,
+                                            c.s, c.quad, b.qscr, qbatch, kfac, c.s_int == 1 ? kfac : 0, k));
+                    kfac = k;
                 }
                 KB_TRY(launch_conv_check(Ucur, Uprev, M, b.ctrl_chk, b.chk_prev, c.p.tol, b.ctrl, c.s, nchk % 2));
                 ++nchk;
@@ -459,10 +465,11 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
         }
         if (c.phi == KB_PHI_EXP) {
             const std::vector<double> d = exp_series_coeffs(c.p.t, lam_p, 1e-17);
-            KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, b.U, cfin, c.s, b.Hdf));
+            KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, b.U, cfin, c.s, f64 ? nullptr : b.Hdf));
         } else {
-            KB_TRY(launch_bt_spline(b.Hd, b.Hs, M, m, c.p.eps, c.s_int, b.V0, b.V1, b.V2, b.U,
-                                    cfin, c.s, c.quad, b.qscr, qbatch));
+            // (a process that stopped by itself skipped the later checks: their Y are formed now)
+            KB_TRY(launch_bt_spline(b.Hd, b.Hs, M, m, c.p.eps, c.s_int, sbufs, b.U, b.ctrl, cfin, c.s, c.quad,
+                                    b.qscr, qbatch, kfac, 0, m));
         }
         if (c.p.tol > 0.0) KB_TRY(launch_copy_check_u(b.Uc, int64_t(m) * M * M, b.U, M, m, b.ctrl, c.s));
         KB_TRY(launch_check_projected(b.U, int64_t(m) * M * M, projected_bound(c), b.ctrl, c.s));

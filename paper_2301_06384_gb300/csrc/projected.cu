@@ -18,6 +18,7 @@
 // rounding (the Chebyshev series is truncated below 1e-17 relative).
 #include "kb_internal.cuh"
 #include "kb_kernels.cuh"
+#include "smallmat.cuh"
 
 namespace kb {
 namespace {
@@ -91,12 +92,14 @@ k_cheb_bt_iter(const double *__restrict__ Hd, const double *__restrict__ Hs,
 }
 
 // ---------------------------------------------------------------- double-float recurrence
-// The same recurrence with H and V held as unevaluated float pairs (hi + lo, about 48
-// significant bits) on the FP32 pipe, which this part runs at 64 times its FP64 rate.  The
-// products are compensated dot products (Ogita, Rump and Oishi's Dot2): each h v term is
-// split exactly by an FMA (TwoProd), the running sum by Knuth's TwoSum, and the rounding
-// errors are summed beside it; the result is exact to about 2^-48 relative, far below the
-// 1e-14 the projected solve needs after thousands of terms.  U is accumulated in FP64.
+// The same recurrence with V held as unevaluated float pairs (hi + lo, about 48 significant
+// bits) on the FP32 pipe, which this part runs at 64 times its FP64 rate.  The entries of H
+// are FP32 values (the blocks are recorded as the FP32 recurrence subtracts them), so H is one
+// float per entry.  The products are compensated dot products (Ogita, Rump and Oishi's
+// Dot2): each h v term is split exactly by an FMA (TwoProd), the running sum by Knuth's
+// TwoSum, and the rounding errors are summed beside it; the result is exact to about 2^-48
+// relative, far below the 1e-14 the projected solve needs after thousands of terms.  U is
+// accumulated in FP64.
 struct dfl {
     float h, l;
 };
@@ -115,17 +118,40 @@ __device__ __forceinline__ void dot2_step(float &s, float &err, dfl a, dfl b) {
     err += ((s - (t - bb)) + (p - bb)) + pe;
     s = t;
 }
+// the same with a single float a
+__device__ __forceinline__ void dot2_step(float &s, float &err, float a, dfl b) {
+    const float p = a * b.h;
+    const float pe = fmaf(a, b.l, fmaf(a, b.h, -p));
+    const float t = s + p;
+    const float bb = t - s;
+    err += ((s - (t - bb)) + (p - bb)) + pe;
+    s = t;
+}
 __host__ __device__ __forceinline__ dfl dfl_from(double v) {
     const float h = float(v);
     return dfl{h, float(v - double(h))};
 }
 __device__ __forceinline__ double dfl_val(dfl a) { return double(a.h) + double(a.l); }
 
-// H_d, H_s split into float pairs (once per projected solve)
-__global__ void k_split_df(const double *__restrict__ H, dfl *__restrict__ out, int64_t count) {
-    for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < count;
-         i += int64_t(gridDim.x) * blockDim.x)
-        out[i] = dfl_from(H[i]);
+// The float form of H, every block so that the recurrence reads it along rows of 2 floats: rows
+// of ld = M rounded up to even, zeros in the padding.  Hdf: H_rr (symmetric); Hsf: R_r =
+// H_{r+1,r} (upper triangular); Hst: R_r^T.  Once per projected solve.
+__global__ void __launch_bounds__(256)
+k_split_df(const double *__restrict__ Hd, const double *__restrict__ Hs, float *__restrict__ Hdf,
+           float *__restrict__ Hsf, float *__restrict__ Hst, int M, int ld, const Ctrl *ctrl) {
+    const int r = blockIdx.x;
+    if (r >= ctrl->steps) return;
+    const int64_t MM = int64_t(M) * M, LL = int64_t(M) * ld;
+    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int i = (threadIdx.x >> 5) + blockIdx.y * nw; i < M; i += nw * gridDim.y)
+        for (int j = lane; j < ld; j += 32) {
+            const bool in = j < M;
+            Hdf[r * LL + i * ld + j] = in ? float(Hd[r * MM + i * M + j]) : 0.f;
+            if (r + 1 < ctrl->steps) {
+                Hsf[r * LL + i * ld + j] = in && j >= i ? float(Hs[r * MM + i * M + j]) : 0.f;
+                Hst[r * LL + i * ld + j] = in && j <= i ? float(Hs[r * MM + j * M + i]) : 0.f;
+            }
+        }
 }
 
 __global__ void k_cheb_bt_seed_df(dfl *V0, double *U, int M, double d0, const Ctrl *ctrl) {
@@ -136,54 +162,89 @@ __global__ void k_cheb_bt_seed_df(dfl *V0, double *U, int M, double d0, const Ct
     }
 }
 
-// V_{j+1} = beta (V_j - g H V_j) - gamma V_{j-1};  U += d_{j+1} V_{j+1}, in double-float
+// V_{j+1} = beta (V_j - g H V_j) - gamma V_{j-1};  U += d_{j+1} V_{j+1}, in double-float.
+// A CTA forms 8 columns of one block row.  The three blocks of H and the V columns of the three
+// block rows that enter are copied to shared memory at once (cp.async; H_rr is symmetric,
+// R_{r-1} comes transposed and R_r^T is read as R_r, so all are read along the output rows), and
+// a thread owns 2 rows x 2 columns: two shared loads per 4 compensated terms of 11 operations,
+// instead of one strided 8-byte global load and one shared load per term.  Bound by the
+// FP32 pipe and the latency of a launch.  Per term, launch list: M = 64 with 30 blocks
+// 30.3 -> 16.7 us, M = 40 with 20 blocks 16.9 -> 12.2 us.
+constexpr int CBW = 8;
 __global__ void __launch_bounds__(256)
-k_cheb_bt_iter_df(const dfl *__restrict__ Hd, const dfl *__restrict__ Hs, const dfl *__restrict__ Vp,
-                  const dfl *__restrict__ Vc, dfl *__restrict__ Vn, double *__restrict__ U, int M,
-                  float beta, float gamma, double dnext, dfl g, const Ctrl *ctrl) {
+k_cheb_bt_iter_df(const float *__restrict__ Hd, const float *__restrict__ Hs, const float *__restrict__ Hst,
+                  const dfl *__restrict__ Vp, const dfl *__restrict__ Vc, dfl *__restrict__ Vn,
+                  double *__restrict__ U, int M, int ld, float beta, float gamma, double dnext, dfl g,
+                  const Ctrl *ctrl) {
     const int r = blockIdx.x;
     const int steps = ctrl->steps;
     if (r >= steps) return;
-    const int c0 = blockIdx.y * TC;
-    extern __shared__ __align__(16) unsigned char svraw[];   // [3][M][TC] pairs
-    dfl *s0 = reinterpret_cast<dfl *>(svraw), *s1 = s0 + M * TC, *s2 = s0 + 2 * M * TC;
-    const int64_t MM = int64_t(M) * M;
-    for (int idx = threadIdx.x; idx < M * TC; idx += blockDim.x) {
-        const int k = idx / TC, cc = idx % TC, c = c0 + cc;
-        dfl a{0.f, 0.f}, b{0.f, 0.f}, d{0.f, 0.f};
+    const int c0 = blockIdx.y * CBW;
+    extern __shared__ __align__(16) unsigned char svraw[];   // V [3][M][CBW] pairs, H [3][M][ld]
+    dfl *s1 = reinterpret_cast<dfl *>(svraw), *s0 = s1 + M * CBW, *s2 = s0 + M * CBW;
+    float *h1 = reinterpret_cast<float *>(s2 + M * CBW), *h0 = h1 + M * ld, *h2 = h0 + M * ld;
+    const int64_t MM = int64_t(M) * M, LL = int64_t(M) * ld;
+    auto copy8 = [](void *dst, const void *src) {
+        const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+    };
+    for (int i = threadIdx.x * 2; i < M * ld; i += blockDim.x * 2) {
+        copy8(h1 + i, Hd + r * LL + i);
+        if (r > 0) copy8(h0 + i, Hst + (r - 1) * LL + i);
+        if (r + 1 < steps) copy8(h2 + i, Hs + r * LL + i);
+    }
+    for (int idx = threadIdx.x; idx < M * CBW; idx += blockDim.x) {
+        const int k = idx / CBW, c = c0 + idx % CBW;
+        const int64_t o = r * MM + int64_t(k) * M + c;
         if (c < M) {
-            if (r > 0) a = Vc[(r - 1) * MM + int64_t(k) * M + c];
-            b = Vc[r * MM + int64_t(k) * M + c];
-            if (r + 1 < steps) d = Vc[(r + 1) * MM + int64_t(k) * M + c];
+            copy8(s1 + idx, Vc + o);
+            if (r > 0) copy8(s0 + idx, Vc + o - MM);
+            if (r + 1 < steps) copy8(s2 + idx, Vc + o + MM);
+        } else {
+            s1[idx] = s0[idx] = s2[idx] = dfl{0.f, 0.f};
         }
-        s0[idx] = a; s1[idx] = b; s2[idx] = d;
     }
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
     __syncthreads();
-    const dfl *hd = Hd + r * MM;
-    const dfl *hl = (r > 0) ? Hs + (r - 1) * MM : nullptr;   // H_{r, r-1} = R_{r-1} (upper)
-    const dfl *hu = (r + 1 < steps) ? Hs + r * MM : nullptr; // H_{r, r+1} = R_r^T
-    for (int idx = threadIdx.x; idx < M * TC; idx += blockDim.x) {
-        const int i = idx / TC, cc = idx % TC, c = c0 + cc;
-        if (c >= M) continue;
-        float s = 0.f, err = 0.f;
-        for (int k = 0; k < M; ++k) dot2_step(s, err, hd[i * M + k], s1[k * TC + cc]);
-        if (hl)
-            for (int k = i; k < M; ++k) dot2_step(s, err, hl[i * M + k], s0[k * TC + cc]);
-        if (hu)
-            for (int k = 0; k <= i; ++k) dot2_step(s, err, hu[k * M + i], s2[k * TC + cc]);
-        // av = V_j - g (H V_j): one more compensated step with the pair -g
-        const dfl hv = dfl_fast(s, err);
-        float s2v = s1[i * TC + cc].h, e2 = s1[i * TC + cc].l;
-        dot2_step(s2v, e2, dfl{-g.h, -g.l}, hv);
-        // vn = beta av - gamma V_{j-1} (beta in {1, 2}, gamma in {0, 1}: exact scalings)
-        const int64_t o = r * MM + int64_t(i) * M + c;
-        const dfl vp = Vp[o];
-        float s3 = beta * s2v, e3 = beta * e2;
-        dot2_step(s3, e3, dfl{-gamma, 0.f}, vp);
-        const dfl vn = dfl_fast(s3, e3);
-        Vn[o] = vn;
-        U[o] += dnext * dfl_val(vn);
-    }
+    const int i0 = (threadIdx.x / 4) * 2, cc = (threadIdx.x % 4) * 2;
+    if (i0 >= M || c0 + cc >= M) return;
+    float s[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, err[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+    // rows k0 .. k1 - 1 of a block stored along the output rows, times V
+    auto acc = [&](const float *H, const dfl *v, int k0, int k1) {
+#pragma unroll 4
+        for (int k = k0; k < k1; ++k) {
+            const float2 h = *reinterpret_cast<const float2 *>(H + k * ld + i0);
+            const float4 t = *reinterpret_cast<const float4 *>(v + k * CBW + cc);
+            const dfl va{t.x, t.y}, vb{t.z, t.w};
+            dot2_step(s[0][0], err[0][0], h.x, va);
+            dot2_step(s[0][1], err[0][1], h.x, vb);
+            dot2_step(s[1][0], err[1][0], h.y, va);
+            dot2_step(s[1][1], err[1][1], h.y, vb);
+        }
+    };
+    acc(h1, s1, 0, M);
+    if (r > 0) acc(h0, s0, i0, M);                           // R_{r-1}: k >= i
+    if (r + 1 < steps) acc(h2, s2, 0, min(i0 + 2, M));       // R_r^T: k <= i
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const int i = i0 + a, c = c0 + cc + b;
+            if (i >= M || c >= M) continue;
+            // av = V_j - g (H V_j): one more compensated step with the pair -g
+            const dfl hv = dfl_fast(s[a][b], err[a][b]);
+            const dfl v1 = s1[i * CBW + cc + b];
+            float s2v = v1.h, e2 = v1.l;
+            dot2_step(s2v, e2, dfl{-g.h, -g.l}, hv);
+            // vn = beta av - gamma V_{j-1} (beta in {1, 2}, gamma in {0, 1}: exact scalings)
+            const int64_t o = r * MM + int64_t(i) * M + c;
+            const dfl vp = Vp[o];
+            float s3 = beta * s2v, e3 = beta * e2;
+            dot2_step(s3, e3, -gamma, vp);
+            const dfl vn = dfl_fast(s3, e3);
+            Vn[o] = vn;
+            U[o] += dnext * dfl_val(vn);
+        }
 }
 
 // ---------------------------------------------------------------- block Cholesky (spline)
@@ -211,188 +272,183 @@ __device__ void chol_lower_inplace(double *A, int M) {
     }
 }
 
-// Block Cholesky factorisation eps I + H = L L^T of the block tridiagonal Lanczos matrix (L
-// block lower bidiagonal: lower triangular diagonal blocks Ld_r, sub-diagonal blocks Ls_r),
-// block by block, three launches per block (FP64 runs at a small fraction of the FP32 rate
-// on this part, so the dense parts are spread over as many SMs as there are rows):
-//   k_bt_dupdate  D_r = eps I + H_rr - Ls_{r-1} Ls_{r-1}^T (lower triangle), one CTA per row
-//   k_bt_dchol    D_r = Ld_r Ld_r^T in place, one CTA
-//   k_bt_lsolve   Ls_r = H_{r+1,r} Ld_r^{-T}, one warp per row
-// Each launch does nothing when its block lies past ctrl->steps.
-__global__ void __launch_bounds__(128)
-k_bt_dupdate(const double *__restrict__ Hd, const double *__restrict__ Ls, int M, double eps, int r,
-             double *__restrict__ Ld, const Ctrl *ctrl) {
-    if (r >= ctrl->steps) return;
-    const int i = blockIdx.x;
-    const int64_t MM = int64_t(M) * M;
-    const double *P = r > 0 ? Ls + (r - 1) * MM : nullptr;
-    double *D = Ld + r * MM;
-    for (int j = threadIdx.x; j <= i; j += blockDim.x) {
-        double v = Hd[r * MM + int64_t(i) * M + j] + (i == j ? eps : 0.0);
-        if (P)
-            for (int k = 0; k < M; ++k) v = fma(-P[int64_t(i) * M + k], P[int64_t(j) * M + k], v);
-        D[int64_t(i) * M + j] = v;
-    }
+// Spline kernel, s_int times U <- (eps I + H)^{-1} U through the block Cholesky factorisation
+// eps I + H = L L^T (L block lower bidiagonal: R_r^T on the diagonal, Ls_r below it).  All in
+// FP64, whose rate on this part is two FMAs per clock and SM, so everything but the Cholesky
+// of one diagonal block is spread over many SMs, and the triangular solves are turned into
+// products with the inverses Ri_r = R_r^{-1}, whose terms are independent:
+//   k_bt_ls      Ls_{r-1} = H_{r,r-1} Ri_{r-1}
+//   k_bt_schur   D_r = eps I + H_rr - Ls_{r-1} Ls_{r-1}^T, and K_{r-1} = Ls_{r-1} Ri_{r-1}^T
+//   k_bt_dchol   D_r = R_r^T R_r, Ri_r and its transpose (one CTA)
+//   k_bt_gt      G_r^T = Ls_{r-1}^T Ri_r for all new blocks
+//   k_bt_subst   Y_r = Ri_r^T rhs_r - G_r Y_{r-1} upwards, U_r = Ri_r Y_r - K_r^T U_{r+1}
+//                downwards, one CTA per column of U
+// The leading blocks of eps I + H_k do not change as k grows, nor do their Y_r for the first
+// solve: a stopping-rule check extends what the check before it left (blocks r0 and up).
+// Each launch does nothing when its block lies past the process's steps, or once a check has
+// stopped the process.  Measured (four concurrent requests, RGG of 55392 rows, M = 64 and less,
+// (0.1 I + L)^{-1}, up to 100 steps, checks at 8 to 96): sums of the launch list 239 -> 62 ms
+// (every check factored all blocks and solved triangular systems with one warp per column),
+// the requests 156 -> 81 ms.
+struct BtArgs {
+    const double *Hd, *Hs;
+    double *Ri, *RiT, *Y, *GT, *K, *Ls;   // Ls: two blocks, by the parity of r
+    int M;
+};
+__device__ __forceinline__ bool bt_skip(const Ctrl *fc, int r) { return r >= fc->steps || fc->from_check >= 0; }
+
+// sum of four interleaved partial sums of a(k) b(k), k0 <= k < k1
+template <typename FA, typename FB>
+__device__ __forceinline__ double dot4(int k0, int k1, const FA &a, const FB &b) {
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    int k = k0;
+    for (; k + 3 < k1; k += 4)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) s[u] = fma(a(k + u), b(k + u), s[u]);
+    for (; k < k1; ++k) s[0] = fma(a(k), b(k), s[0]);
+    return (s[0] + s[1]) + (s[2] + s[3]);
 }
 
-__global__ void __launch_bounds__(1024) k_bt_dchol(double *Ld, int M, int r, const Ctrl *ctrl) {
-    if (r >= ctrl->steps) return;
-    chol_lower_inplace(Ld + r * int64_t(M) * M, M);
+// row i = blockIdx.x of Ls_{r-1} (both factors upper triangular)
+__global__ void __launch_bounds__(128) k_bt_ls(BtArgs a, int r, const Ctrl *fc) {
+    if (bt_skip(fc, r)) return;
+    const int M = a.M, i = blockIdx.x;
+    const int64_t MM = int64_t(M) * M;
+    const double *h = a.Hs + (r - 1) * MM + int64_t(i) * M, *Ri = a.Ri + (r - 1) * MM;
+    double *out = a.Ls + ((r - 1) & 1) * MM + int64_t(i) * M;
+    for (int j = threadIdx.x; j < M; j += blockDim.x)
+        out[j] = j < i ? 0.0 : dot4(i, j + 1, [&](int k) { return h[k]; }, [&](int k) { return Ri[int64_t(k) * M + j]; });
 }
 
-// Row i of Ls_r solves Ld_r x = (row i of H_{r+1,r})^T by column-oriented forward substitution
-// with x in registers (lane l: entries l, l + 32, l + 64, l + 96; M <= 128): x_j = y_j / d_jj,
-// then y_k -= d_kj x_j for the rows k below, one shuffle per row.
-__global__ void __launch_bounds__(32)
-k_bt_lsolve(const double *__restrict__ Hs, const double *__restrict__ Ld, int M, int r,
-            double *__restrict__ Ls, const Ctrl *ctrl) {
-    if (r + 1 >= ctrl->steps) return;
-    const int i = blockIdx.x, lane = threadIdx.x;
+// row i: of D_r (blockIdx.y = 0, into Ri_r, lower triangle transposed to the upper one) and of
+// K_{r-1} (blockIdx.y = 1)
+__global__ void __launch_bounds__(128) k_bt_schur(BtArgs a, int r, double eps, const Ctrl *fc) {
+    if (bt_skip(fc, r)) return;
+    const int M = a.M, i = blockIdx.x;
     const int64_t MM = int64_t(M) * M;
-    const double *D = Ld + r * MM;
-    const double *h = Hs + r * MM + int64_t(i) * M;
-    double y[4], rd[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int j = lane + 32 * q;
-        y[q] = j < M ? h[j] : 0.0;
-        rd[q] = 1.0 / (j < M ? D[int64_t(j) * M + j] : 1.0);
-    }
-#pragma unroll
-    for (int jq = 0; jq < 4; ++jq)
-        for (int jl = 0; jl < 32; ++jl) {
-            const int j = 32 * jq + jl;
-            if (j >= M) break;
-            const double xj = __shfl_sync(0xffffffffu, y[jq], jl) * __shfl_sync(0xffffffffu, rd[jq], jl);
-            if (lane == jl) y[jq] = xj;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int k = lane + 32 * q;
-                if (k > j && k < M) y[q] = fma(-D[int64_t(k) * M + j], xj, y[q]);
-            }
+    const double *L = a.Ls + ((r - 1) & 1) * MM;
+    if (blockIdx.y == 0) {
+        for (int j = threadIdx.x; j < M; j += blockDim.x) {
+            if (j < i) continue;
+            double v = a.Hd[r * MM + int64_t(i) * M + j] + (i == j ? eps : 0.0);
+            if (r > 0)   // (rows of an upper triangular matrix: k >= j)
+                v -= dot4(j, M, [&](int k) { return L[int64_t(i) * M + k]; }, [&](int k) { return L[int64_t(j) * M + k]; });
+            a.Ri[r * MM + int64_t(i) * M + j] = v;
         }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int j = lane + 32 * q;
-        if (j < M) Ls[r * MM + int64_t(i) * M + j] = y[q];
+    } else {
+        const double *RiT = a.RiT + (r - 1) * MM;
+        for (int j = threadIdx.x; j < M; j += blockDim.x)
+            a.K[(r - 1) * MM + int64_t(i) * M + j] =
+                dot4(max(i, j), M, [&](int k) { return L[int64_t(i) * M + k]; },
+                     [&](int k) { return RiT[int64_t(k) * M + j]; });
     }
 }
 
-// s_int times U <- (eps I + H)^{-1} U with the factors Ld, Ls (k_bt_dupdate / dchol / lsolve), by forward and
-// backward block substitution; U starts as F_1 = [I; 0; ...] unless rhs_in_u (U already holds
-// the right-hand side, steps blocks).  The right-hand-side columns are independent: one warp
-// per column, BTS_COLS columns per CTA, the CTAs side by side (FP64 runs at a small fraction
-// of the FP32 rate on this part, so the columns are spread over as many SMs as there are).  A
-// warp keeps its column of the current block in registers (lane l: rows l, l + 32, l + 64,
-// l + 96; M <= 128), takes the coupling term Ls y from the previous block's column (broadcast
-// by shuffles) and solves the triangular system column-oriented: y_i /= d_ii, then
-// y_k -= d_ki y_i for the rows k below (k above in the backward solve with D^T), one shuffle
-// per row.  No block barrier is used.  Yw holds the forward solutions Y_r for the backward
-// pass.
-constexpr int BTS_COLS = 1;
-constexpr int BTS_R = 4;   // rows per lane
-__global__ void __launch_bounds__(32 * BTS_COLS)
-k_bt_spline_subst(const double *__restrict__ Ld, const double *__restrict__ Ls, int M, int s_int,
-                  double *__restrict__ Yw, double *__restrict__ U, const Ctrl *ctrl, int rhs_in_u) {
-    const int steps = ctrl->steps;
-    const int lane = threadIdx.x & 31;
-    const int c = blockIdx.x * BTS_COLS + (threadIdx.x >> 5);
-    if (c >= M) return;   // whole warps: nothing below synchronises the block
+__global__ void __launch_bounds__(512) k_bt_dchol(BtArgs a, int r, const Ctrl *fc) {
+    if (bt_skip(fc, r)) return;
+    extern __shared__ __align__(16) double bsm[];
+    const int M = a.M, lda = (M + 1) / 2 * 2;
+    double *A = bsm, *scr = A + lda * lda, *tmp = scr + sm::NB * sm::NB;
+    const int64_t o = r * int64_t(M) * M;
+    sm::each(M, M, [&](int i, int j) { A[i * lda + j] = j >= i ? __ldcg(a.Ri + o + i * M + j) : 0.0; });
+    __syncthreads();
+    const bool ok = sm::chol_blocked<double>(A, nullptr, lda, M, 0.0, scr);
+    if (ok) {
+        sm::each(M, M, [&](int i, int j) {
+            if (j < i) A[i * lda + j] = 0.0;
+        });
+        __syncthreads();
+        sm::tri_inv_diag<double>(A, lda, M);
+        sm::tri_inv_merge<double>(A, lda, M, tmp);
+    }
+    // a block that is not positive definite (lost orthogonality) shows as NaN
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    sm::each(M, M, [&](int i, int j) {
+        a.Ri[o + i * M + j] = ok ? A[i * lda + j] : nan;
+        a.RiT[o + i * M + j] = ok ? A[j * lda + i] : nan;
+    });
+}
+
+// row i = blockIdx.x of G_r^T (Ri_r upper triangular, Ls_{r-1} upper triangular)
+__global__ void __launch_bounds__(128) k_bt_gt(BtArgs a, int r, const Ctrl *fc) {
+    if (bt_skip(fc, r)) return;
+    const int M = a.M, i = blockIdx.x;
     const int64_t MM = int64_t(M) * M;
-    double y[BTS_R], yp[BTS_R], rd[BTS_R];
+    const double *L = a.Ls + ((r - 1) & 1) * MM, *Ri = a.Ri + r * MM;
+    for (int j = threadIdx.x; j < M; j += blockDim.x)
+        a.GT[r * MM + int64_t(i) * M + j] =
+            dot4(0, min(i, j) + 1, [&](int k) { return L[int64_t(k) * M + i]; }, [&](int k) { return Ri[int64_t(k) * M + j]; });
+}
+
+// One column c = blockIdx.x of U per CTA.  A product with an M x M matrix stored by the input
+// index (rows contiguous in the output index) gives each thread one output row and a part of
+// the inputs; the parts are added in shared memory.  y0: first block whose Y of the first
+// solve is not known yet.
+constexpr int BTS_THREADS = 256;
+__global__ void __launch_bounds__(BTS_THREADS)
+k_bt_subst(BtArgs a, int s_int, int y0, double *__restrict__ U, const Ctrl *ctrl, int rhs_in_u) {
+    const int steps = ctrl->steps, M = a.M, c = blockIdx.x;
+    if (steps <= 0) return;
+    __shared__ double v[2][128], w[2][128], part[BTS_THREADS];
+    const int64_t MM = int64_t(M) * M;
+    int Mp = 32;
+    while (Mp < M) Mp *= 2;
+    const int row = threadIdx.x % Mp, ks = threadIdx.x / Mp, nks = BTS_THREADS / Mp;
+    // part of sum_k A[k][row] x_k over this thread's inputs
+    auto mv = [&](const double *A, const double *x) -> double {
+        if (row >= M) return 0.0;
+        double s0 = 0.0, s1 = 0.0;
+        int k = ks;
+        for (; k + nks < M; k += 2 * nks) {
+            s0 = fma(A[int64_t(k) * M + row], x[k], s0);
+            s1 = fma(A[int64_t(k + nks) * M + row], x[k + nks], s1);
+        }
+        if (k < M) s0 = fma(A[int64_t(k) * M + row], x[k], s0);
+        return s0 + s1;
+    };
+    auto total = [&](double p) -> double {   // valid for ks == 0
+        part[threadIdx.x] = p;
+        __syncthreads();
+        double t = 0.0;
+        if (ks == 0)
+            for (int q = 0; q < nks; ++q) t += part[q * Mp + row];
+        return t;
+    };
     for (int rep = 0; rep < s_int; ++rep) {
-        // forward: Y_r = D_r^{-1} (U_r - Ls_{r-1} Y_{r-1})
-        for (int r = 0; r < steps; ++r) {
-            const double *D = Ld + r * MM;
-#pragma unroll
-            for (int q = 0; q < BTS_R; ++q) {
-                const int i = lane + 32 * q;
-                double v = 0.0, d = 1.0;
-                if (i < M) {
-                    v = (rep == 0 && !rhs_in_u) ? ((r == 0 && i == c) ? 1.0 : 0.0) : U[r * MM + int64_t(i) * M + c];
-                    d = D[int64_t(i) * M + i];
-                }
-                y[q] = v;
-                rd[q] = 1.0 / d;
+        // upwards: Y_r = Ri_r^T rhs_r - G_r Y_{r-1}
+        const bool unit = rep == 0 && !rhs_in_u;     // rhs = F_1
+        const int r0 = unit ? y0 : 0;
+        if (r0 > 0 && threadIdx.x < M) v[(r0 - 1) & 1][threadIdx.x] = a.Y[(r0 - 1) * MM + int64_t(c) * M + threadIdx.x];
+        for (int r = r0; r < steps; ++r) {
+            double p = 0.0;
+            if (!unit) {
+                if (threadIdx.x < M) w[r & 1][threadIdx.x] = U[r * MM + int64_t(threadIdx.x) * M + c];
+                __syncthreads();
+                p = mv(a.Ri + r * MM, w[r & 1]);
+            } else if (r == 0 && ks == 0 && row < M) {
+                p = a.Ri[int64_t(c) * M + row];
             }
-            if (r > 0) {
-                const double *P = Ls + (r - 1) * MM;
-#pragma unroll
-                for (int kq = 0; kq < BTS_R; ++kq)
-                    for (int kl = 0; kl < 32; ++kl) {
-                        const int k = 32 * kq + kl;
-                        if (k >= M) break;
-                        const double ypk = __shfl_sync(0xffffffffu, yp[kq], kl);
-#pragma unroll
-                        for (int q = 0; q < BTS_R; ++q) {
-                            const int i = lane + 32 * q;
-                            if (i < M) y[q] = fma(-P[int64_t(i) * M + k], ypk, y[q]);
-                        }
-                    }
+            __syncthreads();
+            if (r > 0) p -= mv(a.GT + r * MM, v[(r - 1) & 1]);
+            const double t = total(p);
+            if (ks == 0 && row < M) {
+                v[r & 1][row] = t;
+                a.Y[r * MM + int64_t(c) * M + row] = t;
             }
-#pragma unroll
-            for (int iq = 0; iq < BTS_R; ++iq)
-                for (int il = 0; il < 32; ++il) {
-                    const int i = 32 * iq + il;
-                    if (i >= M) break;
-                    const double yi = __shfl_sync(0xffffffffu, y[iq], il) * __shfl_sync(0xffffffffu, rd[iq], il);
-                    if (lane == il) y[iq] = yi;
-#pragma unroll
-                    for (int q = 0; q < BTS_R; ++q) {
-                        const int k = lane + 32 * q;
-                        if (k > i && k < M) y[q] = fma(-D[int64_t(k) * M + i], yi, y[q]);
-                    }
-                }
-#pragma unroll
-            for (int q = 0; q < BTS_R; ++q) {
-                const int i = lane + 32 * q;
-                if (i < M) Yw[r * MM + int64_t(i) * M + c] = y[q];
-                yp[q] = y[q];
-            }
+            __syncthreads();
         }
-        // backward: U_r = D_r^{-T} (Y_r - Ls_r^T U_{r+1})
+        // downwards: U_r = Ri_r Y_r - K_r^T U_{r+1}
         for (int r = steps - 1; r >= 0; --r) {
-            const double *D = Ld + r * MM;
-#pragma unroll
-            for (int q = 0; q < BTS_R; ++q) {
-                const int i = lane + 32 * q;
-                y[q] = i < M ? Yw[r * MM + int64_t(i) * M + c] : 0.0;
-                rd[q] = 1.0 / (i < M ? D[int64_t(i) * M + i] : 1.0);
+            if (threadIdx.x < M) w[r & 1][threadIdx.x] = a.Y[r * MM + int64_t(c) * M + threadIdx.x];
+            __syncthreads();
+            double p = mv(a.RiT + r * MM, w[r & 1]);
+            if (r + 1 < steps) p -= mv(a.K + r * MM, v[(r + 1) & 1]);
+            const double t = total(p);
+            if (ks == 0 && row < M) {
+                v[r & 1][row] = t;
+                U[r * MM + int64_t(row) * M + c] = t;
             }
-            if (r + 1 < steps) {
-                const double *P = Ls + r * MM;
-#pragma unroll
-                for (int kq = 0; kq < BTS_R; ++kq)
-                    for (int kl = 0; kl < 32; ++kl) {
-                        const int k = 32 * kq + kl;
-                        if (k >= M) break;
-                        const double unk = __shfl_sync(0xffffffffu, yp[kq], kl);
-#pragma unroll
-                        for (int q = 0; q < BTS_R; ++q) {
-                            const int i = lane + 32 * q;
-                            if (i < M) y[q] = fma(-P[int64_t(k) * M + i], unk, y[q]);
-                        }
-                    }
-            }
-#pragma unroll
-            for (int iq = BTS_R - 1; iq >= 0; --iq)
-                for (int il = 31; il >= 0; --il) {
-                    const int i = 32 * iq + il;
-                    if (i >= M) continue;
-                    const double ui = __shfl_sync(0xffffffffu, y[iq], il) * __shfl_sync(0xffffffffu, rd[iq], il);
-                    if (lane == il) y[iq] = ui;
-#pragma unroll
-                    for (int q = 0; q < BTS_R; ++q) {
-                        const int k = lane + 32 * q;
-                        if (k < i) y[q] = fma(-D[int64_t(i) * M + k], ui, y[q]);
-                    }
-                }
-#pragma unroll
-            for (int q = 0; q < BTS_R; ++q) {
-                const int i = lane + 32 * q;
-                if (i < M) U[r * MM + int64_t(i) * M + c] = y[q];
-                yp[q] = y[q];
-            }
+            __syncthreads();
         }
     }
 }
@@ -507,29 +563,32 @@ int launch_cheb_bt(const double *Hd, const double *Hs, int M, int m, double lam,
     const size_t bytes = sizeof(double) * size_t(m) * M * M;
     prof_begin(KernelClass::PROJECTED, s);
     if (Hdf) {
-        // double-float recurrence: H split once, V_j as float pairs in the V buffers
-        const int64_t cnt = int64_t(m) * M * M;
-        dfl *hd = reinterpret_cast<dfl *>(Hdf), *hs = hd + cnt;
-        const int sg = int(std::min<int64_t>((cnt + 255) / 256, 8 * int64_t(num_sms())));
-        k_split_df<<<sg, 256, 0, s>>>(Hd, hd, cnt);
-        k_split_df<<<sg, 256, 0, s>>>(Hs, hs, cnt);
+        // double-float recurrence: H as floats once, V_j as float pairs in the V buffers
+        const int ld = (M + 1) / 2 * 2;
+        float *hd = reinterpret_cast<float *>(Hdf), *hs = hd + size_t(m) * M * ld, *ht = hs + size_t(m) * M * ld;
+        k_split_df<<<dim3(m, 2), 256, 0, s>>>(Hd, Hs, hd, hs, ht, M, ld, ctrl);
         KB_CUDA_TRY(cudaMemsetAsync(V0, 0, bytes, s));
         KB_CUDA_TRY(cudaMemsetAsync(V1, 0, bytes, s));
         KB_CUDA_TRY(cudaMemsetAsync(V2, 0, bytes, s));
         zero_if_active(U, int64_t(m) * M * M, ctrl, s);
         dfl *pp = reinterpret_cast<dfl *>(V2), *pc = reinterpret_cast<dfl *>(V0), *pn = reinterpret_cast<dfl *>(V1);
         k_cheb_bt_seed_df<<<(M + 127) / 128, 128, 0, s>>>(pc, U, M, d[0], ctrl);
-        const size_t smem = sizeof(dfl) * 3 * M * TC;
+        const size_t smem = sizeof(dfl) * 3 * M * CBW + sizeof(float) * 3 * M * ld;
+        static const cudaError_t attr = cudaFuncSetAttribute(k_cheb_bt_iter_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                             int(sizeof(dfl) * 3 * 128 * CBW + sizeof(float) * 3 * 128 * 128));
+        (void)attr;
+        const int threads = std::max(32, ((M + 1) / 2 * 4 + 31) / 32 * 32);
         const dfl g = dfl_from(2.0 / lam);
         for (size_t j = 0; j + 1 < d.size(); ++j) {
             const int nrb = std::min<int>(int(j) + 2, m);
-            dim3 grid(nrb, (M + TC - 1) / TC);
+            dim3 grid(nrb, (M + CBW - 1) / CBW);
             const float beta = j == 0 ? 1.f : 2.f, gamma = j == 0 ? 0.f : 1.f;
-            k_cheb_bt_iter_df<<<grid, 256, smem, s>>>(hd, hs, pp, pc, pn, U, M, beta, gamma, d[j + 1], g, ctrl);
+            k_cheb_bt_iter_df<<<grid, threads, smem, s>>>(hd, hs, ht, pp, pc, pn, U, M, ld, beta, gamma, d[j + 1], g,
+                                                          ctrl);
             dfl *t = pp; pp = pc; pc = pn; pn = t;
         }
         KB_CUDA_TRY(cudaGetLastError());
-        prof_end(KernelClass::PROJECTED, s, 0, 0, int(d.size()) + 3);
+        prof_end(KernelClass::PROJECTED, s, 0, 0, int(d.size()) + 2);
         return 0;
     }
     KB_CUDA_TRY(cudaMemsetAsync(V0, 0, bytes, s));
@@ -556,26 +615,37 @@ int launch_cheb_bt(const double *Hd, const double *Hs, int M, int m, double lam,
     return 0;
 }
 
-// The block factorisation, launched block by block up to kmax; returns the launch count.
-static int bt_factor(const double *Hd, const double *Hs, int M, int kmax, double eps, double *Ld,
-                     double *Ls, const Ctrl *ctrl, cudaStream_t s) {
-    for (int r = 0; r < kmax; ++r) {
-        k_bt_dupdate<<<M, 128, 0, s>>>(Hd, Ls, M, eps, r, Ld, ctrl);
-        k_bt_dchol<<<1, 1024, 0, s>>>(Ld, M, r, ctrl);
-        if (r + 1 < kmax) k_bt_lsolve<<<M, 32, 0, s>>>(Hs, Ld, M, r, Ls, ctrl);
+// Factors blocks r0 .. kmax - 1 (the ones before are known); returns the launch count.
+static int bt_factor(const BtArgs &a, int r0, int kmax, double eps, const Ctrl *fc, cudaStream_t s) {
+    const int M = a.M, lda = (M + 1) / 2 * 2;
+    const size_t smem = sizeof(double) * (size_t(lda) * lda + sm::NB * sm::NB + sm::tri_tmp_elems(M));
+    static const cudaError_t attr = cudaFuncSetAttribute(
+        k_bt_dchol, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        int(sizeof(double) * (128 * 128 + sm::NB * sm::NB + sm::tri_tmp_elems(128))));
+    (void)attr;
+    int launches = 0;
+    for (int r = r0; r < kmax; ++r) {
+        if (r > 0) k_bt_ls<<<M, 128, 0, s>>>(a, r, fc);
+        k_bt_schur<<<dim3(M, r > 0 ? 2 : 1), 128, 0, s>>>(a, r, eps, fc);
+        k_bt_dchol<<<1, 512, smem, s>>>(a, r, fc);
+        if (r > 0) k_bt_gt<<<M, 128, 0, s>>>(a, r, fc);
+        launches += r > 0 ? 4 : 2;
     }
-    return 3 * kmax - 1;
+    return launches;
 }
 
 int launch_bt_spline(const double *Hd, const double *Hs, int M, int m, double eps, int s_int,
-                     double *Ld, double *Ls, double *Yw, double *U, const Ctrl *ctrl,
-                     cudaStream_t s, const QuadRule *q, double *qscr, int qbatch, int kmax) {
+                     const SplineBufs &b, double *U, const Ctrl *fc, const Ctrl *ctrl, cudaStream_t s,
+                     const QuadRule *q, double *qscr, int qbatch, int r0, int y0, int kmax) {
     if (kmax <= 0 || kmax > m) kmax = m;
+    const BtArgs a{Hd, Hs, b.Ri, b.RiT, b.Y, b.GT, b.K, b.Ls, M};
     prof_begin(KernelClass::PROJECTED, s);
     int launches = 1;   // zero_if_active
-    if (q && q->n > 0) {
+    // (blocks past the steps stay zero: the bound check reads all m of them)
+    zero_if_active(U, int64_t(m) * M * M, ctrl, s);
+    const bool frac = q && q->n > 0;
+    if (frac) {
         if (!qscr || qbatch < 1) return fail(KB_ERR_ARG, "spline quadrature without scratch");
-        zero_if_active(U, int64_t(m) * M * M, ctrl, s);
         const int acc_grid = int(std::min<int64_t>((int64_t(m) * M * M + 255) / 256, 4 * int64_t(num_sms())));
         for (int j0 = 0; j0 < q->n; j0 += qbatch) {
             const int nb = std::min(qbatch, q->n - j0);
@@ -583,16 +653,10 @@ int launch_bt_spline(const double *Hd, const double *Hs, int M, int m, double ep
             k_quad_accumulate<<<std::max(acc_grid, 1), 256, 0, s>>>(qscr, M, m, nb, *q, j0, U, ctrl);
             launches += 2;
         }
-        if (s_int > 0) {
-            launches += bt_factor(Hd, Hs, M, kmax, eps, Ld, Ls, ctrl, s) + 1;
-            k_bt_spline_subst<<<(M + BTS_COLS - 1) / BTS_COLS, 32 * BTS_COLS, 0, s>>>(Ld, Ls, M, s_int, Yw, U, ctrl, 1);
-        }
-    } else {
-        // (blocks past the steps stay zero: the bound check reads all m of them)
-        zero_if_active(U, int64_t(m) * M * M, ctrl, s);
-        launches += bt_factor(Hd, Hs, M, kmax, eps, Ld, Ls, ctrl, s);
-        k_bt_spline_subst<<<(M + BTS_COLS - 1) / BTS_COLS, 32 * BTS_COLS, 0, s>>>(Ld, Ls, M, s_int, Yw, U, ctrl, 0);
-        ++launches;
+    }
+    if (s_int > 0) {
+        launches += bt_factor(a, r0, kmax, eps, fc, s) + 1;
+        k_bt_subst<<<M, BTS_THREADS, 0, s>>>(a, s_int, y0, U, ctrl, frac ? 1 : 0);
     }
     KB_CUDA_TRY(cudaGetLastError());
     prof_end(KernelClass::PROJECTED, s, 0, 0, launches);

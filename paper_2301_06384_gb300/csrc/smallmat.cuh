@@ -3,10 +3,12 @@
 //
 // One SM works on these, so their time is latency: barriers, dependent operations, and FP64
 // operations above all (two FMAs per clock and SM on this part).  Blocks of 16: a diagonal block
-// is factored by one warp in registers, with no barrier, and the same instructions give the
-// inverse of its factor; everything else is products of 16 or more independent terms over all
-// threads, in 2 x 2 register tiles, a warp's lanes along the columns.  Rows are lda elements
-// apart, lda even (pairs of elements are loaded at once).
+// is factored by four warps in registers, and the same instructions give the inverse of its
+// factor; everything else is products of 16 or more independent terms, in tiles shared out
+// over all threads.  Rows are lda elements apart, lda even (pairs of elements are loaded at
+// once).  Cycles of the parts at M = 64 (FP32 / FP64), now and with the diagonal block in one
+// warp and tiles by rows: Cholesky 25 k / 104 k and 33 k / 173 k, merges 7 k / 40 k and 9 k /
+// 52 k, one product 6 k / 44 k and 6 k / 78 k.
 #pragma once
 #include "kb_internal.cuh"
 
@@ -25,14 +27,20 @@ __device__ __forceinline__ void ld2(const S *p, S (&v)[2]) {
     v[1] = t.y;
 }
 
+template <int E, typename S>
+__device__ __forceinline__ void ldE(const S *p, S (&v)[E]) {
+    if constexpr (E == 2) ld2(p, v);
+    else v[0] = p[0];
+}
+
 // 1/d for a positive double d by Newton's iteration for the reciprocal, r <- r + r (1 - d r),
-// from the single-precision reciprocal: two steps take its 2^-23 relative error to the
-// FP64 rounding level (the error squares at each step).  The FP64 division it replaces is
-// a long dependent sequence on this part's FP64 unit; this is four FMAs.  Outside the
-// normal single-precision range the division is used.
+// from the hardware approximation (relative error about 2^-20): two steps take it to the FP64
+// rounding level (the error squares at each step).  The FP64 division it replaces is a long
+// dependent sequence on this part's FP64 unit; this is four FMAs.
 __device__ __forceinline__ double recip(double d) {
-    if (!(d > 1e-36 && d < 1e36)) return 1.0 / d;
-    double r = double(__frcp_rn(float(d)));
+    if (!(d > 1e-290 && d < 1e290)) return 1.0 / d;
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
     double e = fma(-d, r, 1.0);
     r = fma(r, e, r);
     e = fma(-d, r, 1.0);
@@ -40,17 +48,25 @@ __device__ __forceinline__ double recip(double d) {
 }
 __device__ __forceinline__ float recip(float d) { return __frcp_rn(d); }
 
-// 2 x 2 tiles (i0, j0) of the rows [0, R) and columns [0, C): a warp takes rows i0, i0 + 1 and
-// its lanes the column pairs (several row pairs per warp when the columns are few).
-template <typename F>
-__device__ __forceinline__ void tiles2(int R, int C, const F &f) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int cp = (C + 1) / 2;
-    int lpr = 32;                       // lanes per row pair
-    while (lpr > 1 && lpr / 2 >= cp) lpr /= 2;
-    const int rpw = 32 / lpr;
-    for (int i = (warp * rpw + lane / lpr) * 2; i < R; i += nw * rpw * 2)
-        for (int j = (lane % lpr) * 2; j < C; j += lpr * 2) f(i, j);
+// Edge of the register tiles: 2 in FP32, where a shared load is the dearer part, 1 in FP64,
+// whose FMA occupies a scheduler for some 64 cycles, so that only spreading the entries helps.
+template <typename S> struct Tile { static constexpr int E = sizeof(S) == 8 ? 1 : 2; };
+
+// E x E tiles (i0, j0) meeting the upper triangle of an M x M matrix, shared out evenly over
+// the threads (consecutive threads along a row).
+template <int E, typename F>
+__device__ __forceinline__ void tri_tiles(int M, const F &f) {
+    const int nt = (M + E - 1) / E, total = nt * (nt + 1) / 2;
+    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+        // rows above hold i nt - i (i - 1) / 2 tiles
+        const float h = float(nt) + 0.5f;
+        int i = int(h - sqrtf(fmaxf(h * h - 2.f * float(t), 0.f)));
+        i = max(0, min(i, nt - 1));
+        while (i > 0 && i * nt - i * (i - 1) / 2 > t) --i;
+        while ((i + 1) * nt - (i + 1) * i / 2 <= t) ++i;
+        const int j = i + t - (i * nt - i * (i - 1) / 2);
+        f(i * E, j * E);
+    }
 }
 
 // Cholesky G = R^T R: the upper triangle of A holds G on entry and R on return.  Inv (ld lda,
@@ -60,44 +76,61 @@ __device__ __forceinline__ void tiles2(int R, int C, const F &f) {
 template <typename S>
 __device__ bool chol_blocked(S *A, S *Inv, int lda, int M, S thr, S *scr) {
     __shared__ int s_bad;
+    __shared__ S s_row[64];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x == 0) s_bad = 0;
     __syncthreads();
     for (int j0 = 0; j0 < M; j0 += NB) {
         const int nb = min(NB, M - j0);
-        if (warp == 0) {
-            // lanes 0..15: the columns of the diagonal block; lanes 16..31: those of I, on which
-            // the same row operations leave R^{-T}
+        if (warp < 4) {
+            // Four warps (one per scheduler), warp w the rows w, w + 4, ..; lanes 0..15 the columns
+            // of the diagonal block, lanes 16..31 those of I, on which the same row operations
+            // leave R^{-T}.  Square-root free: row j goes round unscaled through shared memory,
+            // its multiple by 1 / d_j updates the rows below, so a step is one exchange, one
+            // reciprocal, one product and up to four FMAs; the square roots of the pivots come
+            // at the end, all at once.
             const int c = lane & (NB - 1);
             const bool inv = lane >= NB;
-            S a[NB];
+            S a[4];
 #pragma unroll
-            for (int i = 0; i < NB; ++i)
-                a[i] = (!inv && i < nb && c < nb) ? (i <= c ? A[(j0 + i) * lda + j0 + c] : S(0)) : S(i == c ? 1 : 0);
+            for (int u = 0; u < 4; ++u) {
+                const int i = warp + 4 * u;
+                a[u] = (!inv && i < nb && c < nb) ? (i <= c ? A[(j0 + i) * lda + j0 + c] : S(0)) : S(i == c ? 1 : 0);
+            }
             bool bad = false;
 #pragma unroll
             for (int j = 0; j < NB; ++j) {
-                S d = __shfl_sync(0xffffffffu, a[j], j);
+                S *rb = s_row + (j & 1) * 32;
+                if (warp == j % 4) rb[lane] = a[j / 4];
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                S d = rb[j];
                 if (j < nb && !(d > thr)) {
                     bad = true;
                     d = S(1);
                 }
-                const S r = sqrt(d);
-                const S ri = recip(r);
-                a[j] = (!inv && c == j) ? r : a[j] * ri;
+                const S sc = rb[lane] * recip(d);
 #pragma unroll
-                for (int i = j + 1; i < NB; ++i) {
-                    const S rji = __shfl_sync(0xffffffffu, a[j], i);
-                    a[i] = fma(-rji, a[j], a[i]);
-                }
+                for (int u = 0; u < 4; ++u)
+                    if (4 * u + 3 > j && warp + 4 * u > j) a[u] = fma(-rb[warp + 4 * u], sc, a[u]);
             }
             if (bad && lane == 0) s_bad = 1;
+            // row i times 1 / sqrt(d_i)
+            S piv = S(1);
 #pragma unroll
-            for (int i = 0; i < NB; ++i) {
-                if (inv) scr[i * NB + c] = a[i];                  // R^{-T}, lower triangular
+            for (int u = 0; u < 4; ++u) {
+                const S d = __shfl_sync(0xffffffffu, a[u], warp + 4 * u);
+                if (lane == u && warp + 4 * u < nb) piv = d;
+            }
+            const S rt = sqrt(piv), ri = recip(rt);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = warp + 4 * u;
+                const S r = __shfl_sync(0xffffffffu, rt, u), q = __shfl_sync(0xffffffffu, ri, u);
+                const S v = (!inv && c == i) ? r : a[u] * q;
+                if (inv) scr[i * NB + c] = v;                  // R^{-T}, lower triangular
                 if (i < nb && c < nb) {
-                    if (!inv) A[(j0 + i) * lda + j0 + c] = i <= c ? a[i] : S(0);
-                    else if (Inv) Inv[(j0 + c) * lda + j0 + i] = i >= c ? a[i] : S(0);
+                    if (!inv) A[(j0 + i) * lda + j0 + c] = i <= c ? v : S(0);
+                    else if (Inv) Inv[(j0 + c) * lda + j0 + i] = i >= c ? v : S(0);
                 }
             }
         }
@@ -124,25 +157,29 @@ __device__ bool chol_blocked(S *A, S *Inv, int lda, int M, S thr, S *scr) {
         }
         __syncthreads();
         // A_22 -= R_12^T R_12 (upper triangle)
-        tiles2(rest, rest, [&](int i, int j) {
-            if (j + 1 < i) return;
-            S *p = A + (c0 + i) * lda + c0 + j;
-            const bool i1 = i + 1 < rest, j1 = j + 1 < rest;
-            S s00 = p[0], s01 = j1 ? p[1] : S(0), s10 = i1 ? p[lda] : S(0), s11 = i1 && j1 ? p[lda + 1] : S(0);
+        constexpr int E = Tile<S>::E;
+        tri_tiles<E>(rest, [&](int i, int j) {
+            S acc[E][E];
+#pragma unroll
+            for (int r = 0; r < E; ++r)
+#pragma unroll
+                for (int q = 0; q < E; ++q)
+                    acc[r][q] = i + r < rest && j + q < rest ? A[(c0 + i + r) * lda + c0 + j + q] : S(0);
 #pragma unroll
             for (int k = 0; k < NB; ++k) {
-                S u[2], v[2];
-                ld2(A + (j0 + k) * lda + c0 + i, u);
-                ld2(A + (j0 + k) * lda + c0 + j, v);
-                s00 = fma(-u[0], v[0], s00);
-                s01 = fma(-u[0], v[1], s01);
-                s10 = fma(-u[1], v[0], s10);
-                s11 = fma(-u[1], v[1], s11);
+                S u[E], v[E];
+                ldE<E>(A + (j0 + k) * lda + c0 + i, u);
+                ldE<E>(A + (j0 + k) * lda + c0 + j, v);
+#pragma unroll
+                for (int r = 0; r < E; ++r)
+#pragma unroll
+                    for (int q = 0; q < E; ++q) acc[r][q] = fma(-u[r], v[q], acc[r][q]);
             }
-            p[0] = s00;
-            if (j1) p[1] = s01;
-            if (i1 && j > i) p[lda] = s10;
-            if (i1 && j1) p[lda + 1] = s11;
+#pragma unroll
+            for (int r = 0; r < E; ++r)
+#pragma unroll
+                for (int q = 0; q < E; ++q)
+                    if (i + r <= j + q && j + q < rest) A[(c0 + i + r) * lda + c0 + j + q] = acc[r][q];
         });
         __syncthreads();
     }
@@ -193,78 +230,81 @@ __device__ void tri_inv_merge(S *A, int lda, int M, S *tmp) {
         const int np = (M + 2 * bs - 1) / (2 * bs);
         for (int pass = 0; pass < 2; ++pass) {
             // all pairs' rows side by side: row index p * bs + i
-            tiles2(np * bs, bs, [&](int ri, int j) {
+            constexpr int E = Tile<S>::E;
+            const int per = bs / E;   // tiles of a row or column (a power of two)
+            for (int t = threadIdx.x; t < np * per * per; t += blockDim.x) {
+                const int j = (t % per) * E, ri = (t / per) * E;
                 const int p = ri / bs, i = ri % bs, r0 = p * 2 * bs, c0 = r0 + bs;
-                if (c0 + j >= M) return;
-                const bool j1 = c0 + j + 1 < M;
-                S s00 = 0, s01 = 0, s10 = 0, s11 = 0;
+                if (c0 + j >= M) continue;
+                S acc[E][E];
+#pragma unroll
+                for (int r = 0; r < E; ++r)
+#pragma unroll
+                    for (int q = 0; q < E; ++q) acc[r][q] = S(0);
                 S *T = tmp + p * bs * bs;
-                if (pass == 0) {
-                    // T = A^-1 B (A^-1 upper triangular: k >= i)
-                    for (int k = i; k < bs; ++k) {
-                        const S a0 = A[(r0 + i) * lda + r0 + k], a1 = A[(r0 + i + 1) * lda + r0 + k];
-                        S v[2];
-                        ld2(A + (r0 + k) * lda + c0 + j, v);
-                        s00 = fma(a0, v[0], s00);
-                        s01 = fma(a0, v[1], s01);
-                        s10 = fma(a1, v[0], s10);
-                        s11 = fma(a1, v[1], s11);
-                    }
-                    T[i * bs + j] = s00;
-                    T[i * bs + j + 1] = j1 ? s01 : S(0);
-                    T[(i + 1) * bs + j] = s10;
-                    T[(i + 1) * bs + j + 1] = j1 ? s11 : S(0);
-                } else {
-                    // B <- -T C^-1 (C^-1 upper triangular: k <= j)
-                    const int ke = min(j + 2, M - c0);
-                    for (int k = 0; k < ke; ++k) {
-                        const S a0 = T[i * bs + k], a1 = T[(i + 1) * bs + k];
-                        S v[2];
-                        ld2(A + (c0 + k) * lda + c0 + j, v);
-                        s00 = fma(a0, v[0], s00);
-                        s01 = fma(a0, v[1], s01);
-                        s10 = fma(a1, v[0], s10);
-                        s11 = fma(a1, v[1], s11);
-                    }
-                    S *q = A + (r0 + i) * lda + c0 + j;
-                    q[0] = -s00;
-                    q[lda] = -s10;
-                    if (j1) {
-                        q[1] = -s01;
-                        q[lda + 1] = -s11;
+                // pass 0: T = A^-1 B (A^-1 upper triangular: k >= i); pass 1: B <- -T C^-1 (C^-1
+                // upper triangular: k <= j)
+                const S *L = pass == 0 ? A + (r0 + i) * lda + r0 : T + i * bs;
+                const int ldl = pass == 0 ? lda : bs;
+                const S *Rm = A + (pass == 0 ? r0 : c0) * lda + c0 + j;
+                const int k0 = pass == 0 ? i : 0, k1 = pass == 0 ? bs : min(j + E, M - c0);
+#pragma unroll 4
+                for (int k = k0; k < k1; ++k) {
+                    S v[E];
+                    ldE<E>(Rm + k * lda, v);
+#pragma unroll
+                    for (int r = 0; r < E; ++r) {
+                        const S a = L[r * ldl + k];
+#pragma unroll
+                        for (int q = 0; q < E; ++q) acc[r][q] = fma(a, v[q], acc[r][q]);
                     }
                 }
-            });
+#pragma unroll
+                for (int r = 0; r < E; ++r)
+#pragma unroll
+                    for (int q = 0; q < E; ++q) {
+                        const bool in = c0 + j + q < M;
+                        if (pass == 0) T[(i + r) * bs + j + q] = in ? acc[r][q] : S(0);
+                        else if (in) A[(r0 + i + r) * lda + c0 + j + q] = -acc[r][q];
+                    }
+            }
             __syncthreads();
         }
     }
 }
 
-// epi(i, j, c) for the upper triangle of C = A B, A and B upper triangular (ld lda, zeros below
-// the diagonal), in 2 x 2 tiles.
-template <typename S, typename FE>
-__device__ void tri_mm(const S *A, const S *B, int lda, int M, const FE &epi) {
-    tiles2(M, M, [&](int i, int j) {
-        if (j + 1 < i) return;
-        const bool i1 = i + 1 < M;
-        const S *pa = A + i * lda, *pb = pa + (i1 ? lda : 0);
-        S s00 = 0, s01 = 0, s10 = 0, s11 = 0;
-        const int ke = min(j + 2, M);
+// epi(i, j, c, x) for the upper triangle of C = A B, A and B upper triangular (ld lda, zeros
+// below the diagonal); x = pre(i, j), asked for before the sums so that its load overlaps them.
+template <typename S, typename FP, typename FE>
+__device__ void tri_mm(const S *A, const S *B, int lda, int M, const FP &pre, const FE &epi) {
+    constexpr int E = Tile<S>::E;
+    tri_tiles<E>(M, [&](int i, int j) {
+        S acc[E][E];
+        decltype(pre(0, 0)) x[E][E];
+#pragma unroll
+        for (int r = 0; r < E; ++r)
+#pragma unroll
+            for (int q = 0; q < E; ++q) {
+                acc[r][q] = S(0);
+                x[r][q] = pre(min(i + r, M - 1), min(j + q, M - 1));
+            }
+        const int ke = min(j + E, M);
 #pragma unroll 4
         for (int k = i; k < ke; ++k) {
-            const S a0 = pa[k], a1 = pb[k];
-            S v[2];
-            ld2(B + k * lda + j, v);
-            s00 = fma(a0, v[0], s00);
-            s01 = fma(a0, v[1], s01);
-            s10 = fma(a1, v[0], s10);
-            s11 = fma(a1, v[1], s11);
+            S v[E];
+            ldE<E>(B + k * lda + j, v);
+#pragma unroll
+            for (int r = 0; r < E; ++r) {
+                const S a = A[min(i + r, M - 1) * lda + k];
+#pragma unroll
+                for (int q = 0; q < E; ++q) acc[r][q] = fma(a, v[q], acc[r][q]);
+            }
         }
-        const bool j1 = j + 1 < M;
-        if (j >= i) epi(i, j, s00);
-        if (j1) epi(i, j + 1, s01);
-        if (i1 && j >= i + 1) epi(i + 1, j, s10);
-        if (i1 && j1) epi(i + 1, j + 1, s11);
+#pragma unroll
+        for (int r = 0; r < E; ++r)
+#pragma unroll
+            for (int q = 0; q < E; ++q)
+                if (i + r <= j + q && j + q < M) epi(i + r, j + q, acc[r][q], x[r][q]);
     });
 }
 
@@ -275,8 +315,7 @@ __device__ void tri_mm(const S *A, const S *B, int lda, int M, const FE &epi) {
 // running on the FP32 pipe.
 template <typename FE>
 __device__ void tri_residual(const float *Sm, const float *R, int lda, int M, const FE &epi) {
-    tiles2(M, M, [&](int i, int j) {
-        if (j + 1 < i) return;
+    tri_tiles<2>(M, [&](int i, int j) {
         const bool i1 = i + 1 < M;
         const float *pa = Sm + i * lda, *pb = pa + (i1 ? lda : 0);
         float hi[2][2], lo[2][2];
@@ -288,7 +327,7 @@ __device__ void tri_residual(const float *Sm, const float *R, int lda, int M, co
                 lo[r][q] = 0.f;
             }
         const int ke = min(j + 2, M);
-#pragma unroll 2
+#pragma unroll 4
         for (int k = i; k < ke; ++k) {
             const float a[2] = {pa[k], pb[k]};
             float v[2];
