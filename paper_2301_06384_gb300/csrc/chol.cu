@@ -1,6 +1,5 @@
-// Small dense kernels of the classical block Lanczos step (Algorithm 1).
+// Small dense kernel of the classical block Lanczos step (Algorithm 1).
 //
-//  * k_hkk   symmetrised diagonal block H_kk.
 //  * k_chol  reduced QR of the new block by CholeskyQR: Cholesky factor (FP32 first, FP64
 //            fallback), its inverse and the FP64 factor consistent with the applied inverse;
 //            the second pass forms H_{k+1,k} = R2 R1 and the transposed block used by the next
@@ -11,23 +10,6 @@
 #include "smallmat.cuh"
 
 namespace kb {
-
-template <typename T>
-__global__ void k_hkk(const double *__restrict__ G, int M, int W, double *__restrict__ Hd,
-                      T *__restrict__ C, const Ctrl *ctrl) {
-    if (ctrl->stop) return;
-    // rows by warp, columns by lane; both loads of an entry issued before any store
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i = warp; i < W; i += nw)
-        for (int j = lane; j < W; j += 32) {
-            double v = 0.0;
-            if (i < M && j < M) v = 0.5 * (__ldg(G + i * W + j) + __ldg(G + j * W + i));
-            // recorded exactly as the update subtracts it (rounded to the basis precision)
-            const T vt = T(v);
-            if (i < M && j < M) Hd[i * M + j] = double(vt);
-            C[i * W + j] = vt;
-        }
-}
 
 // Reduced QR of the new block by CholeskyQR (Algorithm 1), pass 1 or 2 of CholeskyQR2.
 // Outputs: Rinv (W x W, basis precision) applied by the row-block kernels; pass 1 records
@@ -288,7 +270,7 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
                 Bout[j * W + i] = ht;
             });
         } else {
-            sm::tri_tiles<1>(M, [&](int i, int j) {
+            sm::tri_tiles<1, true>(M, [&](int i, int j) {
                 double h = 0.0;
 #pragma unroll 8
                 for (int k = i; k <= j; ++k) h = fma(A[i * lda + k], __ldcg(R1 + k * M + j), h);
@@ -301,15 +283,6 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
 }
 
 // ---------------------------------------------------------------- launchers
-template <typename T>
-int launch_hkk(const double *G, int M, int W, double *Hd, T *C, const Ctrl *ctrl, cudaStream_t s) {
-    prof_begin(KernelClass::SMALL, s);
-    k_hkk<T><<<1, 1024, 0, s>>>(G, M, W, Hd, C, ctrl);
-    KB_CUDA_TRY(cudaGetLastError());
-    prof_end(KernelClass::SMALL, s, 0, 0);
-    return 0;
-}
-
 template <typename T>
 int launch_chol(const double *G, int M, int W, int pass, int step, double inv_thresh2,
                 double piv_rel2, double *R1, T *Rinv, double *Hs, T *Bout, Ctrl *ctrl,
@@ -327,7 +300,6 @@ int launch_chol(const double *G, int M, int W, int pass, int step, double inv_th
 }
 
 #define KB_INST(T)                                                                              \
-    template int launch_hkk<T>(const double *, int, int, double *, T *, const Ctrl *, cudaStream_t); \
     template int launch_chol<T>(const double *, int, int, int, int, double, double, double *,   \
                                 T *, double *, T *, Ctrl *, cudaStream_t);
 KB_INST(float)

@@ -213,22 +213,34 @@ __device__ int compact_tiles(const int32_t *tgen, int64_t nact, const P &in, int
     return wsum[32];
 }
 
-// The list by distance, one CTA per distance: tiles at distance b = blockIdx.x (b = levels + 1:
-// all that were not reached) into list[acount[b - 1] ..].
+// The lists, one CTA each, all at once.  blockIdx.y = 0: the tiles at distance b = blockIdx.x (b =
+// levels + 1: all that were not reached) into alist[acount[b - 1] ..], so alist holds all tiles by
+// rising distance.  blockIdx.y = 1: the tiles within b hops in index order into lists[b]: in that
+// order neighbouring rows are at work at the same time, and their gathers meet in L2 (128^3
+// grid, sbl, M = 128: @@LS@@).
 __global__ void __launch_bounds__(1024) k_tile_sort(int32_t *tgen, uint8_t *gen, int64_t n, int64_t nact, int levels,
                                                     const int32_t *__restrict__ tcnt, const int32_t *err,
-                                                    int32_t *__restrict__ acount, int32_t *__restrict__ list) {
+                                                    int32_t *__restrict__ acount, int32_t *__restrict__ alist,
+                                                    int32_t *__restrict__ lists) {
     __shared__ int s_before, s_own;
     const int b = blockIdx.x;
     if (*err) {
         // the search gave up: every row counts as reached at once
         const int64_t stride = int64_t(gridDim.x) * blockDim.x, i0 = int64_t(b) * blockDim.x + threadIdx.x;
-        for (int64_t i = i0; i < n; i += stride) gen[i] = 0;
-        for (int64_t i = i0; i < nact; i += stride) {
-            tgen[i] = 0;
-            list[i] = int32_t(i);
+        if (blockIdx.y == 0) {
+            for (int64_t i = i0; i < n; i += stride) gen[i] = 0;
+            for (int64_t i = i0; i < nact; i += stride) {
+                tgen[i] = 0;
+                alist[i] = int32_t(i);
+            }
+            if (b <= levels && threadIdx.x == 0) acount[b] = int32_t(nact);
+        } else if (b <= levels) {
+            for (int64_t i = threadIdx.x; i < nact; i += blockDim.x) lists[b * nact + i] = int32_t(i);
         }
-        if (b <= levels && threadIdx.x == 0) acount[b] = int32_t(nact);
+        return;
+    }
+    if (blockIdx.y == 1) {
+        if (b <= levels) compact_tiles(tgen, nact, [&](int v) { return v <= b; }, 0, lists + b * nact);
         return;
     }
     // tiles nearer than b, by warp 0
@@ -244,14 +256,7 @@ __global__ void __launch_bounds__(1024) k_tile_sort(int32_t *tgen, uint8_t *gen,
     }
     __syncthreads();
     if (s_own == 0) return;
-    compact_tiles(tgen, nact, [&](int v) { return b <= levels ? v == b : v > levels; }, s_before, list);
-}
-
-// The tiles within k hops in index order (solves that keep a fixed order of their sums).
-__global__ void __launch_bounds__(1024) k_tile_list(const int32_t *tgen, int64_t nact, int k, int32_t *list,
-                                                    int32_t *count) {
-    const int c = compact_tiles(tgen, nact, [&](int v) { return v <= k; }, 0, list);
-    if (threadIdx.x == 0) *count = c;
+    compact_tiles(tgen, nact, [&](int v) { return b <= levels ? v == b : v > levels; }, s_before, alist);
 }
 
 // Zeros on the listed tiles.  ring: block b of the stored basis is written on the tiles within
@@ -280,7 +285,9 @@ k_zero_tiles(unsigned char *blocks, int64_t block_bytes, int nblk, int row_bytes
 
 }  // namespace
 
-void plan_frontier(FrontierBufs &f, int64_t n, unsigned char *base, size_t *bytes) {
+void plan_frontier(FrontierBufs &f, int64_t n, int levels, unsigned char *base, size_t *bytes) {
+    f.levels = levels;
+    f.nt = (n + ACT_ROWS - 1) / ACT_ROWS;
     const size_t nt = size_t((n + ACT_ROWS - 1) / ACT_ROWS);
     size_t off = 0;
     auto take = [&](size_t b) {
@@ -299,13 +306,14 @@ void plan_frontier(FrontierBufs &f, int64_t n, unsigned char *base, size_t *byte
     f.gen = take(size_t(n));
     f.tgen = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * nt));
     f.alist = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * nt));
+    f.lists = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * nt * size_t(levels + 1)));
     f.queue = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * size_t(n)));
     *bytes = off;
 }
 
-int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, int levels, cudaStream_t s) {
+int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, cudaStream_t s) {
+    const int levels = f.levels;
     const int64_t nt = (g.n + ACT_ROWS - 1) / ACT_ROWS;
-    f.levels = levels;
     NodeChunk ch;
     if (M > NodeChunk::CAP || levels > FRONTIER_MAX_HOPS + 2) return fail(KB_ERR_ARG, "frontier too large");
     ch.cnt = M;
@@ -328,17 +336,10 @@ int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, in
     cfg.numAttrs = 1;
     KB_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_bfs, g, ch, levels, f.gen, f.tgen, f.vis, f.queue, f.qlev, f.tcnt,
                                    f.sync, f.sync + 1));
-    k_tile_sort<<<levels + 2, 1024, 0, s>>>(f.tgen, f.gen, g.n, nt, levels, f.tcnt, f.sync + 1, f.acount, f.alist);
+    k_tile_sort<<<dim3(levels + 2, 2), 1024, 0, s>>>(f.tgen, f.gen, g.n, nt, levels, f.tcnt, f.sync + 1, f.acount,
+                                                     f.alist, f.lists);
     KB_CUDA_TRY(cudaGetLastError());
     prof_end(KernelClass::OTHER, s, double(g.n) + 4.0 * double(nt), 0, 2);
-    return 0;
-}
-
-int launch_tile_list(const FrontierBufs &f, int64_t n, int k, int32_t *list, int32_t *count, cudaStream_t s) {
-    prof_begin(KernelClass::OTHER, s);
-    k_tile_list<<<1, 1024, 0, s>>>(f.tgen, (n + ACT_ROWS - 1) / ACT_ROWS, k, list, count);
-    KB_CUDA_TRY(cudaGetLastError());
-    prof_end(KernelClass::OTHER, s, double(n) / ACT_ROWS * 4, 0);
     return 0;
 }
 

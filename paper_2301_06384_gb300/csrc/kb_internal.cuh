@@ -118,8 +118,8 @@ bool prof_on();
 // Krylov blocks started from E_W are exactly zero outside the (k-1)-hop ball of W at step
 // k.  gen[i] (uint8) is the hop distance of row i from W (255 = beyond the last hop wanted);
 // tgen[t] is the minimum over the 32-row tile t (0x7f7f7f7f likewise).  Both are known before
-// the first step: alist holds all tiles by rising tgen (equal ones in index order) and
-// acount[k] the number of tiles with tgen <= k, so the tiles active at step k are a prefix.
+// the first step: alist holds all tiles by rising tgen (equal ones in index order), acount[k]
+// the number of tiles with tgen <= k, and for each k there is a list of these in index order.
 // A block that is zero beyond hop b is written on the tiles with tgen <= b only and kept zero
 // on those of the two hops beyond, which the next product's gathers reach; nothing else of
 // it is ever initialised or read.
@@ -276,5 +276,11 @@ int validate_phi(kb_phi phi, const kb_params &p);
 template <typename P>
 int launch_reduce(const P *parts, int nparts, int len, double *out, cudaStream_t s,
                   const Ctrl *ctrl, P *out_p = nullptr, const int32_t *skip = nullptr);
+
+// launch_reduce of the Gram Q_k^T L Q_k into G, and the diagonal block formed from it: Hd (M x M), C (W
+// x W).  cnt: one zeroed word of the solve.
+template <typename P>
+int launch_reduce_hkk(const P *parts, int nparts, int M, int W, double *G, double *Hd, P *C, unsigned *cnt,
+                      const Ctrl *ctrl, cudaStream_t s);
 
 }  // namespace kb

@@ -75,8 +75,6 @@ int launch_scale_copy(T *out, const T *in, int64_t n, int W, double scale, const
 int launch_fill_nan(float *Y, int64_t n, int64_t ldy, int mo, const Ctrl *ctrl, cudaStream_t s);
 
 template <typename T>
-int launch_hkk(const double *G, int M, int W, double *Hd, T *C, const Ctrl *ctrl, cudaStream_t s);
-template <typename T>
 int launch_chol(const double *G, int M, int W, int pass, int step, double inv_thresh2,
                 double piv_rel2, double *R1, T *Rinv, double *Hs, T *Bout, Ctrl *ctrl,
                 cudaStream_t s);
@@ -121,21 +119,23 @@ int launch_assemble_diag(int W, const T *basis, int64_t stride, int nblk, const 
 struct FrontierBufs {
     uint8_t *gen = nullptr;
     int32_t *tgen = nullptr, *alist = nullptr, *acount = nullptr;
+    int32_t *lists = nullptr;          // levels + 1 lists of nt tiles
     unsigned char *zeroed = nullptr;   // qlev, tcnt (the barrier behind it) and vis: cleared first
     size_t zero_bytes = 0;
     int32_t *qlev = nullptr, *tcnt = nullptr, *queue = nullptr;
     int32_t *sync = nullptr;           // barrier count, error flag
     uint32_t *vis = nullptr;
     int levels = 0;
-    // number of tiles within k hops (device)
+    int64_t nt = 0;
+    // the tiles within k hops in index order, and their number (device)
+    const int32_t *list(int k) const { return lists + (k < levels ? k : levels) * nt; }
     const int32_t *count(int k) const { return acount + (k < levels ? k : levels); }
 };
-// Lays the arrays out from base (nullptr: sizes only); *bytes receives their size.
-void plan_frontier(FrontierBufs &f, int64_t n, unsigned char *base, size_t *bytes);
-// Hop distances up to `levels` from the nodes, and the tile list.
-int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, int levels, cudaStream_t s);
-// The tiles within k hops in index order into list, their number into *count.
-int launch_tile_list(const FrontierBufs &f, int64_t n, int k, int32_t *list, int32_t *count, cudaStream_t s);
+// Lays the arrays out from base (nullptr: sizes only) for a search of `levels` hops; *bytes
+// receives their size.
+void plan_frontier(FrontierBufs &f, int64_t n, int levels, unsigned char *base, size_t *bytes);
+// Hop distances up to f.levels from the nodes, and the tile lists.
+int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, cudaStream_t s);
 // Zeros on the tiles within f.levels hops: see k_zero_tiles.
 int launch_zero_tiles(void *blocks, int64_t block_bytes, int nblk, int row_bytes, int64_t n, bool ring,
                       const FrontierBufs &f, cudaStream_t s);

@@ -121,9 +121,10 @@ struct Arena {
         off += bytes;
         return p;
     }
-    void frontier(FrontierBufs &f, int64_t n) {
+    // hops: the last step whose products the search has to cover (0: no restriction)
+    void frontier(FrontierBufs &f, int64_t n, int hops) {
         size_t bytes = 0;
-        plan_frontier(f, n, base ? reinterpret_cast<unsigned char *>(base + off) : nullptr, &bytes);
+        plan_frontier(f, n, hops <= FRONTIER_MAX_HOPS ? hops + 1 : 0, base ? reinterpret_cast<unsigned char *>(base + off) : nullptr, &bytes);
         off += bytes;
     }
 };
@@ -216,7 +217,7 @@ struct CblBufs {
     int32_t *reo_skip;   // ... and the flag that skips the second pass
     Ctrl *ctrl, *ctrl2, *ctrl_chk;
     FrontierBufs fr;
-    int32_t *olist, *ocount;   // ordered solves: the step's tiles in index order
+    unsigned *hcnt;   // CTA counter of the reduction that forms H_kk
 };
 
 template <typename T>
@@ -251,9 +252,8 @@ void plan_cbl(Arena &ar, CblBufs<T> &b, int64_t n, int M, int W, int m, int rb_g
     b.ctrl = ar.take<Ctrl>(1);
     b.ctrl2 = ar.take<Ctrl>(1);
     b.ctrl_chk = ar.take<Ctrl>(1);
-    ar.frontier(b.fr, n);
-    b.olist = ar.take<int32_t>(size_t((n + ACT_ROWS - 1) / ACT_ROWS));
-    b.ocount = ar.take<int32_t>(1);
+    ar.frontier(b.fr, n, m);
+    b.hcnt = ar.take<unsigned>(1);
 }
 
 template <typename T>
@@ -297,7 +297,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             }
             return launch_scatter<T>(b.basis, W, nodes, M, 0, T(1), c.s);
         };
-        if (c.frontier) KB_TRY(launch_frontier(c.g->dev, b.fr, nodes, M, m + 1, c.s));
+        if (c.frontier) KB_TRY(launch_frontier(c.g->dev, b.fr, nodes, M, c.s));
         KB_TRY(start_blocks());
         // slots of steps after a stop are never written: keep them zero
         KB_CUDA_TRY(cudaMemsetAsync(b.Cbs, 0, sizeof(C) * size_t(m) * W * W * 6, c.s));
@@ -308,18 +308,19 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             ra.ordered = c.ordered;
             ra.tgen = tg;
             ra.limit = k;
-            ra.alist = tg ? b.fr.alist : nullptr;
+            ra.alist = tg ? b.fr.list(k) : nullptr;
             ra.acount = tg ? b.fr.count(k) : nullptr;
         };
-        // a launch with a Gram in an ordered solve: the tiles of step k in index order
+        // a launch with a Gram in an ordered solve: all tiles of step k
         auto in_order = [&](RowArgs<T> &ra, int k) {
             if (!ord || !tg) return;
             ra.limit = k;
-            ra.alist = b.olist;
-            ra.acount = b.ocount;
+            ra.alist = b.fr.list(k);
+            ra.acount = b.fr.count(k);
         };
         const size_t WW = size_t(W) * W;
         auto blk = [&](int j) { return b.basis + int64_t(two ? j % 3 : j) * bs; };
+        KB_CUDA_TRY(cudaMemsetAsync(b.hcnt, 0, sizeof(unsigned), c.s));
         int nchk = 0;
         int kfac = 0;   // blocks of the spline kernel's factorisation that earlier checks formed
         const SplineBufs sbufs{b.V0, b.V1, b.V2, b.Hdf, b.Hdf + size_t(m) * M * M, b.bt_ls};
@@ -332,7 +333,6 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             C *Bk = b.Bs + (k - 1) * WW;
             C *S1 = b.Rs1 + (k - 1) * WW, *S2 = b.Rs2 + (k - 1) * WW;
             C *Cl = b.Cloc + 2 * (k - 1) * WW;
-            if (ord && tg) KB_TRY(launch_tile_list(b.fr, n, k, b.olist, b.ocount, c.s));
             // Q_k is supported on rows within k-1 hops of W; L Q_k within k hops
             // block SpMM: W = L Q_k
             LinEpi<T> e;
@@ -342,7 +342,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             e.tgen = tg;
             e.gen = tg ? b.fr.gen : nullptr;
             e.limit = k;
-            e.alist = tg ? b.fr.alist : nullptr;
+            e.alist = tg ? b.fr.list(k) : nullptr;
             e.acount = tg ? b.fr.count(k) : nullptr;
             KB_TRY(launch_spmm<T>(c.g->dev, W, Qk, e, c.s, nullptr, M, 0));
             ++c.spmm;
@@ -353,8 +353,8 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             within(pa, k - 1);   // (Q_k is zero elsewhere)
             in_order(pa, k);
             KB_TRY(launch_rowblock<T>(RB_PROJ, W, pa, c.s, &grid, M));
-            KB_TRY(launch_reduce<C>(b.parts, grid, W * W, b.Gsum, c.s, b.ctrl));
-            KB_TRY(launch_hkk<C>(b.Gsum, M, W, b.Hd + size_t(k - 1) * M * M, Cb, b.ctrl, c.s));
+            KB_TRY(launch_reduce_hkk<C>(b.parts, grid, M, W, b.Gsum, b.Hd + size_t(k - 1) * M * M, Cb, b.hcnt, b.ctrl,
+                                        c.s));
             if (k == m) break;   // Q_{m+1} is never used
             // three-term update: X = L Q_k - Q_{k-1} H_{k-1,k} - Q_k H_kk, then Gram X^T X
             T *X = blk(k);
@@ -479,7 +479,8 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             RowArgs<T> aa;
             aa.n = n; aa.basis = b.basis; aa.block_stride = bs; aa.nblk = m; aa.ca = b.Ut;
             aa.y = Y; aa.ldy = ldy; aa.mo = M; aa.ctrl = b.ctrl;
-            within(aa, m);   // (all tiles are written; the list only orders them)
+            within(aa, m);
+            aa.alist = tg ? b.fr.alist : nullptr;   // all tiles, by rising distance
             int grid = 0;
             KB_TRY(launch_rowblock<T>(RB_ASM, W, aa, c.s, &grid, M));
         } else {
@@ -493,7 +494,8 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                 RowArgs<T> aa;
                 aa.n = n; aa.basis = Qk; aa.block_stride = bs; aa.nblk = 1;
                 aa.ca = b.Ut + (k - 1) * WW; aa.y = Y; aa.ldy = ldy; aa.mo = M;
-                within(aa, k - 1);   // (the first launch writes all of Y)
+                within(aa, k - 1);
+                if (k == 1) aa.alist = tg ? b.fr.alist : nullptr;   // (the first launch writes all of Y)
                 aa.kbase = k - 1; aa.accumulate = k > 1 ? 1 : 0;
                 int grid = 0;
                 KB_TRY(launch_rowblock<T>(RB_ASM, W, aa, c.s, &grid, M));
@@ -505,7 +507,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                 e.tgen = tg;
                 e.gen = tg ? b.fr.gen : nullptr;
                 e.limit = k;
-                e.alist = tg ? b.fr.alist : nullptr;
+                e.alist = tg ? b.fr.list(k) : nullptr;
                 e.acount = tg ? b.fr.count(k) : nullptr;
                 KB_TRY(launch_spmm<T>(c.g->dev, W, Qk, e, c.s, nullptr, M, 0));
                 ++c.spmm;
@@ -571,7 +573,7 @@ void plan_lz(Arena &ar, LzBufs<T> &b, int64_t n, int W, int m, int pgrid, bool t
     b.omega = ar.take<double>(size_t(m) * W);
     b.ctrl = ar.take<Ctrl>(1);
     b.ctrl2 = ar.take<Ctrl>(1);
-    ar.frontier(b.fr, n);
+    ar.frontier(b.fr, n, m);
 }
 
 template <typename T>
@@ -615,7 +617,7 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
             else KB_TRY(launch_zero_tiles(b.basis, bs * sizeof(T), nbuf, W * int(sizeof(T)), n, !two, b.fr, c.s));
             return launch_scatter<T>(b.basis, W, nodes, M, 0, T(1), c.s);
         };
-        if (c.frontier) KB_TRY(launch_frontier(c.g->dev, b.fr, nodes, M, m + 1, c.s));
+        if (c.frontier) KB_TRY(launch_frontier(c.g->dev, b.fr, nodes, M, c.s));
         KB_TRY(start_blocks());
         // coefficients of steps after an invariant stop are never written: keep them zero
         KB_CUDA_TRY(cudaMemsetAsync(b.c1, 0, sizeof(double) * size_t(m + 1) * W, c.s));
@@ -635,7 +637,7 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
             e.tgen = tg;
             e.gen = tg ? b.fr.gen : nullptr;
             e.limit = k;
-            e.alist = tg ? b.fr.alist : nullptr;
+            e.alist = tg ? b.fr.list(k) : nullptr;
             e.acount = tg ? b.fr.count(k) : nullptr;
             e.a1 = b.c1 + int64_t(k - 1) * W;
             e.a2 = b.c2 + int64_t(k - 1) * W;
@@ -652,7 +654,7 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
             if (k == m) break;
             int grid2 = 0;
             KB_TRY(launch_axpy_colnorm<T>(W, X, Pk, b.aupd + int64_t(k - 1) * W, n, b.parts, &grid2,
-                                          b.ctrl, tg, k, M, c.s, tg ? b.fr.alist : nullptr, tg ? b.fr.count(k) : nullptr));
+                                          b.ctrl, tg, k, M, c.s, tg ? b.fr.list(k) : nullptr, tg ? b.fr.count(k) : nullptr));
             KB_TRY(launch_lanczos_beta(b.parts, grid2, W, M, gbl ? 1 : 0, k - 1, f64 ? 0 : 1, thresh, b.beta,
                                        b.sigma, b.alive, b.c1 + int64_t(k) * W, b.c2 + int64_t(k) * W,
                                        b.ctrl, c.s));
@@ -676,7 +678,7 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
                 e.tgen = tg;
                 e.gen = tg ? b.fr.gen : nullptr;
                 e.limit = k;
-                e.alist = tg ? b.fr.alist : nullptr;
+                e.alist = tg ? b.fr.list(k) : nullptr;
                 e.acount = tg ? b.fr.count(k) : nullptr;
                 e.a1 = b.c1 + int64_t(k - 1) * W;
                 e.a2 = b.c2 + int64_t(k - 1) * W;
@@ -690,7 +692,7 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
                 ++c.spmm;
                 int grid2 = 0;
                 KB_TRY(launch_axpy_colnorm<T>(W, X, Pk, b.aupd + int64_t(k - 1) * W, n, b.parts, &grid2,
-                                              b.ctrl2, tg, k, M, c.s, tg ? b.fr.alist : nullptr, tg ? b.fr.count(k) : nullptr));
+                                              b.ctrl2, tg, k, M, c.s, tg ? b.fr.list(k) : nullptr, tg ? b.fr.count(k) : nullptr));
                 KB_TRY(launch_assemble_diag<T>(W, X, bs, 1, b.omega + int64_t(k) * W, n, Y, ldy, M, M,
                                                tg, b.ctrl, c.s, k, 1));
             }
@@ -720,7 +722,7 @@ int cheb_pass(Common &c, const std::vector<double> &coef, double lam, int W, int
     // b_h = w_h S
     int cur_i = 0, prev_i = -1;
     if (Zsrc) {
-        KB_TRY(launch_scale_copy<T>(bufs[0], Zsrc, n, W, w[h], fr ? fr->alist : nullptr,
+        KB_TRY(launch_scale_copy<T>(bufs[0], Zsrc, n, W, w[h], fr ? fr->list(hop0) : nullptr,
                                     fr ? fr->count(hop0) : nullptr, c.s));
     } else {
         if (!fr) KB_CUDA_TRY(cudaMemsetAsync(bufs[0], 0, sizeof(T) * size_t(n) * W, c.s));
@@ -738,7 +740,7 @@ int cheb_pass(Common &c, const std::vector<double> &coef, double lam, int W, int
         e.tgen = fr ? fr->tgen : nullptr;
         e.gen = fr ? fr->gen : nullptr;
         e.limit = hop;
-        e.alist = fr ? fr->alist : nullptr;
+        e.alist = fr ? (last && yout ? fr->alist : fr->list(hop)) : nullptr;
         e.acount = fr ? fr->count(hop) : nullptr;
         e.zero_inactive = last && yout ? 1 : 0;
         e.s1 = (last ? -2.0 : -4.0) / lam;
@@ -764,7 +766,7 @@ int cheb_pass(Common &c, const std::vector<double> &coef, double lam, int W, int
 }
 
 template <typename T>
-void plan_cheb(Arena &ar, int64_t n, int Mmax, bool squared, T **bufs, T **Z, int32_t **marker,
+void plan_cheb(Arena &ar, int64_t n, int Mmax, bool squared, int hops, T **bufs, T **Z, int32_t **marker,
                FrontierBufs &fr) {
     // bufs and Z are consecutive blocks of n Wmax elements
     const int Wmax = width_for(Mmax);
@@ -772,7 +774,7 @@ void plan_cheb(Arena &ar, int64_t n, int Mmax, bool squared, T **bufs, T **Z, in
     for (int i = 0; i < 3; ++i) bufs[i] = p ? p + size_t(i) * n * Wmax : nullptr;
     *Z = squared && p ? p + size_t(3) * n * Wmax : nullptr;
     *marker = ar.take<int32_t>(size_t(n));
-    ar.frontier(fr, n);
+    ar.frontier(fr, n, hops);
 }
 
 template <typename T>
@@ -786,10 +788,10 @@ int run_cheb(Common &c, bool squared, const int32_t *nodes, int M, int m, float 
     T *bufs[3], *Z;
     int32_t *marker;
     FrontierBufs fb;
-    plan_cheb<T>(dry, n, Mmax, squared, bufs, &Z, &marker, fb);
+    plan_cheb<T>(dry, n, Mmax, squared, squared ? 2 * h : h, bufs, &Z, &marker, fb);
     Arena ar;
     KB_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void **>(&ar.base), dry.off, c.s));
-    plan_cheb<T>(ar, n, Mmax, squared, bufs, &Z, &marker, fb);
+    plan_cheb<T>(ar, n, Mmax, squared, squared ? 2 * h : h, bufs, &Z, &marker, fb);
     auto body = [&]() -> int {
         for (int col0 = 0; col0 < M; col0 += Mmax) {
             const int Mc = std::min(Mmax, M - col0);
@@ -799,7 +801,7 @@ int run_cheb(Common &c, bool squared, const int32_t *nodes, int M, int m, float 
             const FrontierBufs *fr = c.frontier ? &fb : nullptr;
             if (c.frontier) {
                 // Clenshaw blocks rotate and are written on reached tiles only: zeros on all of those
-                KB_TRY(launch_frontier(c.g->dev, fb, nodes + col0, Mc, (squared ? 2 * h : h) + 1, c.s));
+                KB_TRY(launch_frontier(c.g->dev, fb, nodes + col0, Mc, c.s));
                 KB_TRY(launch_zero_tiles(bufs[0], int64_t(sizeof(T)) * n * width_for(Mmax), squared ? 4 : 3,
                                          W * int(sizeof(T)), n, false, fb, c.s));
             }
@@ -846,8 +848,8 @@ size_t workspace_bytes_t(int64_t n, kb_method method, int M, int m, bool two, co
             T *bufs[3], *Z;
             int32_t *marker;
             FrontierBufs fb;
-            plan_cheb<T>(dry, n, std::min(M, sizeof(T) == 8 ? 64 : 128), method == KB_CHEB2, bufs, &Z, &marker,
-                         fb);
+            plan_cheb<T>(dry, n, std::min(M, sizeof(T) == 8 ? 64 : 128), method == KB_CHEB2,
+                         method == KB_CHEB2 ? 2 * (m / 2) : m, bufs, &Z, &marker, fb);
             break;
         }
     }

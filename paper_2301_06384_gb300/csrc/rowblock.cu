@@ -22,27 +22,55 @@ extern template int launch_ordered<128>(int, const RowArgs<float> &, cudaStream_
 namespace {
 
 // ---------------------------------------------------------------- deterministic reduction
+// The diagonal block H_kk = (G + G^T) / 2 of Algorithm 1, formed by the reduction's last CTA: Hd (M x
+// M) and C (W x W, the small matrix of the update), rounded to the basis precision, exactly as
+// the update subtracts it.  cnt: a counter that wraps to zero by itself.
+template <typename P>
+struct HkkOut {
+    double *Hd = nullptr;
+    P *C = nullptr;
+    unsigned *cnt = nullptr;
+    int M = 0, W = 0;
+};
+
+// out[e] = sum of the partials' entries e.  32 entries per CTA, its warps over the partials with
+// RU loads in flight per lane (each into its own accumulator, merged in a fixed order), then a
+// fixed-order combination of the warps' sums by warp 0.  FP32 partials are summed in
+// double-float on the FP32 pipe.
 template <typename P>
 __global__ void __launch_bounds__(1024) k_reduce(const P *__restrict__ parts, int nparts, int len,
                                                   double *__restrict__ out, const Ctrl *ctrl,
-                                                  P *__restrict__ out_p, const int32_t *skip) {
-    // 32 columns per CTA, 32 warps over the partials (two loads in flight per lane), then a
-    // fixed-order combination of the warps' sums by warp 0
+                                                  P *__restrict__ out_p, const int32_t *skip, HkkOut<P> h) {
     if ((ctrl && ctrl->stop) || (skip && *skip)) return;
     __shared__ double s[32][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int e = blockIdx.x * 32 + lane;
     if constexpr (std::is_same<P, float>::value) {
-        // double-float accumulation on the FP32 pipe
+        // (two accumulators, each its own partials in rising order: the order of these sums is part
+        // of the ordered form's fixed rounding)
         DF a0{0.f, 0.f}, a1{0.f, 0.f};
         if (e < len) {
             int p = warp;
-            for (; p + nw < nparts; p += 2 * nw) {
-                const float v0 = parts[int64_t(p) * len + e], v1 = parts[int64_t(p + nw) * len + e];
-                df_add(a0, v0);
-                df_add(a1, v1);
+            for (; p + 7 * nw < nparts; p += 8 * nw) {
+                float v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = parts[int64_t(p + u * nw) * len + e];
+#pragma unroll
+                for (int u = 0; u < 8; u += 2) {
+                    df_add(a0, v[u]);
+                    df_add(a1, v[u + 1]);
+                }
             }
-            if (p < nparts) df_add(a0, parts[int64_t(p) * len + e]);
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = p + u * nw < nparts ? parts[int64_t(p + u * nw) * len + e] : 0.f;
+            // the last pair is taken together only when both exist; an odd one goes to a0
+#pragma unroll
+            for (int u = 0; u < 8; u += 2)
+                if (p + u * nw < nparts) {
+                    df_add(a0, v[u]);
+                    if (p + (u + 1) * nw < nparts) df_add(a1, v[u + 1]);
+                }
         }
         df_merge(a0, a1);
         reinterpret_cast<DF *>(&s[warp][0])[lane] = a0;
@@ -66,6 +94,23 @@ __global__ void __launch_bounds__(1024) k_reduce(const P *__restrict__ parts, in
             out[e] = t;
             if (out_p) out_p[e] = P(t);
         }
+    }
+    if (h.cnt) {
+        __shared__ unsigned last;
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicInc(h.cnt, gridDim.x - 1);
+        __syncthreads();
+        if (last != gridDim.x - 1) return;
+        __threadfence();
+        for (int i = warp; i < h.W; i += nw)
+            for (int j = lane; j < h.W; j += 32) {
+                double v = 0.0;
+                if (i < h.M && j < h.M) v = 0.5 * (__ldcg(out + i * h.W + j) + __ldcg(out + j * h.W + i));
+                const P vt = P(v);
+                if (i < h.M && j < h.M) h.Hd[i * h.M + j] = double(vt);
+                h.C[i * h.W + j] = vt;
+            }
     }
 }
 
@@ -158,16 +203,38 @@ int rowblock_max_grid(int W) {
 }
 
 template <typename P>
-int launch_reduce(const P *parts, int nparts, int len, double *out, cudaStream_t s,
-                  const Ctrl *ctrl, P *out_p, const int32_t *skip) {
+static int reduce_impl(const P *parts, int nparts, int len, double *out, cudaStream_t s, const Ctrl *ctrl, P *out_p,
+                       const int32_t *skip, const HkkOut<P> &h) {
     prof_begin(KernelClass::REDUCE, s);
-    k_reduce<P><<<(len + 31) / 32, 1024, 0, s>>>(parts, nparts, len, out, ctrl, out_p, skip);
+    k_reduce<P><<<(len + 31) / 32, 1024, 0, s>>>(parts, nparts, len, out, ctrl, out_p, skip, h);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return cuda_fail(err, "k_reduce launch");
     prof_end(KernelClass::REDUCE, s, double(nparts) * len * sizeof(P), 0);
     return 0;
 }
 
+template <typename P>
+int launch_reduce(const P *parts, int nparts, int len, double *out, cudaStream_t s,
+                  const Ctrl *ctrl, P *out_p, const int32_t *skip) {
+    return reduce_impl<P>(parts, nparts, len, out, s, ctrl, out_p, skip, HkkOut<P>{});
+}
+
+template <typename P>
+int launch_reduce_hkk(const P *parts, int nparts, int M, int W, double *G, double *Hd, P *C, unsigned *cnt,
+                      const Ctrl *ctrl, cudaStream_t s) {
+    HkkOut<P> h;
+    h.Hd = Hd;
+    h.C = C;
+    h.cnt = cnt;
+    h.M = M;
+    h.W = W;
+    return reduce_impl<P>(parts, nparts, W * W, G, s, ctrl, nullptr, nullptr, h);
+}
+
+template int launch_reduce_hkk<float>(const float *, int, int, int, double *, double *, float *, unsigned *,
+                                      const Ctrl *, cudaStream_t);
+template int launch_reduce_hkk<double>(const double *, int, int, int, double *, double *, double *, unsigned *,
+                                       const Ctrl *, cudaStream_t);
 template int launch_rowblock<float>(int, int, const RowArgs<float> &, cudaStream_t, int *, int64_t);
 template int launch_rowblock<double>(int, int, const RowArgs<double> &, cudaStream_t, int *, int64_t);
 template int rowblock_max_grid<float>(int);

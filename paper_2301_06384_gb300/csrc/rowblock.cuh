@@ -56,7 +56,6 @@
 namespace kb {
 namespace rb {
 
-constexpr int RB_THREADS = 256;
 constexpr int NST = 3;   // cp.async stages
 
 template <typename C>
@@ -151,14 +150,14 @@ struct RowGeo {
     int Mk, CG, RG, TR;      // columns in use (multiple of 4), column groups, row groups, rows
     int NI, NJ, NB, NGR;     // Gram blocks along i and j, their number, row groups of the Gram
 };
-template <typename T, int W, int MODE, int RPT, bool ORD = false>
+template <typename T, int W, int MODE, int RPT, bool ORD, int NT>
 __host__ __device__ inline RowGeo row_geo(int M) {
     using G = Geo<T, W, ORD>;
     RowGeo r;
     r.Mk = (M + 3) / 4 * 4;
     r.CG = r.Mk / 4;
     const int cap = 256;     // rows: bounds the shared memory of narrow blocks
-    int tr = (RB_THREADS / r.CG) * RPT;
+    int tr = (NT / r.CG) * RPT;
     tr = (tr < cap ? tr : cap) / 32 * 32;
     r.TR = tr < 32 ? 32 : tr;
     if (ORD) r.TR = G::TO * G::SO;
@@ -172,7 +171,7 @@ __host__ __device__ inline RowGeo row_geo(int M) {
         r.NB = 0;
         for (int b = 0; b < r.NI; ++b) r.NB += r.NJ - 2 * b;
     }
-    r.NGR = RB_THREADS / r.NB;
+    r.NGR = NT / r.NB;
     if (ORD || r.NGR < 1) r.NGR = 1;
     return r;
 }
@@ -197,8 +196,8 @@ inline size_t smem_bytes(const RowGeo &r) {
     return e * sizeof(C);
 }
 
-template <typename T, int W, int MODE, int RPT, bool ORD>
-__global__ void __launch_bounds__(RB_THREADS, sizeof(typename Cmp<T>::type) == 8 ? 1 : 2)
+template <typename T, int W, int MODE, int RPT, bool ORD, int NT>
+__global__ void __launch_bounds__(NT, sizeof(typename Cmp<T>::type) == 8 ? 1 : 512 / NT)
 k_rowblock(RowArgs<T> a) {
     using G = Geo<T, W, ORD>;
     using C = typename G::C;
@@ -206,13 +205,14 @@ k_rowblock(RowArgs<T> a) {
     constexpr bool GRAM = MODE == RB_PROJ || MODE == RB_UPD || MODE == RB_MULGRAM || MODE == RB_ASMSUB;
     constexpr bool SUBX = MODE == RB_UPD || MODE == RB_ASMSUB;     // out = X - product
     constexpr bool MULTI = MODE == RB_ASM || MODE == RB_ASMSUB;    // product over basis blocks
+    constexpr bool ASYNC_X = SUBX && std::is_same<T, typename G::C>::value;   // X comes by cp.async
     constexpr int BI = G::BI, BJ = G::BJ, KC = G::KC, LDA = G::LDA, LDO = G::LDO, VEC = G::VEC;
     if (MODE != RB_ASM && a.ctrl && a.ctrl->stop) return;
     if (a.skip && *a.skip) return;
 
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C *sm = reinterpret_cast<C *>(smem_raw);
-    const RowGeo q = row_geo<T, W, MODE, RPT, ORD>(a.M);
+    const RowGeo q = row_geo<T, W, MODE, RPT, ORD, NT>(a.M);
     const int SE = int(stage_elems<T, W, MODE>(q));
     C *sO = sm + NST * SE;                                          // [TR][LDO]
     C *sG = PROD ? sO + q.TR * LDO : sO;                            // [NGR * NB][BI * BJ] (W = 128)
@@ -326,7 +326,7 @@ k_rowblock(RowArgs<T> a) {
             if (ch < nch) {
                 C *dx = sm + st * SE, *dq = dx + PR * W;
                 constexpr int EPV = std::is_same<T, C>::value ? VEC : 4;   // elements of a copy
-                for (int i = tid; i < PR * W / EPV; i += RB_THREADS) {
+                for (int i = tid; i < PR * W / EPV; i += NT) {
                     const int r = i / (W / EPV), c = (i % (W / EPV)) * EPV;
                     if (c >= q.Mk) continue;   // (columns past M are not read by the sums)
                     const int64_t t = PR >= ACT_ROWS ? tile_at(ch * EPC + r / ACT_ROWS) : tile_at(ch / CPE);
@@ -350,7 +350,7 @@ k_rowblock(RowArgs<T> a) {
             cp_commit();
         };
         // columns Mk .. roundup(M, 8) are read by the blocks at the edge: zero them once
-        for (int i = tid; i < NST * 2 * PR * (W - q.Mk); i += RB_THREADS) {
+        for (int i = tid; i < NST * 2 * PR * (W - q.Mk); i += NT) {
             const int c = q.Mk + i % (W - q.Mk), r = i / (W - q.Mk);
             sm[r * W + c] = C(0);
         }
@@ -363,7 +363,7 @@ k_rowblock(RowArgs<T> a) {
                 if (pvt < olen) {
                     C *dx = sm + s * SE, *dq = dx + PR * W;
                     const int64_t r0 = otile(pvt) * G::TO + ph * PR;
-                    for (int i = tid; i < PR * W / VEC; i += RB_THREADS) {
+                    for (int i = tid; i < PR * W / VEC; i += NT) {
                         const int r = i / (W / VEC), c = (i % (W / VEC)) * VEC;
                         if (c >= q.Mk) continue;
                         const bool in = r0 + r < a.n;
@@ -413,8 +413,9 @@ k_rowblock(RowArgs<T> a) {
         __syncthreads();
     } else {
         // ---------------------------------------------------------------- products
-        // permuted warps: the columns of warps w and w + 4 (one scheduler) are w and 7 - w
-        const int pt = (warp < 4 ? warp : 11 - warp) * 32 + lane;
+        // permuted warps: with eight the columns of warps w and w + 4 (one scheduler) are w and
+        // 7 - w; with four the columns go round from CTA to CTA
+        const int pt = (NT == 128 ? (warp + int(blockIdx.x)) % 4 : warp < 4 ? warp : 11 - warp) * 32 + lane;
         const bool live = pt < q.CG * q.RG;
         const int cg = live ? pt / q.RG : 0, rg = live ? pt % q.RG : 0;
         const int col4 = cg * 4;
@@ -487,7 +488,7 @@ k_rowblock(RowArgs<T> a) {
                 C *dA = sm + st * SE, *dC = dA + q.TR * LDA;
                 constexpr int EPV = std::is_same<T, C>::value ? VEC : 4;
                 constexpr int VPR = KC / EPV;      // copies per row
-                for (int i = tid; i < q.TR * VPR; i += RB_THREADS) {
+                for (int i = tid; i < q.TR * VPR; i += NT) {
                     const int r = i / VPR, c = (i % VPR) * EPV;
                     if (pk0 + c >= q.Mk) continue;
                     const int64_t t = vt_tile(pvt, r / ACT_ROWS);
@@ -503,7 +504,7 @@ k_rowblock(RowArgs<T> a) {
                     }
                 }
                 const int crows = min(KC, q.Mk - pk0);
-                for (int i = tid; i < crows * W / VEC; i += RB_THREADS)
+                for (int i = tid; i < crows * W / VEC; i += NT)
                     cp16(dC + i * VEC, cmat + pk0 * W + i * VEC, true);
                 pk0 += KC;
                 if (pk0 >= q.Mk) {
@@ -517,9 +518,21 @@ k_rowblock(RowArgs<T> a) {
             cp_commit();
         };
         // the columns past Mk of the output tile stay zero
-        for (int i = tid; i < q.TR * (LDO - q.Mk); i += RB_THREADS)
+        for (int i = tid; i < q.TR * (LDO - q.Mk); i += NT)
             sO[(i / (LDO - q.Mk)) * LDO + q.Mk + i % (LDO - q.Mk)] = C(0);
         for (int s = 0; s < NST - 1; ++s) issue(s);
+        // X of a virtual tile to the output tile, asynchronously, once the previous tile is done
+        // with that; its copies belong to the next chunk's group
+        auto load_x = [&](int64_t vt) {
+            for (int i = tid; i < q.TR * (W / VEC); i += NT) {
+                const int r = i / (W / VEC), c = (i % (W / VEC)) * VEC;
+                if (c >= q.Mk) continue;
+                const int64_t t = vt_tile(vt, r / ACT_ROWS);
+                const int64_t row = t * ACT_ROWS + r % ACT_ROWS;
+                const bool in = t >= 0 && row < a.n;
+                cp16(sO + r * LDO + c, a.x + (in ? row * W + c : 0), in);
+            }
+        };
         int st = 0;
         for (int64_t vt = vt0; vt < nvt; vt = vt_next(vt)) {
             const int kb0 = first_kb(vt);
@@ -550,6 +563,9 @@ k_rowblock(RowArgs<T> a) {
                 for (int k0 = 0; k0 < q.Mk; k0 += KC) {
                     cp_wait<NST - 2>();
                     __syncthreads();
+                    if constexpr (ASYNC_X) {
+                        if (kb == kb0 && k0 == 0) load_x(vt);
+                    }
                     issue(st == 0 ? NST - 1 : st - 1);
                     const C *pA = sm + st * SE + rg * LDA;
                     const C *pC = sm + st * SE + q.TR * LDA + col4;
@@ -585,16 +601,32 @@ k_rowblock(RowArgs<T> a) {
             // The register tile goes to shared memory (UPD subtracts it from X on the way).
             // With an empty K loop no barrier has separated this from the previous tile.
             if (kb0 >= nkb) __syncthreads();
+            if constexpr (ASYNC_X) {
+                // (kb0 < nkb: UPD has a block always, ASMSUB the block of the seeds or a nearer one;
+                // otherwise X is loaded here)
+                if (kb0 >= nkb) {
+                    load_x(vt);
+                    cp_commit();
+                }
+                // the chunks after the one X came with may be too few to have waited for it
+                if ((nkb - kb0) * ((q.Mk + KC - 1) / KC) < NST) cp_wait<0>();
+                // other threads' copies
+                __syncthreads();
+            }
             if (live) {
 #pragma unroll
                 for (int r = 0; r < RPT; ++r) {
                     const int lr = rg + q.RG * r;
                     C o[4];
                     if (SUBX) {
-                        const int64_t t = vt_tile(vt, lr / ACT_ROWS);
-                        const int64_t row = t * ACT_ROWS + lr % ACT_ROWS;
                         C xv[4] = {0, 0, 0, 0};
-                        if (t >= 0 && row < a.n) ldg4<T>(a.x + row * W + col4, xv);
+                        if constexpr (std::is_same<T, C>::value) {
+                            ld4<C>(sO + lr * LDO + col4, xv);
+                        } else {
+                            const int64_t t = vt_tile(vt, lr / ACT_ROWS);
+                            const int64_t row = t * ACT_ROWS + lr % ACT_ROWS;
+                            if (t >= 0 && row < a.n) ldg4<T>(a.x + row * W + col4, xv);
+                        }
 #pragma unroll
                         for (int u = 0; u < 4; ++u) o[u] = xv[u] - acc[r][u];
                     } else {
@@ -612,7 +644,7 @@ k_rowblock(RowArgs<T> a) {
             __syncthreads();
             // whole rows to HBM
             constexpr int CPR = W / 4;
-            for (int i = tid; i < q.TR * CPR; i += RB_THREADS) {
+            for (int i = tid; i < q.TR * CPR; i += NT) {
                 const int r = i / CPR, c = (i % CPR) * 4;
                 const int64_t t = vt_tile(vt, r / ACT_ROWS);
                 const int64_t row = t * ACT_ROWS + r % ACT_ROWS;
@@ -663,7 +695,7 @@ k_rowblock(RowArgs<T> a) {
         }
         __syncthreads();
         C *p = a.partials + int64_t(blockIdx.x) * W * W;
-        for (int e = tid; e < W * W; e += RB_THREADS) {
+        for (int e = tid; e < W * W; e += NT) {
             int i = e / W, j = e % W;
             C v = 0;
             if (i < a.M && j < a.M) {
@@ -683,32 +715,32 @@ k_rowblock(RowArgs<T> a) {
     }
 }
 
-constexpr int RB_MAX_CTAS = 4;   // per SM: bounds the Gram partials
+constexpr int RB_MAX_CTAS = 5;   // per SM: bounds the Gram partials
 
 // Resident CTAs per SM of an instance with smem bytes of dynamic shared memory.  The attribute
 // is raised once per instance to the most any block can take.
-template <typename T, int W, int MODE, int RPT, bool ORD>
+template <typename T, int W, int MODE, int RPT, bool ORD, int NT>
 int occupancy(size_t smem) {
     static const cudaError_t attr = cudaFuncSetAttribute(
-        k_rowblock<T, W, MODE, RPT, ORD>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        k_rowblock<T, W, MODE, RPT, ORD, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     (void)attr;
     int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rowblock<T, W, MODE, RPT, ORD>, RB_THREADS, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rowblock<T, W, MODE, RPT, ORD, NT>, NT, smem);
     return std::max(1, std::min(per_sm, RB_MAX_CTAS));
 }
 
-template <typename T, int W, int MODE, int RPT, bool ORD = false>
+template <typename T, int W, int MODE, int RPT, bool ORD, int NT>
 int launch_r(const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
     using G = Geo<T, W, ORD>;
-    const RowGeo q = row_geo<T, W, MODE, RPT, ORD>(a.M);
+    const RowGeo q = row_geo<T, W, MODE, RPT, ORD, NT>(a.M);
     const size_t smem = smem_bytes<T, W, MODE, ORD>(q);
     const int64_t unit = ORD ? G::TO : MODE == RB_PROJ ? G::PR : q.TR;
     const int64_t nvt = (a.n + unit - 1) / unit;
-    const int per_sm = occupancy<T, W, MODE, RPT, ORD>(smem);
+    const int per_sm = occupancy<T, W, MODE, RPT, ORD, NT>(smem);
     int grid = int(std::min<int64_t>(nvt, int64_t(num_sms()) * (ORD ? G::CTAS : per_sm)));
     if (grid < 1) grid = 1;
     if (grid_out) *grid_out = grid;
-    k_rowblock<T, W, MODE, RPT, ORD><<<grid, RB_THREADS, smem, s>>>(a);
+    k_rowblock<T, W, MODE, RPT, ORD, NT><<<grid, NT, smem, s>>>(a);
     return 0;
 }
 
@@ -719,11 +751,15 @@ int launch_r(const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
 template <typename T, int W, int MODE>
 int launch_mode(const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
     constexpr int R = sizeof(typename Cmp<T>::type) == 8 || W == 16 ? 4 : 8;
+    // Threads: two CTAs of 256 per SM, or four of 128 for the narrow blocks, whose tiles are
+    // short of arithmetic between their barriers (128^3 grid, M = 32, 40 steps: 24.8 / 24.0 ms;
+    // RGG of 10^6 rows, M = 64, where the taller tile shares the small matrix: 13.2 / 13.6 ms).
+    constexpr int NT = sizeof(typename Cmp<T>::type) == 8 || MODE == RB_PROJ || W >= 64 ? 256 : 128;
     if constexpr (MODE != RB_PROJ) {
-        const RowGeo q = row_geo<T, W, MODE, R>(a.M);
-        if (a.n < int64_t(q.TR) * num_sms()) return launch_r<T, W, MODE, W == 128 ? 4 : 2>(a, s, grid_out);
+        const RowGeo q = row_geo<T, W, MODE, R, false, 256>(a.M);
+        if (a.n < int64_t(q.TR) * num_sms()) return launch_r<T, W, MODE, W == 128 ? 4 : 2, false, 256>(a, s, grid_out);
     }
-    return launch_r<T, W, MODE, R>(a, s, grid_out);
+    return launch_r<T, W, MODE, R, false, NT>(a, s, grid_out);
 }
 
 template <typename T, int W>
@@ -744,10 +780,10 @@ template <int W>
 int launch_ordered(int mode, const RowArgs<float> &a, cudaStream_t s, int *grid_out) {
     constexpr int R = W == 128 ? 8 : 4;
     switch (mode) {
-        case RB_PROJ: return launch_r<float, W, RB_PROJ, R, true>(a, s, grid_out);
-        case RB_UPD: return launch_r<float, W, RB_UPD, R, true>(a, s, grid_out);
-        case RB_MULGRAM: return launch_r<float, W, RB_MULGRAM, R, true>(a, s, grid_out);
-        case RB_ASMSUB: return launch_r<float, W, RB_ASMSUB, R, true>(a, s, grid_out);
+        case RB_PROJ: return launch_r<float, W, RB_PROJ, R, true, 256>(a, s, grid_out);
+        case RB_UPD: return launch_r<float, W, RB_UPD, R, true, 256>(a, s, grid_out);
+        case RB_MULGRAM: return launch_r<float, W, RB_MULGRAM, R, true, 256>(a, s, grid_out);
+        case RB_ASMSUB: return launch_r<float, W, RB_ASMSUB, R, true, 256>(a, s, grid_out);
     }
     return fail(KB_ERR_ARG, "bad ordered row-block mode");
 }

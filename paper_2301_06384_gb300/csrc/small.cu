@@ -9,8 +9,12 @@
 #include <climits>
 #include <type_traits>
 
+#include <cooperative_groups.h>
+
 #include "kb_internal.cuh"
 #include "kb_kernels.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace kb {
 
@@ -130,66 +134,90 @@ int launch_reorth_decide(const double *G, const double *d0, int M, int W, int32_
 }
 
 // ---------------------------------------------------------------- gbl / sbl scalars
-// Reduce [nparts][W] partials per column (fixed order) into s[W].  df: the partials are
-// double-float pairs (FP32 arithmetic), combined on the FP32 pipe; else doubles.
+// The scalars of a step come from [nparts][W] partial column sums.  A cluster of W / 16 CTAs takes
+// 16 columns each (one CTA reading all partials is bound by its SM's L2 bandwidth: 16 us at W =
+// 64, 27 us at W = 128, now 5 and 6 us); the global method's totals meet in distributed shared
+// memory.  df: the partials are double-float pairs (FP32 arithmetic), combined on the FP32
+// pipe; else doubles.
+constexpr int LZ_THREADS = 512;
+constexpr int LZ_COLS = 16;
+
+// Sum of the partials' column blockIdx.x * 16 + c into s[c], c < 16, in a fixed order: 32 strided
+// subsets of the partials, eight loads in flight per thread, then a fixed-order combination.
 __device__ void reduce_cols(const double *parts, int nparts, int W, double *s, int df) {
-    // one warp per strided subset of the partials (up to 32 warps), eight loads in flight per
-    // lane (each into its own accumulator, merged in a fixed order), then a fixed-order
-    // combination of the warps' sums
-    __shared__ double tmp[32][128];
-    constexpr int U = 8;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int c0 = 0; c0 < W; c0 += 32) {
-        const int c = c0 + lane;
-        if (c >= W) continue;
-        if (df) {
-            const DF *pp = reinterpret_cast<const DF *>(parts);
-            DF a[U];
+    __shared__ double tmp[LZ_THREADS / 32][LZ_COLS];
+    constexpr int U = 8, NG = LZ_THREADS / LZ_COLS;
+    const int c = threadIdx.x % LZ_COLS, g = threadIdx.x / LZ_COLS;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t col = int64_t(blockIdx.x) * LZ_COLS + c;
+    if (df) {
+        const DF *pp = reinterpret_cast<const DF *>(parts);
+        DF a[U];
 #pragma unroll
-            for (int u = 0; u < U; ++u) a[u] = DF{0.f, 0.f};
-            int p = warp;
-            for (; p < nparts; p += U * nw) {
-                DF v[U];
+        for (int u = 0; u < U; ++u) a[u] = DF{0.f, 0.f};
+        for (int p = g; p < nparts; p += U * NG) {
+            DF v[U];
 #pragma unroll
-                for (int u = 0; u < U; ++u)
-                    v[u] = p + u * nw < nparts ? pp[int64_t(p + u * nw) * W + c] : DF{0.f, 0.f};
+            for (int u = 0; u < U; ++u) v[u] = p + u * NG < nparts ? pp[int64_t(p + u * NG) * W + col] : DF{0.f, 0.f};
 #pragma unroll
-                for (int u = 0; u < U; ++u) df_merge(a[u], v[u]);
-            }
-#pragma unroll
-            for (int u = 1; u < U; ++u) df_merge(a[0], a[u]);
-            reinterpret_cast<DF *>(&tmp[warp][0])[c] = a[0];
-        } else {
-            double a[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) a[u] = 0.0;
-            int p = warp;
-            for (; p < nparts; p += U * nw) {
-                double v[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) v[u] = p + u * nw < nparts ? parts[int64_t(p + u * nw) * W + c] : 0.0;
-#pragma unroll
-                for (int u = 0; u < U; ++u) a[u] += v[u];
-            }
-            double t = a[0];
-#pragma unroll
-            for (int u = 1; u < U; ++u) t += a[u];
-            tmp[warp][c] = t;
+            for (int u = 0; u < U; ++u) df_merge(a[u], v[u]);
         }
+#pragma unroll
+        for (int u = 1; u < U; ++u) df_merge(a[0], a[u]);
+        // the warp's two subsets
+        const DF o{__shfl_xor_sync(0xffffffffu, a[0].hi, 16), __shfl_xor_sync(0xffffffffu, a[0].lo, 16)};
+        df_merge(a[0], o);
+        if (lane < LZ_COLS) reinterpret_cast<DF &>(tmp[warp][c]) = a[0];
+    } else {
+        double a[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) a[u] = 0.0;
+        for (int p = g; p < nparts; p += U * NG) {
+            double v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) v[u] = p + u * NG < nparts ? parts[int64_t(p + u * NG) * W + col] : 0.0;
+#pragma unroll
+            for (int u = 0; u < U; ++u) a[u] += v[u];
+        }
+        double t = a[0];
+#pragma unroll
+        for (int u = 1; u < U; ++u) t += a[u];
+        t += __shfl_xor_sync(0xffffffffu, t, 16);
+        if (lane < LZ_COLS) tmp[warp][c] = t;
     }
     __syncthreads();
-    for (int c = threadIdx.x; c < W; c += blockDim.x) {
+    if (threadIdx.x < LZ_COLS) {
         if (df) {
-            DF t = reinterpret_cast<const DF *>(&tmp[0][0])[c];
-            for (int w = 1; w < nw; ++w) df_merge(t, reinterpret_cast<const DF *>(&tmp[w][0])[c]);
+            DF t = reinterpret_cast<const DF &>(tmp[0][c]);
+            for (int w = 1; w < LZ_THREADS / 32; ++w) df_merge(t, reinterpret_cast<const DF &>(tmp[w][c]));
             s[c] = df_value(t);
         } else {
             double t = 0.0;
-            for (int w = 0; w < nw; ++w) t += tmp[w][c];
+            for (int w = 0; w < LZ_THREADS / 32; ++w) t += tmp[w][c];
             s[c] = t;
         }
     }
     __syncthreads();
+}
+
+// Sum of s over the columns of all CTAs of the cluster, in rank order, in every CTA (s holds zeros
+// in padding columns).
+__device__ double cluster_total(const double *s) {
+    __shared__ double own, tot;
+    cg::cluster_group cl = cg::this_cluster();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int c = 0; c < LZ_COLS; ++c) t += s[c];
+        own = t;
+    }
+    cl.sync();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (unsigned r = 0; r < cl.num_blocks(); ++r) t += *cl.map_shared_rank(&own, r);
+        tot = t;
+    }
+    cl.sync();   // (no CTA leaves while another reads its sum)
+    return tot;
 }
 
 // Scale factors sigma (Q_k = sigma_k P_k) are rounded to the basis precision when the
@@ -210,39 +238,20 @@ __global__ void k_lanczos_init(int W, int M, int gbl, int round32, double *sigma
     }
 }
 
-// Sum of s[0..M) by warp 0 (fixed order); the result is returned to lane 0.
-__device__ __forceinline__ double warp0_sum(const double *s, int M) {
-    double t = 0.0;
-    for (int c = threadIdx.x; c < M; c += 32) t += s[c];
-    for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
-    return t;
-}
-
 // alpha_k = <Q_k, X> (gbl: Frobenius, sbl: per column) from SpMM dot partials of P_k . X
-__global__ void k_lanczos_alpha(const double *parts, int nparts, int W, int M, int gbl, int k,
-                                int df, const double *sigma, double *alpha, double *a_upd,
-                                const Ctrl *ctrl) {
+__global__ void __launch_bounds__(LZ_THREADS)
+k_lanczos_alpha(const double *parts, int nparts, int W, int M, int gbl, int k, int df, const double *sigma,
+                double *alpha, double *a_upd, const Ctrl *ctrl) {
     if (ctrl->stop) return;
-    __shared__ double s[128];
+    __shared__ double s[LZ_COLS];
     reduce_cols(parts, nparts, W, s, df);
     const double *sg = sigma + int64_t(k) * W;
-    if (gbl) {
-        __shared__ double tot;
-        if (threadIdx.x < 32) {
-            const double t = warp0_sum(s, M);
-            if (threadIdx.x == 0) tot = sg[0] * t;
-        }
-        __syncthreads();
-        for (int c = threadIdx.x; c < W; c += blockDim.x) {
-            alpha[int64_t(k) * W + c] = c < M ? tot : 0.0;
-            a_upd[c] = c < M ? tot * sg[0] : 0.0;
-        }
-    } else {
-        for (int c = threadIdx.x; c < W; c += blockDim.x) {
-            const double al = c < M ? sg[c] * s[c] : 0.0;
-            alpha[int64_t(k) * W + c] = al;
-            a_upd[c] = al * sg[c];
-        }
+    const double tot = gbl ? sg[0] * cluster_total(s) : 0.0;
+    if (threadIdx.x < LZ_COLS) {
+        const int c = blockIdx.x * LZ_COLS + threadIdx.x;
+        const double al = c < M ? (gbl ? tot : sg[c] * s[threadIdx.x]) : 0.0;
+        alpha[int64_t(k) * W + c] = al;
+        a_upd[c] = al * (gbl ? sg[0] : sg[c]);
     }
 }
 
@@ -250,48 +259,35 @@ __global__ void k_lanczos_alpha(const double *parts, int nparts, int W, int M, i
 // SpMM coefficients of the next step: X = sigma_{k+1} L P_{k+1} - beta_{k+1} sigma_k P_k.
 // sigma_{k+1} is rounded to the basis precision and beta_{k+1} is recorded as its exact
 // reciprocal, so Q_{k+1} = sigma_{k+1} P_{k+1} = X / beta_{k+1} holds for the stored values.
-__global__ void k_lanczos_beta(const double *parts, int nparts, int W, int M, int gbl, int k,
-                               int round32, double thresh, double *beta, double *sigma,
-                               int32_t *alive, double *c1, double *c2, Ctrl *ctrl) {
+__global__ void __launch_bounds__(LZ_THREADS)
+k_lanczos_beta(const double *parts, int nparts, int W, int M, int gbl, int k, int round32, double thresh,
+               double *beta, double *sigma, int32_t *alive, double *c1, double *c2, Ctrl *ctrl) {
     if (ctrl->stop) return;
-    __shared__ double s[128];
+    __shared__ double s[LZ_COLS];
     reduce_cols(parts, nparts, W, s, round32);
     const double *sk = sigma + int64_t(k) * W;
     double *sn = sigma + int64_t(k + 1) * W;
     double *bn = beta + int64_t(k + 1) * W;
-    if (gbl) {
-        __shared__ double b;
-        __shared__ int stop;
-        if (threadIdx.x < 32) {
-            const double t = warp0_sum(s, M);
-            if (threadIdx.x == 0) {
-                b = sqrt(t);
-                stop = !(b > thresh);
-                if (stop) { ctrl->stop = 1; ctrl->steps = k + 1; }
+    const double tot = gbl ? cluster_total(s) : 0.0;   // (a barrier: no CTA has stopped the process before all read stop)
+    if (threadIdx.x < LZ_COLS) {
+        const int c = blockIdx.x * LZ_COLS + threadIdx.x;
+        const double b = sqrt(gbl ? tot : s[threadIdx.x]);
+        bool live = c < M && b > thresh;
+        if (gbl) {
+            if (c == 0 && !(b > thresh)) {
+                ctrl->stop = 1;
+                ctrl->steps = k + 1;
             }
-        }
-        __syncthreads();
-        const double sg = round_to(1.0 / b, round32);
-        const double bt = 1.0 / sg;
-        for (int c = threadIdx.x; c < W; c += blockDim.x) {
-            const bool live = c < M && !stop;
-            bn[c] = live ? bt : 0.0;
-            sn[c] = live ? sg : 0.0;
-            c1[c] = live ? sg : 0.0;
-            c2[c] = live ? -bt * sk[c] : 0.0;
-        }
-    } else {
-        for (int c = threadIdx.x; c < W; c += blockDim.x) {
-            const double b = sqrt(s[c]);
-            const bool live = c < M && alive[c] && (b > thresh);
+        } else {
+            live = live && alive[c];
             if (!live) alive[c] = 0;
-            const double sg = live ? round_to(1.0 / b, round32) : 0.0;
-            const double bt = live ? 1.0 / sg : 0.0;
-            bn[c] = bt;
-            sn[c] = sg;
-            c1[c] = sg;
-            c2[c] = live ? -bt * sk[c] : 0.0;
         }
+        const double sg = live ? round_to(1.0 / b, round32) : 0.0;
+        const double bt = live ? 1.0 / sg : 0.0;
+        bn[c] = bt;
+        sn[c] = sg;
+        c1[c] = sg;
+        c2[c] = live ? -bt * sk[c] : 0.0;
     }
 }
 
@@ -820,12 +816,29 @@ int launch_lanczos_init(int W, int M, int gbl, int round32, double *sigma, int32
     return 0;
 }
 
+// One cluster of n (1, 2, 4 or 8) CTAs.
+template <typename... P, typename... A>
+static cudaError_t launch_cluster(int n, cudaStream_t s, void (*kernel)(P...), A... args) {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = unsigned(n);
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.gridDim = unsigned(n);
+    cfg.blockDim = LZ_THREADS;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 int launch_lanczos_alpha(const double *parts, int nparts, int W, int M, int gbl, int k, int df,
                          const double *sigma, double *alpha, double *a_upd, const Ctrl *ctrl,
                          cudaStream_t s) {
     prof_begin(KernelClass::SMALL, s);
-    k_lanczos_alpha<<<1, 1024, 0, s>>>(parts, nparts, W, M, gbl, k, df, sigma, alpha, a_upd, ctrl);
-    KB_CUDA_TRY(cudaGetLastError());
+    KB_CUDA_TRY(launch_cluster(W / LZ_COLS, s, k_lanczos_alpha, parts, nparts, W, M, gbl, k, df, sigma, alpha, a_upd,
+                               ctrl));
     prof_end(KernelClass::SMALL, s, double(nparts) * W * 8, 0);
     return 0;
 }
@@ -834,9 +847,8 @@ int launch_lanczos_beta(const double *parts, int nparts, int W, int M, int gbl, 
                         double thresh, double *beta, double *sigma, int32_t *alive, double *c1,
                         double *c2, Ctrl *ctrl, cudaStream_t s) {
     prof_begin(KernelClass::SMALL, s);
-    k_lanczos_beta<<<1, 1024, 0, s>>>(parts, nparts, W, M, gbl, k, round32, thresh, beta, sigma,
-                                     alive, c1, c2, ctrl);
-    KB_CUDA_TRY(cudaGetLastError());
+    KB_CUDA_TRY(launch_cluster(W / LZ_COLS, s, k_lanczos_beta, parts, nparts, W, M, gbl, k, round32, thresh, beta, sigma,
+                               alive, c1, c2, ctrl));
     prof_end(KernelClass::SMALL, s, double(nparts) * W * 8, 0);
     return 0;
 }

@@ -46,15 +46,21 @@ __device__ __forceinline__ double recip(double d) {
     e = fma(-d, r, 1.0);
     return fma(r, e, r);
 }
-__device__ __forceinline__ float recip(float d) { return __frcp_rn(d); }
+// (one unit in the last place: the FP32 factors are corrected afterwards)
+__device__ __forceinline__ float recip(float d) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return r;
+}
 
 // Edge of the register tiles: 2 in FP32, where a shared load is the dearer part, 1 in FP64,
 // whose FMA occupies a scheduler for some 64 cycles, so that only spreading the entries helps.
 template <typename S> struct Tile { static constexpr int E = sizeof(S) == 8 ? 1 : 2; };
 
 // E x E tiles (i0, j0) meeting the upper triangle of an M x M matrix, shared out evenly over
-// the threads (consecutive threads along a row).
-template <int E, typename F>
+// the threads: consecutive threads along a row, or (DIAG) along a diagonal, where the sums over
+// k = i0 .. j0 of triangular products are equally long.
+template <int E, bool DIAG, typename F>
 __device__ __forceinline__ void tri_tiles(int M, const F &f) {
     const int nt = (M + E - 1) / E, total = nt * (nt + 1) / 2;
     for (int t = threadIdx.x; t < total; t += blockDim.x) {
@@ -65,7 +71,8 @@ __device__ __forceinline__ void tri_tiles(int M, const F &f) {
         while (i > 0 && i * nt - i * (i - 1) / 2 > t) --i;
         while ((i + 1) * nt - (i + 1) * i / 2 <= t) ++i;
         const int j = i + t - (i * nt - i * (i - 1) / 2);
-        f(i * E, j * E);
+        if (DIAG) f((j - i) * E, j * E);   // (row i of the enumeration: the i-th diagonal)
+        else f(i * E, j * E);
     }
 }
 
@@ -158,7 +165,7 @@ __device__ bool chol_blocked(S *A, S *Inv, int lda, int M, S thr, S *scr) {
         __syncthreads();
         // A_22 -= R_12^T R_12 (upper triangle)
         constexpr int E = Tile<S>::E;
-        tri_tiles<E>(rest, [&](int i, int j) {
+        tri_tiles<E, false>(rest, [&](int i, int j) {
             S acc[E][E];
 #pragma unroll
             for (int r = 0; r < E; ++r)
@@ -278,7 +285,7 @@ __device__ void tri_inv_merge(S *A, int lda, int M, S *tmp) {
 template <typename S, typename FP, typename FE>
 __device__ void tri_mm(const S *A, const S *B, int lda, int M, const FP &pre, const FE &epi) {
     constexpr int E = Tile<S>::E;
-    tri_tiles<E>(M, [&](int i, int j) {
+    tri_tiles<E, true>(M, [&](int i, int j) {
         S acc[E][E];
         decltype(pre(0, 0)) x[E][E];
 #pragma unroll
@@ -315,7 +322,7 @@ __device__ void tri_mm(const S *A, const S *B, int lda, int M, const FP &pre, co
 // running on the FP32 pipe.
 template <typename FE>
 __device__ void tri_residual(const float *Sm, const float *R, int lda, int M, const FE &epi) {
-    tri_tiles<2>(M, [&](int i, int j) {
+    tri_tiles<2, true>(M, [&](int i, int j) {
         const bool i1 = i + 1 < M;
         const float *pa = Sm + i * lda, *pb = pa + (i1 ? lda : 0);
         float hi[2][2], lo[2][2];
