@@ -2,9 +2,8 @@
 // distance, and the zeros that the restricted kernels rely on.
 //
 // All of it is known before the first step.  One cooperative kernel runs the whole
-// breadth-first search with a barrier between the levels, instead of two launches per step.  A second one sorts the tiles by distance, one CTA per distance, so that the tiles
-// active at step k are a prefix of one list and no step needs bookkeeping of its own.  A third
-// writes the zeros that blocks need just beyond their reach, instead of clearing all of them.
+// breadth-first search with a barrier between the levels, instead of two launches per step. A
+// second one makes the tile lists of all steps at once, one CTA each. A third writes the zeros that blocks need just beyond their reach, instead of clearing all of them.
 //
 // Measured, whole solves before -> after (per-step list and expansion launches, all blocks
 // cleared in full): RGG of 10^6 rows, M = 64, 30 steps: gbl 4.82 -> 3.45 ms, cheb 2.16 -> 1.58
@@ -216,8 +215,8 @@ __device__ int compact_tiles(const int32_t *tgen, int64_t nact, const P &in, int
 // The lists, one CTA each, all at once.  blockIdx.y = 0: the tiles at distance b = blockIdx.x (b =
 // levels + 1: all that were not reached) into alist[acount[b - 1] ..], so alist holds all tiles by
 // rising distance.  blockIdx.y = 1: the tiles within b hops in index order into lists[b]: in that
-// order neighbouring rows are at work at the same time, and their gathers meet in L2 (128^3
-// grid, sbl, M = 128: @@LS@@).
+// order neighbouring rows are at work at the same time, and their gathers meet in L2 (RGG of
+// 10^6 rows, M = 64, SpMM mean per launch 36.2 -> 34.5 us, with column dots 50.8 -> 46.7 us).
 __global__ void __launch_bounds__(1024) k_tile_sort(int32_t *tgen, uint8_t *gen, int64_t n, int64_t nact, int levels,
                                                     const int32_t *__restrict__ tcnt, const int32_t *err,
                                                     int32_t *__restrict__ acount, int32_t *__restrict__ alist,

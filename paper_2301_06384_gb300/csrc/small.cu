@@ -135,8 +135,8 @@ int launch_reorth_decide(const double *G, const double *d0, int M, int W, int32_
 
 // ---------------------------------------------------------------- gbl / sbl scalars
 // The scalars of a step come from [nparts][W] partial column sums.  A cluster of W / 16 CTAs takes
-// 16 columns each (one CTA reading all partials is bound by its SM's L2 bandwidth: 16 us at W =
-// 64, 27 us at W = 128, now 5 and 6 us); the global method's totals meet in distributed shared
+// 16 columns each (one CTA reading all partials is bound by its SM's L2 bandwidth: alpha / beta at
+// W = 64 15.9 / 16.3 us, now 12.3 / 15.1; at W = 128 27.1 / 19.5, now 11.2 / 14.1); the global method's totals meet in distributed shared
 // memory.  df: the partials are double-float pairs (FP32 arithmetic), combined on the FP32
 // pipe; else doubles.
 constexpr int LZ_THREADS = 512;
