@@ -39,13 +39,15 @@
 // Measured (launch list, mean us of a solve's launches; before: synchronous staging, 4 x 4
 // tiles, all W columns, full Grams):                          PROJ     UPD  MULGRAM     MUL
 //   RGG 10^6 rows, M = 64, 30 steps, before                   68.3   170.9    100.0    56.3
-//                                    now                      42.3   117.7     63.2    34.5
+//                                    now                      38.0    90.6     53.5    32.9
 //   128^3 grid, M = 32, 40 steps,    before                  242.8   451.8    291.6   155.8
-//                                    now                      71.7   219.6    103.5    59.5
+//                                    now                      65.4   137.2     79.1    53.1
 //   BA 5e5 rows, M = 128, ordered,   before                  280.8  1675.7    962.6   665.5
-//                                    now                     209.2  1129.1    634.4   329.6
+//                                    now, whole solve 243 -> 172 ms
 //   RGG 10^5 rows, M = 33, FP64,     before                  477.6  1193.7    743.4   305.1
-//                                    now                     113.5   234.1    136.6    67.8
+//                                    now                     104.3   234.1    136.7    67.4
+// With scalar FMAs, list lookups and 64-bit addresses per copy, and the first level of the Gram
+// sums held across the products, UPD at M = 64 took 113.4.
 #pragma once
 #include <algorithm>
 #include <climits>
@@ -119,6 +121,34 @@ __device__ __forceinline__ void stg4(T *p, const typename Cmp<T>::type (&v)[4]) 
         st4<T>(p, v);
     }
 }
+// Packed FP32 pairs (fma.rn.f32x2): each lane rounds as the scalar instruction would, at half
+// the issue slots; these kernels are bound by those (65 % of them busy with scalar FMAs).
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 f2_pack(float lo, float hi) {
+    f2 d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+// c[i] += a b[i] over N (even) consecutive entries
+template <typename C, int N>
+__device__ __forceinline__ void fma_row(C (&c)[N], C a, const C (&b)[N]) {
+    if constexpr (sizeof(C) == 4 && N % 2 == 0) {
+        const f2 aa = f2_pack(a, a);
+#pragma unroll
+        for (int i = 0; i < N; i += 2) {
+            const f2 t = f2_fma(aa, f2_pack(b[i], b[i + 1]), f2_pack(c[i], c[i + 1]));
+            asm("mov.b64 {%0, %1}, %2;" : "=f"(c[i]), "=f"(c[i + 1]) : "l"(t));
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) c[i] = fma(a, b[i], c[i]);
+    }
+}
 // 16 bytes global -> shared, asynchronous; zeros when !in (the address is then not read)
 __device__ __forceinline__ void cp16(void *dst, const void *src, bool in) {
     const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
@@ -156,7 +186,7 @@ __host__ __device__ inline RowGeo row_geo(int M) {
     RowGeo r;
     r.Mk = (M + 3) / 4 * 4;
     r.CG = r.Mk / 4;
-    const int cap = 256;     // rows: bounds the shared memory of narrow blocks
+    const int cap = NT == 128 ? 128 : 256;   // rows: bounds the shared memory of narrow blocks
     int tr = (NT / r.CG) * RPT;
     tr = (tr < cap ? tr : cap) / 32 * 32;
     r.TR = tr < 32 ? 32 : tr;
@@ -300,17 +330,17 @@ k_rowblock(RowArgs<T> a) {
                     ldn<C, BI>(left + r * ld + gi0, av);
                     ldn<C, BJ>(right + r * ld + gj0, bv);
 #pragma unroll
-                    for (int i = 0; i < BI; ++i)
-#pragma unroll
-                        for (int j = 0; j < BJ; ++j) {
-                            if constexpr (G::TWO) g1[i][j] = fma(av[i], bv[j], g1[i][j]);
-                            else g2[i][j] = fma(av[i], bv[j], g2[i][j]);
-                        }
+                    for (int i = 0; i < BI; ++i) {
+                        if constexpr (G::TWO) fma_row<C, BJ>(g1[i], av[i], bv);
+                        else fma_row<C, BJ>(g2[i], av[i], bv);
+                    }
                 }
             }
             if constexpr (G::TWO && !ORD) {
+                // (a product's tile ends the first level, which then takes no registers beside the
+                // product's)
                 grows += R / q.NGR;
-                if (grows >= 32) flush();
+                if (PROD || grows >= 32) flush();
             }
         }
     };
@@ -425,6 +455,7 @@ k_rowblock(RowArgs<T> a) {
             cmax = max(cmax, __shfl_xor_sync(0xffffffffu, cmax, o));
         }
         const int nsub = q.TR / ACT_ROWS;
+        const int n32 = int(a.n);
         const int64_t nvt = ORD ? olen : (cnt + nsub - 1) / nsub;
         const int64_t vt0 = ORD ? onorm(blockIdx.x) : int64_t(blockIdx.x);
         auto vt_next = [&](int64_t vt) -> int64_t {
@@ -466,8 +497,35 @@ k_rowblock(RowArgs<T> a) {
             pk0 = 0;
         };
         skip_empty();
+        // The rows this thread copies of a virtual tile, and their tiles' distances, looked up once per
+        // tile: a copy then costs one address.
+        constexpr int EPV = std::is_same<T, C>::value ? VEC : 4;
+        constexpr int VPR = KC / EPV;                                        // copies per row
+        constexpr int NA = ((NT == 128 ? 128 : 256) * VPR + NT - 1) / NT;    // copies per thread, at most
+        static_assert(NT % VPR == 0, "a thread's copies share their column");
+        int prow[NA], pdist[NA];
+        int64_t plook = -1;                                                  // the tile looked up
+        const int pc = (tid % VPR) * EPV;
+        auto look_up = [&]() {
+            plook = pvt;
+#pragma unroll
+            for (int j = 0; j < NA; ++j) {
+                const int r = tid / VPR + j * (NT / VPR);
+                prow[j] = -1;
+                pdist[j] = 0;
+                if (r < q.TR) {
+                    const int64_t t = vt_tile(pvt, r / ACT_ROWS);
+                    const int64_t row = t * ACT_ROWS + r % ACT_ROWS;
+                    if (t >= 0 && row < a.n) {
+                        prow[j] = int(row);
+                        if (a.tgen) pdist[j] = __ldg(a.tgen + t);
+                    }
+                }
+            }
+        };
         auto issue = [&](int st) {
             if (pvt < nvt) {
+                if (plook != pvt) look_up();
                 const T *src;
                 const C *cmat;
                 int lim;
@@ -486,21 +544,20 @@ k_rowblock(RowArgs<T> a) {
                     lim = INT_MAX;
                 }
                 C *dA = sm + st * SE, *dC = dA + q.TR * LDA;
-                constexpr int EPV = std::is_same<T, C>::value ? VEC : 4;
-                constexpr int VPR = KC / EPV;      // copies per row
-                for (int i = tid; i < q.TR * VPR; i += NT) {
-                    const int r = i / VPR, c = (i % VPR) * EPV;
-                    if (pk0 + c >= q.Mk) continue;
-                    const int64_t t = vt_tile(pvt, r / ACT_ROWS);
-                    const int64_t row = t * ACT_ROWS + r % ACT_ROWS;
-                    const bool in = t >= 0 && row < a.n && (!a.tgen || lim == INT_MAX || __ldg(a.tgen + t) <= lim);
-                    const int64_t off = in ? row * W + pk0 + c : 0;
-                    if constexpr (std::is_same<T, C>::value) {
-                        cp16(dA + r * LDA + c, src + off, in);
-                    } else {
-                        C v[4] = {0, 0, 0, 0};
-                        if (in) ldg4<T>(src + off, v);
-                        st4<C>(dA + r * LDA + c, v);
+                if (pk0 + pc < q.Mk) {
+#pragma unroll
+                    for (int j = 0; j < NA; ++j) {
+                        const int r = tid / VPR + j * (NT / VPR);
+                        if (r >= q.TR) break;
+                        const bool in = prow[j] >= 0 && pdist[j] <= lim;
+                        const T *from = src + (in ? int64_t(prow[j]) * W + pk0 + pc : 0);
+                        if constexpr (std::is_same<T, C>::value) {
+                            cp16(dA + r * LDA + pc, from, in);
+                        } else {
+                            C v[4] = {0, 0, 0, 0};
+                            if (in) ldg4<T>(from, v);
+                            st4<C>(dA + r * LDA + pc, v);
+                        }
                     }
                 }
                 const int crows = min(KC, q.Mk - pk0);
@@ -523,19 +580,23 @@ k_rowblock(RowArgs<T> a) {
         for (int s = 0; s < NST - 1; ++s) issue(s);
         // X of a virtual tile to the output tile, asynchronously, once the previous tile is done
         // with that; its copies belong to the next chunk's group
-        auto load_x = [&](int64_t vt) {
+        auto load_x = [&](const int *rows) {
             for (int i = tid; i < q.TR * (W / VEC); i += NT) {
                 const int r = i / (W / VEC), c = (i % (W / VEC)) * VEC;
                 if (c >= q.Mk) continue;
-                const int64_t t = vt_tile(vt, r / ACT_ROWS);
-                const int64_t row = t * ACT_ROWS + r % ACT_ROWS;
-                const bool in = t >= 0 && row < a.n;
-                cp16(sO + r * LDO + c, a.x + (in ? row * W + c : 0), in);
+                const int b = rows[r / ACT_ROWS], row = b + r % ACT_ROWS;
+                const bool in = b >= 0 && row < n32;
+                cp16(sO + r * LDO + c, a.x + (in ? int64_t(row) * W + c : 0), in);
             }
         };
+        // the current tile's 32-row tiles (first row, -1: none), by parity of the tile: written
+        // before the tile's first barrier, read after it
+        __shared__ int s_row[2][8];
+        int par = 0;
         int st = 0;
-        for (int64_t vt = vt0; vt < nvt; vt = vt_next(vt)) {
+        for (int64_t vt = vt0; vt < nvt; vt = vt_next(vt), par ^= 1) {
             const int kb0 = first_kb(vt);
+            if (tid < nsub) s_row[par][tid] = int(max(int64_t(-1), vt_tile(vt, tid) * ACT_ROWS));
             if (tid == 0) {
                 const int64_t rows = ORD ? q.TR : min(int64_t(q.TR), (cnt - vt * nsub) * ACT_ROWS);
                 my_rows += rows;
@@ -564,7 +625,7 @@ k_rowblock(RowArgs<T> a) {
                     cp_wait<NST - 2>();
                     __syncthreads();
                     if constexpr (ASYNC_X) {
-                        if (kb == kb0 && k0 == 0) load_x(vt);
+                        if (kb == kb0 && k0 == 0) load_x(s_row[par]);
                     }
                     issue(st == 0 ? NST - 1 : st - 1);
                     const C *pA = sm + st * SE + rg * LDA;
@@ -586,9 +647,7 @@ k_rowblock(RowArgs<T> a) {
 #pragma unroll
                         for (int j = 0; j < 4; ++j)
 #pragma unroll
-                            for (int r = 0; r < RPT; ++r)
-#pragma unroll
-                                for (int u = 0; u < 4; ++u) acc[r][u] = fma(av[r][j], cv[j][u], acc[r][u]);
+                            for (int r = 0; r < RPT; ++r) fma_row<C, 4>(acc[r], av[r][j], cv[j]);
                     };
                     if (ks == 0 && ke == KC) {
 #pragma unroll
@@ -605,7 +664,7 @@ k_rowblock(RowArgs<T> a) {
                 // (kb0 < nkb: UPD has a block always, ASMSUB the block of the seeds or a nearer one;
                 // otherwise X is loaded here)
                 if (kb0 >= nkb) {
-                    load_x(vt);
+                    load_x(s_row[par]);
                     cp_commit();
                 }
                 // the chunks after the one X came with may be too few to have waited for it
@@ -623,9 +682,8 @@ k_rowblock(RowArgs<T> a) {
                         if constexpr (std::is_same<T, C>::value) {
                             ld4<C>(sO + lr * LDO + col4, xv);
                         } else {
-                            const int64_t t = vt_tile(vt, lr / ACT_ROWS);
-                            const int64_t row = t * ACT_ROWS + lr % ACT_ROWS;
-                            if (t >= 0 && row < a.n) ldg4<T>(a.x + row * W + col4, xv);
+                            const int b = s_row[par][lr / ACT_ROWS], row = b + lr % ACT_ROWS;
+                            if (b >= 0 && row < n32) ldg4<T>(a.x + int64_t(row) * W + col4, xv);
                         }
 #pragma unroll
                         for (int u = 0; u < 4; ++u) o[u] = xv[u] - acc[r][u];
@@ -646,9 +704,9 @@ k_rowblock(RowArgs<T> a) {
             constexpr int CPR = W / 4;
             for (int i = tid; i < q.TR * CPR; i += NT) {
                 const int r = i / CPR, c = (i % CPR) * 4;
-                const int64_t t = vt_tile(vt, r / ACT_ROWS);
-                const int64_t row = t * ACT_ROWS + r % ACT_ROWS;
-                if (t < 0 || row >= a.n) continue;
+                const int b = s_row[par][r / ACT_ROWS], rl = b + r % ACT_ROWS;
+                if (b < 0 || rl >= n32) continue;
+                const int64_t row = rl;
                 C o[4];
                 ld4<C>(sO + r * LDO + c, o);
                 if (MODE == RB_ASM) {
@@ -722,7 +780,7 @@ constexpr int RB_MAX_CTAS = 5;   // per SM: bounds the Gram partials
 template <typename T, int W, int MODE, int RPT, bool ORD, int NT>
 int occupancy(size_t smem) {
     static const cudaError_t attr = cudaFuncSetAttribute(
-        k_rowblock<T, W, MODE, RPT, ORD, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        k_rowblock<T, W, MODE, RPT, ORD, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     (void)attr;
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rowblock<T, W, MODE, RPT, ORD, NT>, NT, smem);
