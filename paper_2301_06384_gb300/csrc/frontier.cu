@@ -18,34 +18,6 @@ namespace {
 constexpr int BFS_THREADS = 512;
 constexpr int BFS_ROWS = 8;    // queue rows a warp expands together
 constexpr int BFS_U = 4;       // edges per lane in flight
-constexpr int BFS_SPINS = 1 << 22;   // polls of the level barrier before giving up
-
-// Barrier of all CTAs of a cooperative launch (co-resident by construction): the arrivals are
-// counted in *bar.  false, with *err set, when the wait runs out; every CTA then leaves by
-// itself, and k_tile_sort turns the restriction off (all rows active), so the solve stays right.
-__device__ __forceinline__ bool level_barrier(int32_t *bar, int32_t *err, int target) {
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(bar, 1);
-        int good = 0;
-        for (int i = 0; i < BFS_SPINS; ++i) {
-            int v;
-            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-            if (v >= target) {
-                good = 1;
-                break;
-            }
-        }
-        if (!good) atomicExch(err, 1);
-        __threadfence();
-        ok = good;
-    }
-    __syncthreads();
-    return ok != 0;
-}
-
 // Breadth-first search from the nodes up to `levels` hops in one cooperative launch.  The queue
 // holds the reached rows level after level; a row is claimed by an atomicOr on its bit of vis,
 // whose 32-bit words are the 32-row tiles, so the claim that finds the word empty has found a
@@ -70,7 +42,7 @@ k_bfs(GraphDev g, NodeChunk seeds, int levels, uint8_t *gen, int32_t *tgen, uint
             atomicAdd(tcnt, 1);
         }
     }
-    if (!level_barrier(bar, err, target += gridDim.x)) return;
+    if (!grid_barrier(bar, err, target += gridDim.x)) return;
     int start = 0, end = seeds.cnt;
     for (int k = 1; k <= levels && start < end; ++k) {
         for (int64_t base = start + int64_t(gw) * BFS_ROWS; base < end; base += int64_t(nw) * BFS_ROWS) {
@@ -137,7 +109,7 @@ k_bfs(GraphDev g, NodeChunk seeds, int levels, uint8_t *gen, int32_t *tgen, uint
                 }
             }
         }
-        if (!level_barrier(bar, err, target += gridDim.x)) return;
+        if (!grid_barrier(bar, err, target += gridDim.x)) return;
         start = end;
         end += __ldcg(qlev + k);
     }

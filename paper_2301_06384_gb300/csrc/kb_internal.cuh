@@ -167,6 +167,35 @@ __device__ __forceinline__ void df_merge(DF &a, const DF &b) {
 }
 __device__ __forceinline__ double df_value(const DF &a) { return double(a.hi) + double(a.lo); }
 
+// ------------------------------------------------------------------ grid barrier
+// Barrier of all CTAs of a cooperative launch (co-resident by construction): the arrivals are
+// counted in *bar, target the count that releases this barrier.  The wait is bounded: false, with
+// *err set, when it runs out; every CTA then leaves by itself and the caller's results have to
+// be marked unusable.
+constexpr int GRID_BARRIER_SPINS = 1 << 22;
+__device__ __forceinline__ bool grid_barrier(int32_t *bar, int32_t *err, int target) {
+    __shared__ int ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1);
+        int good = 0;
+        for (int i = 0; i < GRID_BARRIER_SPINS; ++i) {
+            int v;
+            asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if (v >= target) {
+                good = 1;
+                break;
+            }
+        }
+        if (!good) atomicExch(err, 1);
+        __threadfence();
+        ok = good;
+    }
+    __syncthreads();
+    return ok != 0;
+}
+
 // ------------------------------------------------------------------ launch helpers
 int num_sms();
 inline int width_for(int M) { return M <= 16 ? 16 : M <= 32 ? 32 : M <= 64 ? 64 : 128; }

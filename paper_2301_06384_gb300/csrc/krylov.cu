@@ -218,6 +218,7 @@ struct CblBufs {
     Ctrl *ctrl, *ctrl2, *ctrl_chk;
     FrontierBufs fr;
     unsigned *hcnt;   // CTA counter of the reduction that forms H_kk
+    int32_t *csync;   // grid barrier of the projected series
 };
 
 template <typename T>
@@ -254,6 +255,7 @@ void plan_cbl(Arena &ar, CblBufs<T> &b, int64_t n, int M, int W, int m, int rb_g
     b.ctrl_chk = ar.take<Ctrl>(1);
     ar.frontier(b.fr, n, m);
     b.hcnt = ar.take<unsigned>(1);
+    b.csync = ar.take<int32_t>(2);
 }
 
 template <typename T>
@@ -446,7 +448,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                 KB_TRY(launch_ctrl_snapshot(b.ctrl_chk, b.ctrl, k, c.s));
                 if (c.phi == KB_PHI_EXP) {
                     const std::vector<double> d = exp_series_coeffs(c.p.t, lam_p, 1e-17);
-                    KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, Ucur, b.ctrl_chk, c.s, f64 ? nullptr : b.Hdf));
+                    KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, Ucur, b.ctrl_chk, c.s, f64 ? nullptr : b.Hdf, b.csync, k));
                 } else {
                     KB_TRY(launch_bt_spline(b.Hd, b.Hs, M, m, c.p.eps, c.s_int, sbufs, Ucur, b.ctrl, b.ctrl_chk,
                                             c.s, c.quad, b.qscr, qbatch, kfac, c.s_int == 1 ? kfac : 0, k));
@@ -465,7 +467,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
         }
         if (c.phi == KB_PHI_EXP) {
             const std::vector<double> d = exp_series_coeffs(c.p.t, lam_p, 1e-17);
-            KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, b.U, cfin, c.s, f64 ? nullptr : b.Hdf));
+            KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, b.U, cfin, c.s, f64 ? nullptr : b.Hdf, b.csync));
         } else {
             // (a process that stopped by itself skipped the later checks: their Y are formed now)
             KB_TRY(launch_bt_spline(b.Hd, b.Hs, M, m, c.p.eps, c.s_int, sbufs, b.U, b.ctrl, cfin, c.s, c.quad,

@@ -247,6 +247,146 @@ k_cheb_bt_iter_df(const float *__restrict__ Hd, const float *__restrict__ Hs, co
         }
 }
 
+// The whole series (terms j0 .. j0 + cc.n of it) in one cooperative launch: a CTA keeps up to NI
+// items (8 columns of one block row), its U and V_{j-1} entries in registers and, with one item,
+// the three blocks of H in shared memory for all terms; a term reads the neighbours' V from
+// L2, and a grid barrier separates the terms.  A launch per term costs more than its
+// arithmetic, above all with several solves in flight.  Row r of V_j is zero for r > j and never
+// read.  V_j lives in slot j % 3.  Measured, a whole series, launch list:
+// 65 terms, M = 64, 30 blocks 1085 -> 925 us; 48 terms, M = 40, 20 blocks 585 -> 447 us; the four
+// concurrent requests of the serving mix on a hub graph (5300 terms) 41.0 -> 33.7 ms.
+template <int NI>
+__global__ void __launch_bounds__(256)
+k_cheb_bt_all(const float *__restrict__ Hd, const float *__restrict__ Hs, const float *__restrict__ Hst, dfl *V0,
+              dfl *V1, dfl *V2, double *__restrict__ U, int M, int ld, ChebCoef cc, int j0, dfl g,
+              const Ctrl *ctrl, int32_t *sync) {
+    const int steps = ctrl->steps;
+    if (steps <= 0) return;
+    extern __shared__ __align__(16) unsigned char svraw[];   // V [3][M][CBW] pairs, H [3][M][ld]
+    dfl *s1 = reinterpret_cast<dfl *>(svraw), *s0 = s1 + M * CBW, *s2 = s0 + M * CBW;
+    float *h1 = reinterpret_cast<float *>(s2 + M * CBW), *h0 = h1 + M * ld, *h2 = h0 + M * ld;
+    const int64_t MM = int64_t(M) * M, LL = int64_t(M) * ld;
+    const int slabs = (M + CBW - 1) / CBW, items = steps * slabs;
+    const int i0 = int(threadIdx.x / 4) * 2, cc2 = int(threadIdx.x % 4) * 2;
+    auto slot = [&](int j) { return j % 3 == 0 ? V0 : j % 3 == 1 ? V1 : V2; };
+    dfl vp[NI][2][2];      // V_{j-2} at this thread's entries
+    double u[NI][2][2];
+#pragma unroll
+    for (int n = 0; n < NI; ++n) {
+        const int id = blockIdx.x + n * gridDim.x, r = id % steps, c0 = id / steps * CBW;
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int i = i0 + a, c = c0 + cc2 + b;
+                vp[n][a][b] = dfl{0.f, 0.f};
+                u[n][a][b] = 0.0;
+                if (id >= items || i >= M || c >= M) continue;
+                const int64_t o = r * MM + int64_t(i) * M + c;
+                if (j0 == 0) {
+                    // V_0 = F_1
+                    const float e = r == 0 && i == c ? 1.f : 0.f;
+                    if (r == 0) V0[o] = dfl{e, 0.f};
+                    u[n][a][b] = cc.d[0] * double(e);
+                } else {
+                    u[n][a][b] = U[o];
+                    if (r <= j0 - 2) vp[n][a][b] = slot(j0 - 2)[o];
+                }
+            }
+    }
+    int target = 0;
+    bool good = true;
+    if (j0 == 0) good = grid_barrier(sync, sync + 1, target += gridDim.x);
+    auto copy8 = [](void *dst, const void *src) {
+        const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+    };
+    for (int q = j0 == 0 ? 1 : 0; good && q < cc.n; ++q) {
+        const int j = j0 + q;
+        const dfl *Vc = slot(j - 1);
+        dfl *Vn = slot(j);
+        const float beta = j == 1 ? 1.f : 2.f, gamma = j == 1 ? 0.f : 1.f;
+#pragma unroll
+        for (int n = 0; n < NI; ++n) {
+            const int id = blockIdx.x + n * gridDim.x, r = id % steps, c0 = id / steps * CBW;
+            if (id >= items || r > j) continue;   // (uniform; V_j is zero there)
+            if (NI > 1 || q == (j0 == 0 ? 1 : 0) || r == j) {
+                // H of this item (with one item: once, when its row is first reached)
+                for (int i = threadIdx.x * 2; i < M * ld; i += blockDim.x * 2) {
+                    copy8(h1 + i, Hd + r * LL + i);
+                    if (r > 0) copy8(h0 + i, Hst + (r - 1) * LL + i);
+                    if (r + 1 < steps) copy8(h2 + i, Hs + r * LL + i);
+                }
+            }
+            // (V through L2: its slots are rewritten by other SMs)
+            for (int idx = threadIdx.x; idx < M * CBW; idx += blockDim.x) {
+                const int k = idx / CBW, c = c0 + idx % CBW;
+                const int64_t o = r * MM + int64_t(k) * M + c;
+                float2 a{0.f, 0.f}, b{0.f, 0.f}, d{0.f, 0.f};
+                if (c < M) {
+                    if (r > 0) a = __ldcg(reinterpret_cast<const float2 *>(Vc + o - MM));
+                    if (r <= j - 1) b = __ldcg(reinterpret_cast<const float2 *>(Vc + o));
+                    if (r + 1 <= j - 1 && r + 1 < steps) d = __ldcg(reinterpret_cast<const float2 *>(Vc + o + MM));
+                }
+                s0[idx] = dfl{a.x, a.y};
+                s1[idx] = dfl{b.x, b.y};
+                s2[idx] = dfl{d.x, d.y};
+            }
+            asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+            __syncthreads();
+            if (i0 < M && c0 + cc2 < M) {
+                float s[2][2] = {{0.f, 0.f}, {0.f, 0.f}}, err[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+                auto acc = [&](const float *H, const dfl *v, int k0, int k1) {
+#pragma unroll 4
+                    for (int k = k0; k < k1; ++k) {
+                        const float2 h = *reinterpret_cast<const float2 *>(H + k * ld + i0);
+                        const float4 t = *reinterpret_cast<const float4 *>(v + k * CBW + cc2);
+                        const dfl va{t.x, t.y}, vb{t.z, t.w};
+                        dot2_step(s[0][0], err[0][0], h.x, va);
+                        dot2_step(s[0][1], err[0][1], h.x, vb);
+                        dot2_step(s[1][0], err[1][0], h.y, va);
+                        dot2_step(s[1][1], err[1][1], h.y, vb);
+                    }
+                };
+                if (r <= j - 1) acc(h1, s1, 0, M);
+                if (r > 0) acc(h0, s0, i0, M);                                             // R_{r-1}: k >= i
+                if (r + 1 <= j - 1 && r + 1 < steps) acc(h2, s2, 0, min(i0 + 2, M));       // R_r^T: k <= i
+#pragma unroll
+                for (int a = 0; a < 2; ++a)
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) {
+                        const int i = i0 + a, c = c0 + cc2 + b;
+                        if (i >= M || c >= M) continue;
+                        const dfl hv = dfl_fast(s[a][b], err[a][b]);
+                        const dfl v1 = s1[i * CBW + cc2 + b];
+                        float s2v = v1.h, e2 = v1.l;
+                        dot2_step(s2v, e2, dfl{-g.h, -g.l}, hv);
+                        float s3 = beta * s2v, e3 = beta * e2;
+                        dot2_step(s3, e3, -gamma, vp[n][a][b]);
+                        const dfl vn = dfl_fast(s3, e3);
+                        Vn[r * MM + int64_t(i) * M + c] = vn;
+                        vp[n][a][b] = v1;
+                        u[n][a][b] += cc.d[q] * dfl_val(vn);
+                    }
+            }
+            __syncthreads();
+        }
+        if (q + 1 < cc.n) good = grid_barrier(sync, sync + 1, target += gridDim.x);
+    }
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+#pragma unroll
+    for (int n = 0; n < NI; ++n) {
+        const int id = blockIdx.x + n * gridDim.x, r = id % steps, c0 = id / steps * CBW;
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int i = i0 + a, c = c0 + cc2 + b;
+                if (id < items && i < M && c < M) U[r * MM + int64_t(i) * M + c] = good ? u[n][a][b] : nan;
+            }
+    }
+}
+
 // ---------------------------------------------------------------- block Cholesky (spline)
 // One CTA; all scratch in global memory (L1/L2 resident for the sizes used).
 __device__ void chol_lower_inplace(double *A, int M) {
@@ -559,7 +699,8 @@ k_quad_accumulate(const double *__restrict__ scratch, int M, int mcap, int nb, Q
 
 int launch_cheb_bt(const double *Hd, const double *Hs, int M, int m, double lam,
                    const std::vector<double> &d, double *V0, double *V1, double *V2, double *U,
-                   const Ctrl *ctrl, cudaStream_t s, double *Hdf) {
+                   const Ctrl *ctrl, cudaStream_t s, double *Hdf, int32_t *sync, int kmax) {
+    if (kmax <= 0 || kmax > m) kmax = m;
     const size_t bytes = sizeof(double) * size_t(m) * M * M;
     prof_begin(KernelClass::PROJECTED, s);
     if (Hdf) {
@@ -567,18 +708,58 @@ int launch_cheb_bt(const double *Hd, const double *Hs, int M, int m, double lam,
         const int ld = (M + 1) / 2 * 2;
         float *hd = reinterpret_cast<float *>(Hdf), *hs = hd + size_t(m) * M * ld, *ht = hs + size_t(m) * M * ld;
         k_split_df<<<dim3(m, 2), 256, 0, s>>>(Hd, Hs, hd, hs, ht, M, ld, ctrl);
+        const size_t smem = sizeof(dfl) * 3 * M * CBW + sizeof(float) * 3 * M * ld;
+        const int threads = std::max(32, ((M + 1) / 2 * 4 + 31) / 32 * 32);
+        const dfl g = dfl_from(2.0 / lam);
+        // all terms in one cooperative launch while a CTA has at most four items (the steps known to
+        // the host bound the block rows)
+        const int items = kmax * ((M + CBW - 1) / CBW);
+        constexpr int SMEM_MAX = int(sizeof(dfl) * 3 * 128 * CBW + sizeof(float) * 3 * 128 * 128);
+        static const cudaError_t attrs[] = {
+            cudaFuncSetAttribute(k_cheb_bt_all<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX),
+            cudaFuncSetAttribute(k_cheb_bt_all<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX),
+            cudaFuncSetAttribute(k_cheb_bt_all<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX),
+            cudaFuncSetAttribute(k_cheb_bt_iter_df, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX)};
+        (void)attrs;
+        int per_sm = 0;
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cheb_bt_all<4>, threads, smem);
+        const int cap = per_sm * num_sms();
+        if (sync && cap > 0 && items <= 4 * cap && d.size() >= 2) {
+            zero_if_active(U, int64_t(m) * M * M, ctrl, s);
+            const int ni = items <= cap ? 1 : items <= 2 * cap ? 2 : 4;
+            const int grid = (items + ni - 1) / ni;
+            dfl *v[3] = {reinterpret_cast<dfl *>(V0), reinterpret_cast<dfl *>(V1), reinterpret_cast<dfl *>(V2)};
+            int launches = 2;
+            for (size_t j0 = 0; j0 < d.size(); j0 += ChebCoef::CAP) {
+                ChebCoef cc{};
+                cc.n = int(std::min<size_t>(ChebCoef::CAP, d.size() - j0));
+                for (int q = 0; q < cc.n; ++q) cc.d[q] = d[j0 + q];
+                KB_CUDA_TRY(cudaMemsetAsync(sync, 0, 2 * sizeof(int32_t), s));
+                cudaLaunchConfig_t cfg{};
+                cudaLaunchAttribute at[1];
+                at[0].id = cudaLaunchAttributeCooperative;
+                at[0].val.cooperative = 1;
+                cfg.gridDim = unsigned(grid);
+                cfg.blockDim = unsigned(threads);
+                cfg.dynamicSmemBytes = smem;
+                cfg.stream = s;
+                cfg.attrs = at;
+                cfg.numAttrs = 1;
+                auto kern = ni == 1 ? k_cheb_bt_all<1> : ni == 2 ? k_cheb_bt_all<2> : k_cheb_bt_all<4>;
+                KB_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, (const float *)hd, (const float *)hs, (const float *)ht, v[0],
+                                               v[1], v[2], U, M, ld, cc, int(j0), g, ctrl, sync));
+                ++launches;
+            }
+            KB_CUDA_TRY(cudaGetLastError());
+            prof_end(KernelClass::PROJECTED, s, 0, 0, launches);
+            return 0;
+        }
         KB_CUDA_TRY(cudaMemsetAsync(V0, 0, bytes, s));
         KB_CUDA_TRY(cudaMemsetAsync(V1, 0, bytes, s));
         KB_CUDA_TRY(cudaMemsetAsync(V2, 0, bytes, s));
         zero_if_active(U, int64_t(m) * M * M, ctrl, s);
         dfl *pp = reinterpret_cast<dfl *>(V2), *pc = reinterpret_cast<dfl *>(V0), *pn = reinterpret_cast<dfl *>(V1);
         k_cheb_bt_seed_df<<<(M + 127) / 128, 128, 0, s>>>(pc, U, M, d[0], ctrl);
-        const size_t smem = sizeof(dfl) * 3 * M * CBW + sizeof(float) * 3 * M * ld;
-        static const cudaError_t attr = cudaFuncSetAttribute(k_cheb_bt_iter_df, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                             int(sizeof(dfl) * 3 * 128 * CBW + sizeof(float) * 3 * 128 * 128));
-        (void)attr;
-        const int threads = std::max(32, ((M + 1) / 2 * 4 + 31) / 32 * 32);
-        const dfl g = dfl_from(2.0 / lam);
         for (size_t j = 0; j + 1 < d.size(); ++j) {
             const int nrb = std::min<int>(int(j) + 2, m);
             dim3 grid(nrb, (M + CBW - 1) / CBW);
