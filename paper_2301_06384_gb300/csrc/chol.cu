@@ -63,6 +63,7 @@ template <typename T>
 __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, int W, int pass, int step,
                                               double inv_thresh2, double piv_rel2, double *R1,
                                               T *Rinv, double *Hs, T *Bout, Ctrl *ctrl) {
+    pdl_wait();
     if (ctrl->stop) return;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int bad, small;
@@ -152,6 +153,7 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
             });
             sm::tri_mm(F2, F1, lda, M, none, [&](int i, int j, float c, int) { F0[i * lda + j] = c; });
             __syncthreads();
+            pdl_trigger();   // (not earlier: the next kernel's CTAs would hold their SMs meanwhile)
             // H = (I + F + F^2) R1 = R1 + (C + F C), the corrections of relative size ||E||
             sm::tri_mm(F2, F0, lda, M, [&](int i, int j) { return __ldcg(R1 + i * M + j); },
                        [&](int i, int j, float c2, double r1) {
@@ -189,6 +191,7 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
                     // C1 = R E over S (zeros below the diagonal), then R1 = R + (C1 + C1 E)
                     sm::tri_mm(F0, F2, lda, M, none, [&](int i, int j, float c, int) { F1[i * lda + j] = c; });
                     __syncthreads();
+                    pdl_trigger();
                     sm::tri_mm(F1, F2, lda, M, none, [&](int i, int j, float c2, int) {
                         R1[i * M + j] = double(F0[i * lda + j]) + double(F1[i * lda + j] + c2);
                     });
@@ -246,6 +249,7 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
         sm::tri_inv_merge<T>(B, lda, M, Bt);
         sm::each(W, W, [&](int i, int j) { Rinv[i * W + j] = (i < M && j < M && j >= i) ? B[i * lda + j] : T(0); });
     }
+    pdl_trigger();
     // A: the upper triangular R whose inverse is applied (FP64)
     if (pass == 1) {
         sm::each(M, M, [&](int i, int j) { R1[i * M + j] = j >= i ? A[i * lda + j] : 0.0; });
@@ -293,8 +297,8 @@ int launch_chol(const double *G, int M, int W, int pass, int step, double inv_th
         k_chol<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(chol_layout<T>(sizeof(T) == 8 ? 64 : 128).total));
     (void)attr;
     prof_begin(KernelClass::SMALL, s);
-    k_chol<T><<<1, CHOL_THREADS, smem, s>>>(G, M, W, pass, step, inv_thresh2, piv_rel2, R1, Rinv, Hs, Bout, ctrl);
-    KB_CUDA_TRY(cudaGetLastError());
+    KB_CUDA_TRY(launch_dep(k_chol<T>, dim3(1), CHOL_THREADS, smem, s, 0, G, M, W, pass, step, inv_thresh2, piv_rel2, R1,
+                           Rinv, Hs, Bout, ctrl));
     prof_end(KernelClass::SMALL, s, 0, 0);
     return 0;
 }

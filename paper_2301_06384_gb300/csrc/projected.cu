@@ -451,7 +451,9 @@ __device__ __forceinline__ double dot4(int k0, int k1, const FA &a, const FB &b)
 
 // row i = blockIdx.x of Ls_{r-1} (both factors upper triangular)
 __global__ void __launch_bounds__(128) k_bt_ls(BtArgs a, int r, const Ctrl *fc) {
+    pdl_wait();
     if (bt_skip(fc, r)) return;
+    pdl_trigger();
     const int M = a.M, i = blockIdx.x;
     const int64_t MM = int64_t(M) * M;
     const double *h = a.Hs + (r - 1) * MM + int64_t(i) * M, *Ri = a.Ri + (r - 1) * MM;
@@ -463,7 +465,9 @@ __global__ void __launch_bounds__(128) k_bt_ls(BtArgs a, int r, const Ctrl *fc) 
 // row i: of D_r (blockIdx.y = 0, into Ri_r, lower triangle transposed to the upper one) and of
 // K_{r-1} (blockIdx.y = 1)
 __global__ void __launch_bounds__(128) k_bt_schur(BtArgs a, int r, double eps, const Ctrl *fc) {
+    pdl_wait();
     if (bt_skip(fc, r)) return;
+    pdl_trigger();
     const int M = a.M, i = blockIdx.x;
     const int64_t MM = int64_t(M) * M;
     const double *L = a.Ls + ((r - 1) & 1) * MM;
@@ -485,6 +489,7 @@ __global__ void __launch_bounds__(128) k_bt_schur(BtArgs a, int r, double eps, c
 }
 
 __global__ void __launch_bounds__(512) k_bt_dchol(BtArgs a, int r, const Ctrl *fc) {
+    pdl_wait();
     if (bt_skip(fc, r)) return;
     extern __shared__ __align__(16) double bsm[];
     const int M = a.M, lda = (M + 1) / 2 * 2;
@@ -501,6 +506,7 @@ __global__ void __launch_bounds__(512) k_bt_dchol(BtArgs a, int r, const Ctrl *f
         sm::tri_inv_diag<double>(A, lda, M);
         sm::tri_inv_merge<double>(A, lda, M, tmp);
     }
+    pdl_trigger();
     // a block that is not positive definite (lost orthogonality) shows as NaN
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
     sm::each(M, M, [&](int i, int j) {
@@ -511,7 +517,9 @@ __global__ void __launch_bounds__(512) k_bt_dchol(BtArgs a, int r, const Ctrl *f
 
 // row i = blockIdx.x of G_r^T (Ri_r upper triangular, Ls_{r-1} upper triangular)
 __global__ void __launch_bounds__(128) k_bt_gt(BtArgs a, int r, const Ctrl *fc) {
+    pdl_wait();
     if (bt_skip(fc, r)) return;
+    pdl_trigger();
     const int M = a.M, i = blockIdx.x;
     const int64_t MM = int64_t(M) * M;
     const double *L = a.Ls + ((r - 1) & 1) * MM, *Ri = a.Ri + r * MM;
@@ -806,10 +814,11 @@ static int bt_factor(const BtArgs &a, int r0, int kmax, double eps, const Ctrl *
     (void)attr;
     int launches = 0;
     for (int r = r0; r < kmax; ++r) {
-        if (r > 0) k_bt_ls<<<M, 128, 0, s>>>(a, r, fc);
-        k_bt_schur<<<dim3(M, r > 0 ? 2 : 1), 128, 0, s>>>(a, r, eps, fc);
-        k_bt_dchol<<<1, 512, smem, s>>>(a, r, fc);
-        if (r > 0) k_bt_gt<<<M, 128, 0, s>>>(a, r, fc);
+        // (a failed launch shows in the caller's cudaGetLastError)
+        if (r > 0) (void)launch_dep(k_bt_ls, dim3(M), 128, 0, s, 0, a, r, fc);
+        (void)launch_dep(k_bt_schur, dim3(M, r > 0 ? 2 : 1), 128, 0, s, 0, a, r, eps, fc);
+        (void)launch_dep(k_bt_dchol, dim3(1), 512, smem, s, 0, a, r, fc);
+        if (r > 0) (void)launch_dep(k_bt_gt, dim3(M), 128, 0, s, 0, a, r, fc);
         launches += r > 0 ? 4 : 2;
     }
     return launches;

@@ -41,6 +41,7 @@ template <typename P>
 __global__ void __launch_bounds__(1024) k_reduce(const P *__restrict__ parts, int nparts, int len,
                                                   double *__restrict__ out, const Ctrl *ctrl,
                                                   P *__restrict__ out_p, const int32_t *skip, HkkOut<P> h) {
+    pdl_wait();
     if ((ctrl && ctrl->stop) || (skip && *skip)) return;
     __shared__ double s[32][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -95,6 +96,7 @@ __global__ void __launch_bounds__(1024) k_reduce(const P *__restrict__ parts, in
             if (out_p) out_p[e] = P(t);
         }
     }
+    pdl_trigger();
     if (h.cnt) {
         __shared__ unsigned last;
         __threadfence();
@@ -206,8 +208,8 @@ template <typename P>
 static int reduce_impl(const P *parts, int nparts, int len, double *out, cudaStream_t s, const Ctrl *ctrl, P *out_p,
                        const int32_t *skip, const HkkOut<P> &h) {
     prof_begin(KernelClass::REDUCE, s);
-    k_reduce<P><<<(len + 31) / 32, 1024, 0, s>>>(parts, nparts, len, out, ctrl, out_p, skip, h);
-    cudaError_t err = cudaGetLastError();
+    const cudaError_t err = launch_dep(k_reduce<P>, dim3((len + 31) / 32), 1024, 0, s, 0, parts, nparts, len, out, ctrl,
+                                       out_p, skip, h);
     if (err != cudaSuccess) return cuda_fail(err, "k_reduce launch");
     prof_end(KernelClass::REDUCE, s, double(nparts) * len * sizeof(P), 0);
     return 0;

@@ -237,6 +237,7 @@ k_rowblock(RowArgs<T> a) {
     constexpr bool MULTI = MODE == RB_ASM || MODE == RB_ASMSUB;    // product over basis blocks
     constexpr bool ASYNC_X = SUBX && std::is_same<T, typename G::C>::value;   // X comes by cp.async
     constexpr int BI = G::BI, BJ = G::BJ, KC = G::KC, LDA = G::LDA, LDO = G::LDO, VEC = G::VEC;
+    pdl_wait();
     if (MODE != RB_ASM && a.ctrl && a.ctrl->stop) return;
     if (a.skip && *a.skip) return;
 
@@ -735,6 +736,7 @@ k_rowblock(RowArgs<T> a) {
         cp_wait<0>();
         __syncthreads();
     }
+    pdl_trigger();
     if (tid == 0 && a.prof.rows) {
         atomicAdd(a.prof.rows, my_rows);
         atomicAdd(a.prof.nnz, my_units);
@@ -798,8 +800,8 @@ int launch_r(const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
     int grid = int(std::min<int64_t>(nvt, int64_t(num_sms()) * (ORD ? G::CTAS : per_sm)));
     if (grid < 1) grid = 1;
     if (grid_out) *grid_out = grid;
-    k_rowblock<T, W, MODE, RPT, ORD, NT><<<grid, NT, smem, s>>>(a);
-    return 0;
+    const cudaError_t e = launch_dep(k_rowblock<T, W, MODE, RPT, ORD, NT>, dim3(grid), NT, smem, s, 0, a);
+    return e == cudaSuccess ? 0 : cuda_fail(e, "k_rowblock launch");
 }
 
 // Rows per thread.  FP32: 8 (12 shared loads per 128 FMAs instead of 8 per 64), 4 at W = 16

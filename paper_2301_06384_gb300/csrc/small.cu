@@ -242,9 +242,11 @@ __global__ void k_lanczos_init(int W, int M, int gbl, int round32, double *sigma
 __global__ void __launch_bounds__(LZ_THREADS)
 k_lanczos_alpha(const double *parts, int nparts, int W, int M, int gbl, int k, int df, const double *sigma,
                 double *alpha, double *a_upd, const Ctrl *ctrl) {
+    pdl_wait();
     if (ctrl->stop) return;
     __shared__ double s[LZ_COLS];
     reduce_cols(parts, nparts, W, s, df);
+    pdl_trigger();
     const double *sg = sigma + int64_t(k) * W;
     const double tot = gbl ? sg[0] * cluster_total(s) : 0.0;
     if (threadIdx.x < LZ_COLS) {
@@ -262,9 +264,11 @@ k_lanczos_alpha(const double *parts, int nparts, int W, int M, int gbl, int k, i
 __global__ void __launch_bounds__(LZ_THREADS)
 k_lanczos_beta(const double *parts, int nparts, int W, int M, int gbl, int k, int round32, double thresh,
                double *beta, double *sigma, int32_t *alive, double *c1, double *c2, Ctrl *ctrl) {
+    pdl_wait();
     if (ctrl->stop) return;
     __shared__ double s[LZ_COLS];
     reduce_cols(parts, nparts, W, s, round32);
+    pdl_trigger();
     const double *sk = sigma + int64_t(k) * W;
     double *sn = sigma + int64_t(k + 1) * W;
     double *bn = beta + int64_t(k + 1) * W;
@@ -493,6 +497,7 @@ __global__ void __launch_bounds__(256) k_axpy_colnorm(T *X, const T *P, const do
                                                        const int32_t *tgen, int limit,
                                                        const int32_t *alist, const int32_t *acount,
                                                        ProfCount pc) {
+    pdl_wait();
     if (ctrl->stop) return;
     using C = typename Cmp<T>::type;
     constexpr int CG = W / 4;
@@ -559,6 +564,7 @@ __global__ void __launch_bounds__(256) k_axpy_colnorm(T *X, const T *P, const do
             stv4(X + (h ? row2 : row) * W + c4, xv[h]);
         }
     }
+    pdl_trigger();
     if (pc.rows && cg == 0 && my_rows) atomicAdd(pc.rows, my_rows);
     if constexpr (std::is_same<C, float>::value) {
         // double-float column sums on the FP32 pipe; partials written as DF pairs
@@ -816,28 +822,11 @@ int launch_lanczos_init(int W, int M, int gbl, int round32, double *sigma, int32
     return 0;
 }
 
-// One cluster of n (1, 2, 4 or 8) CTAs.
-template <typename... P, typename... A>
-static cudaError_t launch_cluster(int n, cudaStream_t s, void (*kernel)(P...), A... args) {
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = unsigned(n);
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = unsigned(n);
-    cfg.blockDim = LZ_THREADS;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-}
-
 int launch_lanczos_alpha(const double *parts, int nparts, int W, int M, int gbl, int k, int df,
                          const double *sigma, double *alpha, double *a_upd, const Ctrl *ctrl,
                          cudaStream_t s) {
     prof_begin(KernelClass::SMALL, s);
-    KB_CUDA_TRY(launch_cluster(W / LZ_COLS, s, k_lanczos_alpha, parts, nparts, W, M, gbl, k, df, sigma, alpha, a_upd,
+    KB_CUDA_TRY(launch_dep(k_lanczos_alpha, dim3(W / LZ_COLS), LZ_THREADS, 0, s, W / LZ_COLS, parts, nparts, W, M, gbl, k, df, sigma, alpha, a_upd,
                                ctrl));
     prof_end(KernelClass::SMALL, s, double(nparts) * W * 8, 0);
     return 0;
@@ -847,7 +836,7 @@ int launch_lanczos_beta(const double *parts, int nparts, int W, int M, int gbl, 
                         double thresh, double *beta, double *sigma, int32_t *alive, double *c1,
                         double *c2, Ctrl *ctrl, cudaStream_t s) {
     prof_begin(KernelClass::SMALL, s);
-    KB_CUDA_TRY(launch_cluster(W / LZ_COLS, s, k_lanczos_beta, parts, nparts, W, M, gbl, k, round32, thresh, beta, sigma,
+    KB_CUDA_TRY(launch_dep(k_lanczos_beta, dim3(W / LZ_COLS), LZ_THREADS, 0, s, W / LZ_COLS, parts, nparts, W, M, gbl, k, round32, thresh, beta, sigma,
                                alive, c1, c2, ctrl));
     prof_end(KernelClass::SMALL, s, double(nparts) * W * 8, 0);
     return 0;
@@ -891,14 +880,15 @@ int launch_axpy_colnorm(int W, T *X, const T *P, const double *a, int64_t n, dou
     const int grid = int(std::min<int64_t>((n + rpp - 1) / rpp, int64_t(num_sms()) * 4));
     *grid_out = std::max(grid, 1);
     const ProfCount pc = prof_begin(KernelClass::ROWBLOCK, s);
+    cudaError_t err = cudaSuccess;
     switch (W) {
-        case 16: k_axpy_colnorm<T, 16><<<*grid_out, 256, 0, s>>>(X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
-        case 32: k_axpy_colnorm<T, 32><<<*grid_out, 256, 0, s>>>(X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
-        case 64: k_axpy_colnorm<T, 64><<<*grid_out, 256, 0, s>>>(X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
-        case 128: k_axpy_colnorm<T, 128><<<*grid_out, 256, 0, s>>>(X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
+        case 16: err = launch_dep(k_axpy_colnorm<T, 16>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
+        case 32: err = launch_dep(k_axpy_colnorm<T, 32>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
+        case 64: err = launch_dep(k_axpy_colnorm<T, 64>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
+        case 128: err = launch_dep(k_axpy_colnorm<T, 128>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
         default: return fail(KB_ERR_ARG, "bad width");
     }
-    KB_CUDA_TRY(cudaGetLastError());
+    KB_CUDA_TRY(err);
     const double row = double(M_alg) * sizeof(T);
     prof_end(KernelClass::ROWBLOCK, s, 3.0 * double(n) * row, 3.0 * double(n) * M_alg, 1, 3.0 * row,
              0.0, 3.0 * M_alg, 0.0);

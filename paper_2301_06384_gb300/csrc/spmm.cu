@@ -144,6 +144,7 @@ k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo, in
     constexpr int LPR = G::LPR, RPW = G::RPW, UPT = G::UPT;
     constexpr int CPL = LPR >= 8 ? 1 : 8 / LPR;   // neighbour indices a lane loads at once
     constexpr int CHUNK = LPR * CPL;
+    pdl_wait();
     if (e.ctrl && e.ctrl->stop) return;
     __shared__ __align__(16) C s_coef[5][W];       // c1 hi, c1 lo, c0, c2 hi, c2 lo
     __shared__ C s_sc[2];                          // s3, wE in the arithmetic type
@@ -372,6 +373,7 @@ k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo, in
         end = nend;
         act = nact;
     }
+    pdl_trigger();
     if (e.prof.rows && my_rows) {
         atomicAdd(e.prof.rows, (unsigned long long)my_rows);
         atomicAdd(e.prof.nnz, (unsigned long long)my_nnz);
@@ -438,9 +440,10 @@ int launch_wd(const GraphDev &g, const T *x, const LinEpi<T> &e, int64_t ldo, in
     int grid = int(std::min<int64_t>((units + WARPS - 1) / WARPS, int64_t(num_sms()) * occupancy_spmm<T, W, DOT>()));
     if (grid < 1) grid = 1;
     if (grid_out) *grid_out = grid;
-    if (g.w) k_spmm<T, W, DOT, true><<<grid, SPMM_THREADS, 0, s>>>(g, x, e, ldo, mo, mcols);
-    else k_spmm<T, W, DOT, false><<<grid, SPMM_THREADS, 0, s>>>(g, x, e, ldo, mo, mcols);
-    return 0;
+    const cudaError_t err =
+        launch_dep(g.w ? k_spmm<T, W, DOT, true> : k_spmm<T, W, DOT, false>, dim3(grid), SPMM_THREADS, 0, s, 0, g, x, e, ldo,
+                   mo, mcols);
+    return err == cudaSuccess ? 0 : cuda_fail(err, "k_spmm launch");
 }
 
 template <typename T, int W>
@@ -459,15 +462,15 @@ int launch_spmm(const GraphDev &g, int W, const T *x, const LinEpi<T> &e, cudaSt
     LinEpi<T> ee = e;
     ee.prof = prof_begin(KernelClass::SPMM, s);
     const int mcols = int(M_alg);
+    int rc = 0;
     switch (W) {
-        case 16: launch_w<T, 16>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
-        case 32: launch_w<T, 32>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
-        case 64: launch_w<T, 64>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
-        case 128: launch_w<T, 128>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
+        case 16: rc = launch_w<T, 16>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
+        case 32: rc = launch_w<T, 32>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
+        case 64: rc = launch_w<T, 64>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
+        case 128: rc = launch_w<T, 128>(g, x, ee, ldo, mo, mcols, s, grid_out); break;
         default: return fail(KB_ERR_ARG, "unsupported block width");
     }
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess) return cuda_fail(err, "k_spmm launch");
+    if (rc) return rc;
     // algorithmic bytes: CSR (+weights, +diagonal excess) once, the gathered block once,
     // the other dense inputs once each, the output once; flops 3 per nonzero per column
     double csr = 4.0 * double(g.n + 1) + 4.0 * double(g.nnz) + (g.w ? 4.0 * double(g.nnz) : 0.0) +
