@@ -77,7 +77,8 @@ typedef struct {
                            FP64 arithmetic throughout); any other value is KB_ERR_ARG         */
     int32_t no_frontier;/* 0 (default): the products and block updates of step k touch only
                            rows within k hops of W (the Krylov blocks are exactly zero
-                           elsewhere); 1: every step touches all n rows                           */
+                           elsewhere) where blocks of n x W are large enough for that to pay;
+                           1: every step touches all n rows                                       */
     int32_t two_pass;   /* 0 (default): the Krylov basis is stored (m blocks of n x W); 1: the
                            Lanczos methods keep three blocks and run the recurrence twice,
                            the second time with the recorded coefficients, adding each block
@@ -98,7 +99,8 @@ typedef struct {
     int32_t steps_done;      /* products with L whose blocks enter the result (<= m); smaller
                                 than m when the Krylov space became invariant (exact result)     */
     int32_t breakdown_step;  /* step of a rank-deficient block, or -1                             */
-    int32_t spmm_launches;   /* SpMM kernels launched by the call                                  */
+    int32_t spmm_launches;   /* products with L of the call (of all m steps, also when a stopping rule
+                                ends the process earlier)                                         */
     double  lambda_used;     /* Lambda used for the Chebyshev methods (0 for Lanczos)              */
     double  est_change;      /* KB_CBL with params.tol > 0: ||U_k - [U_k'; 0]||_F / ||U_k||_F at the
                                 last stopping-rule check that ran (the estimate of the change of Y
@@ -193,7 +195,7 @@ int kb_graph_lambda_bounds(const kb_graph *g, double *gershgorin, double *projec
  * Other errors: KB_ERR_ARG, KB_ERR_NODES, KB_ERR_NOMEM, KB_ERR_CUDA (also when an opt-in
  * tensor-core kernel gives up waiting for its MMA completion).
  *
- * Environment: KB_TENSOR_CORES=1 (read at every launch) runs the tall-skinny products of
+ * Environment: KB_TENSOR_CORES=1 (read at the start of a solve) runs the tall-skinny products of
  * KB_CBL with FP32 blocks of width 64 (M in 33..64) on the tcgen05 tensor cores (BF16 x 6
  * split products, FP32 accumulation).  It is not the default: with the frontier restriction
  * it is slower than the SIMT kernels, and on sensitive kernels its error is several times
