@@ -493,7 +493,7 @@ def job_value(cols_per_step: int, world: int, ms: float) -> float:
 def main():
     a = parse()
     if a.tensor_cores:
-        os.environ["KB_TENSOR_CORES"] = "1"   # read by the library at each row-block launch
+        os.environ["KB_TENSOR_CORES"] = "1"   # read by the library at each solve
     rank = int(os.environ.get("RANK", "0"))
     world = int(os.environ.get("WORLD_SIZE", "1"))
     local = int(os.environ.get("LOCAL_RANK", "0"))
