@@ -169,6 +169,9 @@ struct SplineBufs {
 int launch_bt_spline(const double *Hd, const double *Hs, int M, int m, double eps, int s_int,
                      const SplineBufs &b, double *U, const Ctrl *fc, const Ctrl *ctrl, cudaStream_t s,
                      const QuadRule *q, double *qscr, int qbatch, int r0, int y0, int kmax);
+// Blocks r0 .. kmax - 1 of that factorisation alone.
+int launch_bt_factor(const double *Hd, const double *Hs, int M, double eps, const SplineBufs &b, const Ctrl *fc,
+                     cudaStream_t s, int r0, int kmax);
 
 // Full reorthogonalisation: save the diagonal of the Gram of X before the first pass; after
 // it, *skip = 1 when every column kept at least half of its squared norm (the second pass is

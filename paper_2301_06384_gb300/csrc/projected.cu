@@ -824,6 +824,16 @@ static int bt_factor(const BtArgs &a, int r0, int kmax, double eps, const Ctrl *
     return launches;
 }
 
+int launch_bt_factor(const double *Hd, const double *Hs, int M, double eps, const SplineBufs &b, const Ctrl *fc,
+                     cudaStream_t s, int r0, int kmax) {
+    const BtArgs a{Hd, Hs, b.Ri, b.RiT, b.Y, b.GT, b.K, b.Ls, M};
+    prof_begin(KernelClass::PROJECTED, s);
+    const int launches = bt_factor(a, r0, kmax, eps, fc, s);
+    KB_CUDA_TRY(cudaGetLastError());
+    prof_end(KernelClass::PROJECTED, s, 0, 0, launches);
+    return 0;
+}
+
 int launch_bt_spline(const double *Hd, const double *Hs, int M, int m, double eps, int s_int,
                      const SplineBufs &b, double *U, const Ctrl *fc, const Ctrl *ctrl, cudaStream_t s,
                      const QuadRule *q, double *qscr, int qbatch, int r0, int y0, int kmax) {
