@@ -160,8 +160,12 @@ class CheckWatch {
             if (!p.tried) {
                 p.tried = true;
                 void *mem = nullptr;
+                // (an allocation must not disturb a capture that another thread has begun)
+                cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+                cudaThreadExchangeStreamCaptureMode(&mode);
                 if (cudaHostAlloc(&mem, sizeof(Ctrl) * 64, cudaHostAllocPortable) == cudaSuccess) p.base = static_cast<Ctrl *>(mem);
                 else (void)cudaGetLastError();
+                cudaThreadExchangeStreamCaptureMode(&mode);
             }
             for (int i = 0; p.base && i < 64 && slot_ < 0; ++i)
                 if (!p.used[i]) {

@@ -429,7 +429,8 @@ __device__ void chol_lower_inplace(double *A, int M) {
 // stopped the process.  Measured (four concurrent requests, RGG of 55392 rows, M = 64 and less,
 // (0.1 I + L)^{-1}, up to 100 steps, checks at 8 to 96): sums of the launch list 239 -> 62 ms
 // (every check factored all blocks and solved triangular systems with one warp per column),
-// the requests 156 -> 81 ms.
+// the requests 156 -> 81 ms; with the blocks factored beside the Lanczos steps, as krylov.cu has
+// it, and the steps' other changes 62 ms.
 struct BtArgs {
     const double *Hd, *Hs;
     double *Ri, *RiT, *Y, *GT, *K, *Ls;   // Ls: two blocks, by the parity of r
