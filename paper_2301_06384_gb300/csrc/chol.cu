@@ -18,11 +18,13 @@ namespace kb {
 //
 // Pass 1 of the FP32 path (G = X^T X, any conditioning) factors G in FP32: it only has to
 // bring X close to orthonormal, the second pass corrects what is left, and R1 is the inverse
-// of the applied FP32 inverse S whatever R it came from: with S R = I - E,
+// of the applied FP32 inverse S whatever R it came from.  M <= 64: with S R = I - E,
 // S^{-1} = R (I - E)^{-1} = R + R E + R E^2 + O(E^3), E (of the order of the FP32 rounding)
-// from a residual in pairs of floats, the corrections in FP32.  A pivot below 1e-5 of the
-// largest diagonal entry, or max |E_ij| >= 1e-3, is not trusted in FP32: the factorisation is
-// then done in FP64 (which alone decides a breakdown) and S is inverted in FP64.
+// from a residual in pairs of floats, the corrections in FP32 (relative error of R1 1e-14 to
+// 4e-14, below the FP32 rounding of H by six orders).  M > 64: S is inverted in FP64 (2e-16 to
+// 7e-16; the corrected form reaches 1e-13 there).  A pivot below 1e-5 of the largest diagonal
+// entry, or max |E_ij| >= 1e-3, is not trusted in FP32: the factorisation is then done in FP64
+// (which alone decides a breakdown) and S is inverted in FP64.
 // Pass 2 of the FP32 path (G = I + E, ||E|| of the order of the FP32 rounding of pass 1): to
 // first order R2 = I + Phi(E) with Phi = strict upper part plus half the diagonal,
 // R2^{-1} = I - Phi(E) (the orthogonality of Q = X1 (I - Phi(E)) is then I + O(||E||^2)); the
@@ -34,6 +36,7 @@ namespace kb {
 // pass 2 (us, launch list): 31 / 15 at M = 40, 17 / 9 at M = 16; with one barrier per column
 // and 4 x 4 tiles on few threads 69 / 19 and 43 / 11.  FP64, M = 33: 58 / 49, before 112 / 90.
 constexpr int CHOL_THREADS = 512;
+constexpr int CORRECTED_MAX = 64;   // widest block whose R1 is the corrected FP32 factor
 
 struct CholLayout {
     // byte offsets of the dynamic shared memory: three FP32 matrices (general FP32 path), or one
@@ -81,6 +84,8 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
     constexpr bool FP32 = sizeof(T) == 4;
     auto none = [](int, int) { return 0; };
     const bool try_small = pass == 2 && FP32;
+    // pass 1 in FP32: S is inverted in FP64 (its copy in the second region is at F2)
+    bool inverted = FP32 && pass == 1 && M > CORRECTED_MAX;
     if (threadIdx.x == 0) {
         emax_bits = 0u;
         bad = 0;
@@ -165,7 +170,7 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
             return;
         }
         if (pass == 1) {
-            // ---- FP32 factor, its inverse and the corrected FP64 inverse of that
+            // ---- FP32 factor, its inverse and the FP64 inverse of that
             sm::each(M, M, [&](int i, int j) { F1[i * lda + j] = 0.f; });
             __syncthreads();
             if (sm::chol_blocked<float>(F0, F1, lda, M, 1e-5f * float(maxdiag), reinterpret_cast<float *>(scr))) {
@@ -177,41 +182,49 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
                 __syncthreads();
                 sm::tri_inv_merge<float>(F1, lda, M, Ft);
                 sm::each(W, W, [&](int i, int j) {
-                    Rinv[i * W + j] = (i < M && j < M && j >= i) ? F1[i * lda + j] : 0.f;
-                    if (i < M && j < i) F2[i * lda + j] = 0.f;
+                    const bool in = i < M && j < M;
+                    const float v = in && j >= i ? F1[i * lda + j] : 0.f;
+                    Rinv[i * W + j] = v;
+                    if (in && (inverted || j < i)) F2[i * lda + j] = v;   // (S, or E's zeros below the diagonal)
                 });
-                unsigned my = 0u;
-                sm::tri_residual(F1, F0, lda, M, [&](int i, int j, float e) {
-                    F2[i * lda + j] = e;
-                    my = max(my, __float_as_uint(fabsf(e)));
-                });
-                atomicMax(&emax_bits, my);
-                __syncthreads();
-                if (__uint_as_float(emax_bits) < 1e-3f) {
-                    // C1 = R E over S (zeros below the diagonal), then R1 = R + (C1 + C1 E)
-                    sm::tri_mm(F0, F2, lda, M, none, [&](int i, int j, float c, int) { F1[i * lda + j] = c; });
+                if (!inverted) {
+                    unsigned my = 0u;
+                    sm::tri_residual(F1, F0, lda, M, [&](int i, int j, float e) {
+                        F2[i * lda + j] = e;
+                        my = max(my, __float_as_uint(fabsf(e)));
+                    });
+                    atomicMax(&emax_bits, my);
                     __syncthreads();
-                    pdl_trigger();
-                    sm::tri_mm(F1, F2, lda, M, none, [&](int i, int j, float c2, int) {
-                        R1[i * M + j] = double(F0[i * lda + j]) + double(F1[i * lda + j] + c2);
-                    });
-                    sm::each(M, M, [&](int i, int j) {
-                        if (j < i) R1[i * M + j] = 0.0;
-                    });
-                    return;
+                    if (__uint_as_float(emax_bits) < 1e-3f) {
+                        // C1 = R E over S (zeros below the diagonal), then R1 = R + (C1 + C1 E)
+                        sm::tri_mm(F0, F2, lda, M, none, [&](int i, int j, float c, int) { F1[i * lda + j] = c; });
+                        __syncthreads();
+                        pdl_trigger();
+                        sm::tri_mm(F1, F2, lda, M, none, [&](int i, int j, float c2, int) {
+                            R1[i * M + j] = double(F0[i * lda + j]) + double(F1[i * lda + j] + c2);
+                        });
+                        sm::each(M, M, [&](int i, int j) {
+                            if (j < i) R1[i * M + j] = 0.0;
+                        });
+                        return;
+                    }
                 }
+            } else {
+                inverted = false;
             }
             __syncthreads();
         }
-        // ---- FP64 factorisation (from G again)
-        sm::load_square(G, W, M, [&](int i, int j, double g) { A[i * lda + j] = g; });
-        __syncthreads();
+        if (!inverted) {
+            // ---- FP64 factorisation (from G again)
+            sm::load_square(G, W, M, [&](int i, int j, double g) { A[i * lda + j] = g; });
+            __syncthreads();
+        }
     }
     T *B = reinterpret_cast<T *>(smem + L.second);   // the applied inverse
     T *Bt = B + size_t(lda) * ((M + 1) / 2 * 2);     // scratch of its merge levels
     bool ok;
     if constexpr (FP32) {
-        ok = sm::chol_blocked<double>(A, nullptr, lda, M, piv_rel2 * maxdiag, scr);
+        ok = inverted || sm::chol_blocked<double>(A, nullptr, lda, M, piv_rel2 * maxdiag, scr);
     } else {
         sm::each(M, M, [&](int i, int j) { B[i * lda + j] = 0.0; });
         __syncthreads();
@@ -228,15 +241,16 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
     }
     if constexpr (FP32) {
         // S = the FP32 inverse of the rounded factor; A = the FP64 inverse of S
-        sm::each(M, M, [&](int i, int j) { B[i * lda + j] = j >= i ? float(A[i * lda + j]) : 0.f; });
-        __syncthreads();
-        sm::tri_inv_diag<float>(B, lda, M);
-        sm::tri_inv_merge<float>(B, lda, M, Bt);
-        sm::each(W, W, [&](int i, int j) {
-            const bool in = i < M && j < M, up = in && j >= i;
-            Rinv[i * W + j] = up ? B[i * lda + j] : 0.f;
-            if (in) A[i * lda + j] = up ? double(B[i * lda + j]) : 0.0;
-        });
+        if (!inverted) {
+            sm::each(M, M, [&](int i, int j) { B[i * lda + j] = j >= i ? float(A[i * lda + j]) : 0.f; });
+            __syncthreads();
+            sm::tri_inv_diag<float>(B, lda, M);
+            sm::tri_inv_merge<float>(B, lda, M, Bt);
+            sm::each(W, W, [&](int i, int j) {
+                Rinv[i * W + j] = i < M && j < M && j >= i ? B[i * lda + j] : 0.f;
+            });
+        }
+        sm::each(M, M, [&](int i, int j) { A[i * lda + j] = j >= i ? double(B[i * lda + j]) : 0.0; });
         __syncthreads();
         sm::tri_inv_diag<double>(A, lda, M);
         sm::tri_inv_merge<double>(A, lda, M, reinterpret_cast<double *>(smem + L.second));
