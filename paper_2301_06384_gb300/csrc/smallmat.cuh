@@ -46,12 +46,7 @@ __device__ __forceinline__ double recip(double d) {
     e = fma(-d, r, 1.0);
     return fma(r, e, r);
 }
-// (one unit in the last place: the FP32 factors are corrected afterwards)
-__device__ __forceinline__ float recip(float d) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-    return r;
-}
+__device__ __forceinline__ float recip(float d) { return __frcp_rn(d); }   // (rounded to nearest)
 
 // Edge of the register tiles: 2 in FP32, where a shared load is the dearer part, 1 in FP64,
 // whose FMA occupies a scheduler for some 64 cycles, so that only spreading the entries helps.

@@ -1,5 +1,6 @@
 """The CholeskyQR kernel against extended precision, through the library's own launcher: R1 as the
-inverse of the applied inverse on both sides of the width where its form changes."""
+inverse of the applied inverse on both sides of the width where its form changes, and the
+reciprocals of the pivots."""
 import ctypes
 
 import numpy as np
@@ -62,3 +63,20 @@ def test_r1_is_the_inverse_of_the_applied_inverse(lib, M, kind):
     ref = R.astype(ld) + R.astype(ld) @ (np.eye(M) - S.astype(ld) @ R.astype(ld))
     err = float(np.abs(R1 - ref).max() / np.abs(ref).max())
     assert err < (4 * M ** 0.5 * U64 if kind == "d" or M > 64 else max(8, M) * U32 ** 2 * 8), err
+
+
+@pytest.mark.parametrize("kind", ["f", "d"])
+def test_pivot_reciprocals_are_rounded(lib, kind):
+    # diagonal G: S holds the reciprocals of the (correctly rounded) square roots: half a unit in
+    # the last place, and in FP64 a term of the squared error before the last Newton step
+    rng = np.random.default_rng(3)
+    dt, ulp = (np.float32, 2 * U32) if kind == "f" else (np.float64, 2 * U64)
+    for rep in range(20):
+        d = 10.0 ** rng.uniform(0, 4 if kind == "f" else 200, 64) * (1 if kind == "f" else 1e-100)
+        if kind == "f":
+            d = d.astype(np.float32).astype(np.float64)
+        S, _ = _pass1(lib, np.diag(d), kind)
+        rt = np.sqrt(d.astype(dt)).astype(np.longdouble)
+        exact = 1 / rt
+        unit = np.exp2(np.floor(np.log2(exact.astype(np.float64)))) * ulp
+        assert np.all(np.abs(np.diag(S) - exact) <= 0.51 * unit)
