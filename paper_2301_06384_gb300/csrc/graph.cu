@@ -246,6 +246,10 @@ extern "C" int kb_graph_create(int64_t n, const int32_t *rowptr, const int32_t *
             h_rdiag[i] = float(excess);
             if (h_rdiag[i] != 0.f) zero_excess = false;
         }
+        const int32_t long_row = long_row_degree(h_rowptr.data(), n);
+        std::vector<int32_t> h_longs;
+        for (int64_t i = 0; i < n; ++i)
+            if (h_rowptr[i + 1] - h_rowptr[i] > long_row) h_longs.push_back(int32_t(i));
         int dev = 0;
         KB_CUDA_TRY(cudaGetDevice(&dev));
         cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -254,16 +258,19 @@ extern "C" int kb_graph_create(int64_t n, const int32_t *rowptr, const int32_t *
         g->device = dev;
         auto cleanup = [&]() {
             cudaFree(g->d_rowptr); cudaFree(g->d_col); cudaFree(g->d_w); cudaFree(g->d_rdiag);
+            cudaFree(g->d_longs);
             delete g;
         };
         cudaError_t e = cudaMalloc(&g->d_rowptr, sizeof(int32_t) * (n + 1));
         if (e == cudaSuccess) e = cudaMalloc(&g->d_col, sizeof(int32_t) * std::max<int64_t>(noff, 1));
         if (e == cudaSuccess && !unit) e = cudaMalloc(&g->d_w, sizeof(float) * std::max<int64_t>(noff, 1));
         if (e == cudaSuccess && !zero_excess) e = cudaMalloc(&g->d_rdiag, sizeof(float) * n);
+        if (e == cudaSuccess && !h_longs.empty()) e = cudaMalloc(&g->d_longs, sizeof(int32_t) * h_longs.size());
         if (e == cudaSuccess) e = cudaMemcpyAsync(g->d_rowptr, h_rowptr.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess && noff) e = cudaMemcpyAsync(g->d_col, h_col.data(), sizeof(int32_t) * noff, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess && !unit && noff) e = cudaMemcpyAsync(g->d_w, h_w.data(), sizeof(float) * noff, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess && !zero_excess) e = cudaMemcpyAsync(g->d_rdiag, h_rdiag.data(), sizeof(float) * n, cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess && !h_longs.empty()) e = cudaMemcpyAsync(g->d_longs, h_longs.data(), sizeof(int32_t) * h_longs.size(), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) {
             cleanup();
@@ -271,6 +278,9 @@ extern "C" int kb_graph_create(int64_t n, const int32_t *rowptr, const int32_t *
         }
         g->dev.n = n;
         g->dev.nnz = noff;
+        g->dev.longs = g->d_longs;
+        g->dev.nlong = int32_t(h_longs.size());
+        g->dev.long_row = long_row;
         g->dev.rowptr = g->d_rowptr;
         g->dev.col = g->d_col;
         g->dev.w = g->d_w;
@@ -318,6 +328,7 @@ extern "C" void kb_graph_destroy(kb_graph *g) {
     cudaFree(g->d_col);
     cudaFree(g->d_w);
     cudaFree(g->d_rdiag);
+    cudaFree(g->d_longs);
     delete g;
 }
 

@@ -26,6 +26,9 @@ namespace kb {
 struct GraphDev {
     int64_t n = 0;
     int64_t nnz = 0;                  // stored off-diagonal entries
+    const int32_t *longs = nullptr;   // rows of more than long_row entries (spmm.cu), by index
+    int32_t nlong = 0;
+    int32_t long_row = 0;
     const int32_t *rowptr = nullptr;  // n+1
     const int32_t *col = nullptr;     // nnz
     const float *w = nullptr;         // nnz or nullptr (unit weights)
@@ -40,6 +43,7 @@ struct kb_graph {
     int32_t *d_col = nullptr;
     float *d_w = nullptr;
     float *d_rdiag = nullptr;
+    int32_t *d_longs = nullptr;
     double lambda = 0.0;     // Gershgorin bound
     double lambda_proj = 0.0;// spectral bound for the Lanczos projected step: the Gershgorin
                              // bound, or for a unit-weight D - A the smaller edge bound
@@ -254,12 +258,15 @@ struct LinEpi {
     int zero_inactive = 0;            // write zeros on the tiles beyond the limit (final output)
     const int32_t *alist = nullptr;   // with tgen: the tiles by rising hop distance and the number
     const int32_t *acount = nullptr;  // of them within the limit (device)
+    int one_group = 0;                // long rows too are summed by one lane group, in index order
     ProfCount prof;
 };
 
 // ldo <= 0: output is an internal n x W block; otherwise out has leading dimension ldo
 // and only columns < mo are written.  n_dense_in counts the dense inputs besides x
 // (y, z) for the algorithmic byte count.
+// Rows of more entries than this are the graph's long rows (rowptr on the host).
+int32_t long_row_degree(const int32_t *rowptr, int64_t n);
 template <typename T>
 int launch_spmm(const GraphDev &g, int W, const T *x, const LinEpi<T> &e, cudaStream_t s,
                 int *grid_out, int64_t M_alg, int n_dense_in, int64_t ldo = 0, int mo = 0);

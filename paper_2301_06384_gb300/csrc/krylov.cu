@@ -495,6 +495,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             LinEpi<T> e;
             e.s1 = 1.0;
             e.out = b.wbuf;
+            e.one_group = c.ordered;
             e.ctrl = b.ctrl;
             e.tgen = tg;
             e.gen = tg ? b.fr.gen : nullptr;

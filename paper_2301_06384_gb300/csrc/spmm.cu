@@ -15,6 +15,14 @@
 // in shared memory (three barriers per tile) and 32-row units that left half of the warps idle
 // at W = 32: RGG of 2e4 rows, M = 37, 30 products 447 -> 345 us.
 //
+// Long rows (hubs).  A lane group's row is a serial chain of one gather latency per U neighbours,
+// and its warp waits for it.  Rows above long_row_degree are therefore listed at graph creation and
+// taken first, a CTA each: its 256 / LPR lane groups share the row's neighbours, and the partial
+// sums meet by shuffles and in shared memory in a fixed order.  Preferential attachment (5 edges a
+// node, 4e5 rows, rows up to some 3000 long), 10 products, ms: M = 16 7.1 -> 1.0, M = 64 12.7 -> 2.5,
+// with column dots 10.9 -> 4.3; the tiles with staged indices took 6.4, 9.0 and 12.0.  A star of
+// 3e4 rows, M = 16: 40 -> 0.5.  A warp per long row was slower (M = 64 7.9, with dots 11.4).
+//
 // The Laplacian is applied in difference form (L x)_i = sum_j w_ij (x_i - x_j) + r_i x_i,
 // which gives L 1 = 0 exactly for D - A and drops the diagonal load for standard
 // Laplacians.  Epilogue coefficients arrive in FP64; in the FP32 path each is split into
@@ -135,8 +143,9 @@ struct SpmmOcc {
     static constexpr int value = sizeof(typename Cmp<T>::type) == 8 ? 3 : (DOT ? 3 : 4);
 };
 
-// WGT: the graph stores edge weights (false: unit weights, w_ij = 1).
-template <typename T, int W, bool DOT, bool WGT>
+// WGT: the graph stores edge weights (false: unit weights, w_ij = 1).  LONG: the graph has long
+// rows (a variant of its own: graphs without them keep the registers of the loop over units).
+template <typename T, int W, bool DOT, bool WGT, bool LONG>
 __global__ void __launch_bounds__(SPMM_THREADS, (SpmmOcc<T, DOT>::value))
 k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo, int mcols) {
     using G = SpmmGeo<W>;
@@ -149,6 +158,7 @@ k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo, in
     __shared__ __align__(16) C s_coef[5][W];       // c1 hi, c1 lo, c0, c2 hi, c2 lo
     __shared__ C s_sc[2];                          // s3, wE in the arithmetic type
     __shared__ double s_dot[DOT ? WARPS : 1][W];
+    __shared__ C s_part[LONG ? WARPS : 1][LONG ? W : 1];   // sums of a long row, by warp
     if (threadIdx.x == 0) {
         s_sc[0] = C(e.s3);
         s_sc[1] = C(e.wE);
@@ -211,99 +221,169 @@ k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo, in
         on = w / UPT < active && (!e.tgen || int(__ldg(e.gen + r)) <= e.limit);
         b = __ldg(g.rowptr + r);
         en = __ldg(g.rowptr + r + 1);
+        if (LONG && on && en - b > g.long_row) {
+            r = -1;   // (done by a CTA)
+            on = false;
+        }
     };
     const int64_t w0 = int64_t(blockIdx.x) * WARPS + warp;
     fetch(w0, row, beg, end, act);
-    for (int64_t w = w0; w < nunits; w += step) {
+    int64_t lnext = blockIdx.x;   // (of the long rows; uniform in the CTA)
+    for (int64_t w = w0; w < nunits || (LONG && lnext < g.nlong); w += step) {
         int64_t nrow;
         int nbeg, nend;
         bool nact;
-        fetch(w + step, nrow, nbeg, nend, nact);
-        const int deg = act ? end - beg : 0;
-        if (sub == 0 && act) {
-            ++my_rows;
-            my_nnz += unsigned(deg);
-        }
         V4<T> xi[VPL];
         C acc[VPL][4];
+        if (LONG && lnext < g.nlong) {
+            // a long row, by all lane groups of the CTA: each takes U neighbours in turn; the unit waits
+            nrow = row;
+            nbeg = beg;
+            nend = end;
+            nact = act;
+            w -= step;
+            row = __ldg(g.longs + lnext);
+            lnext += gridDim.x;
+            act = !e.tgen || int(__ldg(e.gen + row)) <= e.limit;   // (else its unit writes the zeros)
+            const int lbeg = __ldg(g.rowptr + row), deg = act ? __ldg(g.rowptr + row + 1) - lbeg : 0;
 #pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-            xi[v] = act && cin[v] ? V4<T>::load(x + row * W + KB_COL(v)) : V4<T>{};
+            for (int v = 0; v < VPL; ++v) {
+                xi[v] = act && cin[v] ? V4<T>::load(x + row * W + KB_COL(v)) : V4<T>{};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) acc[v][q] = C(0);
-        }
-        // neighbours: the lanes of a group load the indices (and weights) of a chunk of 8 or
-        // LPR; the group then takes them in order by shuffles.  The loop runs to the longest row of the
-        // warp; slots past a row's end contribute x_i - x_i, an exact zero.
-        const int maxdeg = __reduce_max_sync(0xffffffffu, deg);
-        for (int p0 = 0; p0 < maxdeg; p0 += CHUNK) {
-            int mj[CPL];
-            float mw[CPL];
+                for (int q = 0; q < 4; ++q) acc[v][q] = C(0);
+            }
+            for (int p0 = (warp * RPW + grp) * U; p0 < deg; p0 += WARPS * RPW * U) {
+                V4<T> xj[U][VPL];
+                C wv[U];
 #pragma unroll
-            for (int q = 0; q < CPL; ++q) {
-                const int p = p0 + q * LPR + sub;
-                mj[q] = p < deg ? __ldg(g.col + beg + p) : 0;
-                if (WGT) mw[q] = p < deg ? __ldg(g.w + beg + p) : 0.f;
+                for (int u = 0; u < U; ++u) {
+                    const bool in = p0 + u < deg;
+                    const int j = in ? __ldg(g.col + lbeg + p0 + u) : 0;
+                    wv[u] = WGT && in ? C(__ldg(g.w + lbeg + p0 + u)) : C(1);
+#pragma unroll
+                    for (int v = 0; v < VPL; ++v)
+                        xj[u][v] = in && cin[v] ? V4<T>::load(x + int64_t(j) * W + KB_COL(v)) : xi[v];
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int v = 0; v < VPL; ++v)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const C d = xi[v].v[q] - xj[u][v].v[q];
+                            acc[v][q] = WGT ? fma(wv[u], d, acc[v][q]) : acc[v][q] + d;
+                        }
+            }
+            __syncthreads();   // (the sums of the row before are read)
+#pragma unroll
+            for (int v = 0; v < VPL; ++v)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+#pragma unroll
+                    for (int off = LPR; off < 32; off <<= 1) acc[v][q] += __shfl_xor_sync(0xffffffffu, acc[v][q], off);
+                    if (grp == 0) s_part[warp][KB_COL(v) + q] = acc[v][q];
+                }
+            __syncthreads();
+            // the first group finishes the row
+            if (warp != 0 || grp != 0 || !act) {
+                row = -1;
+            } else {
+#pragma unroll
+                for (int v = 0; v < VPL; ++v)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        for (int w2 = 1; w2 < WARPS; ++w2) acc[v][q] += s_part[w2][KB_COL(v) + q];
+                if (sub == 0) {
+                    ++my_rows;
+                    my_nnz += unsigned(deg);
+                }
+            }
+        } else {
+            fetch(w + step, nrow, nbeg, nend, nact);
+            const int deg = act ? end - beg : 0;
+            if (sub == 0 && act) {
+                ++my_rows;
+                my_nnz += unsigned(deg);
             }
 #pragma unroll
-            for (int u0 = 0; u0 < CHUNK; u0 += U) {
-                if (p0 + u0 >= maxdeg) break;
-                if constexpr (std::is_same<T, float>::value) {
-                    f2 xj[U][VPL][2], xi2[VPL][2];
-                    f2 wv[U];
+            for (int v = 0; v < VPL; ++v) {
+                xi[v] = act && cin[v] ? V4<T>::load(x + row * W + KB_COL(v)) : V4<T>{};
 #pragma unroll
-                    for (int v = 0; v < VPL; ++v) {
-                        xi2[v][0] = f2_pack(xi[v].v[0], xi[v].v[1]);
-                        xi2[v][1] = f2_pack(xi[v].v[2], xi[v].v[3]);
-                    }
+                for (int q = 0; q < 4; ++q) acc[v][q] = C(0);
+            }
+            // neighbours: the lanes of a group load the indices (and weights) of a chunk of 8 or
+            // LPR; the group then takes them in order by shuffles.  The loop runs to the longest row of the
+            // warp; slots past a row's end contribute x_i - x_i, an exact zero.
+            const int maxdeg = __reduce_max_sync(0xffffffffu, deg);
+            for (int p0 = 0; p0 < maxdeg; p0 += CHUNK) {
+                int mj[CPL];
+                float mw[CPL];
 #pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int j = __shfl_sync(0xffffffffu, mj[(u0 + u) / LPR], (u0 + u) % LPR, LPR);
-                        if (WGT) {
-                            const float wj = __shfl_sync(0xffffffffu, mw[(u0 + u) / LPR], (u0 + u) % LPR, LPR);
-                            wv[u] = f2_pack(wj, wj);
-                        }
-                        const bool in = p0 + u0 + u < deg;
-                        const float *xr = reinterpret_cast<const float *>(x) + int64_t(j) * W;
+                for (int q = 0; q < CPL; ++q) {
+                    const int p = p0 + q * LPR + sub;
+                    mj[q] = p < deg ? __ldg(g.col + beg + p) : 0;
+                    if (WGT) mw[q] = p < deg ? __ldg(g.w + beg + p) : 0.f;
+                }
+#pragma unroll
+                for (int u0 = 0; u0 < CHUNK; u0 += U) {
+                    if (p0 + u0 >= maxdeg) break;
+                    if constexpr (std::is_same<T, float>::value) {
+                        f2 xj[U][VPL][2], xi2[VPL][2];
+                        f2 wv[U];
 #pragma unroll
                         for (int v = 0; v < VPL; ++v) {
-                            xj[u][v][0] = xi2[v][0];
-                            xj[u][v][1] = xi2[v][1];
-                            if (in && cin[v]) ldg_f2x2(xr + KB_COL(v), xj[u][v][0], xj[u][v][1]);
+                            xi2[v][0] = f2_pack(xi[v].v[0], xi[v].v[1]);
+                            xi2[v][1] = f2_pack(xi[v].v[2], xi[v].v[3]);
                         }
-                    }
-#pragma unroll
-                    for (int v = 0; v < VPL; ++v) {
-                        f2 a0 = f2_pack(acc[v][0], acc[v][1]), a1 = f2_pack(acc[v][2], acc[v][3]);
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
-                            const f2 d0 = f2_sub(xi2[v][0], xj[u][v][0]), d1 = f2_sub(xi2[v][1], xj[u][v][1]);
-                            a0 = WGT ? f2_fma(wv[u], d0, a0) : f2_add(a0, d0);
-                            a1 = WGT ? f2_fma(wv[u], d1, a1) : f2_add(a1, d1);
+                            const int j = __shfl_sync(0xffffffffu, mj[(u0 + u) / LPR], (u0 + u) % LPR, LPR);
+                            if (WGT) {
+                                const float wj = __shfl_sync(0xffffffffu, mw[(u0 + u) / LPR], (u0 + u) % LPR, LPR);
+                                wv[u] = f2_pack(wj, wj);
+                            }
+                            const bool in = p0 + u0 + u < deg;
+                            const float *xr = reinterpret_cast<const float *>(x) + int64_t(j) * W;
+#pragma unroll
+                            for (int v = 0; v < VPL; ++v) {
+                                xj[u][v][0] = xi2[v][0];
+                                xj[u][v][1] = xi2[v][1];
+                                if (in && cin[v]) ldg_f2x2(xr + KB_COL(v), xj[u][v][0], xj[u][v][1]);
+                            }
                         }
-                        f2_unpack(a0, acc[v][0], acc[v][1]);
-                        f2_unpack(a1, acc[v][2], acc[v][3]);
+#pragma unroll
+                        for (int v = 0; v < VPL; ++v) {
+                            f2 a0 = f2_pack(acc[v][0], acc[v][1]), a1 = f2_pack(acc[v][2], acc[v][3]);
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                const f2 d0 = f2_sub(xi2[v][0], xj[u][v][0]), d1 = f2_sub(xi2[v][1], xj[u][v][1]);
+                                a0 = WGT ? f2_fma(wv[u], d0, a0) : f2_add(a0, d0);
+                                a1 = WGT ? f2_fma(wv[u], d1, a1) : f2_add(a1, d1);
+                            }
+                            f2_unpack(a0, acc[v][0], acc[v][1]);
+                            f2_unpack(a1, acc[v][2], acc[v][3]);
+                        }
+                    } else {
+                        V4<T> xj[U][VPL];
+                        C wv[U];
+#pragma unroll
+                        for (int u = 0; u < U; ++u) {
+                            const int j = __shfl_sync(0xffffffffu, mj[(u0 + u) / LPR], (u0 + u) % LPR, LPR);
+                            wv[u] = WGT ? C(__shfl_sync(0xffffffffu, mw[(u0 + u) / LPR], (u0 + u) % LPR, LPR)) : C(1);
+                            const bool in = p0 + u0 + u < deg;
+#pragma unroll
+                            for (int v = 0; v < VPL; ++v)
+                                xj[u][v] = in && cin[v] ? V4<T>::load(x + int64_t(j) * W + KB_COL(v)) : xi[v];
+                        }
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+#pragma unroll
+                            for (int v = 0; v < VPL; ++v)
+#pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    acc[v][q] = WGT ? fma(wv[u], xi[v].v[q] - xj[u][v].v[q], acc[v][q])
+                                                    : acc[v][q] + (xi[v].v[q] - xj[u][v].v[q]);
                     }
-                } else {
-                    V4<T> xj[U][VPL];
-                    C wv[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int j = __shfl_sync(0xffffffffu, mj[(u0 + u) / LPR], (u0 + u) % LPR, LPR);
-                        wv[u] = WGT ? C(__shfl_sync(0xffffffffu, mw[(u0 + u) / LPR], (u0 + u) % LPR, LPR)) : C(1);
-                        const bool in = p0 + u0 + u < deg;
-#pragma unroll
-                        for (int v = 0; v < VPL; ++v)
-                            xj[u][v] = in && cin[v] ? V4<T>::load(x + int64_t(j) * W + KB_COL(v)) : xi[v];
-                    }
-#pragma unroll
-                    for (int u = 0; u < U; ++u)
-#pragma unroll
-                        for (int v = 0; v < VPL; ++v)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                acc[v][q] = WGT ? fma(wv[u], xi[v].v[q] - xj[u][v].v[q], acc[v][q])
-                                                : acc[v][q] + (xi[v].v[q] - xj[u][v].v[q]);
                 }
             }
         }
@@ -421,39 +501,63 @@ k_spmm(GraphDev g, const T *__restrict__ x, LinEpi<T> e, int64_t ldo, int mo, in
 
 #undef KB_COL
 
-template <typename T, int W, bool DOT>
+template <typename T, int W, bool DOT, bool LONG>
 int occupancy_spmm() {
     // the weighted and unweighted kernels share the launch bounds
     // function-local static: computed once, thread-safe (several serving workers)
     static const int per_sm = [] {
         int v = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_spmm<T, W, DOT, true>, SPMM_THREADS, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_spmm<T, W, DOT, true, LONG>, SPMM_THREADS, 0);
         return v < 1 ? 1 : v;
     }();
     return per_sm;
 }
 
-template <typename T, int W, bool DOT>
+template <typename T, int W, bool DOT, bool LONG>
 int launch_wd(const GraphDev &g, const T *x, const LinEpi<T> &e, int64_t ldo, int mo, int mcols,
               cudaStream_t s, int *grid_out) {
     const int64_t units = (g.n + SpmmGeo<W>::RPW - 1) / SpmmGeo<W>::RPW;
-    int grid = int(std::min<int64_t>((units + WARPS - 1) / WARPS, int64_t(num_sms()) * occupancy_spmm<T, W, DOT>()));
+    int grid = int(std::min<int64_t>((units + WARPS - 1) / WARPS, int64_t(num_sms()) * occupancy_spmm<T, W, DOT, LONG>()));
     if (grid < 1) grid = 1;
     if (grid_out) *grid_out = grid;
     const cudaError_t err =
-        launch_dep(g.w ? k_spmm<T, W, DOT, true> : k_spmm<T, W, DOT, false>, dim3(grid), SPMM_THREADS, 0, s, 0, g, x, e, ldo,
-                   mo, mcols);
+        launch_dep(g.w ? k_spmm<T, W, DOT, true, LONG> : k_spmm<T, W, DOT, false, LONG>, dim3(grid), SPMM_THREADS, 0, s, 0,
+                   g, x, e, ldo, mo, mcols);
     return err == cudaSuccess ? 0 : cuda_fail(err, "k_spmm launch");
 }
 
 template <typename T, int W>
 int launch_w(const GraphDev &g, const T *x, const LinEpi<T> &e, int64_t ldo, int mo, int mcols,
              cudaStream_t s, int *grid_out) {
-    return e.dot_partials ? launch_wd<T, W, true>(g, x, e, ldo, mo, mcols, s, grid_out)
-                          : launch_wd<T, W, false>(g, x, e, ldo, mo, mcols, s, grid_out);
+    if (g.nlong && !e.one_group)
+        return e.dot_partials ? launch_wd<T, W, true, true>(g, x, e, ldo, mo, mcols, s, grid_out)
+                              : launch_wd<T, W, false, true>(g, x, e, ldo, mo, mcols, s, grid_out);
+    return e.dot_partials ? launch_wd<T, W, true, false>(g, x, e, ldo, mo, mcols, s, grid_out)
+                          : launch_wd<T, W, false, false>(g, x, e, ldo, mo, mcols, s, grid_out);
+}
+
+// CTAs per SM of the kernels that write dot partials
+template <typename T, int W>
+int max_occupancy() {
+    return std::max(occupancy_spmm<T, W, true, false>(), occupancy_spmm<T, W, true, true>());
 }
 
 }  // namespace
+
+// The line between the two.  A CTA spends about as long on any long row of less than some 500
+// entries, so they have to be few: at most one row in 64, and longer than four mean rows (with every
+// row of mean degree 100 taken by a CTA, 5e4 rows, M = 24: 1.70 ms for 10 products, 0.63 by units; one
+// row in 20 of 105 entries, 4e5 rows, column dots, M = 24: 2.54 and 2.30).  Between 64 and 256 as the
+// smallest length, preferential attachment of 4e5 rows, M = 64: 2.52 at 64, 2.65 at 128, 3.03 at 256;
+// at 32 2.77.
+int32_t long_row_degree(const int32_t *rowptr, int64_t n) {
+    int64_t t = std::max<int64_t>(64, 4 * int64_t(rowptr[n]) / n);
+    for (;; t *= 2) {
+        int64_t above = 0;
+        for (int64_t i = 0; i < n; ++i) above += rowptr[i + 1] - rowptr[i] > t;
+        if (above <= n / 64 || above <= 1) return int32_t(std::min<int64_t>(t, INT32_MAX));
+    }
+}
 
 template <typename T>
 int launch_spmm(const GraphDev &g, int W, const T *x, const LinEpi<T> &e, cudaStream_t s,
@@ -491,10 +595,10 @@ template <typename T>
 int spmm_max_grid(int W) {
     // dot partials are written only by the DOT variant; its grid bounds the buffer
     switch (W) {
-        case 16: return num_sms() * occupancy_spmm<T, 16, true>();
-        case 32: return num_sms() * occupancy_spmm<T, 32, true>();
-        case 64: return num_sms() * occupancy_spmm<T, 64, true>();
-        default: return num_sms() * occupancy_spmm<T, 128, true>();
+        case 16: return num_sms() * max_occupancy<T, 16>();
+        case 32: return num_sms() * max_occupancy<T, 32>();
+        case 64: return num_sms() * max_occupancy<T, 64>();
+        default: return num_sms() * max_occupancy<T, 128>();
     }
 }
 
