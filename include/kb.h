@@ -192,8 +192,8 @@ int kb_graph_lambda_bounds(const kb_graph *g, double *gershgorin, double *projec
  * Not implemented (KB_ERR_UNSUPPORTED): the Lanczos methods with KB_PHI_SPLINE and s >= 65,
  * or with (eps + Lambda) / eps so large that 240 quadrature nodes do not reach 1e-14;
  * reorth with methods other than KB_CBL; KB_CBL / KB_GBL with M > 128 (M > 64 for KB_F64).
- * Other errors: KB_ERR_ARG, KB_ERR_NODES, KB_ERR_NOMEM, KB_ERR_CUDA (also when an opt-in
- * tensor-core kernel gives up waiting for its MMA completion).
+ * Other errors: KB_ERR_ARG, KB_ERR_NODES, KB_ERR_NOMEM, KB_ERR_CUDA (also when the projected
+ * step's grid barrier, or an opt-in tensor-core kernel's wait for its MMA completion, gives up).
  *
  * Environment: KB_TENSOR_CORES=1 (read at the start of a solve) runs the tall-skinny products of
  * KB_CBL with FP32 blocks of width 64 (M in 33..64) on the tcgen05 tensor cores (BF16 x 6

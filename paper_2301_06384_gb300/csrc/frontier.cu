@@ -27,7 +27,7 @@ constexpr int BFS_U = 4;       // edges per lane in flight
 // level.
 __global__ void __launch_bounds__(BFS_THREADS)
 k_bfs(GraphDev g, NodeChunk seeds, int levels, uint8_t *gen, int32_t *tgen, uint32_t *vis, int32_t *queue,
-      int32_t *qlev, int32_t *tcnt, int32_t *bar, int32_t *err) {
+      int32_t *qlev, int32_t *tcnt, int32_t *bar, int32_t *err, int spins) {
     const int lane = threadIdx.x & 31;
     const int gw = (int(blockIdx.x) * BFS_THREADS + int(threadIdx.x)) >> 5;
     const int nw = int(gridDim.x) * (BFS_THREADS / 32);
@@ -42,7 +42,7 @@ k_bfs(GraphDev g, NodeChunk seeds, int levels, uint8_t *gen, int32_t *tgen, uint
             atomicAdd(tcnt, 1);
         }
     }
-    if (!grid_barrier(bar, err, target += gridDim.x)) return;
+    if (!grid_barrier(bar, err, target += gridDim.x, spins)) return;
     int start = 0, end = seeds.cnt;
     for (int k = 1; k <= levels && start < end; ++k) {
         for (int64_t base = start + int64_t(gw) * BFS_ROWS; base < end; base += int64_t(nw) * BFS_ROWS) {
@@ -109,7 +109,7 @@ k_bfs(GraphDev g, NodeChunk seeds, int levels, uint8_t *gen, int32_t *tgen, uint
                 }
             }
         }
-        if (!grid_barrier(bar, err, target += gridDim.x)) return;
+        if (!grid_barrier(bar, err, target += gridDim.x, spins)) return;
         start = end;
         end += __ldcg(qlev + k);
     }
@@ -283,7 +283,7 @@ void plan_frontier(FrontierBufs &f, int64_t n, int levels, unsigned char *base, 
     *bytes = off;
 }
 
-int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, cudaStream_t s) {
+int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, cudaStream_t s, int spins) {
     const int levels = f.levels;
     const int64_t nt = (g.n + ACT_ROWS - 1) / ACT_ROWS;
     NodeChunk ch;
@@ -307,7 +307,7 @@ int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, in
     cfg.attrs = at;
     cfg.numAttrs = 1;
     KB_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_bfs, g, ch, levels, f.gen, f.tgen, f.vis, f.queue, f.qlev, f.tcnt,
-                                   f.sync, f.sync + 1));
+                                   f.sync, f.sync + 1, spins));
     k_tile_sort<<<dim3(levels + 2, 2), 1024, 0, s>>>(f.tgen, f.gen, g.n, nt, levels, f.tcnt, f.sync + 1, f.acount,
                                                      f.alist, f.lists);
     KB_CUDA_TRY(cudaGetLastError());

@@ -26,13 +26,13 @@ namespace kb {
 struct GraphDev {
     int64_t n = 0;
     int64_t nnz = 0;                  // stored off-diagonal entries
-    const int32_t *longs = nullptr;   // rows of more than long_row entries (spmm.cu), by index
-    int32_t nlong = 0;
-    int32_t long_row = 0;
     const int32_t *rowptr = nullptr;  // n+1
     const int32_t *col = nullptr;     // nnz
     const float *w = nullptr;         // nnz or nullptr (unit weights)
     const float *rdiag = nullptr;     // n or nullptr (zero diagonal excess)
+    const int32_t *longs = nullptr;   // rows of more than long_row entries (spmm.cu), by index
+    int32_t nlong = 0;
+    int32_t long_row = 0;
 };
 
 }  // namespace kb
@@ -69,7 +69,7 @@ int cuda_fail(cudaError_t e, const char *what);
 // ------------------------------------------------------------------ device control block
 // One per solve, in device memory.  Kernels after a stop or a breakdown return early.
 struct Ctrl {
-    int32_t status;          // KB_OK / KB_ERR_BREAKDOWN
+    int32_t status;          // KB_OK, or why the result is unusable (KB_ERR_BREAKDOWN, ...)
     int32_t stop;            // 1 once the process stopped (invariant space or breakdown)
     int32_t steps;           // blocks entering the result
     int32_t breakdown_step;  // -1 or step index
@@ -173,18 +173,18 @@ __device__ __forceinline__ double df_value(const DF &a) { return double(a.hi) + 
 
 // ------------------------------------------------------------------ grid barrier
 // Barrier of all CTAs of a cooperative launch (co-resident by construction): the arrivals are
-// counted in *bar, target the count that releases this barrier.  The wait is bounded: false, with
-// *err set, when it runs out; every CTA then leaves by itself and the caller's results have to
-// be marked unusable.
+// counted in *bar, target the count that releases this barrier.  The wait is bounded by `spins`
+// polls: false, with *err set, when it runs out; every CTA then leaves by itself and the caller's
+// results have to be marked unusable.
 constexpr int GRID_BARRIER_SPINS = 1 << 22;
-__device__ __forceinline__ bool grid_barrier(int32_t *bar, int32_t *err, int target) {
+__device__ __forceinline__ bool grid_barrier(int32_t *bar, int32_t *err, int target, int spins) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
         atomicAdd(bar, 1);
         int good = 0;
-        for (int i = 0; i < GRID_BARRIER_SPINS; ++i) {
+        for (int i = 0; i < spins; ++i) {
             int v;
             asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
             if (v >= target) {

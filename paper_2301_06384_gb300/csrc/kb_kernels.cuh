@@ -134,8 +134,10 @@ struct FrontierBufs {
 // Lays the arrays out from base (nullptr: sizes only) for a search of `levels` hops; *bytes
 // receives their size.
 void plan_frontier(FrontierBufs &f, int64_t n, int levels, unsigned char *base, size_t *bytes);
-// Hop distances up to f.levels from the nodes, and the tile lists.
-int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, cudaStream_t s);
+// Hop distances up to f.levels from the nodes, and the tile lists; every row at distance 0 when a
+// barrier of the search runs out of its polls.
+int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, cudaStream_t s,
+                    int spins = GRID_BARRIER_SPINS);
 // Zeros on the tiles within f.levels hops: see k_zero_tiles.
 int launch_zero_tiles(void *blocks, int64_t block_bytes, int nblk, int row_bytes, int64_t n, bool ring,
                       const FrontierBufs &f, cudaStream_t s);
@@ -146,10 +148,12 @@ int launch_u_convert(const double *U, int M, int W, int m, T *Ut, const Ctrl *ct
 // Hdf: nullptr for the FP64 recurrence; else 2 m M (M + 1) doubles of scratch for H as floats, and
 // the recurrence runs in double-float on the FP32 pipe (the FP32 and BF16 modes), with sync (two
 // words of scratch) in one cooperative launch.  kmax: a host-side bound on ctrl->steps (0: m).
+// proc: control block of the process, stopped with KB_ERR_CUDA when a barrier of that launch runs
+// out of its polls.
 int launch_cheb_bt(const double *Hd, const double *Hs, int M, int m, double lam,
                    const std::vector<double> &d, double *V0, double *V1, double *V2, double *U,
                    const Ctrl *ctrl, cudaStream_t s, double *Hdf = nullptr, int32_t *sync = nullptr,
-                   int kmax = 0);
+                   int kmax = 0, Ctrl *proc = nullptr, int spins = GRID_BARRIER_SPINS);
 // U = (eps I + H_m)^{-s} F_1.  Integer s: s_int block Cholesky solves (q == nullptr or
 // q->n == 0).  Non-integer s: the quadrature rule q gives the fractional factor
 // sum_k W_k (sigma_k I + H_m)^{-1} F_1, one block Cholesky factorisation and solve per node

@@ -609,7 +609,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
                 KB_TRY(launch_ctrl_snapshot(b.ctrl_chk, b.ctrl, k, c.s));
                 if (c.phi == KB_PHI_EXP) {
                     const std::vector<double> d = exp_series_coeffs(c.p.t, lam_p, 1e-17);
-                    KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, Ucur, b.ctrl_chk, c.s, f64 ? nullptr : b.Hdf, b.csync, k));
+                    KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, Ucur, b.ctrl_chk, c.s, f64 ? nullptr : b.Hdf, b.csync, k, b.ctrl));
                 } else {
                     KB_TRY(side.join());
                     KB_TRY(launch_bt_spline(b.Hd, b.Hs, M, m, c.p.eps, c.s_int, sbufs, Ucur, b.ctrl, b.ctrl_chk,
@@ -636,7 +636,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
         if (formed) {
         } else if (c.phi == KB_PHI_EXP) {
             const std::vector<double> d = exp_series_coeffs(c.p.t, lam_p, 1e-17);
-            KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, b.U, cfin, c.s, f64 ? nullptr : b.Hdf, b.csync, kend));
+            KB_TRY(launch_cheb_bt(b.Hd, b.Hs, M, m, lam_p, d, b.V0, b.V1, b.V2, b.U, cfin, c.s, f64 ? nullptr : b.Hdf, b.csync, kend, b.ctrl));
         } else {
             // (a process that stopped by itself skipped the later checks: their Y are formed now)
             KB_TRY(side.join());
@@ -1161,7 +1161,7 @@ int apply_device(kb_graph *g, kb_method method, kb_phi phi, const kb_params *par
         return fail(info->status, "the projected matrix left the spectral interval [0, Lambda] "
                                   "(loss of orthogonality of the Lanczos basis); use reorth");
     if (info->status == KB_ERR_CUDA)
-        return fail(info->status, "a tensor-core kernel gave up waiting for its MMA completion");
+        return fail(info->status, "a kernel gave up waiting (grid barrier, or completion of a tensor-core product)");
     if (info->status != KB_OK) return fail(info->status, "Lanczos breakdown: rank-deficient block");
     return KB_OK;
 }

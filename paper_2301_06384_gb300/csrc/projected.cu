@@ -259,7 +259,7 @@ template <int NI>
 __global__ void __launch_bounds__(256)
 k_cheb_bt_all(const float *__restrict__ Hd, const float *__restrict__ Hs, const float *__restrict__ Hst, dfl *V0,
               dfl *V1, dfl *V2, double *__restrict__ U, int M, int ld, ChebCoef cc, int j0, dfl g,
-              const Ctrl *ctrl, int32_t *sync) {
+              const Ctrl *ctrl, int32_t *sync, Ctrl *proc, int spins) {
     const int steps = ctrl->steps;
     if (steps <= 0) return;
     extern __shared__ __align__(16) unsigned char svraw[];   // V [3][M][CBW] pairs, H [3][M][ld]
@@ -296,7 +296,7 @@ k_cheb_bt_all(const float *__restrict__ Hd, const float *__restrict__ Hs, const 
     }
     int target = 0;
     bool good = true;
-    if (j0 == 0) good = grid_barrier(sync, sync + 1, target += gridDim.x);
+    if (j0 == 0) good = grid_barrier(sync, sync + 1, target += gridDim.x, spins);
     auto copy8 = [](void *dst, const void *src) {
         const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
@@ -371,7 +371,13 @@ k_cheb_bt_all(const float *__restrict__ Hd, const float *__restrict__ Hs, const 
             }
             __syncthreads();
         }
-        if (q + 1 < cc.n) good = grid_barrier(sync, sync + 1, target += gridDim.x);
+        if (q + 1 < cc.n) good = grid_barrier(sync, sync + 1, target += gridDim.x, spins);
+    }
+    // a barrier ran out: U is not to be used, and the process ends
+    if (!good && proc && threadIdx.x == 0) {
+        proc->status = KB_ERR_CUDA;
+        proc->steps = steps;
+        proc->stop = 1;
     }
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
 #pragma unroll
@@ -708,7 +714,8 @@ k_quad_accumulate(const double *__restrict__ scratch, int M, int mcap, int nb, Q
 
 int launch_cheb_bt(const double *Hd, const double *Hs, int M, int m, double lam,
                    const std::vector<double> &d, double *V0, double *V1, double *V2, double *U,
-                   const Ctrl *ctrl, cudaStream_t s, double *Hdf, int32_t *sync, int kmax) {
+                   const Ctrl *ctrl, cudaStream_t s, double *Hdf, int32_t *sync, int kmax, Ctrl *proc,
+                   int spins) {
     if (kmax <= 0 || kmax > m) kmax = m;
     const size_t bytes = sizeof(double) * size_t(m) * M * M;
     prof_begin(KernelClass::PROJECTED, s);
@@ -756,7 +763,7 @@ int launch_cheb_bt(const double *Hd, const double *Hs, int M, int m, double lam,
                 cfg.numAttrs = 1;
                 auto kern = ni == 1 ? k_cheb_bt_all<1> : ni == 2 ? k_cheb_bt_all<2> : k_cheb_bt_all<4>;
                 KB_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, (const float *)hd, (const float *)hs, (const float *)ht, v[0],
-                                               v[1], v[2], U, M, ld, cc, int(j0), g, ctrl, sync));
+                                               v[1], v[2], U, M, ld, cc, int(j0), g, ctrl, sync, proc, spins));
                 ++launches;
             }
             KB_CUDA_TRY(cudaGetLastError());
