@@ -704,7 +704,8 @@ __global__ void __launch_bounds__(1024) k_conv_check(const double *U, const doub
         double D = 0.0, N = 0.0;
         for (int w = 0; w < int(blockDim.x >> 5); ++w) { D += sd[w]; N += sn[w]; }
         if (ps > 0) {
-            const double change = N > 0.0 ? sqrt(D) / sqrt(N) : 0.0;
+            // (a U with NaN or infinite entries has not converged: no change <= tol holds then)
+            const double change = N == 0.0 ? 0.0 : isfinite(N) ? sqrt(D) / sqrt(N) : N - N;
             ctrl->est_change = change;
             if (change <= tol) {
                 ctrl->stop = 1;

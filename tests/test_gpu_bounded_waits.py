@@ -1,5 +1,6 @@
 """Grid barriers that run out of their polls (none allowed: every CTA gives up at the first one),
-through the library's own launchers: the projected series ends the process with KB_ERR_CUDA."""
+through the library's own launchers: the projected series ends the process with KB_ERR_CUDA.  And the stopping
+rule on a solution that is not finite."""
 import ctypes
 
 import numpy as np
@@ -84,3 +85,30 @@ def test_projected_series_gives_up(lib, M, m):
         else:
             assert (p.status, p.stop, p.steps) == (KB_ERR_CUDA, 1, m)
             assert np.isnan(u).all()
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_check_of_unusable_u_does_not_converge(lib, bad):
+    """The stopping rule on a U that holds a NaN or an infinity: the process goes on (the test of the
+    projected solution reports it), and the change is not a number."""
+    import torch
+    f = lib["_ZN2kb17launch_conv_checkEPKdS1_iPKNS_4CtrlEPidPS2_P11CUstream_sti"]
+    f.restype, f.argtypes = I32, [VP, VP, I32, VP, VP, DBL, VP, VP, I32]
+    M, steps, before = 5, 4, 3
+    rng = np.random.default_rng(1)
+    for value in (None, bad):
+        Up = torch.from_numpy(rng.standard_normal(before * M * M)).cuda()
+        U = torch.cat([Up, torch.zeros((steps - before) * M * M, dtype=torch.float64, device="cuda")])
+        if value is not None:
+            U[7] = value
+        prev = torch.tensor([before], dtype=torch.int32, device="cuda")
+        chk, ctrl = Ctrl.on_device(steps), Ctrl.on_device(20)
+        torch.cuda.synchronize()
+        assert f(U.data_ptr(), Up.data_ptr(), M, chk.data_ptr(), prev.data_ptr(), 1e-6, ctrl.data_ptr(), None, 1) == 0
+        torch.cuda.synchronize()
+        c = Ctrl.read(ctrl)
+        if value is None:
+            assert (c.stop, c.steps, c.from_check, c.est_change) == (1, steps, 1, 0.0)
+        else:
+            assert (c.stop, c.steps, c.from_check) == (0, 20, -1) and np.isnan(c.est_change)
+        assert int(prev) == steps
