@@ -1,7 +1,9 @@
 """Grid barriers that run out of their polls (none allowed: every CTA gives up at the first one),
-through the library's own launchers: the projected series ends the process with KB_ERR_CUDA.  And the stopping
+through the library's own launchers: the projected series ends the process with KB_ERR_CUDA, the search
+reaches every row.  And the stopping
 rule on a solution that is not finite."""
 import ctypes
+import subprocess
 
 import numpy as np
 import pytest
@@ -112,3 +114,90 @@ def test_check_of_unusable_u_does_not_converge(lib, bad):
         else:
             assert (c.stop, c.steps, c.from_check) == (0, 20, -1) and np.isnan(c.est_change)
         assert int(prev) == steps
+
+
+class GraphDev(ctypes.Structure):
+    _fields_ = [("n", ctypes.c_int64), ("nnz", ctypes.c_int64), ("rowptr", VP), ("col", VP), ("w", VP), ("rdiag", VP),
+                ("longs", VP), ("nlong", I32), ("long_row", I32)]
+
+
+class FrontierBufs(ctypes.Structure):
+    _fields_ = [(f, VP) for f in ("gen", "tgen", "alist", "acount", "lists", "zeroed")] + [("zero_bytes", ctypes.c_size_t)] + \
+               [(f, VP) for f in ("qlev", "tcnt", "queue", "sync", "vis")] + [("levels", I32), ("nt", ctypes.c_int64)]
+
+
+@pytest.fixture(scope="module")
+def layouts(tmp_path_factory):
+    """The two structures' layouts by the compiler, before anything is launched with the ones above."""
+    from paper_2301_06384_gb300 import build
+    d = tmp_path_factory.mktemp("layout")
+    lines = []
+    for cls in (GraphDev, FrontierBufs):
+        name = cls.__name__
+        lines.append(f'printf("{name} %zu\\n", sizeof(kb::{name}));')
+        lines += [f'printf("{name}.{f[0]} %zu\\n", offsetof(kb::{name}, {f[0]}));' for f in cls._fields_]
+    (d / "layout.cu").write_text("#include <cstddef>\n#include <cstdio>\n#include \"kb_internal.cuh\"\n#include "
+                                 "\"kb_kernels.cuh\"\nint main() {\n" + "\n".join(lines) + "\n}\n")
+    subprocess.run([build.nvcc(), *build._flags(), "-c", str(d / "layout.cu"), "-o", str(d / "layout.o")], check=True)
+    subprocess.run([build.nvcc(), build.ARCH, str(d / "layout.o"), "-o", str(d / "layout")], check=True)
+    got = dict(x.split() for x in subprocess.run([str(d / "layout")], check=True, capture_output=True, text=True).stdout.splitlines())
+    for cls in (GraphDev, FrontierBufs):
+        assert int(got[cls.__name__]) == ctypes.sizeof(cls)
+        for f in cls._fields_:
+            assert int(got[f"{cls.__name__}.{f[0]}"]) == getattr(cls, f[0]).offset, f[0]
+
+
+@pytest.mark.parametrize("n", [31, 5000])
+@pytest.mark.parametrize("levels", [2, 9])
+def test_search_that_gives_up_reaches_every_row(lib, layouts, n, levels):
+    """Distances and tile lists of the search; without polls every row counts as reached at once, and
+    the lists hold every tile."""
+    import torch
+    # a path with a few chords: rows in hop order of node 0 only near the start
+    src = np.concatenate([np.arange(n - 1), np.arange(0, n - 40, 37)])
+    dst = np.concatenate([np.arange(1, n), np.arange(0, n - 40, 37) + 29])
+    r, c = np.concatenate([src, dst]), np.concatenate([dst, src])
+    order = np.argsort(r, kind="stable")
+    ptr = np.concatenate([[0], np.cumsum(np.bincount(r, minlength=n))]).astype(np.int32)
+    col = c[order].astype(np.int32)
+    nodes = np.array([n // 2, 3, n - 1], dtype=np.int32)
+    dist = np.full(n, 255)
+    dist[nodes] = 0
+    for k in range(1, levels + 1):
+        near = np.concatenate([col[:0]] + [col[ptr[i]:ptr[i + 1]] for i in np.nonzero(dist == k - 1)[0]])
+        near = near[dist[near] == 255]
+        dist[near] = k
+
+    plan = lib["_ZN2kb13plan_frontierERNS_12FrontierBufsEliPhPm"]
+    plan.restype, plan.argtypes = None, [VP, ctypes.c_int64, I32, VP, VP]
+    launch = lib["_ZN2kb15launch_frontierERKNS_8GraphDevERNS_12FrontierBufsEPKiiP11CUstream_sti"]
+    launch.restype, launch.argtypes = I32, [VP, VP, VP, I32, VP, I32]
+    dptr, dcol = torch.from_numpy(ptr).cuda(), torch.from_numpy(col).cuda()
+    g = GraphDev(n, col.size, dptr.data_ptr(), dcol.data_ptr(), None, None, None, 0, 64)
+    fr, size = FrontierBufs(), ctypes.c_size_t()
+    plan(ctypes.byref(fr), n, levels, None, ctypes.byref(size))
+    buf = torch.zeros(size.value, dtype=torch.uint8, device="cuda")
+    plan(ctypes.byref(fr), n, levels, buf.data_ptr(), ctypes.byref(size))
+    nt = (n + 31) // 32
+    assert (fr.levels, fr.nt) == (levels, nt)
+
+    def ints(p, count):
+        return buf[p - buf.data_ptr():][:4 * count].cpu().numpy().view(np.int32)
+
+    for spins in (1 << 22, 0):
+        buf.fill_(0xA5)
+        torch.cuda.synchronize()
+        assert launch(ctypes.byref(g), ctypes.byref(fr), nodes.ctypes.data, nodes.size, None, spins) == 0
+        torch.cuda.synchronize()
+        want = dist if spins else np.zeros(n, dtype=int)
+        gen = buf[fr.gen - buf.data_ptr():][:n].cpu().numpy()
+        assert np.array_equal(gen, want)
+        tile = np.array([want[32 * t:32 * t + 32].min() for t in range(nt)])
+        tgen = ints(fr.tgen, nt)
+        assert np.array_equal(np.where(tgen > levels, 255, tgen), tile)
+        assert np.array_equal(ints(fr.alist, nt), np.argsort(tile, kind="stable"))
+        count = ints(fr.acount, levels + 1)
+        lists = ints(fr.lists, (levels + 1) * nt).reshape(levels + 1, nt)
+        for k in range(levels + 1):
+            assert count[k] == np.sum(tile <= k)
+            assert np.array_equal(lists[k, :count[k]], np.nonzero(tile <= k)[0])
