@@ -27,6 +27,7 @@ int fail(int code, const std::string &msg) {
 }
 int cuda_fail(cudaError_t e, const char *what) {
     g_last_error = std::string(what) + ": " + cudaGetErrorString(e);
+    (void)cudaGetLastError();   // (else the next launch check of this thread would report it again)
     if (e == cudaErrorMemoryAllocation) return KB_ERR_NOMEM;
     return KB_ERR_CUDA;
 }
