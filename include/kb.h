@@ -325,7 +325,8 @@ int kb_rls_predict(kb_graph *g, kb_method method, kb_phi phi, const kb_params *p
 /* ------------------------------------------------------------------ scratch size */
 /* Bytes of device scratch one kb_krylov_apply call with these arguments takes from the
  * stream-ordered pool (the result Y excluded).  Host-only; validates the arguments as
- * kb_krylov_apply does, except the node list. */
+ * kb_krylov_apply does, except the node list.  Where the pool cannot give that much, a call
+ * restricted to the reached rows does with what it takes under no_frontier = 1. */
 int kb_workspace_bytes(kb_graph *g, kb_method method, kb_phi phi, const kb_params *params,
                        int32_t M, int32_t m, uint64_t *bytes);
 
@@ -345,7 +346,8 @@ int kb_workspace_bytes(kb_graph *g, kb_method method, kb_phi phi, const kb_param
  * and must not touch the device array Y (n x M float32, as for kb_krylov_apply) until the
  * request has been polled as finished.  It returns a ticket, or KB_ERR_BUSY when
  * queue_capacity requests are pending or unpolled, or KB_ERR_NOMEM when the request alone
- * exceeds the memory budget.  Argument errors of the solve itself are reported by poll.
+ * exceeds the memory budget (one that exceeds it only with the scratch of the restriction to
+ * reached rows runs under no_frontier = 1).  Argument errors of the solve itself are reported by poll.
  *
  * kb_server_poll waits up to wait_ms milliseconds (0: do not wait, < 0: wait until done).
  * It returns KB_PENDING while the request runs or waits, otherwise the solve's status; a

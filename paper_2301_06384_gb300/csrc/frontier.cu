@@ -257,7 +257,13 @@ k_zero_tiles(unsigned char *blocks, int64_t block_bytes, int nblk, int row_bytes
 
 }  // namespace
 
-void plan_frontier(FrontierBufs &f, int64_t n, int levels, unsigned char *base, size_t *bytes) {
+// qlev, tcnt (with the barrier behind them) and vis; the queue
+constexpr size_t LV = FRONTIER_MAX_HOPS + 6;
+static size_t zeroed_bytes(int64_t n) { return sizeof(int32_t) * 2 * LV + sizeof(uint32_t) * size_t((n + ACT_ROWS - 1) / ACT_ROWS); }
+static size_t queue_offset(int64_t n) { return (zeroed_bytes(n) + 255) & ~size_t(255); }
+size_t frontier_search_bytes(int64_t n) { return queue_offset(n) + sizeof(int32_t) * size_t(n); }
+
+void plan_frontier(FrontierBufs &f, int64_t n, int levels, unsigned char *base, size_t *bytes, unsigned char *search) {
     f.levels = levels;
     f.nt = (n + ACT_ROWS - 1) / ACT_ROWS;
     const size_t nt = size_t((n + ACT_ROWS - 1) / ACT_ROWS);
@@ -267,19 +273,18 @@ void plan_frontier(FrontierBufs &f, int64_t n, int levels, unsigned char *base, 
         off += (b + 255) & ~size_t(255);
         return p;
     };
-    constexpr size_t LV = FRONTIER_MAX_HOPS + 6;
-    f.zeroed = take(sizeof(int32_t) * 2 * LV + sizeof(uint32_t) * nt);
-    f.zero_bytes = sizeof(int32_t) * 2 * LV + sizeof(uint32_t) * nt;
+    f.zeroed = search;
+    f.zero_bytes = zeroed_bytes(n);
     f.qlev = reinterpret_cast<int32_t *>(f.zeroed);
     f.tcnt = f.qlev + LV;
     f.sync = f.tcnt + LV - 2;
     f.vis = reinterpret_cast<uint32_t *>(f.tcnt + LV);
+    f.queue = reinterpret_cast<int32_t *>(search ? search + queue_offset(n) : nullptr);
     f.acount = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * LV));
     f.gen = take(size_t(n));
     f.tgen = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * nt));
     f.alist = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * nt));
     f.lists = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * nt * size_t(levels + 1)));
-    f.queue = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * size_t(n)));
     *bytes = off;
 }
 

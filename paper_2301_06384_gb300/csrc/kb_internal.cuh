@@ -312,6 +312,8 @@ struct RowArgs {
     int M = 0;                        // columns in use (set by launch_rowblock)
     int ordered = 0;                  // sums in a fixed order (rowblock.cuh): alist is in index order
     int tc = 0;                       // tensor-core kernels allowed (rowblock_tc.cu)
+    int max_grid = INT32_MAX;         // rows of the partials buffer (modes with a Gram)
+    int plan = 0;                     // report the grid only
     int kbase = 0;                    // ASM: index of the first block (frontier reach)
     int accumulate = 0;               // ASM: y += product (the accumulator starts from y)
     const int32_t *skip = nullptr;    // the launch does nothing when *skip != 0 (device flag)
@@ -321,7 +323,8 @@ template <typename T>
 int launch_rowblock(int mode, int W, const RowArgs<T> &a, cudaStream_t s, int *grid_out,
                     int64_t M_alg);
 template <typename T>
-int rowblock_max_grid(int W);
+// Largest grid of the modes with a Gram (rows of the partials buffer) for blocks of n x M.
+int rowblock_max_grid(int W, int M, int64_t n, bool ordered, bool tc);
 // Tensor-core (tcgen05) variant of PROJ, UPD, MULGRAM and MUL for FP32 blocks of width 64
 // (rowblock_tc.cu); launch_rowblock uses it where rowblock_tc_supported says so.  Gram
 // partials: grid <= max_grid rows of [W*W].

@@ -120,6 +120,7 @@ struct FrontierBufs {
     uint8_t *gen = nullptr;
     int32_t *tgen = nullptr, *alist = nullptr, *acount = nullptr;
     int32_t *lists = nullptr;          // levels + 1 lists of nt tiles
+    // of the search alone:
     unsigned char *zeroed = nullptr;   // qlev, tcnt (the barrier behind it) and vis: cleared first
     size_t zero_bytes = 0;
     int32_t *qlev = nullptr, *tcnt = nullptr, *queue = nullptr;
@@ -132,8 +133,10 @@ struct FrontierBufs {
     const int32_t *count(int k) const { return acount + (k < levels ? k : levels); }
 };
 // Lays the arrays out from base (nullptr: sizes only) for a search of `levels` hops; *bytes
-// receives their size.
-void plan_frontier(FrontierBufs &f, int64_t n, int levels, unsigned char *base, size_t *bytes);
+// receives their size.  search: frontier_search_bytes(n) bytes that only launch_frontier uses (the
+// solves give it block memory, which the steps write afterwards).
+size_t frontier_search_bytes(int64_t n);
+void plan_frontier(FrontierBufs &f, int64_t n, int levels, unsigned char *base, size_t *bytes, unsigned char *search);
 // Hop distances up to f.levels from the nodes, and the tile lists; every row at distance 0 when a
 // barrier of the search runs out of its polls.
 int launch_frontier(const GraphDev &g, FrontierBufs &f, const int32_t *nodes, int M, cudaStream_t s,

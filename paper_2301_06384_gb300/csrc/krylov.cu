@@ -121,12 +121,19 @@ struct Arena {
         off += bytes;
         return p;
     }
-    // hops: the last step whose products the search has to cover (0: no restriction)
+    // `count` values of block memory, which also serves the search for reached rows
+    template <typename T>
+    T *take_blocks(size_t count, int64_t n, bool restricted) {
+        blocks = base ? reinterpret_cast<unsigned char *>(base + off) : nullptr;
+        return reinterpret_cast<T *>(take<char>(std::max(count * sizeof(T), restricted ? frontier_search_bytes(n) : 0)));
+    }
+    // hops: the last step whose products the search has to cover
     void frontier(FrontierBufs &f, int64_t n, int hops) {
         size_t bytes = 0;
-        plan_frontier(f, n, hops <= FRONTIER_MAX_HOPS ? hops + 1 : 0, base ? reinterpret_cast<unsigned char *>(base + off) : nullptr, &bytes);
+        plan_frontier(f, n, hops + 1, base ? reinterpret_cast<unsigned char *>(base + off) : nullptr, &bytes, blocks);
         off += bytes;
     }
+    unsigned char *blocks = nullptr;
 };
 
 void ensure_pool(int dev) {
@@ -335,6 +342,9 @@ double projected_bound(const Common &c) {
 }
 
 // ---------------------------------------------------------------- cbl
+// W x W matrices kept per step (CblBufs)
+static int step_mats(const Common &c) { return c.p.reorth == 2 ? 6 : 4; }
+
 template <typename T>
 struct CblBufs {
     using C = typename Cmp<T>::type;   // small matrices and Gram partials
@@ -360,13 +370,12 @@ struct CblBufs {
 };
 
 template <typename T>
-void plan_cbl(Arena &ar, CblBufs<T> &b, int64_t n, int M, int W, int m, int rb_grid, bool two_pass,
-              int qbatch) {
-    b.basis = ar.take<T>(size_t(two_pass ? 3 : m) * n * W);
+void plan_cbl(Arena &ar, CblBufs<T> &b, const Common &c, int64_t n, int M, int W, int m, int rb_grid, int qbatch) {
+    b.basis = ar.take_blocks<T>(size_t(c.p.two_pass ? 3 : m) * n * W, n, c.frontier);
     b.wbuf = ar.take<T>(size_t(n) * W);
     using C = typename Cmp<T>::type;
     b.parts = ar.take<C>(size_t(rb_grid) * W * W);
-    b.Cbs = ar.take<C>(size_t(m) * W * W * 6);   // Cbs | Bs | Rs1 | Rs2 | Cloc (2 per step)
+    b.Cbs = ar.take<C>(size_t(m) * W * W * step_mats(c));   // Cbs | Bs | Rs1 | Rs2 | Cloc (2 per step)
     b.Bs = b.Cbs + size_t(m) * W * W;
     b.Rs1 = b.Bs + size_t(m) * W * W;
     b.Rs2 = b.Rs1 + size_t(m) * W * W;
@@ -376,24 +385,31 @@ void plan_cbl(Arena &ar, CblBufs<T> &b, int64_t n, int M, int W, int m, int rb_g
     b.Hd = ar.take<double>(size_t(m) * M * M);
     b.Hs = ar.take<double>(size_t(m) * M * M);
     b.R1 = ar.take<double>(size_t(M) * M);
-    b.Cstk = ar.take<C>(size_t(m) * W * W);
+    b.Cstk = c.p.reorth == 1 ? ar.take<C>(size_t(m) * W * W) : nullptr;
     b.V0 = ar.take<double>(size_t(m) * M * M);
     b.V1 = ar.take<double>(size_t(m) * M * M);
     b.V2 = ar.take<double>(size_t(m) * M * M);
     b.U = ar.take<double>(size_t(m) * M * M);
-    b.Uc = ar.take<double>(size_t(2) * m * M * M);
+    b.Uc = c.p.tol > 0.0 ? ar.take<double>(size_t(2) * m * M * M) : nullptr;
     b.qscr = qbatch > 0 ? ar.take<double>(size_t(qbatch) * bt_quad_node_doubles(M, m)) : nullptr;
-    b.Hdf = ar.take<double>(size_t(2) * m * M * (M + 1));
-    b.bt_ls = ar.take<double>(size_t(2) * M * M);
+    const bool spline = c.phi == KB_PHI_SPLINE;
+    b.Hdf = spline ? ar.take<double>(size_t(2) * m * M * M)
+                   : sizeof(C) == 4 ? ar.take<double>(size_t(2) * m * M * (M + 1)) : nullptr;
+    b.bt_ls = spline ? ar.take<double>(size_t(2) * M * M) : nullptr;
     b.chk_prev = ar.take<int32_t>(1);
     b.reo_d0 = ar.take<double>(size_t(W));
     b.reo_skip = ar.take<int32_t>(1);
     b.ctrl = ar.take<Ctrl>(1);
     b.ctrl2 = ar.take<Ctrl>(1);
     b.ctrl_chk = ar.take<Ctrl>(1);
-    ar.frontier(b.fr, n, m);
+    if (c.frontier) ar.frontier(b.fr, n, m);
     b.hcnt = ar.take<unsigned>(1);
     b.csync = ar.take<int32_t>(2);
+}
+
+template <typename T>
+int cbl_grid(const Common &c, int W, int M, int64_t n) {
+    return rowblock_max_grid<T>(W, M, n, c.ordered != 0, c.tc != 0);
 }
 
 template <typename T>
@@ -402,15 +418,15 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
     const int64_t n = c.g->dev.n;
     const int W = width_for(M);
     const bool f64 = sizeof(C) == 8;
-    const int rb_grid = rowblock_max_grid<T>(W);
+    const int rb_grid = cbl_grid<T>(c, W, M, n);
     const bool two = c.p.two_pass != 0;
     const int qbatch = quad_batch(c.quad, M, m);
     Arena dry;
     CblBufs<T> b{};
-    plan_cbl<T>(dry, b, n, M, W, m, rb_grid, two, qbatch);
+    plan_cbl<T>(dry, b, c, n, M, W, m, rb_grid, qbatch);
     Arena ar;
     KB_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void **>(&ar.base), dry.off, c.s));
-    plan_cbl<T>(ar, b, n, M, W, m, rb_grid, two, qbatch);
+    plan_cbl<T>(ar, b, c, n, M, W, m, rb_grid, qbatch);
     auto body = [&]() -> int {
         const double lam = c.g->lambda;        // thresholds (scale of L)
         const double lam_p = c.g->lambda_proj; // interval of the projected series
@@ -440,10 +456,11 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
         if (c.frontier) KB_TRY(launch_frontier(c.g->dev, b.fr, nodes, M, c.s));
         KB_TRY(start_blocks());
         // slots of steps after a stop are never written: keep them zero
-        KB_CUDA_TRY(cudaMemsetAsync(b.Cbs, 0, sizeof(C) * size_t(m) * W * W * 6, c.s));
+        KB_CUDA_TRY(cudaMemsetAsync(b.Cbs, 0, sizeof(C) * size_t(m) * W * W * step_mats(c), c.s));
         // the frontier arguments of a row-block launch over the tiles within k hops
         const int32_t *tg = c.frontier ? b.fr.tgen : nullptr;
         auto within = [&](RowArgs<T> &ra, int k) {
+            ra.max_grid = rb_grid;
             ra.tc = c.tc;
             ra.ordered = c.ordered;
             ra.tgen = tg;
@@ -729,9 +746,9 @@ struct LzBufs {
 };
 
 template <typename T>
-void plan_lz(Arena &ar, LzBufs<T> &b, int64_t n, int W, int m, int pgrid, bool two_pass, int nquad) {
+void plan_lz(Arena &ar, LzBufs<T> &b, const Common &c, int64_t n, int W, int m, int pgrid, int nquad) {
     // two-pass: three rotating blocks; the coefficients of every step are kept for the replay
-    b.basis = ar.take<T>(size_t(two_pass ? 3 : m + 1) * n * W);
+    b.basis = ar.take_blocks<T>(size_t(c.p.two_pass ? 3 : m + 1) * n * W, n, c.frontier);
     b.parts = ar.take<double>(size_t(pgrid) * W);
     b.sigma = ar.take<double>(size_t(m + 1) * W);
     b.alpha = ar.take<double>(size_t(m + 1) * W);
@@ -745,7 +762,7 @@ void plan_lz(Arena &ar, LzBufs<T> &b, int64_t n, int W, int m, int pgrid, bool t
     b.omega = ar.take<double>(size_t(m) * W);
     b.ctrl = ar.take<Ctrl>(1);
     b.ctrl2 = ar.take<Ctrl>(1);
-    ar.frontier(b.fr, n, m);
+    if (c.frontier) ar.frontier(b.fr, n, m);
 }
 
 template <typename T>
@@ -774,10 +791,10 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
     const bool two = c.p.two_pass != 0;
     Arena dry;
     LzBufs<T> b{};
-    plan_lz<T>(dry, b, n, W, m, pgrid, two, nquad);
+    plan_lz<T>(dry, b, c, n, W, m, pgrid, nquad);
     Arena ar;
     KB_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void **>(&ar.base), dry.off, c.s));
-    plan_lz<T>(ar, b, n, W, m, pgrid, two, nquad);
+    plan_lz<T>(ar, b, c, n, W, m, pgrid, nquad);
     auto body = [&]() -> int {
         const double thresh = (f64 ? 1e-12 : 1e-6) * c.g->lambda;
         KB_TRY(launch_ctrl_init(b.ctrl, m, c.s));
@@ -938,15 +955,15 @@ int cheb_pass(Common &c, const std::vector<double> &coef, double lam, int W, int
 }
 
 template <typename T>
-void plan_cheb(Arena &ar, int64_t n, int Mmax, bool squared, int hops, T **bufs, T **Z, int32_t **marker,
-               FrontierBufs &fr) {
+void plan_cheb(Arena &ar, const Common &c, int64_t n, int Mmax, bool squared, int hops, T **bufs, T **Z,
+               int32_t **marker, FrontierBufs &fr) {
     // bufs and Z are consecutive blocks of n Wmax elements
     const int Wmax = width_for(Mmax);
-    T *p = ar.take<T>(size_t(squared ? 4 : 3) * n * Wmax);
+    T *p = ar.take_blocks<T>(size_t(squared ? 4 : 3) * n * Wmax, n, c.frontier);
     for (int i = 0; i < 3; ++i) bufs[i] = p ? p + size_t(i) * n * Wmax : nullptr;
     *Z = squared && p ? p + size_t(3) * n * Wmax : nullptr;
     *marker = ar.take<int32_t>(size_t(n));
-    ar.frontier(fr, n, hops);
+    if (c.frontier) ar.frontier(fr, n, hops);
 }
 
 template <typename T>
@@ -960,10 +977,10 @@ int run_cheb(Common &c, bool squared, const int32_t *nodes, int M, int m, float 
     T *bufs[3], *Z;
     int32_t *marker;
     FrontierBufs fb;
-    plan_cheb<T>(dry, n, Mmax, squared, squared ? 2 * h : h, bufs, &Z, &marker, fb);
+    plan_cheb<T>(dry, c, n, Mmax, squared, squared ? 2 * h : h, bufs, &Z, &marker, fb);
     Arena ar;
     KB_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void **>(&ar.base), dry.off, c.s));
-    plan_cheb<T>(ar, n, Mmax, squared, squared ? 2 * h : h, bufs, &Z, &marker, fb);
+    plan_cheb<T>(ar, c, n, Mmax, squared, squared ? 2 * h : h, bufs, &Z, &marker, fb);
     auto body = [&]() -> int {
         for (int col0 = 0; col0 < M; col0 += Mmax) {
             const int Mc = std::min(Mmax, M - col0);
@@ -996,13 +1013,15 @@ int run_cheb(Common &c, bool squared, const int32_t *nodes, int M, int m, float 
 
 // Scratch bytes of one solve (the same plans the runs allocate).
 template <typename T>
-size_t workspace_bytes_t(int64_t n, kb_method method, int M, int m, bool two, const QuadRule *q) {
+size_t workspace_bytes_t(const Common &c, kb_method method, int M, int m) {
     Arena dry;
+    const int64_t n = c.g->dev.n;
+    const QuadRule *q = c.quad;
     const int W = width_for(M);
     switch (method) {
         case KB_CBL: {
             CblBufs<T> b{};
-            plan_cbl<T>(dry, b, n, M, W, m, rowblock_max_grid<T>(W), two, quad_batch(q, M, m));
+            plan_cbl<T>(dry, b, c, n, M, W, m, cbl_grid<T>(c, W, M, n), quad_batch(q, M, m));
             break;
         }
         case KB_GBL:
@@ -1011,8 +1030,7 @@ size_t workspace_bytes_t(int64_t n, kb_method method, int M, int m, bool two, co
             const int Mg = method == KB_SBL ? std::min(M, sizeof(T) == 8 ? 64 : 128) : M;
             const int Wg = width_for(Mg);
             LzBufs<T> b{};
-            plan_lz<T>(dry, b, n, Wg, m, std::max(spmm_max_grid<T>(Wg), axpy_max_grid()), two,
-                       q ? q->n : 0);
+            plan_lz<T>(dry, b, c, n, Wg, m, std::max(spmm_max_grid<T>(Wg), axpy_max_grid()), q ? q->n : 0);
             break;
         }
         case KB_CHEB:
@@ -1020,7 +1038,7 @@ size_t workspace_bytes_t(int64_t n, kb_method method, int M, int m, bool two, co
             T *bufs[3], *Z;
             int32_t *marker;
             FrontierBufs fb;
-            plan_cheb<T>(dry, n, std::min(M, sizeof(T) == 8 ? 64 : 128), method == KB_CHEB2,
+            plan_cheb<T>(dry, c, n, std::min(M, sizeof(T) == 8 ? 64 : 128), method == KB_CHEB2,
                          method == KB_CHEB2 ? 2 * (m / 2) : m, bufs, &Z, &marker, fb);
             break;
         }
@@ -1079,8 +1097,27 @@ int validate(kb_graph *g, kb_method method, kb_phi phi, const kb_params *params,
     return KB_OK;
 }
 
-int apply_device(kb_graph *g, kb_method method, kb_phi phi, const kb_params *params,
-                 const int32_t *nodes, int32_t M, int32_t m, float *Y, void *stream, kb_info *info) {
+// A solve's settings.  restricted: the per-step kernels may keep to the rows reached from W.
+Common solve_of(kb_graph *g, kb_method method, kb_phi phi, const kb_params &params, int M, int m, int s_int,
+                cudaStream_t s, const QuadRule &quad, bool restricted) {
+    Common c{g, phi, params, s_int, s, 0, nullptr, true};
+    if (quad.n > 0) c.quad = &quad;
+    // exact restriction of the per-step kernels to rows reached from W (hop distances are kept
+    // in 8 bits).  It costs a breadth-first search and a sort (about 5 us per hop), so blocks
+    // below 16 MiB, which stay in L2, run on all rows: measured with 20 steps on random
+    // geometric graphs, restricted / all rows (us): 16384 rows, M = 64, cheb 308 / 222, cbl
+    // 5061 / 4975; 65536 rows, M = 64 (16 MiB), cheb 456 / 429, cbl 6290 / 7050; 262144 rows,
+    // M = 16 (16 MiB), cheb 321 / 552, cbl 2558 / 3598.  FP64 products cost some 16 times as
+    // much per row.
+    const int64_t blk_bytes = g->dev.n * width_for(std::min(M, 128)) * (params.basis == KB_F64 ? 128 : 4);
+    c.ordered = method == KB_CBL && params.reorth == 1 && params.basis == KB_F32 ? 1 : 0;
+    c.frontier = restricted && !params.no_frontier && m <= FRONTIER_MAX_HOPS && (blk_bytes >= (int64_t(16) << 20) || c.ordered);
+    c.tc = rowblock_tc_enabled() ? 1 : 0;
+    return c;
+}
+
+int apply_once(kb_graph *g, kb_method method, kb_phi phi, const kb_params *params, const int32_t *nodes, int32_t M,
+               int32_t m, float *Y, void *stream, kb_info *info, bool &restricted) {
     int s_int = 0;
     int rc = validate(g, method, phi, params, nodes, M, m, Y, &s_int);
     if (rc) return rc;
@@ -1090,19 +1127,8 @@ int apply_device(kb_graph *g, kb_method method, kb_phi phi, const kb_params *par
     auto quad = std::make_unique<QuadRule>();
     rc = quad_setup(g, method, phi, *params, *quad);
     if (rc) return rc;
-    Common c{g, phi, *params, s_int, static_cast<cudaStream_t>(stream), 0, nullptr, true};
-    if (quad->n > 0) c.quad = quad.get();
-    // exact restriction of the per-step kernels to rows reached from W (hop distances are kept
-    // in 8 bits).  It costs a breadth-first search and a sort (about 5 us per hop), so blocks
-    // below 16 MiB, which stay in L2, run on all rows: measured with 20 steps on random
-    // geometric graphs, restricted / all rows (us): 16384 rows, M = 64, cheb 308 / 222, cbl
-    // 5061 / 4975; 65536 rows, M = 64 (16 MiB), cheb 456 / 429, cbl 6290 / 7050; 262144 rows,
-    // M = 16 (16 MiB), cheb 321 / 552, cbl 2558 / 3598.  FP64 products cost some 16 times as
-    // much per row.
-    const int64_t blk_bytes = g->dev.n * width_for(std::min(M, 128)) * (params->basis == KB_F64 ? 128 : 4);
-    c.ordered = method == KB_CBL && params->reorth == 1 && params->basis == KB_F32 ? 1 : 0;
-    c.frontier = !params->no_frontier && m <= FRONTIER_MAX_HOPS && (blk_bytes >= (int64_t(16) << 20) || c.ordered);
-    c.tc = rowblock_tc_enabled() ? 1 : 0;
+    Common c = solve_of(g, method, phi, *params, M, m, s_int, static_cast<cudaStream_t>(stream), *quad, restricted);
+    restricted = c.frontier;
     const bool f64 = params->basis == KB_F64;
     const bool bf16 = params->basis == KB_BF16;
     const int chunk = f64 ? 64 : 128;
@@ -1166,6 +1192,19 @@ int apply_device(kb_graph *g, kb_method method, kb_phi phi, const kb_params *par
     return KB_OK;
 }
 
+// The restriction takes scratch of its own (the tile lists: n / 8 bytes per step), which memory that
+// is nearly full may not hold: the solve then runs on all rows.
+int apply_device(kb_graph *g, kb_method method, kb_phi phi, const kb_params *params, const int32_t *nodes, int32_t M,
+                 int32_t m, float *Y, void *stream, kb_info *info) {
+    bool restricted = true;
+    int rc = apply_once(g, method, phi, params, nodes, M, m, Y, stream, info, restricted);
+    if (rc == KB_ERR_NOMEM && restricted) {
+        restricted = false;
+        rc = apply_once(g, method, phi, params, nodes, M, m, Y, stream, info, restricted);
+    }
+    return rc;
+}
+
 }  // namespace
 
 extern "C" int kb_krylov_apply(kb_graph *g, kb_method method, kb_phi phi, const kb_params *params,
@@ -1219,16 +1258,14 @@ extern "C" int kb_workspace_bytes(kb_graph *g, kb_method method, kb_phi phi, con
         const float probe = 0.f;
         int rc = validate(g, method, phi, params, dummy.data(), M, m, &probe, &s_int);
         if (rc) return rc;
-        const int64_t n = g->dev.n;
         auto quad = std::make_unique<QuadRule>();
         rc = quad_setup(g, method, phi, *params, *quad);
         if (rc) return rc;
-        const QuadRule *q = quad->n > 0 ? quad.get() : nullptr;
-        const bool two = params->two_pass != 0;
+        const Common c = solve_of(g, method, phi, *params, M, m, s_int, nullptr, *quad, true);
         switch (params->basis) {
-            case KB_F64: *bytes = workspace_bytes_t<double>(n, method, M, m, two, q); break;
-            case KB_BF16: *bytes = workspace_bytes_t<__nv_bfloat16>(n, method, M, m, two, q); break;
-            default: *bytes = workspace_bytes_t<float>(n, method, M, m, two, q); break;
+            case KB_F64: *bytes = workspace_bytes_t<double>(c, method, M, m); break;
+            case KB_BF16: *bytes = workspace_bytes_t<__nv_bfloat16>(c, method, M, m); break;
+            default: *bytes = workspace_bytes_t<float>(c, method, M, m); break;
         }
         return KB_OK;
     } catch (...) {

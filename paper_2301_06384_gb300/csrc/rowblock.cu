@@ -128,6 +128,28 @@ bool rowblock_tc_enabled() {
 }
 
 template <typename T>
+static int launch_simt(int mode, int W, const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
+    if constexpr (std::is_same<T, float>::value) {
+        if (a.ordered && mode != RB_MUL && mode != RB_ASM) {
+            switch (W) {
+                case 16: return rb::launch_ordered<16>(mode, a, s, grid_out);
+                case 32: return rb::launch_ordered<32>(mode, a, s, grid_out);
+                case 64: return rb::launch_ordered<64>(mode, a, s, grid_out);
+                default: return rb::launch_ordered<128>(mode, a, s, grid_out);
+            }
+        }
+    }
+    switch (W) {
+        case 16: return rb::launch_w<T, 16>(mode, a, s, grid_out);
+        case 32: return rb::launch_w<T, 32>(mode, a, s, grid_out);
+        case 64: return rb::launch_w<T, 64>(mode, a, s, grid_out);
+        case 128:
+            if constexpr (sizeof(typename Cmp<T>::type) == 4) return rb::launch_w<T, 128>(mode, a, s, grid_out);
+    }
+    return fail(KB_ERR_ARG, "unsupported block width");
+}
+
+template <typename T>
 int launch_rowblock(int mode, int W, const RowArgs<T> &a, cudaStream_t s, int *grid_out,
                     int64_t M_alg) {
     if (sizeof(typename Cmp<T>::type) == 8 && W > 64) return fail(KB_ERR_UNSUPPORTED, "FP64 blocks wider than 64");
@@ -140,33 +162,11 @@ int launch_rowblock(int mode, int W, const RowArgs<T> &a, cudaStream_t s, int *g
     // (launches under a device skip flag take the SIMT kernels, which read the flag)
     if constexpr (std::is_same<T, float>::value)
         tc = a.tc && !a.skip && rowblock_tc_supported(mode, W);
-    bool done = false;
-    if constexpr (std::is_same<T, float>::value) {
-        if (a.ordered && !tc && mode != RB_MUL && mode != RB_ASM) {
-            done = true;
-            switch (W) {
-                case 16: rc = rb::launch_ordered<16>(mode, aa, s, grid_out); break;
-                case 32: rc = rb::launch_ordered<32>(mode, aa, s, grid_out); break;
-                case 64: rc = rb::launch_ordered<64>(mode, aa, s, grid_out); break;
-                default: rc = rb::launch_ordered<128>(mode, aa, s, grid_out); break;
-            }
-        }
-    }
-    if (done) {
-    } else if (tc) {
+    if (tc) {
         // FP32 blocks of width 64: tensor-core kernel (rowblock_tc.cu)
-        if constexpr (std::is_same<T, float>::value)
-            rc = launch_rowblock_tc(mode, aa, s, rowblock_max_grid<T>(W), grid_out);
+        if constexpr (std::is_same<T, float>::value) rc = launch_rowblock_tc(mode, aa, s, aa.max_grid, grid_out);
     } else {
-        switch (W) {
-            case 16: rc = rb::launch_w<T, 16>(mode, aa, s, grid_out); break;
-            case 32: rc = rb::launch_w<T, 32>(mode, aa, s, grid_out); break;
-            case 64: rc = rb::launch_w<T, 64>(mode, aa, s, grid_out); break;
-            case 128:
-                if constexpr (sizeof(typename Cmp<T>::type) == 4) { rc = rb::launch_w<T, 128>(mode, aa, s, grid_out); break; }
-                [[fallthrough]];
-            default: return fail(KB_ERR_ARG, "unsupported block width");
-        }
+        rc = launch_simt<T>(mode, W, aa, s, grid_out);
     }
     if (rc) return rc;
     cudaError_t err = cudaGetLastError();
@@ -199,9 +199,21 @@ int launch_rowblock(int mode, int W, const RowArgs<T> &a, cudaStream_t s, int *g
 }
 
 template <typename T>
-int rowblock_max_grid(int W) {
-    (void)W;
-    return num_sms() * rb::RB_MAX_CTAS;
+int rowblock_max_grid(int W, int M, int64_t n, bool ordered, bool tc) {
+    int most = 0;
+    for (const int mode : {RB_PROJ, RB_UPD, RB_MULGRAM, RB_ASMSUB}) {
+        RowArgs<T> a;
+        a.n = n;
+        a.M = M;
+        a.ordered = ordered ? 1 : 0;
+        a.plan = 1;
+        int grid = 0;
+        if (launch_simt<T>(mode, W, a, nullptr, &grid) == 0) most = std::max(most, grid);
+    }
+    if constexpr (std::is_same<T, float>::value) {
+        if (tc && rowblock_tc_supported(RB_PROJ, W)) most = std::max(most, rowblock_tc_max_grid());
+    }
+    return most;
 }
 
 template <typename P>
@@ -239,10 +251,10 @@ template int launch_reduce_hkk<double>(const double *, int, int, int, double *, 
                                        const Ctrl *, cudaStream_t);
 template int launch_rowblock<float>(int, int, const RowArgs<float> &, cudaStream_t, int *, int64_t);
 template int launch_rowblock<double>(int, int, const RowArgs<double> &, cudaStream_t, int *, int64_t);
-template int rowblock_max_grid<float>(int);
-template int rowblock_max_grid<double>(int);
+template int rowblock_max_grid<float>(int, int, int64_t, bool, bool);
+template int rowblock_max_grid<double>(int, int, int64_t, bool, bool);
 template int launch_rowblock<__nv_bfloat16>(int, int, const RowArgs<__nv_bfloat16> &, cudaStream_t, int *, int64_t);
-template int rowblock_max_grid<__nv_bfloat16>(int);
+template int rowblock_max_grid<__nv_bfloat16>(int, int, int64_t, bool, bool);
 template int launch_reduce<float>(const float *, int, int, double *, cudaStream_t, const Ctrl *, float *,
                                   const int32_t *);
 template int launch_reduce<double>(const double *, int, int, double *, cudaStream_t, const Ctrl *, double *,

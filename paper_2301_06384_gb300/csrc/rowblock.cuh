@@ -775,7 +775,7 @@ k_rowblock(RowArgs<T> a) {
     }
 }
 
-constexpr int RB_MAX_CTAS = 5;   // per SM: bounds the Gram partials
+constexpr int RB_MAX_CTAS = 5;   // per SM
 
 // Resident CTAs per SM of an instance with smem bytes of dynamic shared memory.  The attribute
 // is raised once per instance to the most any block can take.
@@ -798,8 +798,10 @@ int launch_r(const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
     const int64_t nvt = (a.n + unit - 1) / unit;
     const int per_sm = occupancy<T, W, MODE, RPT, ORD, NT>(smem);
     int grid = int(std::min<int64_t>(nvt, int64_t(num_sms()) * (ORD ? G::CTAS : per_sm)));
+    if (MODE == RB_PROJ || MODE == RB_UPD || MODE == RB_MULGRAM || MODE == RB_ASMSUB) grid = std::min(grid, a.max_grid);
     if (grid < 1) grid = 1;
     if (grid_out) *grid_out = grid;
+    if (a.plan) return 0;
     const cudaError_t e = launch_dep(k_rowblock<T, W, MODE, RPT, ORD, NT>, dim3(grid), NT, smem, s, 0, a);
     return e == cudaSuccess ? 0 : cuda_fail(e, "k_rowblock launch");
 }

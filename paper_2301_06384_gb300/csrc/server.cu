@@ -8,6 +8,7 @@
 // the completion time.  Requests therefore complete out of submission order, but they are
 // started in submission order (no request overtakes an older one that does not fit yet).
 // Latency is measured on the host from kb_server_submit to the end of the solve.
+#include <algorithm>
 #include <chrono>
 #include <condition_variable>
 #include <deque>
@@ -59,6 +60,24 @@ struct kb_server {
 
 namespace {
 
+// Scratch of a request.  Where it exceeds the limit with what the restriction to reached rows takes,
+// the request runs without that.
+int scratch_within(kb_graph *g, kb_method method, kb_phi phi, kb_params &p, int32_t M, int32_t m, size_t limit,
+                   size_t *bytes) {
+    int rc = kb_workspace_bytes(g, method, phi, &p, M, m, bytes);
+    if (rc || *bytes <= limit || p.no_frontier) return rc;
+    p.no_frontier = 1;
+    return kb_workspace_bytes(g, method, phi, &p, M, m, bytes);
+}
+
+// The rerun of a request as one Lanczos process per column: the stopping rule and the
+// reorthogonalisation are cbl features, sbl runs the m steps.
+kb_params fallback_params(kb_params p) {
+    p.reorth = 0;
+    p.tol = 0.0;
+    return p;
+}
+
 void worker_loop(kb_server *sv, int w) {
     cudaSetDevice(sv->device);
     std::unique_lock<std::mutex> lk(sv->mu);
@@ -90,11 +109,9 @@ void worker_loop(kb_server *sv, int w) {
         if (rc == KB_ERR_BREAKDOWN && sv->fallback_sbl && (method == KB_CBL || method == KB_GBL)) {
             // rank-deficient block: one Lanczos process per column instead, when its scratch
             // fits what the request was admitted with
-            kb_params p2 = params;
-            p2.reorth = 0;
-            p2.tol = 0.0;   // the stopping rule is a cbl feature: sbl runs the m steps
-            uint64_t need = 0;
-            if (kb_workspace_bytes(g, KB_SBL, phi, &p2, M, m, &need) == KB_OK && need <= r_bytes) {
+            kb_params p2 = fallback_params(params);
+            size_t need = 0;
+            if (scratch_within(g, KB_SBL, phi, p2, M, m, r_bytes, &need) == KB_OK && need <= r_bytes) {
                 const int32_t bstep = info.breakdown_step;
                 kb_info info2{};
                 rc = kb_krylov_apply(g, KB_SBL, phi, &p2, nodes, M, m, Y, sv->streams[w], &info2);
@@ -178,9 +195,15 @@ extern "C" int kb_server_submit(kb_server *sv, kb_graph *g, kb_method method, kb
     try {
         if (!sv || !g || !params || !nodes || !Y || !ticket) return fail(KB_ERR_ARG, "NULL argument");
         if (M < 1 || M > g->dev.n) return fail(KB_ERR_ARG, "M out of range");
-        size_t bytes = 0;
-        int rc = kb_workspace_bytes(g, method, phi, params, M, m, &bytes);
+        size_t bytes = 0, need = 0;
+        kb_params p = *params;
+        int rc = scratch_within(g, method, phi, p, M, m, sv->budget, &bytes);
         if (rc) return rc;
+        if (sv->fallback_sbl && (method == KB_CBL || method == KB_GBL)) {
+            kb_params p2 = fallback_params(p);
+            if (scratch_within(g, KB_SBL, phi, p2, M, m, sv->budget, &need) == KB_OK && need <= sv->budget)
+                bytes = std::max(bytes, need);
+        }
         if (bytes > sv->budget) return fail(KB_ERR_NOMEM, "request scratch exceeds the server memory budget");
         std::lock_guard<std::mutex> lk(sv->mu);
         if (sv->stopping) return fail(KB_ERR_ARG, "server is shutting down");
@@ -190,7 +213,7 @@ extern "C" int kb_server_submit(kb_server *sv, kb_graph *g, kb_method method, kb
         r.g = g;
         r.method = method;
         r.phi = phi;
-        r.params = *params;
+        r.params = p;
         r.nodes.assign(nodes, nodes + M);
         r.m = m;
         r.Y = Y;

@@ -168,16 +168,19 @@ def test_search_that_gives_up_reaches_every_row(lib, layouts, n, levels):
         near = near[dist[near] == 255]
         dist[near] = k
 
-    plan = lib["_ZN2kb13plan_frontierERNS_12FrontierBufsEliPhPm"]
-    plan.restype, plan.argtypes = None, [VP, ctypes.c_int64, I32, VP, VP]
+    plan = lib["_ZN2kb13plan_frontierERNS_12FrontierBufsEliPhPmS2_"]
+    plan.restype, plan.argtypes = None, [VP, ctypes.c_int64, I32, VP, VP, VP]
+    search = lib["_ZN2kb21frontier_search_bytesEl"]
+    search.restype, search.argtypes = ctypes.c_size_t, [ctypes.c_int64]
     launch = lib["_ZN2kb15launch_frontierERKNS_8GraphDevERNS_12FrontierBufsEPKiiP11CUstream_sti"]
     launch.restype, launch.argtypes = I32, [VP, VP, VP, I32, VP, I32]
     dptr, dcol = torch.from_numpy(ptr).cuda(), torch.from_numpy(col).cuda()
     g = GraphDev(n, col.size, dptr.data_ptr(), dcol.data_ptr(), None, None, None, 0, 64)
     fr, size = FrontierBufs(), ctypes.c_size_t()
-    plan(ctypes.byref(fr), n, levels, None, ctypes.byref(size))
+    plan(ctypes.byref(fr), n, levels, None, ctypes.byref(size), None)
     buf = torch.zeros(size.value, dtype=torch.uint8, device="cuda")
-    plan(ctypes.byref(fr), n, levels, buf.data_ptr(), ctypes.byref(size))
+    scratch = torch.zeros(search(n), dtype=torch.uint8, device="cuda")
+    plan(ctypes.byref(fr), n, levels, buf.data_ptr(), ctypes.byref(size), scratch.data_ptr())
     nt = (n + 31) // 32
     assert (fr.levels, fr.nt) == (levels, nt)
 
@@ -186,6 +189,7 @@ def test_search_that_gives_up_reaches_every_row(lib, layouts, n, levels):
 
     for spins in (1 << 22, 0):
         buf.fill_(0xA5)
+        scratch.fill_(0xA5)
         torch.cuda.synchronize()
         assert launch(ctypes.byref(g), ctypes.byref(fr), nodes.ctypes.data, nodes.size, None, spins) == 0
         torch.cuda.synchronize()
