@@ -3,6 +3,7 @@
 // such solves (rowblock.cuh, ordered form).
 #include "kb_internal.cuh"
 #include "kb_kernels.cuh"
+#include "smallmat.cuh"
 
 namespace kb {
 namespace {
@@ -240,28 +241,6 @@ __device__ void tri_residual_df(const float *Sm, const float *Rm, int lda, int M
     }
 }
 
-// Copy an M x M row-major matrix (leading dimension ldg) from global memory through
-// store(i, j, v): rows by warp, columns by lane (coalesced), eight rows in flight per warp
-// before their stores.
-template <typename FS>
-__device__ __forceinline__ void load_square(const double *g, int ldg, int M, const FS &store) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int i0 = warp; i0 < M; i0 += 8 * nw)
-        for (int j = lane; j < M; j += 32) {
-            double v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int i = i0 + u * nw;
-                v[u] = i < M ? __ldg(g + i * ldg + j) : 0.0;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const int i = i0 + u * nw;
-                if (i < M) store(i, j, v[u]);
-            }
-        }
-}
-
 // Cholesky G = R^T R of an M x M symmetric matrix in shared memory, upper R overwriting A
 // and the lower part zeroed.  Square-root-free form: step j needs the pivot d_j (the
 // diagonal of the current Schur complement) and one reciprocal; the Schur complement update
@@ -385,15 +364,15 @@ __device__ bool chol_upper_inplace(S *A, int lda, int M, S piv_rel2, S maxdiag, 
 // pass 1 records R1 = the FP64 inverse of the applied inverse; pass 2 records
 // H_{k+1,k} = R2 R1 (rounded to the basis precision) and B = H^T.
 //
-// Pass 1 (G = X^T X, any conditioning): FP64 Cholesky; in the FP32 path the inverse is
-// formed in FP32 from R1 and R1 is then recomputed as the FP64 inverse of that FP32
-// inverse, so that X = X1 R1 holds for the applied matrices.
-// Pass 2 of the FP32 path (G = I + E, ||E|| of the order of the FP32 rounding of pass 1):
+// Pass 1 (G = X^T X, any conditioning): Cholesky in FP32, or in FP64 where a pivot is small; the
+// inverse is formed in FP32 and R1 is then the inverse of that FP32 inverse, so that X = X1 R1
+// holds for the applied matrices.
+// Pass 2 (G = I + E, ||E|| of the order of the FP32 rounding of pass 1):
 // to first order R2 = I + Phi(E) with Phi = strict upper part plus half the diagonal,
 // R2^{-1} = I - Phi(E) (the orthogonality of Q = X1 (I - Phi(E)) is then I + O(||E||^2));
 // the applied inverse I - F has the inverse I + F + F^2 + O(F^3), so H = R1 + F R1 + F (F R1),
-// the corrections formed in FP32.  When ||E|| is not small (max |E_ij| >= 1e-4), and always
-// in the FP64 mode, pass 2 uses the pass-1 algorithm.
+// the corrections formed in FP32.  When ||E|| is not small (max |E_ij| >= 1e-4) pass 2 uses the
+// pass-1 algorithm.
 //
 // The kernel runs on one SM, so its time is latency: the matrices are loaded with several
 // loads in flight per thread, the triangular products run as 4 x 4 register tiles (16
@@ -403,21 +382,20 @@ __device__ bool chol_upper_inplace(S *A, int lda, int M, S piv_rel2, S maxdiag, 
 // order-preserving bit patterns of non-negative doubles) and the Cholesky factorisation needs
 // one division per column.
 constexpr int CHOL_NEWTON_MAX = 64;   // widest block with the corrected-inverse scratch
-template <typename T>
 __global__ void __launch_bounds__(256) k_chol_ordered(const double *G, int M, int W, int pass, int step,
                                               double inv_thresh2, double piv_rel2, double *R1,
-                                              T *Rinv, double *Hs, T *Bout, Ctrl *ctrl) {
+                                              float *Rinv, double *Hs, float *Bout, Ctrl *ctrl) {
     if (ctrl->stop) return;
-    // [M][M+1] FP64, then [M][M+1] T, then 3 M + 2 doubles of scratch
+    // [M][M+1] FP64, then [M][M+1] FP32, then 3 M + 2 doubles of scratch
     extern __shared__ __align__(16) double A[];
     __shared__ int bad, small;
     __shared__ int pivot_bad[2];   // chol_upper_inplace's per-parity pivot failure flags
     __shared__ double maxdiag;
     __shared__ unsigned long long emax_bits;
     const int lda = M + 1;
-    T *Sf = reinterpret_cast<T *>(A + M * lda);
-    double *t = reinterpret_cast<double *>(Sf + M * lda + (sizeof(T) == 4 ? (M * lda) % 2 : 0));
-    const bool try_small = pass == 2 && sizeof(T) == 4;
+    float *Sf = reinterpret_cast<float *>(A + M * lda);
+    double *t = reinterpret_cast<double *>(Sf + M * lda + (M * lda) % 2);
+    const bool try_small = pass == 2;
     if (threadIdx.x == 0) {
         emax_bits = 0ull;
         bad = 0;
@@ -426,7 +404,7 @@ __global__ void __launch_bounds__(256) k_chol_ordered(const double *G, int M, in
     }
     __syncthreads();
     unsigned long long my_e = 0ull;
-    load_square(G, W, M, [&](int i, int j, double g) {
+    sm::load_square(G, W, M, [&](int i, int j, double g) {
         A[i * lda + j] = g;
         if (try_small) {
             double e = g;
@@ -472,52 +450,52 @@ __global__ void __launch_bounds__(256) k_chol_ordered(const double *G, int M, in
     __syncthreads();
     if (bad) return;
     if (small) {
-        // ---- pass 2, first order (FP32 path): S = I - Phi(E) applied; F = I - S exactly
+        // ---- pass 2, first order: S = I - Phi(E) applied; F = I - S exactly
         for (int i = threadIdx.x >> 5; i < W; i += blockDim.x >> 5)
             for (int j = threadIdx.x & 31; j < W; j += 32) {
                 const int idx = i * W + j;
                 // one FP64 subtraction per entry (E is small: the rest is exact or FP32-level)
-                T v = T(0);
+                float v = 0.f;
                 if (i < M && j < M && j >= i) {
                     const float e = float(A[i * lda + j] - (i == j ? 1.0 : 0.0));
-                    v = (i == j) ? T(1.f - 0.5f * e) : T(-e);
+                    v = (i == j) ? 1.f - 0.5f * e : -e;
                 }
                 Rinv[idx] = v;
-                if (i < M && j < M) Sf[i * lda + j] = (j >= i) ? T((i == j ? 1.f : 0.f) - float(v)) : T(0);
+                if (i < M && j < M) Sf[i * lda + j] = (j >= i) ? (i == j ? 1.f : 0.f) - v : 0.f;
             }
         __syncthreads();
-        // A is free now: R1 rounded to T, and C = F R1 (both upper triangular, zeros below)
-        T *R1t = reinterpret_cast<T *>(A);
-        T *Ct = R1t + M * lda;
-        load_square(R1, M, M, [&](int i, int j, double v) {
-            R1t[i * lda + j] = (j >= i) ? T(v) : T(0);
-            Ct[i * lda + j] = T(0);
+        // A is free now: R1 rounded to FP32, and C = F R1 (both upper triangular, zeros below)
+        float *R1t = reinterpret_cast<float *>(A);
+        float *Ct = R1t + M * lda;
+        sm::load_square(R1, M, M, [&](int i, int j, double v) {
+            R1t[i * lda + j] = (j >= i) ? float(v) : 0.f;
+            Ct[i * lda + j] = 0.f;
         });
         __syncthreads();
         auto sf = [&](int i, int k) { return Sf[i * lda + k]; };
-        auto zero = [](int, int) { return T(0); };
-        tri_mm_upper<T>(M, sf, [&](int k, int j) { return R1t[k * lda + j]; }, zero,
-                        [&](int i, int j, T c) { Ct[i * lda + j] = c; });
+        auto zero = [](int, int) { return 0.f; };
+        tri_mm_upper<float>(M, sf, [&](int k, int j) { return R1t[k * lda + j]; }, zero,
+                        [&](int i, int j, float c) { Ct[i * lda + j] = c; });
         // entries of Hs and B outside H's upper triangle are zero
         for (int i = threadIdx.x >> 5; i < W; i += blockDim.x >> 5)
             for (int j = threadIdx.x & 31; j < W; j += 32) {
                 if (i < M && j < M && j >= i) continue;
                 if (i < M && j < M) Hs[i * M + j] = 0.0;
-                Bout[j * W + i] = T(0);
+                Bout[j * W + i] = 0.f;
             }
         __syncthreads();
         // H = (I + F + F^2) R1 = R1 + (C + F C), the corrections of relative size ||E||
-        tri_mm_upper<T>(M, sf, [&](int k, int j) { return Ct[k * lda + j]; }, zero,
-                        [&](int i, int j, T corr2) {
+        tri_mm_upper<float>(M, sf, [&](int k, int j) { return Ct[k * lda + j]; }, zero,
+                        [&](int i, int j, float corr2) {
                             const double h = __ldg(R1 + i * M + j) + double(Ct[i * lda + j] + corr2);
-                            const T ht = T(h);
+                            const float ht = float(h);
                             Hs[i * M + j] = double(ht);
                             Bout[j * W + i] = ht;
                         });
         return;
     }
     // ---- general CholeskyQR pass
-    // Pass 1 of the FP32 path first factors G in FP32 (the FP32 pipe runs 64 times the FP64
+    // Pass 1 first factors G in FP32 (the FP32 pipe runs 64 times the FP64
     // rate): the first pass only has to bring X close to orthonormal, the second pass
     // corrects what is left (its first-order form when max |G2 - I| < 1e-4, a full
     // factorisation otherwise), and R1 below is the FP64 inverse of the applied inverse
@@ -525,8 +503,8 @@ __global__ void __launch_bounds__(256) k_chol_ordered(const double *G, int M, in
     // trusted in FP32: the factorisation is then redone in FP64 (which alone decides a
     // breakdown).
     bool factored = false;
-    if (sizeof(T) == 4 && pass == 1) {
-        float *Af = reinterpret_cast<float *>(Sf);   // Sf is free until the inverse below
+    if (pass == 1) {
+        float *Af = Sf;   // Sf is free until the inverse below
         float *tf = reinterpret_cast<float *>(t);
         for (int i = threadIdx.x >> 5; i < M; i += blockDim.x >> 5)
             for (int j = threadIdx.x & 31; j < M; j += 32) {
@@ -556,97 +534,93 @@ __global__ void __launch_bounds__(256) k_chol_ordered(const double *G, int M, in
         }
         return;
     }
-    const bool newton = sizeof(T) == 4 && M <= CHOL_NEWTON_MAX;
+    const bool newton = M <= CHOL_NEWTON_MAX;
     double *Sd = t + 3 * M + 2;                               // [M][M+1] (newton only)
     float *Rf = reinterpret_cast<float *>(Sd + M * lda);      // [M][M+1]
     float *C1 = Rf + M * lda;                                 // [M][M+1]
     for (int i = threadIdx.x >> 5; i < M; i += blockDim.x >> 5)
         for (int j = threadIdx.x & 31; j < M; j += 32) {
-            Sf[i * lda + j] = T(A[i * lda + j]);
-            if (newton) Rf[i * lda + j] = float(Sf[i * lda + j]);
+            Sf[i * lda + j] = float(A[i * lda + j]);
+            if (newton) Rf[i * lda + j] = Sf[i * lda + j];
         }
     __syncthreads();
     {
         // scratch after the Newton region (launch_chol sizes it)
         unsigned char *after = reinterpret_cast<unsigned char *>(t + 3 * M + 2) + (newton ? 16 * size_t(M) * lda : 0);
-        tri_inv_upper_blocked<T>(Sf, lda, M, reinterpret_cast<T *>(after));
+        tri_inv_upper_blocked<float>(Sf, lda, M, reinterpret_cast<float *>(after));
     }
     for (int i = threadIdx.x >> 5; i < W; i += blockDim.x >> 5)
         for (int j = threadIdx.x & 31; j < W; j += 32) {
             const int idx = i * W + j;
-            Rinv[idx] = (i < M && j < M && j >= i) ? Sf[i * lda + j] : T(0);
+            Rinv[idx] = (i < M && j < M && j >= i) ? Sf[i * lda + j] : 0.f;
         }
-    if (sizeof(T) == 4) {
-        // R := the FP64 inverse of the applied FP32 inverse S.
-        bool exact = !newton;
-        if (newton) {
-            // With S R = I - E (E upper triangular, of the order of the FP32 rounding),
-            // S^{-1} = R (I - E)^{-1} = R + R E + R E^2 + O(E^3): E is formed from S and R with
-            // a residual more precise than FP32 (pairs of floats when R is the FP32 factor,
-            // FP64 when the factorisation fell back to FP64), the corrections in FP32.  When
-            // max |E_ij| >= 1e-3 the exact FP64 inverse below is used instead.
-            __shared__ unsigned int emax_e;
-            float *Sff = reinterpret_cast<float *>(Sf);
-            // E goes to the Sd region (pair residual; S stays in Sf) or, with the FP64
-            // residual, which reads S from Sd, over S in Sf
-            float *Ef = factored ? reinterpret_cast<float *>(Sd) : Sff;
-            if (threadIdx.x == 0) emax_e = 0u;
-            for (int i = threadIdx.x >> 5; i < M; i += blockDim.x >> 5)
-                for (int j = threadIdx.x & 31; j < M; j += 32) {
-                    if (factored) {
-                        if (j < i) Ef[i * lda + j] = 0.f;
-                    } else {
-                        Sd[i * lda + j] = (j >= i) ? double(Sff[i * lda + j]) : 0.0;
-                    }
+    // R := the FP64 inverse of the applied FP32 inverse S.
+    bool exact = !newton;
+    if (newton) {
+        // With S R = I - E (E upper triangular, of the order of the FP32 rounding),
+        // S^{-1} = R (I - E)^{-1} = R + R E + R E^2 + O(E^3): E is formed from S and R with
+        // a residual more precise than FP32 (pairs of floats when R is the FP32 factor,
+        // FP64 when the factorisation fell back to FP64), the corrections in FP32.  When
+        // max |E_ij| >= 1e-3 the exact FP64 inverse below is used instead.
+        __shared__ unsigned int emax_e;
+        // E goes to the Sd region (pair residual; S stays in Sf) or, with the FP64
+        // residual, which reads S from Sd, over S in Sf
+        float *Ef = factored ? reinterpret_cast<float *>(Sd) : Sf;
+        if (threadIdx.x == 0) emax_e = 0u;
+        for (int i = threadIdx.x >> 5; i < M; i += blockDim.x >> 5)
+            for (int j = threadIdx.x & 31; j < M; j += 32) {
+                if (factored) {
+                    if (j < i) Ef[i * lda + j] = 0.f;
+                } else {
+                    Sd[i * lda + j] = (j >= i) ? double(Sf[i * lda + j]) : 0.0;
                 }
-            __syncthreads();
-            unsigned int my = 0u;
-            auto put_e = [&](int i, int j, float ef) {
-                Ef[i * lda + j] = ef;
-                const unsigned int bits = __float_as_uint(fabsf(ef));
-                my = bits > my ? bits : my;
-            };
-            if (factored) {
-                tri_residual_df(Sff, Rf, lda, M, put_e);
-            } else {
-                tri_mm_upper<double>(
-                    M, [&](int i, int k) { return -Sd[i * lda + k]; }, [&](int k, int j) { return A[k * lda + j]; },
-                    [](int i, int j) { return i == j ? 1.0 : 0.0; },
-                    [&](int i, int j, double e) { put_e(i, j, float(e)); });
             }
-            atomicMax(&emax_e, my);
-            __syncthreads();
-            if (__uint_as_float(emax_e) < 1e-3f) {
-                auto ef = [&](int k, int j) { return Ef[k * lda + j]; };
-                auto zero = [](int, int) { return 0.f; };
-                for (int i = threadIdx.x >> 5; i < M; i += blockDim.x >> 5)
-                    for (int j = threadIdx.x & 31; j < M; j += 32) {
-                        if (j < i) C1[i * lda + j] = 0.f;
-                    }
-                tri_mm_upper<float>(M, [&](int i, int k) { return Rf[i * lda + k]; }, ef, zero,
-                                    [&](int i, int j, float c) { C1[i * lda + j] = c; });
-                __syncthreads();
-                tri_mm_upper<float>(M, [&](int i, int k) { return C1[i * lda + k]; }, ef, zero,
-                                    [&](int i, int j, float c2) { A[i * lda + j] += double(C1[i * lda + j] + c2); });
-                __syncthreads();
-            } else {
-                exact = true;
-                for (int i = threadIdx.x >> 5; i < M; i += blockDim.x >> 5)
-                    for (int j = threadIdx.x & 31; j < M; j += 32) {
-                        A[i * lda + j] = factored ? ((j >= i) ? double(Sff[i * lda + j]) : 0.0) : Sd[i * lda + j];
-                    }
-                __syncthreads();
-            }
+        __syncthreads();
+        unsigned int my = 0u;
+        auto put_e = [&](int i, int j, float ef) {
+            Ef[i * lda + j] = ef;
+            const unsigned int bits = __float_as_uint(fabsf(ef));
+            my = bits > my ? bits : my;
+        };
+        if (factored) {
+            tri_residual_df(Sf, Rf, lda, M, put_e);
         } else {
+            tri_mm_upper<double>(
+                M, [&](int i, int k) { return -Sd[i * lda + k]; }, [&](int k, int j) { return A[k * lda + j]; },
+                [](int i, int j) { return i == j ? 1.0 : 0.0; },
+                [&](int i, int j, double e) { put_e(i, j, float(e)); });
+        }
+        atomicMax(&emax_e, my);
+        __syncthreads();
+        if (__uint_as_float(emax_e) < 1e-3f) {
+            auto ef = [&](int k, int j) { return Ef[k * lda + j]; };
+            auto zero = [](int, int) { return 0.f; };
             for (int i = threadIdx.x >> 5; i < M; i += blockDim.x >> 5)
                 for (int j = threadIdx.x & 31; j < M; j += 32) {
-                    A[i * lda + j] = (j >= i) ? double(Sf[i * lda + j]) : 0.0;
+                    if (j < i) C1[i * lda + j] = 0.f;
+                }
+            tri_mm_upper<float>(M, [&](int i, int k) { return Rf[i * lda + k]; }, ef, zero,
+                                [&](int i, int j, float c) { C1[i * lda + j] = c; });
+            __syncthreads();
+            tri_mm_upper<float>(M, [&](int i, int k) { return C1[i * lda + k]; }, ef, zero,
+                                [&](int i, int j, float c2) { A[i * lda + j] += double(C1[i * lda + j] + c2); });
+            __syncthreads();
+        } else {
+            exact = true;
+            for (int i = threadIdx.x >> 5; i < M; i += blockDim.x >> 5)
+                for (int j = threadIdx.x & 31; j < M; j += 32) {
+                    A[i * lda + j] = factored ? ((j >= i) ? double(Sf[i * lda + j]) : 0.0) : Sd[i * lda + j];
                 }
             __syncthreads();
         }
-        if (exact) tri_inv_upper_inplace<double>(A, lda, M, t);
+    } else {
+        for (int i = threadIdx.x >> 5; i < M; i += blockDim.x >> 5)
+            for (int j = threadIdx.x & 31; j < M; j += 32) {
+                A[i * lda + j] = (j >= i) ? double(Sf[i * lda + j]) : 0.0;
+            }
+        __syncthreads();
     }
-    // (FP64 basis: the inverse is applied in FP64, R needs no correction)
+    if (exact) tri_inv_upper_inplace<double>(A, lda, M, t);
     if (pass == 1) {
         for (int i = threadIdx.x >> 5; i < M; i += blockDim.x >> 5)
             for (int j = threadIdx.x & 31; j < M; j += 32) {
@@ -660,13 +634,13 @@ __global__ void __launch_bounds__(256) k_chol_ordered(const double *G, int M, in
             for (int j = threadIdx.x & 31; j < W; j += 32) {
                 if (i < M && j < M && j >= i) continue;
                 if (i < M && j < M) Hs[i * M + j] = 0.0;
-                Bout[j * W + i] = T(0);
+                Bout[j * W + i] = 0.f;
             }
         tri_mm_upper<double>(
             M, [&](int i, int k) { return A[i * lda + k]; }, [&](int k, int j) { return __ldg(R1 + k * M + j); },
             [](int, int) { return 0.0; },
             [&](int i, int j, double h) {
-                const T ht = T(h);
+                const float ht = float(h);
                 Hs[i * M + j] = double(ht);
                 Bout[j * W + i] = ht;
             });
@@ -679,24 +653,22 @@ int launch_chol_ordered(const double *G, int M, int W, int pass, int step, doubl
                 double piv_rel2, double *R1, float *Rinv, double *Hs, float *Bout, Ctrl *ctrl,
                 cudaStream_t s) {
     auto bytes_for = [](int m) {
-        const bool newton = sizeof(float) == 4 && m <= CHOL_NEWTON_MAX;
+        const bool newton = m <= CHOL_NEWTON_MAX;
         return sizeof(double) * size_t(m) * (m + 1) + sizeof(float) * (size_t(m) * (m + 1) + 2) +
                sizeof(double) * size_t(3 * m + 2) +
                (newton ? (sizeof(double) + 2 * sizeof(float)) * size_t(m) * (m + 1) : 0) +
                sizeof(float) * size_t(tri_inv_tmp_elems(m));
     };
     const size_t smem = bytes_for(M);
-    // FP64 blocks are at most 64 wide; function-local static: set once, thread-safe
+    // function-local static: set once, thread-safe
     static const cudaError_t attr = cudaFuncSetAttribute(
-        k_chol_ordered<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes_for(sizeof(float) == 8 ? 64 : 128)));
+        k_chol_ordered, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes_for(128)));
     (void)attr;
     prof_begin(KernelClass::SMALL, s);
-    k_chol_ordered<float><<<1, 256, smem, s>>>(G, M, W, pass, step, inv_thresh2, piv_rel2, R1, Rinv, Hs,
-                                   Bout, ctrl);
+    k_chol_ordered<<<1, 256, smem, s>>>(G, M, W, pass, step, inv_thresh2, piv_rel2, R1, Rinv, Hs, Bout, ctrl);
     KB_CUDA_TRY(cudaGetLastError());
     prof_end(KernelClass::SMALL, s, 0, 0);
     return 0;
 }
-
 
 }  // namespace kb

@@ -64,8 +64,7 @@ int launch_conv_check(const double *U, const double *Up, int M, const Ctrl *chk,
 // dst = src, with steps = 0 when src->from_check >= 0 (the final projected solve is then
 // skipped); launch_copy_check_u copies that check's U (buffers of per doubles) into U.
 int launch_ctrl_final(Ctrl *dst, const Ctrl *src, cudaStream_t s);
-int launch_copy_check_u(const double *Uc, int64_t per, double *U, int M, int m, const Ctrl *ctrl,
-                        cudaStream_t s);
+int launch_copy_check_u(const double *Uc, int64_t per, double *U, const Ctrl *ctrl, cudaStream_t s);
 template <typename T>
 int launch_scatter(T *block, int64_t ld, const int32_t *nodes, int M, int col0, T val, cudaStream_t s);
 int launch_marker(int32_t *marker, const int32_t *nodes, int M, cudaStream_t s);
@@ -104,9 +103,8 @@ int launch_tridiag_phi(int W, int M, int m, int gbl, const double *alpha, const 
                        double bound, cudaStream_t s, const std::vector<double> *series = nullptr);
 template <typename T>
 int launch_axpy_colnorm(int W, T *X, const T *P, const double *a, int64_t n, double *parts,
-                        int *grid_out, const Ctrl *ctrl, const int32_t *tgen, int limit,
-                        int64_t M_alg, cudaStream_t s, const int32_t *alist = nullptr,
-                        const int32_t *acount = nullptr);
+                        int *grid_out, const Ctrl *ctrl, int64_t M_alg, cudaStream_t s,
+                        const int32_t *alist = nullptr, const int32_t *acount = nullptr);
 int axpy_max_grid();
 template <typename T>
 int launch_assemble_diag(int W, const T *basis, int64_t stride, int nblk, const double *omega,

@@ -9,8 +9,9 @@
 //         reads/writes per product instead of 5).
 //   cheb2 Section 3.4.1: the interpolant of sqrt(phi) of degree floor(m/2) applied twice.
 //
-// Every step runs on the device; the host only enqueues work.  No host synchronisation
-// happens inside a solve (breakdown and early stops travel through a device control block).
+// Every step runs on the device; the host only enqueues work (breakdown and early stops travel
+// through a device control block).  It waits for the device in the middle of a solve only where
+// that has a stopping rule and reports to the caller (CheckWatch).
 #include "kb_internal.cuh"
 #include "kb_kernels.cuh"
 
@@ -660,7 +661,7 @@ int run_cbl(Common &c, const int32_t *nodes, int M, int m, float *Y, int64_t ldy
             KB_TRY(launch_bt_spline(b.Hd, b.Hs, M, m, c.p.eps, c.s_int, sbufs, b.U, b.ctrl, cfin, c.s, c.quad,
                                     b.qscr, qbatch, std::min(kfac, kend), 0, kend));
         }
-        if (c.p.tol > 0.0) KB_TRY(launch_copy_check_u(b.Uc, int64_t(m) * M * M, b.U, M, m, b.ctrl, c.s));
+        if (c.p.tol > 0.0) KB_TRY(launch_copy_check_u(b.Uc, int64_t(m) * M * M, b.U, b.ctrl, c.s));
         KB_TRY(launch_check_projected(b.U, int64_t(m) * M * M, projected_bound(c), b.ctrl, c.s));
         KB_TRY(launch_u_convert<C>(b.U, M, W, m, b.Ut, b.ctrl, c.s));
         // assembly: Y = [Q_1 .. Q_m] U
@@ -843,7 +844,7 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
             if (k == m) break;
             int grid2 = 0;
             KB_TRY(launch_axpy_colnorm<T>(W, X, Pk, b.aupd + int64_t(k - 1) * W, n, b.parts, &grid2,
-                                          b.ctrl, tg, k, M, c.s, tg ? b.fr.list(k) : nullptr, tg ? b.fr.count(k) : nullptr));
+                                          b.ctrl, M, c.s, tg ? b.fr.list(k) : nullptr, tg ? b.fr.count(k) : nullptr));
             KB_TRY(launch_lanczos_beta(b.parts, grid2, W, M, gbl ? 1 : 0, k - 1, f64 ? 0 : 1, thresh, b.beta,
                                        b.sigma, b.alive, b.c1 + int64_t(k) * W, b.c2 + int64_t(k) * W,
                                        b.ctrl, c.s));
@@ -881,7 +882,7 @@ int run_lanczos_scalar(Common &c, bool gbl, const int32_t *nodes, int M, int m, 
                 ++c.spmm;
                 int grid2 = 0;
                 KB_TRY(launch_axpy_colnorm<T>(W, X, Pk, b.aupd + int64_t(k - 1) * W, n, b.parts, &grid2,
-                                              b.ctrl2, tg, k, M, c.s, tg ? b.fr.list(k) : nullptr, tg ? b.fr.count(k) : nullptr));
+                                              b.ctrl2, M, c.s, tg ? b.fr.list(k) : nullptr, tg ? b.fr.count(k) : nullptr));
                 KB_TRY(launch_assemble_diag<T>(W, X, bs, 1, b.omega + int64_t(k) * W, n, Y, ldy, M, M,
                                                tg, b.ctrl, c.s, k, 1));
             }

@@ -494,7 +494,6 @@ __global__ void __launch_bounds__(TRI_THREADS) k_tridiag_phi(int W, int M, int m
 template <typename T, int W>
 __global__ void __launch_bounds__(256) k_axpy_colnorm(T *X, const T *P, const double *a, int64_t n,
                                                        double *parts, const Ctrl *ctrl,
-                                                       const int32_t *tgen, int limit,
                                                        const int32_t *alist, const int32_t *acount,
                                                        ProfCount pc) {
     pdl_wait();
@@ -513,7 +512,7 @@ __global__ void __launch_bounds__(256) k_axpy_colnorm(T *X, const T *P, const do
     }
     C acc[4] = {0, 0, 0, 0};
     unsigned long long my_rows = 0;
-    if (alist && tgen) {
+    if (alist) {
         // active 32-row tiles only: RPP rows per pass
         const int cnt = *acount;
         for (int it = blockIdx.x; it < cnt; it += gridDim.x) {
@@ -537,22 +536,19 @@ __global__ void __launch_bounds__(256) k_axpy_colnorm(T *X, const T *P, const do
     }
     // two rows per iteration, 16-byte vector accesses: four loads in flight per thread
     const int64_t stride = int64_t(gridDim.x) * RPP;
-    for (int64_t row = int64_t(blockIdx.x) * RPP + rr; !(alist && tgen) && row < n; row += 2 * stride) {
+    for (int64_t row = int64_t(blockIdx.x) * RPP + rr; !alist && row < n; row += 2 * stride) {
         const int64_t row2 = row + stride;
-        const bool act0 = !tgen || __ldg(tgen + row / ACT_ROWS) <= limit;
-        const bool act1 = row2 < n && (!tgen || __ldg(tgen + row2 / ACT_ROWS) <= limit);
+        const bool second = row2 < n;
         C xv[2][4], pv[2][4];
-        if (act0) {
-            ldv4(X + row * W + c4, xv[0]);
-            ldv4(P + row * W + c4, pv[0]);
-        }
-        if (act1) {
+        ldv4(X + row * W + c4, xv[0]);
+        ldv4(P + row * W + c4, pv[0]);
+        if (second) {
             ldv4(X + row2 * W + c4, xv[1]);
             ldv4(P + row2 * W + c4, pv[1]);
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            if (!(h ? act1 : act0)) continue;
+            if (h && !second) continue;
             if (cg == 0) ++my_rows;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -732,10 +728,9 @@ __global__ void k_ctrl_final(Ctrl *dst, const Ctrl *src) {
     if (c.from_check >= 0) c.steps = 0;
     *dst = c;
 }
-__global__ void k_copy_check_u(const double *Uc, int64_t per, double *U, int M, const Ctrl *ctrl) {
+__global__ void k_copy_check_u(const double *Uc, int64_t per, double *U, const Ctrl *ctrl) {
     const int b = ctrl->from_check;
     if (b < 0) return;
-    (void)M;
     const int64_t cnt = per;   // the check zeroed its whole buffer: copy it all
     for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < cnt; i += int64_t(gridDim.x) * blockDim.x)
         U[i] = Uc[b * per + i];
@@ -746,10 +741,9 @@ int launch_ctrl_final(Ctrl *dst, const Ctrl *src, cudaStream_t s) {
     KB_CUDA_TRY(cudaGetLastError());
     return 0;
 }
-int launch_copy_check_u(const double *Uc, int64_t per, double *U, int M, int m, const Ctrl *ctrl,
-                        cudaStream_t s) {
-    const int grid = int(std::max<int64_t>(1, std::min<int64_t>((int64_t(m) * M * M + 255) / 256, 4 * int64_t(num_sms()))));
-    k_copy_check_u<<<grid, 256, 0, s>>>(Uc, per, U, M, ctrl);
+int launch_copy_check_u(const double *Uc, int64_t per, double *U, const Ctrl *ctrl, cudaStream_t s) {
+    const int grid = int(std::max<int64_t>(1, std::min<int64_t>((per + 255) / 256, 4 * int64_t(num_sms()))));
+    k_copy_check_u<<<grid, 256, 0, s>>>(Uc, per, U, ctrl);
     count_launches(1);
     KB_CUDA_TRY(cudaGetLastError());
     return 0;
@@ -875,18 +869,18 @@ int launch_tridiag_phi(int W, int M, int m, int gbl, const double *alpha, const 
 
 template <typename T>
 int launch_axpy_colnorm(int W, T *X, const T *P, const double *a, int64_t n, double *parts,
-                        int *grid_out, const Ctrl *ctrl, const int32_t *tgen, int limit,
-                        int64_t M_alg, cudaStream_t s, const int32_t *alist, const int32_t *acount) {
+                        int *grid_out, const Ctrl *ctrl, int64_t M_alg, cudaStream_t s,
+                        const int32_t *alist, const int32_t *acount) {
     const int rpp = 256 / (W / 4);
     const int grid = int(std::min<int64_t>((n + rpp - 1) / rpp, int64_t(num_sms()) * 4));
     *grid_out = std::max(grid, 1);
     const ProfCount pc = prof_begin(KernelClass::ROWBLOCK, s);
     cudaError_t err = cudaSuccess;
     switch (W) {
-        case 16: err = launch_dep(k_axpy_colnorm<T, 16>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
-        case 32: err = launch_dep(k_axpy_colnorm<T, 32>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
-        case 64: err = launch_dep(k_axpy_colnorm<T, 64>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
-        case 128: err = launch_dep(k_axpy_colnorm<T, 128>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, tgen, limit, alist, acount, pc); break;
+        case 16: err = launch_dep(k_axpy_colnorm<T, 16>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, alist, acount, pc); break;
+        case 32: err = launch_dep(k_axpy_colnorm<T, 32>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, alist, acount, pc); break;
+        case 64: err = launch_dep(k_axpy_colnorm<T, 64>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, alist, acount, pc); break;
+        case 128: err = launch_dep(k_axpy_colnorm<T, 128>, dim3(*grid_out), 256, 0, s, 0, X, P, a, n, parts, ctrl, alist, acount, pc); break;
         default: return fail(KB_ERR_ARG, "bad width");
     }
     KB_CUDA_TRY(err);
@@ -944,7 +938,7 @@ int launch_u_convert(const double *U, int M, int W, int m, T *Ut, const Ctrl *ct
     template int launch_scale_copy<T>(T *, const T *, int64_t, int, double, const int32_t *,    \
                                       const int32_t *, cudaStream_t);                           \
     template int launch_axpy_colnorm<T>(int, T *, const T *, const double *, int64_t, double *,  \
-                                        int *, const Ctrl *, const int32_t *, int, int64_t,     \
+                                        int *, const Ctrl *, int64_t,                           \
                                         cudaStream_t, const int32_t *, const int32_t *);        \
     template int launch_assemble_diag<T>(int, const T *, int64_t, int, const double *, int64_t, \
                                          float *, int64_t, int, int64_t, const int32_t *,       \
@@ -960,7 +954,7 @@ template int launch_scale_copy<__nv_bfloat16>(__nv_bfloat16 *, const __nv_bfloat
                                               double, const int32_t *, const int32_t *, cudaStream_t);
 template int launch_axpy_colnorm<__nv_bfloat16>(int, __nv_bfloat16 *, const __nv_bfloat16 *,
                                                 const double *, int64_t, double *, int *,
-                                                const Ctrl *, const int32_t *, int, int64_t,
+                                                const Ctrl *, int64_t,
                                                 cudaStream_t, const int32_t *, const int32_t *);
 template int launch_assemble_diag<__nv_bfloat16>(int, const __nv_bfloat16 *, int64_t, int,
                                                  const double *, int64_t, float *, int64_t, int,
