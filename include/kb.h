@@ -20,8 +20,10 @@
  *   - Device pointers are plain CUDA device addresses of the current device; host
  *     pointers are ordinary host memory.  `stream` is a cudaStream_t passed as void*
  *     (NULL = the legacy default stream).
- *   - All GPU work of a call is enqueued on `stream`.  A call returns without waiting for
- *     the GPU unless it is documented to synchronise.
+ *   - All GPU work of a call is ordered by `stream`: what a call runs beside it on a stream of
+ *     its own waits for `stream` first, and `stream` waits for it before the result and the
+ *     scratch are complete.  A call returns without waiting for the GPU unless it is documented
+ *     to synchronise.
  *   - The library never frees memory it does not own and never keeps a caller pointer
  *     beyond the call.
  */
@@ -174,7 +176,7 @@ int kb_graph_lambda_bounds(const kb_graph *g, double *gershgorin, double *projec
  *           degree floor(m/2) interpolant of sqrt(phi).
  *   Y       device, n x M float32, row-major with leading dimension M (Y[i*M + j] is
  *           entry (node i, column j)); written completely; caller-owned.
- *   stream  all work is enqueued here; scratch memory is taken from and returned to the
+ *   stream  all work is ordered by this stream; scratch memory is taken from and returned to the
  *           device's stream-ordered memory pool on this stream.
  *   info    NULL, or receives facts about the run.  When non-NULL the call synchronises
  *           `stream` and returns KB_ERR_BREAKDOWN if the Lanczos process met a

@@ -276,8 +276,8 @@ __global__ void __launch_bounds__(CHOL_THREADS) k_chol(const double *G, int M, i
             Bout[j * W + i] = T(0);
         });
         __syncthreads();
-        // R1 over the second region where it fits beside A (FP64 mode, and FP32 up to M = 96), else
-        // over the product's own loads from global memory
+        // R1 over the second region where it fits beside A (FP64 mode; FP32 up to M = 8, whose second
+        // region is sized for floats), else over the product's own loads from global memory
         double *R = reinterpret_cast<double *>(smem + L.second);
         if (L.second + size_t(lda) * ((M + 1) / 2 * 2) * sizeof(double) <= L.scr) {
             sm::load_square(R1, M, M, [&](int i, int j, double v) { R[i * lda + j] = j >= i ? v : 0.0; });

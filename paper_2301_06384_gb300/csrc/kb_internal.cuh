@@ -256,8 +256,8 @@ struct LinEpi {
                                       // are written as zeros, without their gathers
     int limit = 0;                    // process tiles with tgen <= limit
     int zero_inactive = 0;            // write zeros on the tiles beyond the limit (final output)
-    const int32_t *alist = nullptr;   // with tgen: the tiles by rising hop distance and the number
-    const int32_t *acount = nullptr;  // of them within the limit (device)
+    const int32_t *alist = nullptr;   // with tgen: the tiles within the limit (in index order; all tiles by
+    const int32_t *acount = nullptr;  // rising hop distance with zero_inactive), their number (device)
     int one_group = 0;                // long rows too are summed by one lane group, in index order
     ProfCount prof;
 };
@@ -304,8 +304,8 @@ struct RowArgs {
     const Ctrl *ctrl = nullptr;
     const int32_t *tgen = nullptr;    // frontier tiles (nullptr: all rows)
     int limit = 0;                    // process tiles with tgen <= limit (ASM: all tiles)
-    const int32_t *alist = nullptr;   // the frontier tiles by rising hop distance and the number
-    const int32_t *acount = nullptr;  // of them within the limit (ASM walks all of them)
+    const int32_t *alist = nullptr;   // the frontier tiles within the limit in index order (ASM that writes
+    const int32_t *acount = nullptr;  // all of y: all tiles by rising hop distance) and their number
     int lim_a = INT32_MAX;            // UPD: qa / qb are zero (and not read) in tiles beyond these
     int lim_b = INT32_MAX;            // hop distances; ASM, ASMSUB: block k beyond kbase + k
     int tri_a = 0;                    // UPD: ca is lower triangular

@@ -178,7 +178,7 @@ int launch_rowblock(int mode, int W, const RowArgs<T> &a, cudaStream_t s, int *g
     const double mm = double(a.n) * fr;
     // algorithmic flops count the structure of the small matrices: a product with a
     // triangular factor (H_{k-1,k}, R^{-1}) is half of a general one, a Gram X^T X is
-    // symmetric (half); the kernels compute more than this (full products, full Gram)
+    // symmetric (half); the kernels compute little more (the blocks that meet the half, M rounded up to 4)
     switch (mode) {
         case RB_PROJ: bytes = 2 * blk; flops = mm; per_row = 2 * row; frow = fr; break;
         case RB_UPD:

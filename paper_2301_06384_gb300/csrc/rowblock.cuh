@@ -33,8 +33,13 @@
 // (one row group), a CTA's tiles by rising index from the step's list in index order, a fixed
 // number of CTAs per SM.  (Products have no freedom: a chain over k per entry.)
 //
-// Bound: the shared-memory data path (8 x 4 register tiles: 12 16-byte loads of 4 wavefronts
-// per 128 FMAs) for W >= 64, HBM below; the FP64 pipe in FP64.
+// Bound, W >= 64: latency between a stage's arrival, its shared loads and the FMAs that depend on
+// them at 16 warps per SM (M = 64: FMA pipe 47 to 58 % busy, no pipe saturated); 8 x 4 register tiles take 12 16-byte
+// loads of 4 wavefronts per 128 FMAs.  HBM below; the FP64 pipe in FP64.
+//
+// CTAs per SM, from the shared memory that the geometry takes: two of 256 threads at M = 37..64 and 121..128, one
+// at M = 33..36 (tiles of 224 rows) and 65..120 (two to five Gram row groups beside the tile); whole cbl
+// solves there, RGG of 3e5 rows, 12 steps, before -> now: M = 33 3.46 -> 1.87 ms, 72 11.2 -> 5.1, 112 17.1 -> 10.2.
 //
 // Measured (launch list, mean us of a solve's launches; before: synchronous staging, 4 x 4
 // tiles, all W columns, full Grams):                          PROJ     UPD  MULGRAM     MUL
@@ -813,7 +818,7 @@ int launch_r(const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
 template <typename T, int W, int MODE>
 int launch_mode(const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
     constexpr int R = sizeof(typename Cmp<T>::type) == 8 || W == 16 ? 4 : 8;
-    // Threads: two CTAs of 256 per SM, or four of 128 for the narrow blocks, whose tiles are
+    // Threads: CTAs of 256, two per SM where they fit, or four of 128 for the narrow blocks, whose tiles are
     // short of arithmetic between their barriers (128^3 grid, M = 32, 40 steps: 24.8 / 24.0 ms;
     // RGG of 10^6 rows, M = 64, where the taller tile shares the small matrix: 13.2 / 13.6 ms).
     constexpr int NT = sizeof(typename Cmp<T>::type) == 8 || MODE == RB_PROJ || W >= 64 ? 256 : 128;
