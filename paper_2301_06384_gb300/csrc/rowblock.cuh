@@ -55,6 +55,7 @@
 // sums held across the products, UPD at M = 64 took 113.4.
 #pragma once
 #include <algorithm>
+#include <atomic>
 #include <climits>
 #include <type_traits>
 
@@ -782,16 +783,22 @@ k_rowblock(RowArgs<T> a) {
 
 constexpr int RB_MAX_CTAS = 5;   // per SM
 
-// Resident CTAs per SM of an instance with smem bytes of dynamic shared memory.  The attribute
-// is raised once per instance to the most any block can take.
+// Resident CTAs per SM of an instance with the shared memory that blocks of M columns take.  The
+// runtime is asked once (several microseconds, and a solve needs it for every launch and for its plan);
+// devices are taken to be alike, as in num_sms().  The attribute is raised once per instance to the
+// most any block can take.
 template <typename T, int W, int MODE, int RPT, bool ORD, int NT>
-int occupancy(size_t smem) {
+int occupancy(int M, size_t smem) {
+    static std::atomic<int> known[W + 1];   // (zero: not asked yet)
+    if (const int v = known[M].load(std::memory_order_relaxed)) return v;
     static const cudaError_t attr = cudaFuncSetAttribute(
         k_rowblock<T, W, MODE, RPT, ORD, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     (void)attr;
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_rowblock<T, W, MODE, RPT, ORD, NT>, NT, smem);
-    return std::max(1, std::min(per_sm, RB_MAX_CTAS));
+    const int v = std::max(1, std::min(per_sm, RB_MAX_CTAS));
+    if (per_sm > 0) known[M].store(v, std::memory_order_relaxed);
+    return v;
 }
 
 template <typename T, int W, int MODE, int RPT, bool ORD, int NT>
@@ -801,7 +808,7 @@ int launch_r(const RowArgs<T> &a, cudaStream_t s, int *grid_out) {
     const size_t smem = smem_bytes<T, W, MODE, ORD>(q);
     const int64_t unit = ORD ? G::TO : MODE == RB_PROJ ? G::PR : q.TR;
     const int64_t nvt = (a.n + unit - 1) / unit;
-    const int per_sm = occupancy<T, W, MODE, RPT, ORD, NT>(smem);
+    const int per_sm = occupancy<T, W, MODE, RPT, ORD, NT>(a.M, smem);
     int grid = int(std::min<int64_t>(nvt, int64_t(num_sms()) * (ORD ? G::CTAS : per_sm)));
     if (MODE == RB_PROJ || MODE == RB_UPD || MODE == RB_MULGRAM || MODE == RB_ASMSUB) grid = std::min(grid, a.max_grid);
     if (grid < 1) grid = 1;
