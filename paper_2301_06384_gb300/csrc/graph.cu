@@ -215,7 +215,9 @@ extern "C" int kb_graph_create(int64_t n, const int32_t *rowptr, const int32_t *
                 }
         }
         // build the stored form
-        std::vector<int32_t> h_rowptr(n + 1);
+        std::vector<int32_t> h_rowptr;
+        h_rowptr.reserve(n + 2 + n / 64);   // (the long rows follow)
+        h_rowptr.resize(n + 1);
         std::vector<int32_t> h_col(noff);
         std::vector<float> h_w(unit ? 0 : noff);
         std::vector<float> h_rdiag(n);
@@ -247,10 +249,9 @@ extern "C" int kb_graph_create(int64_t n, const int32_t *rowptr, const int32_t *
             h_rdiag[i] = float(excess);
             if (h_rdiag[i] != 0.f) zero_excess = false;
         }
-        const int32_t long_row = long_row_degree(h_rowptr.data(), n);
         std::vector<int32_t> h_longs;
-        for (int64_t i = 0; i < n; ++i)
-            if (h_rowptr[i + 1] - h_rowptr[i] > long_row) h_longs.push_back(int32_t(i));
+        const int32_t long_row = long_row_degree(h_rowptr.data(), n, &h_longs);
+        h_rowptr.insert(h_rowptr.end(), h_longs.begin(), h_longs.end());   // (one upload)
         int dev = 0;
         KB_CUDA_TRY(cudaGetDevice(&dev));
         cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -259,19 +260,16 @@ extern "C" int kb_graph_create(int64_t n, const int32_t *rowptr, const int32_t *
         g->device = dev;
         auto cleanup = [&]() {
             cudaFree(g->d_rowptr); cudaFree(g->d_col); cudaFree(g->d_w); cudaFree(g->d_rdiag);
-            cudaFree(g->d_longs);
             delete g;
         };
-        cudaError_t e = cudaMalloc(&g->d_rowptr, sizeof(int32_t) * (n + 1));
+        cudaError_t e = cudaMalloc(&g->d_rowptr, sizeof(int32_t) * h_rowptr.size());
         if (e == cudaSuccess) e = cudaMalloc(&g->d_col, sizeof(int32_t) * std::max<int64_t>(noff, 1));
         if (e == cudaSuccess && !unit) e = cudaMalloc(&g->d_w, sizeof(float) * std::max<int64_t>(noff, 1));
         if (e == cudaSuccess && !zero_excess) e = cudaMalloc(&g->d_rdiag, sizeof(float) * n);
-        if (e == cudaSuccess && !h_longs.empty()) e = cudaMalloc(&g->d_longs, sizeof(int32_t) * h_longs.size());
-        if (e == cudaSuccess) e = cudaMemcpyAsync(g->d_rowptr, h_rowptr.data(), sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(g->d_rowptr, h_rowptr.data(), sizeof(int32_t) * h_rowptr.size(), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess && noff) e = cudaMemcpyAsync(g->d_col, h_col.data(), sizeof(int32_t) * noff, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess && !unit && noff) e = cudaMemcpyAsync(g->d_w, h_w.data(), sizeof(float) * noff, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess && !zero_excess) e = cudaMemcpyAsync(g->d_rdiag, h_rdiag.data(), sizeof(float) * n, cudaMemcpyHostToDevice, s);
-        if (e == cudaSuccess && !h_longs.empty()) e = cudaMemcpyAsync(g->d_longs, h_longs.data(), sizeof(int32_t) * h_longs.size(), cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) {
             cleanup();
@@ -279,7 +277,7 @@ extern "C" int kb_graph_create(int64_t n, const int32_t *rowptr, const int32_t *
         }
         g->dev.n = n;
         g->dev.nnz = noff;
-        g->dev.longs = g->d_longs;
+        g->dev.longs = g->d_rowptr + n + 1;
         g->dev.nlong = int32_t(h_longs.size());
         g->dev.long_row = long_row;
         g->dev.rowptr = g->d_rowptr;
@@ -329,7 +327,6 @@ extern "C" void kb_graph_destroy(kb_graph *g) {
     cudaFree(g->d_col);
     cudaFree(g->d_w);
     cudaFree(g->d_rdiag);
-    cudaFree(g->d_longs);
     delete g;
 }
 

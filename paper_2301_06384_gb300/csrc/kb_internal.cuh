@@ -39,11 +39,10 @@ struct GraphDev {
 
 struct kb_graph {
     kb::GraphDev dev;
-    int32_t *d_rowptr = nullptr;
+    int32_t *d_rowptr = nullptr;   // row pointers, then the long rows
     int32_t *d_col = nullptr;
     float *d_w = nullptr;
     float *d_rdiag = nullptr;
-    int32_t *d_longs = nullptr;
     double lambda = 0.0;     // Gershgorin bound
     double lambda_proj = 0.0;// spectral bound for the Lanczos projected step: the Gershgorin
                              // bound, or for a unit-weight D - A the smaller edge bound
@@ -265,8 +264,8 @@ struct LinEpi {
 // ldo <= 0: output is an internal n x W block; otherwise out has leading dimension ldo
 // and only columns < mo are written.  n_dense_in counts the dense inputs besides x
 // (y, z) for the algorithmic byte count.
-// Rows of more entries than this are the graph's long rows (rowptr on the host).
-int32_t long_row_degree(const int32_t *rowptr, int64_t n);
+// The graph's long rows, by index, and the number of entries that they all exceed (rowptr on the host).
+int32_t long_row_degree(const int32_t *rowptr, int64_t n, std::vector<int32_t> *rows);
 template <typename T>
 int launch_spmm(const GraphDev &g, int W, const T *x, const LinEpi<T> &e, cudaStream_t s,
                 int *grid_out, int64_t M_alg, int n_dense_in, int64_t ldo = 0, int mo = 0);

@@ -27,6 +27,7 @@
 // which gives L 1 = 0 exactly for D - A and drops the diagonal load for standard
 // Laplacians.  Epilogue coefficients arrive in FP64; in the FP32 path each is split into
 // a float pair (hi + lo) so that c * (L x) carries only the rounding of the final sum.
+#include <algorithm>
 #include <type_traits>
 
 #include "kb_internal.cuh"
@@ -572,13 +573,17 @@ int max_occupancy() {
 // row in 20 of 105 entries, 4e5 rows, column dots, M = 24: 2.54 and 2.30).  Between 64 and 256 as the
 // smallest length, preferential attachment of 4e5 rows, M = 64: 2.52 at 64, 2.65 at 128, 3.03 at 256;
 // at 32 2.77.
-int32_t long_row_degree(const int32_t *rowptr, int64_t n) {
+int32_t long_row_degree(const int32_t *rowptr, int64_t n, std::vector<int32_t> *rows) {
     int64_t t = std::max<int64_t>(64, 4 * int64_t(rowptr[n]) / n);
-    for (;; t *= 2) {
-        int64_t above = 0;
-        for (int64_t i = 0; i < n; ++i) above += rowptr[i + 1] - rowptr[i] > t;
-        if (above <= n / 64 || above <= 1) return int32_t(std::min<int64_t>(t, INT32_MAX));
+    rows->clear();
+    for (int64_t i = 0; i < n; ++i)
+        if (rowptr[i + 1] - rowptr[i] > t) rows->push_back(int32_t(i));
+    while (int64_t(rows->size()) > std::max<int64_t>(1, n / 64)) {
+        t *= 2;
+        rows->erase(std::remove_if(rows->begin(), rows->end(), [&](int32_t i) { return rowptr[i + 1] - rowptr[i] <= t; }),
+                    rows->end());
     }
+    return int32_t(std::min<int64_t>(t, INT32_MAX));
 }
 
 template <typename T>

@@ -28,11 +28,15 @@ def kb():
     ([3] * 10 + [70, 600], 233),                      # small: one long row at most (4 * 700 / 12)
 ])
 def test_rule_lists_few_rows(kb, degrees, line):
-    f = ctypes.CDLL(kb.LIB_PATH)["_ZN2kb15long_row_degreeEPKil"]
-    f.restype, f.argtypes = ctypes.c_int32, [ctypes.c_void_p, ctypes.c_int64]
+    f = ctypes.CDLL(kb.LIB_PATH)["_ZN2kb15long_row_degreeEPKilPSt6vectorIiSaIiEE"]
+    f.restype, f.argtypes = ctypes.c_int32, [ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
     ptr = np.concatenate([[0], np.cumsum(degrees)]).astype(np.int32)
-    assert f(ptr.ctypes.data, len(degrees)) == line
-    assert sum(d > line for d in degrees) <= max(1, len(degrees) // 64)
+    rows = (ctypes.c_void_p * 3)()   # an empty std::vector<int32_t>
+    assert f(ptr.ctypes.data, len(degrees), ctypes.addressof(rows)) == line
+    count = ((rows[1] or 0) - (rows[0] or 0)) // 4
+    got = list((ctypes.c_int32 * count).from_address(rows[0])) if count else []
+    assert got == [i for i, d in enumerate(degrees) if d > line]
+    assert count <= max(1, len(degrees) // 64)
 
 
 # rows of the hubs: the line itself (64: an ordinary row) and around it; one round of the 128 groups of 4
