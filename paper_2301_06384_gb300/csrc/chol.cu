@@ -34,7 +34,8 @@ namespace kb {
 //
 // Bound: latency of one CTA (smallmat.cuh).  Per launch, FP32, pass 1 and
 // pass 2 (us, launch list): 31 / 15 at M = 40, 17 / 9 at M = 16; with one barrier per column
-// and 4 x 4 tiles on few threads 69 / 19 and 43 / 11.  FP64, M = 33: 58 / 49, before 112 / 90.
+// and 4 x 4 tiles on few threads 69 / 19 and 43 / 11.  FP64, M = 33: 58 / 49, before 112 / 90.  (Pivot
+// reciprocals rounded to nearest add 1 us to pass 1 at M = 16, 3 us at M = 64.)
 constexpr int CHOL_THREADS = 512;
 constexpr int CORRECTED_MAX = 64;   // widest block whose R1 is the corrected FP32 factor
 
