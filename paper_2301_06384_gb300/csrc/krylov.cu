@@ -1259,6 +1259,9 @@ extern "C" int kb_workspace_bytes(kb_graph *g, kb_method method, kb_phi phi, con
         const float probe = 0.f;
         int rc = validate(g, method, phi, params, dummy.data(), M, m, &probe, &s_int);
         if (rc) return rc;
+        // (the plan asks for the occupancy of kernels, which sets their attributes: on the graph's device)
+        DeviceGuard dg;
+        KB_CUDA_TRY(dg.set(g->device));
         auto quad = std::make_unique<QuadRule>();
         rc = quad_setup(g, method, phi, *params, *quad);
         if (rc) return rc;
